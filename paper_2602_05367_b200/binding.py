@@ -1,5 +1,6 @@
-"""ctypes binding of the C ABI in include/rabit.h.  Marshalling only: every step of the layer
-runs inside the CUDA library."""
+"""Binding of the C ABI in include/rabit.h.  Marshalling only: every step of the layer runs inside the
+CUDA library.  The calls of a decoder's inner loop go through the native module _rabit_binding
+(csrc/rabit_binding.cpp: checks, output, stream and call in one), the others through ctypes."""
 from __future__ import annotations
 
 import ctypes
@@ -7,6 +8,7 @@ import os
 from typing import Optional, Tuple
 
 import numpy as np
+import torch                                   # (before the native module: it links against torch's libraries)
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 # RABIT_LIBRARY selects another build of the same library (e.g. librabit_trace.so, built with --trace)
@@ -83,6 +85,21 @@ def _load() -> ctypes.CDLL:
 
 _lib = _load()
 
+try:
+    from . import _rabit_binding as _native
+except ImportError as e:
+    raise ImportError(f"the native binding module is missing or does not load ({e}): build it with "
+                      "`python paper_2602_05367_b200/build.py`") from e
+_native.init(RabitError, *(ctypes.cast(getattr(_lib, name), _c_void_p).value for name in
+                           ("rabit_linear", "rabit_linear_group", "rabit_linear_group_host", "rabit_layer_M", "rabit_layer_N", "rabit_last_error")))
+
+
+def _stream_of(device, stream: Optional[int]) -> int:
+    """The stream argument as a handle: torch's current stream on `device` when it is None."""
+    if stream is not None:
+        return stream
+    return _native.current_stream(torch.cuda.current_device() if device.index is None else device.index)
+
 
 def lib_path() -> str:
     return _LIB_PATH
@@ -149,6 +166,7 @@ class RabitLayer:
 
     def __init__(self, handle: int, dev_buf, K: int, M: int, N: int):
         self._handle = _c_void_p(handle)
+        self._addr = handle             # the same as an integer, for the native module; None once freed
         self.dev_buf = dev_buf          # keeps the device memory alive
         self.K, self.M, self.N = K, M, N
         self._stage = None              # device staging buffer of rabit_linear_host
@@ -179,7 +197,7 @@ class RabitLayer:
     def free(self) -> None:
         if self._handle is not None:
             _lib.rabit_free(self._handle)
-            self._handle = None
+            self._handle = self._addr = None
             self.dev_buf = None
             self._stage = None
 
@@ -192,15 +210,13 @@ class RabitLayer:
 
 def rabit_pack(planes, g, h, device="cuda:0", stream: Optional[int] = None) -> RabitLayer:
     """Pack on the host, upload into a torch-allocated device buffer, return the layer."""
-    import torch
-
     planes, g16, h16, K, M, N = _host_arrays(planes, g, h)
     nbytes = packed_bytes(K, M, N)
     if nbytes == 0:
         raise RabitError(-2, f"unsupported shape K={K} M={M} N={N}")
     dev = torch.device(device)
     buf = torch.empty(nbytes, dtype=torch.uint8, device=dev)
-    st = torch.cuda.current_stream(dev).cuda_stream if stream is None else stream
+    st = _stream_of(dev, stream)
     out = _c_void_p()
     with torch.cuda.device(dev):
         _check(_lib.rabit_pack(planes.ctypes.data, g16.ctypes.data, h16.ctypes.data, K, M, N,
@@ -211,8 +227,6 @@ def rabit_pack(planes, g, h, device="cuda:0", stream: Optional[int] = None) -> R
 def rabit_derive_pack(W, g, h, stream: Optional[int] = None) -> RabitLayer:
     """Derive the sign planes of every path from the CUDA float32 weight W [M][N] and the fp16 scales
     g [K][M], h [K][N] (host arrays) on the device, packed in place; returns the layer."""
-    import torch
-
     if W.dtype != torch.float32 or not W.is_cuda or not W.is_contiguous() or W.dim() != 2:
         raise ValueError("W must be a contiguous CUDA float32 matrix")
     g16 = np.ascontiguousarray(g, dtype=np.float16).view(np.uint16)
@@ -225,7 +239,7 @@ def rabit_derive_pack(W, g, h, stream: Optional[int] = None) -> RabitLayer:
     if nbytes == 0:
         raise RabitError(-2, f"unsupported shape K={K} M={M} N={N}")
     buf = torch.empty(nbytes, dtype=torch.uint8, device=W.device)
-    st = torch.cuda.current_stream(W.device).cuda_stream if stream is None else stream
+    st = _stream_of(W.device, stream)
     out = _c_void_p()
     with torch.cuda.device(W.device):
         _check(_lib.rabit_derive_pack(_c_void_p(W.data_ptr()), g16.ctypes.data, h16.ctypes.data, K, M, N,
@@ -235,50 +249,18 @@ def rabit_derive_pack(W, g, h, stream: Optional[int] = None) -> RabitLayer:
 
 def rabit_linear(layer: RabitLayer, x, y=None, stream: Optional[int] = None):
     """y[b] = layer(x[b]); x is a CUDA fp16 tensor [batch][N] (or [N]); returns y [batch][M]."""
-    import torch
-
-    if x.dtype != torch.float16 or not x.is_cuda or not x.is_contiguous():
-        raise ValueError("x must be a contiguous CUDA float16 tensor")
-    xb = x if x.dim() == 2 else x.view(1, -1)
-    if xb.shape[1] != layer.N:
-        raise ValueError(f"x has {xb.shape[1]} columns, layer expects {layer.N}")
-    batch = xb.shape[0]
-    if y is None:
-        y = torch.empty((batch, layer.M), dtype=torch.float16, device=x.device)
-    elif y.dtype != torch.float16 or not y.is_cuda or not y.is_contiguous() or y.numel() != batch * layer.M:
-        raise ValueError("y must be a contiguous CUDA float16 tensor of batch*M elements")
-    st = torch.cuda.current_stream(x.device).cuda_stream if stream is None else stream
-    _check(_lib.rabit_linear(layer.handle, _c_void_p(xb.data_ptr()), _c_void_p(y.data_ptr()), batch, _c_void_p(st)))
-    return y if x.dim() == 2 else y.view(-1)
+    return _native.linear(layer, x, y, stream)
 
 
 def rabit_linear_group(layers, xs, ys, stream: Optional[int] = None):
     """Independent layers in one launch: ys[l] = layers[l](xs[l]).  xs may repeat one tensor (projections
     that share their input).  All tensors are contiguous CUDA float16, [batch][N_l] and [batch][M_l]."""
-    import torch
-
-    n = len(layers)
-    if n < 1 or len(xs) != n or len(ys) != n:
-        raise ValueError("layers, xs and ys must have the same, non-zero length")
-    batch = 1 if xs[0].dim() == 1 else xs[0].shape[0]
-    for L, x, y in zip(layers, xs, ys):
-        if x.dtype != torch.float16 or not x.is_cuda or not x.is_contiguous() or x.numel() != batch * L.N:
-            raise ValueError("every x must be a contiguous CUDA float16 tensor of batch*N elements")
-        if y.dtype != torch.float16 or not y.is_cuda or not y.is_contiguous() or y.numel() != batch * L.M:
-            raise ValueError("every y must be a contiguous CUDA float16 tensor of batch*M elements")
-    st = torch.cuda.current_stream(xs[0].device).cuda_stream if stream is None else stream
-    h = (_c_void_p * n)(*[L.handle for L in layers])
-    xp = (_c_void_p * n)(*[x.data_ptr() for x in xs])
-    yp = (_c_void_p * n)(*[y.data_ptr() for y in ys])
-    _check(_lib.rabit_linear_group(h, xp, yp, n, batch, _c_void_p(st)))
-    return ys
+    return _native.linear_group(layers, xs, ys, stream)
 
 
 def rabit_linear_group_host(layers, xs_host, ys_host, stream: Optional[int] = None):
     """Host-buffer form of rabit_linear_group: CPU float16 tensors in and out (pinned for asynchronous copies);
     an input tensor that occurs several times is copied once.  Returns without synchronising."""
-    import torch
-
     n = len(layers)
     if n < 1 or len(xs_host) != n or len(ys_host) != n:
         raise ValueError("layers, xs_host and ys_host must have the same, non-zero length")
@@ -293,7 +275,7 @@ def rabit_linear_group_host(layers, xs_host, ys_host, stream: Optional[int] = No
     first = layers[0]
     if first._stage is None or first._stage.numel() < need:
         first._stage = torch.empty(need, dtype=torch.uint8, device=first.dev_buf.device)
-    st = torch.cuda.current_stream(first.dev_buf.device).cuda_stream if stream is None else stream
+    st = _stream_of(first.dev_buf.device, stream)
     xp = (_c_void_p * n)(*[x.data_ptr() for x in xs_host])
     yp = (_c_void_p * n)(*[y.data_ptr() for y in ys_host])
     _check(_lib.rabit_linear_group_host(h, xp, yp, n, batch, _c_void_p(first._stage.data_ptr()), need, _c_void_p(st)))
@@ -306,8 +288,6 @@ class PreparedGroupHost:
     without the per-call checks of rabit_linear_group_host.  Returns without synchronising."""
 
     def __init__(self, layers, xs_host, ys_host):
-        import torch
-
         n = len(layers)
         if n < 1 or len(xs_host) != n or len(ys_host) != n:
             raise ValueError("layers, xs_host and ys_host must have the same, non-zero length")
@@ -325,16 +305,12 @@ class PreparedGroupHost:
         self._n, self._batch = n, batch
         self._need = int(_lib.rabit_group_stage_bytes(self._h, n, batch))
         self._stage = torch.empty(self._need, dtype=torch.uint8, device=self._device)
-        self._stage_ptr = _c_void_p(self._stage.data_ptr())
+        self._call = (ctypes.addressof(self._h), ctypes.addressof(self._xp), ctypes.addressof(self._yp), n, batch,
+                      self._stage.data_ptr(), self._need, self._device.index)
         self.ys_host = ys_host
 
     def __call__(self, stream: Optional[int] = None):
-        if stream is None:
-            import torch
-            stream = torch.cuda.current_stream(self._device).cuda_stream
-        rc = _lib.rabit_linear_group_host(self._h, self._xp, self._yp, self._n, self._batch, self._stage_ptr, self._need, _c_void_p(stream))
-        if rc != 0:
-            _check(rc)
+        _native.group_host(self._call, stream)
         return self.ys_host
 
 
@@ -342,8 +318,6 @@ def rabit_linear_host(layer: RabitLayer, x_host, y_host, stream: Optional[int] =
     """Host-buffer form: x_host / y_host are CPU float16 tensors (pinned for asynchronous copies)
     of shape [batch][N] (or [N]) and [batch][M]; the copies and the kernel are enqueued on the
     stream and the call returns without synchronising."""
-    import torch
-
     if x_host.dtype != torch.float16 or x_host.is_cuda or not x_host.is_contiguous():
         raise ValueError("x_host must be a contiguous CPU float16 tensor")
     if y_host.dtype != torch.float16 or y_host.is_cuda or not y_host.is_contiguous():
@@ -354,7 +328,7 @@ def rabit_linear_host(layer: RabitLayer, x_host, y_host, stream: Optional[int] =
     need = int(_lib.rabit_stage_bytes(layer.handle, batch))
     if layer._stage is None or layer._stage.numel() < need:
         layer._stage = torch.empty(need, dtype=torch.uint8, device=layer.dev_buf.device)
-    st = torch.cuda.current_stream(layer.dev_buf.device).cuda_stream if stream is None else stream
+    st = _stream_of(layer.dev_buf.device, stream)
     _check(_lib.rabit_linear_host(layer.handle, _c_void_p(x_host.data_ptr()), _c_void_p(y_host.data_ptr()), batch,
                                   _c_void_p(layer._stage.data_ptr()), need, _c_void_p(st)))
     return y_host
@@ -364,8 +338,6 @@ def rabit_linear_static_scratch(layer: RabitLayer, x, y, stream: Optional[int] =
     """rabit_linear for batch 1..16 that keeps its reduction scratch in the library's own fixed
     4 MiB device array, so nothing is allocated for the call (the caller passes x and y).  All
     calls share that array: keep them on one stream."""
-    import torch
-
     if x.dtype != torch.float16 or not x.is_cuda or not x.is_contiguous():
         raise ValueError("x must be a contiguous CUDA float16 tensor")
     if y.dtype != torch.float16 or not y.is_cuda or not y.is_contiguous():
@@ -373,7 +345,7 @@ def rabit_linear_static_scratch(layer: RabitLayer, x, y, stream: Optional[int] =
     batch = 1 if x.dim() == 1 else x.shape[0]
     if x.numel() != batch * layer.N or y.numel() != batch * layer.M:
         raise ValueError("x / y sizes do not match the layer")
-    st = torch.cuda.current_stream(x.device).cuda_stream if stream is None else stream
+    st = _stream_of(x.device, stream)
     with torch.cuda.device(x.device):
         _check(_lib.rabit_linear_static_scratch(layer.handle, _c_void_p(x.data_ptr()), _c_void_p(y.data_ptr()), batch, _c_void_p(st)))
     return y
