@@ -167,9 +167,8 @@ extern "C" int rabit_linear(const rabit_layer* layer, const void* x, void* y, in
         const double packed_mb = (double)G.K * G.Mp * G.N / 8.0e6;
         if (rabit_gemv_lut_supports(*layer, batch)) {
             variant = 5;
-        } else if (batch <= 2 * RABIT_MAX_GEMV_BATCH && rabit_gemv_f16_supports(*layer, RABIT_MAX_GEMV_BATCH)) {
-            variant = 6;                    // 3..16 rows: one pass over the weights with the batch in the MMA's N dimension;
-                                            // 17..32: two passes, which measured faster than one GEMM launch on every shape tried
+        } else if (batch <= RABIT_MAX_GEMV_BATCH && rabit_gemv_f16_supports(*layer, RABIT_MAX_GEMV_BATCH)) {
+            variant = 6;                    // 3..16 rows: one pass over the weights with the batch in the MMA's N dimension
         } else if (batch <= 4 && packed_mb <= 8.0 && rabit_gemv_lut_supports(*layer, 1)) {
             variant = 5;                    // two passes of the table-driven kernel
         } else if (batch <= RABIT_MAX_GEMV_BATCH) {
@@ -217,13 +216,10 @@ extern "C" int rabit_linear(const rabit_layer* layer, const void* x, void* y, in
                                           batch - b0 >= rows ? rows : batch - b0, st);
             break;
         }
-        case 6:
-            if (!rabit_gemv_f16_supports(*layer, batch < RABIT_MAX_GEMV_BATCH ? batch : RABIT_MAX_GEMV_BATCH))
+        case 6:                             // beyond 16 rows the GEMM: one launch of it beats two passes on every shape measured
+            if (!rabit_gemv_f16_supports(*layer, batch < RABIT_MAX_GEMV_BATCH ? batch : RABIT_MAX_GEMV_BATCH))   // (14336 x 4096 at batch 32: 24 us against 39)
                 return rabit_fail(RABIT_INVALID_ARG, "rabit_linear: f16 tensor-core GEMV cannot run this layer");
-            e = cudaSuccess;
-            for (int b0 = 0; b0 < batch && e == cudaSuccess; b0 += RABIT_MAX_GEMV_BATCH)   // up to 16 batch rows share one pass over the weights
-                e = rabit_launch_gemv_f16(*layer, (const char*)x + (size_t)b0 * G.N * 2, (char*)y + (size_t)b0 * G.M * 2,
-                                          batch - b0 >= RABIT_MAX_GEMV_BATCH ? RABIT_MAX_GEMV_BATCH : batch - b0, st);
+            e = batch <= RABIT_MAX_GEMV_BATCH ? rabit_launch_gemv_f16(*layer, x, y, batch, st) : rabit_launch_gemm_tc(*layer, x, y, batch, st);
             break;
         default:
             e = rabit_launch_plain(*layer, x, y, batch, st);

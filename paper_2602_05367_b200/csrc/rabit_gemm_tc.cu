@@ -2,93 +2,100 @@
 //
 //   y[b][i] = sum_k g_k[i] * sum_j (B_k[i][j] * h_k[j]) * x[b][j]                       (Section 4.1, Eq. 2)
 //
-// For many activation rows the layer is a dense contraction.  Per path k the A operand is the
-// sign tile with the input scale folded in, A_k[i][j] = +-h_k[j]: an fp16 value with its sign
-// bit flipped by the weight bit, so the expansion is exact.  The B operand is x itself (fp16,
-// loaded by TMA, shared by all paths), products are exact in fp32 and accumulate in fp32 in
-// tensor memory; the epilogue applies g_k, adds the paths and rounds once to fp16.
+// For many activation rows the layer is a dense contraction.  Per path k the A operand is the sign tile with the input
+// scale folded in, A_k[i][j] = +-h_k[j]: an fp16 value with its sign bit flipped by the weight bit, so the expansion is
+// exact.  The B operand is x itself (fp16, loaded by TMA, shared by all paths), products are exact in fp32 and
+// accumulate in fp32 in tensor memory; the epilogue applies g_k, adds the paths and rounds once to fp16.
 //
-// One CTA per SM, persistent over output tiles of 128 weight rows x 256 batch rows:
-//   warp 0      producer: per 64-column step, one TMA tile of x (128B swizzle) plus bulk copies of
-//               the packed sign tiles and the h slices of that step, into a ring of up to 8 steps
-//   warp 1      allocates tensor memory, issues tcgen05.mma (M=128, N=256, K=16, kind::f16) for every
-//               path into that path's accumulator, commits stages back to the producer
-//   warps 2..9  expand packed signs to +-h fp16 in the canonical K-major 128B-swizzled layout (two A stages), then
-//               (same warps) read the accumulators with tcgen05.ld for the epilogue
-// Every wait is bounded; on a time-out the CTA sets the status word, skips the remaining waits,
-// frees its tensor memory and returns.
+// A lives in TENSOR MEMORY.  The expander warps write +-h straight from registers with tcgen05.st and the MMAs read it
+// there, so the expanded operand (16 bits per weight and path) crosses shared memory neither on its way in nor out.
+// Measured on B200: an M = 128, K = 16 MMA with N batch columns takes N/2 clocks all the way down to N = 16 (9.2) with A in
+// tensor memory, and stores to tensor memory from other warps do not slow it; with A in shared memory N/2 only down to
+// N = 128, then 32 + N/4 (its 4 KB through the shared-memory port).  Both figures need the issuing warp to be converged (one
+// elected lane of a uniform loop): from a divergent single thread an MMA costs 90 to 125 clocks of issue whatever its N.
 //
-// Two more forms of the same kernel:
-//   * split contraction: when a launch has fewer tiles than half the SMs, clusters of 2, 4 or 8 CTAs share the 64-column
-//     steps of one tile and add their partial results through distributed shared memory (fixed order, no atomics);
-//     tiles left over beyond whole waves of the persistent form are launched that way too;
-//   * DEQ: the expander forms the dequantised weight sum_k +-g_k h_k in fp16 and one contraction serves all paths
-//     (rabit_set_variant 4; half the tensor work, one fp16 rounding per partial product and weight).
+// Warps of a CTA:
+//   0      producer: per 64-column step the x rows by TMA (128-byte swizzle) into one ring, per eight steps the packed sign
+//          tiles and the h slices of every path by bulk copies into another; the first weights set off before the
+//          dependency wait.  (Few, large copies: with one per step and path, and x in boxes of 16 rows, this warp was
+//          what the CTA waited for: 28672 x 8192 at batch 512 390 us with boxes of 16 rows, 350 with two boxes a step.)
+//   1..3   warp 1 allocates tensor memory; each issues the MMAs of the units of one accumulator and commits units and stages
+//          back (a unit is a step of one path; one path uses two accumulators for alternate steps, added in the epilogue).
+//          One issuing warp took about 430 clocks per unit, mostly its own waits, where the four MMAs need 2 N.
+//   4..19  expanders: four warpgroups (three if there are three paths) take the units in turn; warp q of a group owns
+//          tensor-memory lanes 32q..32q+31, i.e. the row blocks p = 2q, 2q + 1 of a sign tile.  tcgen05.st.16x256b takes a
+//          warp's registers in the same arrangement in which the tile keeps them (lane (gq, tq): rows gq, gq + 8, four
+//          consecutive columns at 4 tq), so a word of the tile becomes two operand registers with one byte permute, one
+//          shift and one logic instruction each.  Then (same warps) the epilogue: tcgen05.ld, g_k, sum of the paths, fp16,
+//          store.
+//
+// Work.  One CTA per SM.  An output tile is 128 weight rows x N batch columns, N a multiple of 16 chosen for the call.
+// make_plan() picks between: whole tiles; tiles whose contraction is split over a cluster of 2, 4 or 8 CTAs that add their partial
+// results through distributed shared memory (fixed order, no atomics); and, for long batches, contiguous ranges of
+// 16-column groups in (row tile, group) order, one per SM, so that no last wave is left over.
+//
+// Every wait is bounded; on a time-out the CTA sets the status word, skips the remaining waits, frees its tensor memory
+// and returns.  DEQ (rabit_set_variant 4): the expander forms the dequantised weight sum_k +-g_k h_k in fp16 and one
+// contraction serves all paths (a K-th of the tensor work, one fp16 rounding per partial product and weight).
 #include <cuda.h>
 #include <cuda_fp16.h>
+
+#include <algorithm>
+#include <type_traits>
+#include <vector>
 
 #include "rabit_internal.h"
 
 namespace {
 
 constexpr int kTileM = 128;                 // weight rows per output tile
-// batch rows per output tile (MMA N) and paths: TB = 256 with up to 2 paths or TB = 128 with 3 (template parameters):
-// paths x TB accumulator columns must fit the 512 columns of tensor memory
 constexpr int kStepCols = 64;               // input columns per pipeline step (128 bytes of fp16: one swizzle row)
-// Expanded A tiles: double-buffered, or four stages where there is one tile per step (KA == 1, the dequantised form),
-// whose expander warps work as two groups on alternate steps.
-__host__ __device__ constexpr int a_stages(int ka) { return ka == 1 ? 4 : 2; }
-constexpr int kExpandWarps = 8;
-constexpr int kThreads = (2 + kExpandWarps) * 32;
+constexpr int kGroupCols = 16;              // batch columns come in groups of 16 (MMA N granularity)
+constexpr int kUnitCols = kStepCols / 2;    // tensor-memory columns of one expanded unit (128 rows x 64 columns of fp16)
+constexpr int kMaxStages = 8, kMaxUnits = 8;
+constexpr int kWSteps = 8;                  // steps per stage of the weight ring
+constexpr int kWTiles = 2 * kWSteps, kWBytes = kWTiles * (RABIT_TILE_BYTES + RABIT_TILE_COLS * 2);   // per path
+constexpr int kMaxWStages = 4;
+constexpr int kExpandGroups = 4;            // of four warps each
+constexpr int kExpandWarps = 4 * kExpandGroups;
+constexpr int kThreads = (4 + kExpandWarps) * 32;
 constexpr long long kWaitLimitCycles = 1LL << 31;
 
-// What the copy engine brings per 64-column step (deep ring: it hides the global-memory latency) ...
-template <int TB, int KP>
-struct __align__(1024) InStage {
-    __half x[TB * kStepCols];                         // 8..32 KB, swizzled by TMA
-    uint4 bits[KP][2][32];                            // packed sign tiles: 2 column tiles per step per path
-    __half h[KP][kStepCols];
-};
-// ... and what the expander warps make of it (two steps: one being multiplied, one being written).
-template <int KA>
-struct __align__(1024) AStage {
-    __half a[KA][kTileM * kStepCols];                 // 16 KB per expanded operand tile (one per path, or one in all), swizzled
-};
-
-// Input-ring depth: as many steps as fit beside the A ring in 222 KB, at most 8.
-template <int TB, int KP, int KA>
-struct GemmCfg {
-    static constexpr int kInBytes = (int)sizeof(InStage<TB, KP>);
-    static constexpr int kFit = (222 * 1024 - a_stages(KA) * (int)sizeof(AStage<KA>)) / kInBytes;
-    static constexpr int kStages = kFit > 8 ? 8 : kFit;
-};
-
-template <int TB, int KP, int KA>
-struct Smem {
-    AStage<KA> astage[a_stages(KA)];
-    InStage<TB, KP> stage[GemmCfg<TB, KP, KA>::kStages];
-    unsigned long long full[8];                       // TMA bytes landed (x, bits, h)
-    unsigned long long empty[8];                      // MMAs that read the input stage retired
-    unsigned long long a_ready[4];                    // expanders done (a_stages(KA) in use)
-    unsigned long long a_empty[4];                    // MMAs that read the A stage retired
-    unsigned long long acc_ready;                     // all MMAs of the tile retired
-    unsigned long long acc_empty;                     // epilogue has read the accumulators
-    uint32_t tmem_base;
-    int abort_flag;
-};
-
 struct GemmParams {
-    RabitGeom G;
     const unsigned char* bits;
     const __half* g;
     const __half* h;
     __half* y;
     unsigned int* status;
+    int M, N, Mp, n_ct;
     int batch;
-    int n_bt;                                         // batch tiles
-    int tile_lo, tile_hi;                             // this launch covers tiles tile_lo .. tile_hi - 1 of the n_rt * n_bt
-    int split;                                        // CTAs (one cluster) that share the contraction of one tile: 1, 2, 4 or 8
+    int n16;                                // groups of 16 batch columns
+    int n_tasks;                            // tasks of the grid: one per CTA, or one per cluster if split > 1
+    int chunks, chunk16;                    // > 0: a task is (row tile, chunk of chunk16 groups); 0: a contiguous range of groups
+    long long n_groups;                     // row tiles * n16
+    int max16;                              // most groups one pass can accumulate
+    int split;                              // CTAs (one cluster) that share the contraction of a task: 1, 2, 4 or 8
+    int stages, stage_bytes;                // x ring (stage_bytes: one stage)
+    int w_stages;                           // weight ring, behind the x ring: per stage the sign tiles [K][8][512], then h [K][256]
+    int box16;                              // groups of 16 batch columns per TMA box
+    int n_acc;                              // accumulators (and issuing warps)
+    int units, a_col;                       // expanded-unit ring in tensor memory: unit u % units at columns a_col + 32 * that
 };
+
+struct Control {                            // ahead of the ring in shared memory
+    unsigned long long full[kMaxStages];    // x of the stage landed
+    unsigned long long empty[kMaxStages];   // MMAs that read it retired
+    unsigned long long w_full[kMaxWStages]; // weights of the stage landed
+    unsigned long long w_empty[kMaxWStages];// every expander warp has read them
+    unsigned long long a_ready[kMaxUnits];  // unit expanded
+    unsigned long long a_empty[kMaxUnits];  // MMAs that read the unit retired
+    unsigned long long acc_ready;           // all MMAs of the pass retired
+    unsigned long long acc_empty;           // epilogue has read the accumulators
+    uint32_t tmem_base;
+    int abort_flag;
+};
+constexpr int kControlBytes = 1024;
+static_assert(sizeof(Control) <= kControlBytes, "control block");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(uint32_t bar, int count) {
@@ -103,6 +110,12 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {   // never blocks
+    uint32_t ok;
+    asm volatile("{ .reg .pred p; mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
                  : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
@@ -121,6 +134,11 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                  ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(bar) : "memory");
 }
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{ .reg .pred p; elect.sync _|p, 0xFFFFFFFF; selp.u32 %0, 1, 0, p; }" : "=r"(p));
+    return p != 0;
+}
 
 // Shared-memory operand descriptor: K-major tile whose rows are 128 bytes, 128-byte swizzle,
 // 8-row groups 1024 bytes apart; descriptor version 1.
@@ -132,31 +150,30 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t smem_addr) {
     d |= (uint64_t)2 << 61;                        // 128-byte swizzle
     return d;
 }
-// Instruction descriptor: D fp32, A and B fp16, both K-major, N = batch tile, M = 128.
+// Instruction descriptor: D fp32, A and B fp16, both K-major, N batch columns, M = 128.
 __device__ __forceinline__ uint32_t umma_idesc(int n) {
     return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
 }
-__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile("{ .reg .pred p; setp.ne.b32 p, %4, 0; tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p; }"
-                 ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+__device__ __forceinline__ void umma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile("{ .reg .pred p; setp.ne.b32 p, %4, 0; tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p; }"
+                 ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-                 "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+// (no memory clobber: only tcgen05.wait::st and the fences, which follow in program order, give these stores a meaning)
+__device__ __forceinline__ void tmem_st_16x256b_x2(uint32_t taddr, const uint32_t (&r)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.16x256b.x2.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]));
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
                  : "r"(taddr) : "memory");
 }
-
-// DEQ = false: one operand tile +-h_k and one accumulator per path (exact products, g_k applied in the epilogue).
-// DEQ = true:  one operand tile holding the dequantised weight sum_k +-g_k h_k rounded to fp16 and one accumulator:
-//              half the tensor-core work and half the shared-memory operand traffic, at the price of one fp16
-//              rounding per partial product and per weight (relative 2^-11 each).
+__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -171,323 +188,412 @@ __device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
 
-template <int TB, int KP, bool DEQ>
+// One role's walk through a ring: every `stride`-th slot, with the parity of the slot's current lap.  A ring is a multiple of
+// every stride in use, so a slot is met by the same warps in every lap and a warp that waits for a slot's barrier is
+// never two laps from it (the parity would not tell the two apart).
+struct Walk {
+    int slot;
+    uint32_t lap = 0;
+    __device__ __forceinline__ void step(int stride, int size) {
+        slot += stride;
+        if (slot >= size) { slot -= size; lap ^= 1u; }
+    }
+};
+
+// A task's passes: runs of groups inside one row tile, at most max16 groups each, cut evenly.
+struct Pass {
+    int rt, c16, n;                         // row tile, first group, groups
+};
+struct PassWalker {
+    long long g, g1;
+    __device__ PassWalker(const GemmParams& P, int task) {
+        if (P.chunks > 0) {
+            const int rt = task / P.chunks, c = (task - rt * P.chunks) * P.chunk16;
+            g = (long long)rt * P.n16 + c;
+            g1 = g + min(P.chunk16, P.n16 - c);
+        } else {
+            g = P.n_groups * task / P.n_tasks;
+            g1 = P.n_groups * (task + 1) / P.n_tasks;
+        }
+    }
+    __device__ bool next(const GemmParams& P, Pass& ps) {
+        if (g >= g1) return false;
+        ps.rt = (int)(g / P.n16);
+        ps.c16 = (int)(g - (long long)ps.rt * P.n16);
+        const int run = (int)min(g1 - g, (long long)(P.n16 - ps.c16));
+        const int pieces = (run + P.max16 - 1) / P.max16;
+        ps.n = (run + pieces - 1) / pieces;
+        g += ps.n;
+        return true;
+    }
+};
+
+// K paths; DEQ: see above.
+template <int K, bool DEQ>
 __global__ void __launch_bounds__(kThreads, 1)
-rabit_gemm_tc_kernel(const GemmParams P, const __grid_constant__ CUtensorMap x_map) {
-    constexpr int KA = DEQ ? 1 : KP;
-    using Stage = InStage<TB, KP>;
-    using Smem = Smem<TB, KP, KA>;
-    constexpr int kStages = GemmCfg<TB, KP, KA>::kStages;
-    constexpr int kAStages = a_stages(KA);
-    constexpr int kGroupWarps = DEQ ? kExpandWarps / 2 : kExpandWarps;   // expander warps that build one step's operand
-    constexpr int kTileB = TB;
-    constexpr int kMaxPaths = KP;
+rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtensorMap x_map) {
     extern __shared__ unsigned char smem_raw[];
-    // the swizzled operand tiles need 1024-byte alignment; the launch reserves the slack
-    Smem& S = *reinterpret_cast<Smem*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
-    const RabitGeom& G = P.G;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int K = G.K;
-    const int n_steps = (G.N + kStepCols - 1) / kStepCols;        // N % 32 == 0: the last step may hold one column tile only
+    // the swizzled x tiles need 1024-byte alignment; the launch reserves the slack
+    unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    Control& S = *reinterpret_cast<Control*>(smem);
+    unsigned char* ring = smem + kControlBytes;
+    unsigned char* w_ring = ring + P.stages * P.stage_bytes;
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
+    constexpr int n_ops = DEQ ? 1 : K;                            // operand units (and accumulators) per step
+    constexpr int n_groups = n_ops == 3 ? 3 : 4;                  // expander groups at work
+    const int stages = P.stages, w_stages = P.w_stages, units = P.units;
+    const int stage_bytes = P.stage_bytes, n_ct = P.n_ct;
+    const int n_steps = (P.N + kStepCols - 1) / kStepCols;        // N % 32 == 0: the last step may hold one column tile only
     volatile int* abort_flag = &S.abort_flag;
-    // Split contraction: the `split` CTAs of a cluster work on the same output tile, rank r taking the r-th part of
-    // the 64-column steps; their partial results meet through distributed shared memory at the end.  Each CTA
-    // then has exactly one tile.  split == 1 is the persistent form (a CTA walks tiles blockIdx.x, +gridDim.x, ...).
+    // Split contraction: the CTAs of a cluster work on the same task, rank r taking the r-th part of the steps; their
+    // partial results meet through distributed shared memory at the end (such a task is one pass).
     const int split = P.split;
     uint32_t crank = 0;
     if (split > 1) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
-    const int t_first = P.tile_lo + (split > 1 ? (int)blockIdx.x / split : (int)blockIdx.x);
-    const int t_stride = split > 1 ? P.tile_hi - P.tile_lo : (int)gridDim.x;
-    const int s_lo = split > 1 ? (int)((long long)n_steps * crank / split) : 0;
-    const int s_hi = split > 1 ? (int)((long long)n_steps * (crank + 1) / split) : n_steps;
+    const int task = split > 1 ? (int)blockIdx.x / split : (int)blockIdx.x;
+    const int s_lo = __shfl_sync(0xFFFFFFFFu, (int)((long long)n_steps * crank / split), 0);
+    const int s_hi = __shfl_sync(0xFFFFFFFFu, (int)((long long)n_steps * (crank + 1) / split), 0);
 
     if (tid == 0) {
-        for (int s = 0; s < kStages; ++s) {
+        for (int s = 0; s < stages; ++s) {
             mbar_init(smem_u32(&S.full[s]), 1);
-            mbar_init(smem_u32(&S.empty[s]), 1);
+            mbar_init(smem_u32(&S.empty[s]), n_ops);
         }
-        for (int s = 0; s < kAStages; ++s) {
-            mbar_init(smem_u32(&S.a_ready[s]), kGroupWarps);
-            mbar_init(smem_u32(&S.a_empty[s]), 1);
+        for (int s = 0; s < w_stages; ++s) {
+            mbar_init(smem_u32(&S.w_full[s]), 1);
+            mbar_init(smem_u32(&S.w_empty[s]), 4 * n_groups);
         }
-        mbar_init(smem_u32(&S.acc_ready), 1);
+        for (int u = 0; u < units; ++u) {
+            mbar_init(smem_u32(&S.a_ready[u]), 4);
+            mbar_init(smem_u32(&S.a_empty[u]), 1);
+        }
+        mbar_init(smem_u32(&S.acc_ready), P.n_acc);
         mbar_init(smem_u32(&S.acc_empty), kExpandWarps);
         S.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1) {                                            // one warp allocates all 512 columns of tensor memory
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.tmem_base)), "r"(512) : "memory");
+    __syncthreads();
+
+    const int n_w = (s_hi - s_lo + kWSteps - 1) / kWSteps;        // weight stages of a pass
+    // weight stage j of a pass over row tile rt into slot `slot` (these do not depend on the stream's past)
+    auto load_weights = [&](int rt, int j, int slot) {
+        const int ct0 = 2 * (s_lo + kWSteps * j), cts = min(kWTiles, min(2 * s_hi, n_ct) - ct0);
+        const uint32_t bar = smem_u32(&S.w_full[slot]), dst = smem_u32(w_ring + slot * (K * kWBytes));
+        mbar_expect_tx(bar, (uint32_t)(K * cts * (RABIT_TILE_BYTES + RABIT_TILE_COLS * 2)));
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            bulk_g2s(dst + k * kWTiles * RABIT_TILE_BYTES, P.bits + (((size_t)rt * K + k) * n_ct + ct0) * RABIT_TILE_BYTES, cts * RABIT_TILE_BYTES, bar);
+            bulk_g2s(dst + K * kWTiles * RABIT_TILE_BYTES + k * kWTiles * RABIT_TILE_COLS * 2, P.h + (size_t)k * P.N + (size_t)ct0 * RABIT_TILE_COLS,
+                     cts * RABIT_TILE_COLS * 2, bar);
+        }
+    };
+    // the weight stages of all passes in order; `next` starts one if its slot is free or becomes free
+    struct WeightFeed {
+        PassWalker w;
+        Pass ps;
+        int j, issued;
+        Walk at;
+        bool more;
+    };
+    WeightFeed feed{PassWalker(P, task), Pass{}, 0, 0, Walk{0}, false};
+    auto feed_next = [&](bool elected) {
+        if (feed.issued >= w_stages) mbar_wait(smem_u32(&S.w_empty[feed.at.slot]), feed.at.lap ^ 1u, abort_flag);
+        if (elected) load_weights(feed.ps.rt, feed.j, feed.at.slot);
+        __syncwarp();
+        ++feed.issued;
+        feed.at.step(1, w_stages);
+        if (++feed.j == n_w) { feed.j = 0; feed.more = feed.w.next(P, feed.ps); }
+    };
+    if (warp == 0) {
+        const bool elected = elect_one();
+        feed.more = feed.w.next(P, feed.ps);
+        while (feed.more && feed.issued < w_stages) feed_next(elected);
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // Tensor memory is taken only after the dependency wait: a CTA that held some while the kernel before it in the stream
+    // still had CTAs about to allocate would keep that kernel, and with it itself, waiting for good.
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&S.tmem_base)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    fence_before();
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem_base = S.tmem_base;
+    fence_after();
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const uint32_t tmem_base = __shfl_sync(0xFFFFFFFFu, S.tmem_base, 0);   // (one value per warp: the MMA operands then live in uniform registers)
 
     if (warp == 0) {
         // ===================================== producer =====================================
-        if (lane == 0) {
-            int it = 0;                                          // global step counter of this CTA
-            for (int t = t_first; t < P.tile_hi; t += t_stride) {
-                const int rt = t / P.n_bt, bt = t % P.n_bt;
-                for (int s = s_lo; s < s_hi; ++s, ++it) {
-                    const int slot = it % kStages;
-                    if (it >= kStages) mbar_wait(smem_u32(&S.empty[slot]), ((it / kStages) - 1) & 1, abort_flag);
-                    Stage& st = S.stage[slot];
-                    const int cts = min(2, G.n_ct - 2 * s);      // column tiles in this step
-                    const uint32_t bar = smem_u32(&S.full[slot]);
-                    const uint32_t bytes = (uint32_t)(kTileB * kStepCols * 2) + (uint32_t)K * cts * (RABIT_TILE_BYTES + RABIT_TILE_COLS * 2);
-                    mbar_expect_tx(bar, bytes);
-                    tma_load_2d(smem_u32(st.x), &x_map, s * kStepCols, bt * kTileB, bar);
-                    for (int k = 0; k < K; ++k) {
-                        bulk_g2s(smem_u32(&st.bits[k][0][0]), P.bits + rabit_tile_pos(G, rt, k, 2 * s) * RABIT_TILE_BYTES,
-                                 cts * RABIT_TILE_BYTES, bar);
-                        bulk_g2s(smem_u32(&st.h[k][0]), P.h + (size_t)k * G.N + (size_t)s * kStepCols, cts * RABIT_TILE_COLS * 2, bar);
-                    }
+        const bool elected = elect_one();
+        int it = 0, w_at = 0;                                    // steps and weight stages begun, over all passes
+        Walk at{0};
+        PassWalker w(P, task);
+        Pass ps;
+        while (w.next(P, ps)) {
+            const int boxes = (ps.n + P.box16 - 1) / P.box16;
+            for (int s = s_lo; s < s_hi; ++s, ++it) {
+                if ((s - s_lo) % kWSteps == 0) {
+                    ++w_at;                                      // two stages behind the ring's depth: never held up by the stage in use
+                    while (feed.more && feed.issued < w_at + w_stages - 2) feed_next(elected);
                 }
+                const uint32_t bar = smem_u32(&S.full[at.slot]), dst = smem_u32(ring + at.slot * stage_bytes);
+                if (it >= stages) mbar_wait(smem_u32(&S.empty[at.slot]), at.lap ^ 1u, abort_flag);
+                if (elected) {
+                    mbar_expect_tx(bar, (uint32_t)(boxes * P.box16 * (kGroupCols * kStepCols * 2)));
+                    for (int c = 0; c < boxes; ++c)
+                        tma_load_2d(dst + c * P.box16 * (kGroupCols * kStepCols * 2), &x_map, s * kStepCols, (ps.c16 + c * P.box16) * kGroupCols, bar);
+                }
+                __syncwarp();
+                at.step(1, stages);
             }
         }
-    } else if (warp == 1) {
-        // ===================================== MMA issuer =====================================
-        if (lane == 0) {
-            const uint32_t idesc = umma_idesc(kTileB);
-            int it = 0, tile_i = 0;
-            for (int t = t_first; t < P.tile_hi; t += t_stride, ++tile_i) {
-                if (tile_i > 0) mbar_wait(smem_u32(&S.acc_empty), (tile_i - 1) & 1, abort_flag);   // epilogue has drained the accumulators
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                for (int s = s_lo; s < s_hi; ++s, ++it) {
-                    const int slot = it % kStages, aslot = it % kAStages;
-                    mbar_wait(smem_u32(&S.full[slot]), (it / kStages) & 1, abort_flag);
-                    mbar_wait(smem_u32(&S.a_ready[aslot]), (it / kAStages) & 1, abort_flag);
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    Stage& st = S.stage[slot];
-                    const int ksub = min(2, G.n_ct - 2 * s) * 2;                                   // MMAs of K = 16 in this step (2 per column tile)
-                    const uint64_t bdesc = umma_desc(smem_u32(st.x));
-                    const int n_acc = DEQ ? 1 : K;
-                    for (int k = 0; k < n_acc; ++k) {
-                        const uint64_t adesc = umma_desc(smem_u32(S.astage[aslot].a[k]));
-                        for (int kk = 0; kk < ksub; ++kk)
-                            umma_f16(tmem_base + (uint32_t)k * kTileB, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), idesc,
-                                     (s > s_lo || kk > 0) ? 1u : 0u);
+    } else if (warp < 4) {
+        // ===================================== MMA issuers =====================================
+        // Warp 1 + m issues the units u = m, m + n_acc, ... into accumulator m.  (The whole warp walks the loop, one elected lane
+        // issues: see the header.)
+        auto issue_units = [&](auto acc) {
+            constexpr int m = decltype(acc)::value;
+            const int n_acc = P.n_acc;
+            const bool elected = elect_one();
+            int pass_i = 0, u = m, u_end = 0;
+            Walk uw{m}, xw{n_ops == 1 ? m : 0};                  // units and x stages of this accumulator
+            const int x_stride = n_ops == 1 ? n_acc : 1;
+            const uint32_t full0 = smem_u32(&S.full[0]), empty0 = smem_u32(&S.empty[0]), a_ready0 = smem_u32(&S.a_ready[0]), a_empty0 = smem_u32(&S.a_empty[0]);
+            const uint64_t bdesc0 = umma_desc(smem_u32(ring));
+            const uint32_t a0 = tmem_base + (uint32_t)P.a_col, d = tmem_base + (uint32_t)(m * P.max16 * kGroupCols);
+            PassWalker w(P, task);
+            Pass ps;
+            while (w.next(P, ps)) {
+                const uint32_t idesc = __shfl_sync(0xFFFFFFFFu, umma_idesc(ps.n * kGroupCols), 0);
+                if (pass_i > 0) mbar_wait(smem_u32(&S.acc_empty), (pass_i - 1) & 1, abort_flag);   // epilogue has drained the accumulators
+                ++pass_i;
+                const int u_short = (n_ct & 1) && s_hi == n_steps ? u_end + (s_hi - s_lo - 1) * n_ops : 0x7FFFFFFF;   // units from here on hold one column tile
+                u_end += (s_hi - s_lo) * n_ops;
+                uint32_t accumulate = 0u;
+                bool ready = mbar_test(a_ready0 + uw.slot * 8, uw.lap), x_ready = mbar_test(full0 + xw.slot * 8, xw.lap);
+                for (; u < u_end; u += n_acc) {
+                    const int us = uw.slot, slot = xw.slot;
+                    if (!x_ready) mbar_wait(full0 + slot * 8, xw.lap, abort_flag);
+                    if (!ready) mbar_wait(a_ready0 + us * 8, uw.lap, abort_flag);
+                    fence_after();
+                    uw.step(n_acc, units);
+                    xw.step(x_stride, stages);
+                    ready = mbar_test(a_ready0 + uw.slot * 8, uw.lap);                             // asked early, used next time round
+                    x_ready = mbar_test(full0 + xw.slot * 8, xw.lap);
+                    const uint64_t bdesc = bdesc0 + (uint64_t)((slot * stage_bytes) >> 4);
+                    const uint32_t a = a0 + us * kUnitCols;
+                    if (elected) {
+                        umma_f16_ts(d, a, bdesc, idesc, accumulate);
+                        umma_f16_ts(d, a + 8, bdesc + 2, idesc, 1u);
+                        if (u < u_short) {
+                            umma_f16_ts(d, a + 16, bdesc + 4, idesc, 1u);
+                            umma_f16_ts(d, a + 24, bdesc + 6, idesc, 1u);
+                        }
+                        umma_commit(a_empty0 + us * 8);
+                        umma_commit(empty0 + slot * 8);
                     }
-                    umma_commit(smem_u32(&S.empty[slot]));                                         // frees both stages when these MMAs retire
-                    umma_commit(smem_u32(&S.a_empty[aslot]));
+                    accumulate = 1u;
+                    __syncwarp();
                 }
-                umma_commit(smem_u32(&S.acc_ready));
+                if (elected) umma_commit(smem_u32(&S.acc_ready));
+                __syncwarp();
             }
-        }
-    } else {
+        };
+        if (warp == 1) issue_units(std::integral_constant<int, 0>{});
+        else if (warp == 2 && P.n_acc > 1) issue_units(std::integral_constant<int, 1>{});
+        else if (warp == 3 && P.n_acc > 2) issue_units(std::integral_constant<int, 2>{});
+    } else if (warp >= 4) {
         // ============================ expanders, then epilogue ============================
-        const int e = warp - 2;                               // 0..7
-        const int quarter = warp & 3;                         // tensor-memory lanes this warp may read: 32*quarter .. +31
-        const int col_half = e >> 2;                          // which half of the tile's batch columns this warp drains
-        // expander role of this thread, the same in every step: one packed word position per path
-        // (dequantised form: the warps are two groups that take alternate steps; a thread then covers both column tiles of its step)
-        const int grp = e >> 2;
-        // Exact form: warp e takes the words of packed lanes gq = e; its lanes spread over both column tiles, the two column
-        // halves, the four tq and the two row halves, so that one 8-byte store per lane covers two whole 128-byte rows of
-        // the swizzled tile.  An 8-byte store is served half a warp at a time: lanes 0..15 must fill ONE row (16 x 8 bytes,
-        // all 32 banks once), so the row half is chosen by lane bit 4 and the position in the row by bits 0..3 (with the
-        // row half in bit 0 every half warp wrote two half rows on the same banks: 25 M of 42 M wavefronts were conflicts).
-        // Dequantised form: a group has four warps, so warp e & 3 takes gq = 2*(e & 3) and 2*(e & 3) + 1 in turn.
-        const int x_ct2 = (lane >> 3) & 1;
-        const int x_a = 2 * ((lane >> 2) & 1) + (lane >> 4);
-        const int x_tq = lane & 3;
-        const int x_gq = DEQ ? 2 * (e & 3) : e;
-        const int x_l = 4 * x_gq + x_tq;
-        const int x_hoff = 32 * x_ct2 + 16 * (x_a >> 1) + 4 * x_tq;
-        const uint32_t x_aoff = (uint32_t)((x_gq + 8 * (x_a & 1)) * 128 + (((4 * x_ct2 + 2 * (x_a >> 1) + (x_tq >> 1)) ^ x_gq) << 4) + 8 * (x_tq & 1));
-        int it = 0, tile_i = 0;
-        for (int t = t_first; t < P.tile_hi; t += t_stride, ++tile_i) {
-            const int rt = t / P.n_bt, bt = t % P.n_bt;
-            __half2 g_rows[kMaxPaths][2][8];                  // DEQ: output scales of this thread's 2 x 8 rows, both halves alike
+        const int grp = (warp - 4) >> 2, q = warp & 3;        // tensor-memory lanes this warp may touch: 32q .. 32q + 31
+        const int gq = lane >> 2, tq = lane & 3;
+        const uint32_t lane_base = tmem_base + ((uint32_t)(32 * q) << 16);
+        const int shift = 6 - 2 * q;                          // bit p of a byte to its top: a shift by 7 - p, this for p = 2q + 1 and one more for p = 2q
+        const uint32_t w_full0 = smem_u32(&S.w_full[0]), w_empty0 = smem_u32(&S.w_empty[0]), a_ready0 = smem_u32(&S.a_ready[0]), a_empty0 = smem_u32(&S.a_empty[0]);
+        const uint32_t a0 = lane_base + (uint32_t)P.a_col;
+        Walk uw{grp}, ww{0};
+        int pass_i = 0, u0 = 0, u = grp;                      // u: this group's next unit, counted over all passes
+        PassWalker w(P, task);
+        Pass ps;
+        while (w.next(P, ps)) {
+            __half2 g_rows[DEQ ? K : 1][2][2];                 // DEQ: output scales of this thread's rows (row block, row half), both halves alike
             if (DEQ) {
 #pragma unroll
-                for (int k = 0; k < kMaxPaths; ++k)
+                for (int k = 0; k < K; ++k)
 #pragma unroll
-                    for (int gi = 0; gi < 2; ++gi)
+                    for (int pi = 0; pi < 2; ++pi)
 #pragma unroll
-                        for (int p = 0; p < 8; ++p) {
-                            const int r = rt * kTileM + 16 * p + x_gq + gi + 8 * (x_a & 1);
-                            g_rows[k][gi][p] = __half2half2((k < K && r < G.Mp) ? P.g[(size_t)k * G.Mp + r] : __float2half(0.f));
-                        }
+                        for (int rh = 0; rh < 2; ++rh)
+                            g_rows[k][pi][rh] = __half2half2(P.g[(size_t)k * P.Mp + ps.rt * kTileM + 32 * q + 16 * pi + gq + 8 * rh]);
             }
-            for (int s = s_lo; s < s_hi; ++s, ++it) {
-                if (DEQ && (it & 1) != grp) continue;                 // the other group's step
-                const int slot = it % kStages, aslot = it % kAStages;
-                mbar_wait(smem_u32(&S.full[slot]), (it / kStages) & 1, abort_flag);
-                if (it >= kAStages) mbar_wait(smem_u32(&S.a_empty[aslot]), ((it / kAStages) - 1) & 1, abort_flag);
-                Stage& st = S.stage[slot];
-                AStage<KA>& ast = S.astage[aslot];
-                const int cts = min(2, G.n_ct - 2 * s);
-                if (DEQ) {
-                    // dequantised operand: for each of this thread's 8 rows and 4 columns, sum_k +-g_k[row] h_k[col],
-                    // accumulated from the last (smallest) path to the first with one fused multiply-add per path
-#pragma unroll
-                    for (int gi = 0; gi < 2; ++gi) {
-                        const int gq = x_gq + gi, l = x_l + 4 * gi;
-                        uint32_t u01[kMaxPaths], u23[kMaxPaths];
-                        uint2 hv[kMaxPaths];
-#pragma unroll
-                        for (int k = 0; k < kMaxPaths; ++k) {
-                            uint32_t w = 0;
-                            hv[k] = make_uint2(0u, 0u);
-                            if (k < K && x_ct2 < cts) {
-                                w = reinterpret_cast<const uint32_t*>(&st.bits[k][x_ct2][l])[x_a];
-                                hv[k] = *reinterpret_cast<const uint2*>(&st.h[k][x_hoff]);
-                            }
-                            u01[k] = __byte_perm(w, 0u, 0x1404);
-                            u23[k] = __byte_perm(w, 0u, 0x3424);
-                        }
-                        const uint32_t aoff = (uint32_t)((gq + 8 * (x_a & 1)) * 128 + (((4 * x_ct2 + 2 * (x_a >> 1) + (x_tq >> 1)) ^ gq) << 4) + 8 * (x_tq & 1));
-                        const uint32_t dst = smem_u32(ast.a[0]) + aoff;
-#pragma unroll
-                        for (int p = 0; p < 8; ++p) {
-                            __half2 s01 = __float2half2_rn(0.f), s23 = __float2half2_rn(0.f);
-#pragma unroll
-                            for (int k = kMaxPaths - 1; k >= 0; --k) {
-                                if (k >= K) continue;
-                                const uint32_t ox = hv[k].x ^ ((u01[k] << (7 - p)) & 0x80008000u);   // +-h: sign flipped where the weight is -1
-                                const uint32_t oy = hv[k].y ^ ((u23[k] << (7 - p)) & 0x80008000u);
-                                s01 = __hfma2(g_rows[k][gi][p], *reinterpret_cast<const __half2*>(&ox), s01);
-                                s23 = __hfma2(g_rows[k][gi][p], *reinterpret_cast<const __half2*>(&oy), s23);
-                            }
-                            asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dst + p * 16 * 128), "r"(*reinterpret_cast<const uint32_t*>(&s01)),
-                                         "r"(*reinterpret_cast<const uint32_t*>(&s23)) : "memory");
-                        }
-                    }
-                } else
-                {
-                // This thread's packed word (column tile ct2, lane l, word a) of every path: rows 16*p + gq + 8*(a&1),
-                // columns 32*ct2 + 16*(a>>1) + 4*tq + c (c = 0..3) = bytes 0..7 of 16-byte chunk 4*ct2 + 2*(a>>1) + (tq>>1)
-                // of the row (second half if tq is odd); the chunk is XOR-swizzled with the row.
-#pragma unroll
-                for (int k = 0; k < kMaxPaths; ++k) {
-                    if (k >= K) break;
-                    uint32_t w = 0;
-                    uint2 hv = make_uint2(0u, 0u);
-                    if (x_ct2 < cts) {
-                        w = reinterpret_cast<const uint32_t*>(&st.bits[k][x_ct2][x_l])[x_a];
-                        hv = *reinterpret_cast<const uint2*>(&st.h[k][x_hoff]);
-                    }
-                    const uint32_t u01 = __byte_perm(w, 0u, 0x1404);                       // bytes [0, c0, 0, c1]: bit p of a column -> bit 8+p / 24+p
-                    const uint32_t u23 = __byte_perm(w, 0u, 0x3424);                       // bytes [0, c2, 0, c3]
-                    const uint32_t dst = smem_u32(ast.a[k]) + x_aoff;
-#pragma unroll
-                    for (int p = 0; p < 8; ++p) {
-                        const uint32_t ox = hv.x ^ ((u01 << (7 - p)) & 0x80008000u);       // flip the fp16 sign where the weight is -1
-                        const uint32_t oy = hv.y ^ ((u23 << (7 - p)) & 0x80008000u);
-                        asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dst + p * 16 * 128), "r"(ox), "r"(oy) : "memory");
-                    }
+            const int u_end = u0 + (s_hi - s_lo) * n_ops;
+            for (int j = 0; j < n_w && grp < n_groups; ++j) {
+              const unsigned char* w_stage = w_ring + ww.slot * (K * kWBytes) + lane * 16;
+              const unsigned char* h_stage = w_ring + ww.slot * (K * kWBytes) + K * kWTiles * RABIT_TILE_BYTES + 8 * tq;
+              const int uj = u0 + j * kWSteps * n_ops, uj_end = min(uj + kWSteps * n_ops, u_end);
+              mbar_wait(w_full0 + ww.slot * 8, ww.lap, abort_flag);
+              for (; u < uj_end; u += n_groups) {
+                const int sj = (u - uj) / n_ops, k = (u - uj) - sj * n_ops, us = uw.slot;
+                const unsigned char* bits = w_stage + sj * 2 * RABIT_TILE_BYTES;
+                const unsigned char* hs = h_stage + sj * kStepCols * 2;
+                if (u >= units) {
+                    mbar_wait(a_empty0 + us * 8, uw.lap ^ 1u, abort_flag);
+                    fence_after();
                 }
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");              // generic-proxy writes -> visible to the tensor core
+                const uint32_t dst = a0 + us * kUnitCols;
+                auto expand_tile = [&](int ct2) {
+                    uint32_t o[2][8];                                                      // [row block][16-column half, row half, column pair]
+                    // dequantised: sum_k +-g_k[row] h_k[col], accumulated from the last (smallest) path to the first with one
+                    // fused multiply-add per path
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) o[0][i] = o[1][i] = 0u;
+#pragma unroll
+                    for (int kk = DEQ ? K - 1 : 0; kk >= 0; --kk) {
+                        const int kp = DEQ ? kk : k;
+                        const uint4 wv = *reinterpret_cast<const uint4*>(bits + (kp * kWTiles + ct2) * RABIT_TILE_BYTES);
+                        const uint32_t word[4] = {wv.x, wv.y, wv.z, wv.w};
+#pragma unroll
+                        for (int ah = 0; ah < 2; ++ah) {
+                            const uint2 hv = *reinterpret_cast<const uint2*>(hs + (kp * kWTiles * RABIT_TILE_COLS + 32 * ct2 + 16 * ah) * 2);
+#pragma unroll
+                            for (int rh = 0; rh < 2; ++rh)
+#pragma unroll
+                                for (int pair = 0; pair < 2; ++pair) {
+                                    // bytes [0, c0, 0, c1]: bit p of the pair's columns at 8 + p and 24 + p
+                                    const uint32_t v = __byte_perm(word[2 * ah + rh], 0u, pair ? 0x3424 : 0x1404) << shift;
+                                    const uint32_t hp = pair ? hv.y : hv.x;
+#pragma unroll
+                                    for (int pi = 0; pi < 2; ++pi) {
+                                        const uint32_t m = ((pi ? v : v << 1) & 0x80008000u) ^ hp;
+                                        uint32_t& a = o[pi][4 * ah + 2 * rh + pair];
+                                        if (DEQ) {
+                                            const __half2 sum = __hfma2(g_rows[kk][pi][rh], *reinterpret_cast<const __half2*>(&m), *reinterpret_cast<const __half2*>(&a));
+                                            a = *reinterpret_cast<const uint32_t*>(&sum);
+                                        } else {
+                                            a = m;
+                                        }
+                                    }
+                                }
+                        }
+                    }
+                    tmem_st_16x256b_x2(dst + ct2 * 16, o[0]);
+                    tmem_st_16x256b_x2(dst + ct2 * 16 + (16u << 16), o[1]);
+                };
+                expand_tile(0);
+                if (2 * (s_lo + j * kWSteps + sj) + 1 < n_ct) expand_tile(1);
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&S.a_ready[aslot]));
+                if (lane == 0) mbar_arrive(a_ready0 + us * 8);
+                uw.step(n_groups, units);
+              }
+              if (lane == 0) mbar_arrive(w_empty0 + ww.slot * 8);
+              ww.step(1, w_stages);
             }
+            u0 = u_end;
             if (split > 1) break;                              // the cluster's epilogue follows the role branches
-            // ---- epilogue of this tile
-            mbar_wait(smem_u32(&S.acc_ready), tile_i & 1, abort_flag);
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int row = rt * kTileM + quarter * 32 + lane;
-            float gk[kMaxPaths];
+            // ---- epilogue of this pass
+            mbar_wait(smem_u32(&S.acc_ready), pass_i & 1, abort_flag);
+            ++pass_i;
+            fence_after();
+            const int row = ps.rt * kTileM + q * 32 + lane;
+            float gk[K];
 #pragma unroll
-            for (int k = 0; k < kMaxPaths; ++k) gk[k] = (k < K && row < G.Mp) ? __half2float(P.g[(size_t)k * G.Mp + row]) : 0.f;
+            for (int k = 0; k < K; ++k) gk[k] = __half2float(P.g[(size_t)k * P.Mp + row]);
 #pragma unroll 1
-            for (int c0 = 0; c0 < kTileB / 2; c0 += 32) {
-                const int col = col_half * (kTileB / 2) + c0;
-                if (bt * kTileB + col >= P.batch) break;                          // batch rows beyond the batch: nothing to drain or store
-                float v[32];
+            for (int c = grp; c < ps.n; c += kExpandGroups) {
+                float v[16];
 #pragma unroll
-                for (int c = 0; c < 32; ++c) v[c] = 0.f;
+                for (int i = 0; i < 16; ++i) v[i] = 0.f;
 #pragma unroll
-                for (int k = 0; k < kMaxPaths; ++k) {
-                    if (k >= (DEQ ? 1 : K)) break;
-                    uint32_t d[32];
-                    tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(k * kTileB + col), d);
+                for (int m = 0; m < (n_ops == 1 ? 2 : n_ops); ++m) {
+                    if (n_ops == 1 && m >= P.n_acc) break;
+                    uint32_t d[16];
+                    tmem_ld16(lane_base + (uint32_t)((m * P.max16 + c) * kGroupCols), d);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    const float gm = DEQ ? 1.f : gk[n_ops == 1 ? 0 : m];
 #pragma unroll
-                    for (int c = 0; c < 32; ++c) v[c] = DEQ ? __uint_as_float(d[c]) : fmaf(gk[k], __uint_as_float(d[c]), v[c]);
+                    for (int i = 0; i < 16; ++i) v[i] = fmaf(gm, __uint_as_float(d[i]), v[i]);
                 }
+                const int b0 = (ps.c16 + c) * kGroupCols;
+                __half* yp = P.y + (size_t)b0 * P.M + row;
+                if (row < P.M) {
 #pragma unroll
-                for (int c = 0; c < 32; ++c) {
-                    const int b = bt * kTileB + col + c;
-                    if (b < P.batch && row < G.M) P.y[(size_t)b * G.M + row] = __float2half_rn(v[c]);
+                    for (int i = 0; i < 16; ++i)
+                        if (b0 + i < P.batch) yp[(size_t)i * P.M] = __float2half_rn(v[i]);
                 }
             }
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&S.acc_empty));
         }
     }
 
     if (split > 1) {
-        // ---- epilogue of a split tile.  Every CTA of the cluster holds a partial 128 x TB result in tensor memory.
-        //      CTA `o` finishes the batch columns [o*W, (o+1)*W), W = TB / split: all CTAs send it their slice of
-        //      those columns (already scaled by g_k and summed over the paths), into its receive buffer
-        //      recv[source rank][column][row] (the input ring's memory: nothing uses it once every CTA's MMAs have
-        //      retired, which the first cluster barrier establishes).  After the second barrier each CTA adds the
-        //      slices it received in rank order and stores fp16.
-        const int rt = t_first / P.n_bt, bt = t_first % P.n_bt;
-        const int W = kTileB / split;
-        if (warp >= 2) {
+        // ---- epilogue of a split task.  Every CTA of the cluster holds a partial result in tensor memory.  Group c of 16
+        //      batch columns is finished by CTA c % split: all CTAs send it that group's columns (already scaled by g_k and
+        //      summed over the paths) into its receive buffer recv[its c / split][source rank][column][row] (the input ring's
+        //      memory: nothing uses it once every CTA's MMAs have retired, which the first cluster barrier
+        //      establishes).  After the second barrier each CTA adds what it received in rank order and stores fp16.
+        PassWalker w(P, task);
+        Pass ps;
+        w.next(P, ps);
+        if (warp >= 4) {
             mbar_wait(smem_u32(&S.acc_ready), 0, abort_flag);
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            fence_after();
         }
         __syncwarp();
         cluster_sync_all();
-        float* recv = reinterpret_cast<float*>(&S.stage[0]);
-        if (warp >= 2) {
-            const int e = warp - 2, quarter = warp & 3, col_half = e >> 2;
-            const int r_in = quarter * 32 + lane;                                  // row of the tile this thread reads from tensor memory
-            const int row = rt * kTileM + r_in;
-            float gk[kMaxPaths];
+        float* recv = reinterpret_cast<float*>(ring);
+        if (warp >= 4) {
+            const int grp = (warp - 4) >> 2, q = warp & 3, r_in = q * 32 + lane;
+            const int row = ps.rt * kTileM + r_in;
+            float gk[K];
 #pragma unroll
-            for (int k = 0; k < kMaxPaths; ++k) gk[k] = (k < K && row < G.Mp) ? __half2float(P.g[(size_t)k * G.Mp + row]) : 0.f;
+            for (int k = 0; k < K; ++k) gk[k] = __half2float(P.g[(size_t)k * P.Mp + row]);
 #pragma unroll 1
-            for (int c0 = 0; c0 < kTileB / 2; c0 += 32) {
-                const int col = col_half * (kTileB / 2) + c0;
-                if (bt * kTileB + col >= P.batch) break;                          // batch rows beyond the batch: nothing to drain or store
-                float v[32];
+            for (int c = grp; c < ps.n; c += kExpandGroups) {
+                float v[16];
 #pragma unroll
-                for (int c = 0; c < 32; ++c) v[c] = 0.f;
+                for (int i = 0; i < 16; ++i) v[i] = 0.f;
 #pragma unroll
-                for (int k = 0; k < kMaxPaths; ++k) {
-                    if (k >= (DEQ ? 1 : K)) break;
-                    uint32_t d[32];
-                    tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(k * kTileB + col), d);
+                for (int m = 0; m < (n_ops == 1 ? 2 : n_ops); ++m) {
+                    if (n_ops == 1 && m >= P.n_acc) break;
+                    uint32_t d[16];
+                    tmem_ld16(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)((m * P.max16 + c) * kGroupCols), d);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    const float gm = DEQ ? 1.f : gk[n_ops == 1 ? 0 : m];
 #pragma unroll
-                    for (int c = 0; c < 32; ++c) v[c] = DEQ ? __uint_as_float(d[c]) : fmaf(gk[k], __uint_as_float(d[c]), v[c]);
+                    for (int i = 0; i < 16; ++i) v[i] = fmaf(gm, __uint_as_float(d[i]), v[i]);
                 }
-                const int owner = col / W, lc0 = col % W;                         // 32 divides W: the chunk has one owner
-                const uint32_t dst = cluster_map(smem_u32(recv + ((size_t)crank * W + lc0) * kTileM + r_in), (uint32_t)owner);
+                const uint32_t dst = cluster_map(smem_u32(recv + ((size_t)((c / split) * split + crank) * kGroupCols) * kTileM + r_in), (uint32_t)(c % split));
 #pragma unroll
-                for (int c = 0; c < 32; ++c) st_cluster_f32(dst + (uint32_t)(c * kTileM * 4), v[c]);
+                for (int i = 0; i < 16; ++i) st_cluster_f32(dst + (uint32_t)(i * kTileM * 4), v[i]);
             }
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            fence_before();
         }
         __syncwarp();
         cluster_sync_all();
-        if (warp >= 2) {
-            const int et = (warp - 2) * 32 + lane;
-            const int r_in = et & (kTileM - 1), hh = et >> 7;                     // two threads per row, half of the W columns each
-            const int row = rt * kTileM + r_in;
-            for (int lc = hh * (W / 2); lc < (hh + 1) * (W / 2); ++lc) {
-                float sum = 0.f;
-                for (int src = 0; src < split; ++src) sum += recv[((size_t)src * W + lc) * kTileM + r_in];
-                const int b = bt * kTileB + (int)crank * W + lc;
-                if (b < P.batch && row < G.M) P.y[(size_t)b * G.M + row] = __float2half_rn(sum);
-            }
+        if (warp >= 4) {
+            const int et = (warp - 4) * 32 + lane, r_in = et & (kTileM - 1), hh = et >> 7;  // four threads per row, every fourth column each
+            const int row = ps.rt * kTileM + r_in;
+            for (int c = (int)crank; c < ps.n; c += split)
+#pragma unroll
+                for (int i = hh; i < kGroupCols; i += kExpandGroups) {
+                    const float* src = recv + ((size_t)((c / split) * split) * kGroupCols + i) * kTileM + r_in;
+                    float sum = 0.f;
+                    for (int r = 0; r < split; ++r) sum += src[(size_t)r * kGroupCols * kTileM];
+                    const int b = (ps.c16 + c) * kGroupCols + i;
+                    if (b < P.batch && row < P.M) P.y[(size_t)b * P.M + row] = __float2half_rn(sum);
+                }
         }
     }
 
     // ---- teardown: everyone meets, then the allocating warp frees the tensor memory
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    fence_before();
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    fence_after();
     if (warp == 1) {
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
     }
     if (tid == 0 && *abort_flag) atomicExch(P.status, 1u);
 }
@@ -497,151 +603,233 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 EncodeTiledFn encode_tiled_fn() {
-    static EncodeTiledFn fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
+    static const EncodeTiledFn fn = [] {
         void* p = nullptr;
         cudaDriverEntryPointQueryResult q;
         if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
-            fn = (EncodeTiledFn)p;
-    }
+            return (EncodeTiledFn)p;
+        return (EncodeTiledFn) nullptr;
+    }();
     return fn;
 }
 
-}  // namespace
+// Descriptor of x [batch][N] in boxes of 16 * box16 rows x 64 columns.  A pure function of its arguments; the last few are
+// remembered per thread (encoding one costs about a microsecond of host time).
+cudaError_t x_tensor_map(const void* x, int N, int batch, int box16, CUtensorMap* out) {
+    struct Entry { const void* x; int N, batch, box16; CUtensorMap map; };
+    static thread_local Entry recent[8];
+    static thread_local int next = 0;
+    for (const Entry& e : recent)
+        if (e.x == x && e.N == N && e.batch == batch && e.box16 == box16) { *out = e.map; return cudaSuccess; }
+    EncodeTiledFn encode = encode_tiled_fn();
+    if (!encode) return cudaErrorNotSupported;
+    const cuuint64_t dims[2] = {(cuuint64_t)N, (cuuint64_t)batch};
+    const cuuint64_t strides[1] = {(cuuint64_t)N * 2};
+    const cuuint32_t box[2] = {(cuuint32_t)kStepCols, (cuuint32_t)(box16 * kGroupCols)};
+    const cuuint32_t estr[2] = {1, 1};
+    if (encode(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(x), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    recent[next] = Entry{x, N, batch, box16, *out};
+    next = (next + 1) & 7;
+    return cudaSuccess;
+}
 
-// CTAs per cluster that share one tile's contraction: doubled while every CTA keeps at least 8 steps, the
-// slices stay 32 columns wide and the whole grid is resident at once.
-// Clusters of 2 / 4 / 8 of these one-per-SM CTAs that the device places at once (index log2 of the size); cautious
-// defaults until a launch has asked the runtime (a cluster must sit inside one GPC, so 8-CTA clusters are few).
-static int g_cluster_limit[4] = {1 << 30, 64, 28, 8};
+// ---- choosing the work split -------------------------------------------------------------------------
 
-static int choose_split(int n_tiles, int N, int tb, int sms) {
-    const int n_steps = (N + kStepCols - 1) / kStepCols;
-    int best = 1;
-    for (int lg = 1; lg <= 3; ++lg) {
-        const int split = 1 << lg;
-        if (n_tiles * split <= sms && n_tiles <= g_cluster_limit[lg] && n_steps / split >= 8 && tb / split >= 32) best = split;
+struct Plan {
+    int chunks, chunk16, split, max16, tasks;        // chunks == 0: contiguous group ranges
+    int stages, stage_bytes, w_stages, box16, units, n_acc;
+    size_t smem;
+    double clocks;                                   // estimate
+};
+
+// Ring, tensor-memory and shared-memory figures of passes of up to max16 groups; false if they do not fit.  The units are a
+// multiple of the expander groups and of the accumulators (see Walk), the x stages of two for the same reason.
+bool fill_resources(Plan& p, int K, int n_ops, int steps) {
+    if (p.max16 * kGroupCols > 256) return false;
+    const int turn = n_ops == 3 ? 3 : 4;
+    auto free_units = [&](int n_acc) { return (512 - n_acc * p.max16 * kGroupCols) / kUnitCols; };
+    p.n_acc = n_ops > 1 ? n_ops : steps >= 2 && free_units(2) >= turn ? 2 : 1;
+    if (free_units(p.n_acc) < turn) return false;
+    p.units = free_units(p.n_acc) >= 2 * turn ? 2 * turn : turn;
+    p.stage_bytes = (p.max16 + p.box16 - 1) / p.box16 * p.box16 * kGroupCols * kStepCols * 2;
+    const int room = (226 - 1) * 1024 - kControlBytes;
+    p.stages = std::min(kMaxStages, (room - 3 * K * kWBytes) / p.stage_bytes / 2 * 2);
+    if (p.stages < 4) return false;
+    p.w_stages = std::min(kMaxWStages, (room - p.stages * p.stage_bytes) / (K * kWBytes));
+    // Never so little that two CTAs could share an SM: each takes all of its tensor memory, and of two clusters waiting
+    // crosswise for each other's neither would ever get it.
+    p.smem = std::max<size_t>(1024 + kControlBytes + (size_t)p.stages * p.stage_bytes + (size_t)p.w_stages * K * kWBytes, 152 * 1024);
+    return true;
+}
+
+// Clocks of a (step, path) unit: four MMAs of n16 groups of batch columns, or the expansion of its two sign tiles (measured
+// 270 to 290 per unit and SM up to 128 columns: about 165 clocks of integer issue, the rest hand-over).
+double unit_clocks(int n16) { return std::max(32.0 * n16 + 40.0, 280.0); }
+
+const void* kernel_for(int K, bool deq) {
+    if (K == 1) return deq ? (const void*)rabit_gemm_tc_kernel<1, true> : (const void*)rabit_gemm_tc_kernel<1, false>;
+    if (K == 2) return deq ? (const void*)rabit_gemm_tc_kernel<2, true> : (const void*)rabit_gemm_tc_kernel<2, false>;
+    return deq ? (const void*)rabit_gemm_tc_kernel<3, true> : (const void*)rabit_gemm_tc_kernel<3, false>;
+}
+
+// Function attributes are per device.
+cudaError_t prepare_kernel(int K, bool deq, int device) {
+    static bool done[64][6] = {};
+    const int slot = device >= 0 && device < 64 ? device : 0, inst = 2 * (K - 1) + (deq ? 1 : 0);
+    if (done[slot][inst] && slot == device) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(kernel_for(K, deq), cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+    if (e == cudaSuccess) done[slot][inst] = true;
+    return e;
+}
+
+// How many clusters of `split` CTAs of this kernel the device places at once (a cluster sits inside one GPC).
+int resident_clusters(const void* kernel, int split, size_t smem, int sms) {
+    cudaLaunchConfig_t q = {};
+    q.gridDim = dim3((unsigned int)((sms / split) * split));
+    q.blockDim = dim3(kThreads);
+    q.dynamicSmemBytes = smem;
+    cudaLaunchAttribute qa[1];
+    qa[0].id = cudaLaunchAttributeClusterDimension;
+    qa[0].val.clusterDim.x = (unsigned int)split;
+    qa[0].val.clusterDim.y = 1;
+    qa[0].val.clusterDim.z = 1;
+    q.attrs = qa;
+    q.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &q) != cudaSuccess) { cudaGetLastError(); n = 0; }
+    return n;
+}
+
+constexpr double kPassClocks = 3000.0;               // pipeline fill and epilogue of a pass that nothing overlaps
+constexpr double kLaunchClocks = 5000.0;             // launch, first loads, last epilogue
+constexpr double kExchangeClocks = 1500.0;           // cluster barriers and exchange of a split task
+
+Plan make_plan(int n_rt, int n_steps, int K, bool deq, int n16, int sms, int device) {
+    const int n_ops = deq ? 1 : K;
+    Plan best = {};
+    best.clocks = 1e300;
+    // (a) uniform tasks: every row tile in `chunks` chunks, the contraction of a task over `split` CTAs
+    for (int chunks = 1; chunks <= n16; ++chunks) {
+        Plan p = {};
+        p.max16 = p.chunk16 = p.box16 = (n16 + chunks - 1) / chunks;
+        p.chunks = (n16 + p.chunk16 - 1) / p.chunk16;
+        if (p.chunks != chunks || !fill_resources(p, K, n_ops, n_steps / 8)) continue;
+        for (int split = 1; split <= 8; split *= 2) {
+            p.split = split;
+            p.tasks = n_rt * chunks;
+            const long long ctas = (long long)p.tasks * split;
+            if (split > 1) {
+                if (n_steps / split < 4 || ctas > sms) continue;
+                if ((size_t)((p.chunk16 + split - 1) / split * split) * kGroupCols * kTileM * 4 > (size_t)p.stages * p.stage_bytes + (size_t)p.w_stages * K * kWBytes) continue;
+                if (prepare_kernel(K, deq, device) != cudaSuccess || resident_clusters(kernel_for(K, deq), split, p.smem, sms) < p.tasks) continue;
+            }
+            const double rounds = (double)((ctas + sms - 1) / sms);
+            p.clocks = kLaunchClocks + (split > 1 ? kExchangeClocks : 0.0) + rounds * ((n_steps + split - 1) / split) * n_ops * unit_clocks(p.chunk16) +
+                       (rounds - 1.0) * kPassClocks;
+            if (p.clocks < best.clocks) best = p;
+        }
+        if (p.chunk16 <= 4) break;                   // narrower passes cost as much as these
+    }
+    // (b) contiguous ranges of groups, one per SM: no last wave
+    const long long groups = (long long)n_rt * n16;
+    if (groups >= 2LL * sms) {
+        Plan p = {};
+        p.split = 1;
+        p.tasks = sms;
+        const int per_sm = (int)((groups + sms - 1) / sms);
+        for (p.max16 = std::min(16, n16); p.max16 > 1; --p.max16) {
+            // most passes of a range are cut to this size: two boxes of it make one step
+            const int run = std::min(per_sm, n16), pieces = (run + p.max16 - 1) / p.max16;
+            p.box16 = ((run + pieces - 1) / pieces + 1) / 2;
+            if (fill_resources(p, K, n_ops, n_steps)) break;
+        }
+        if (fill_resources(p, K, n_ops, n_steps)) {
+            double worst = 0.0;
+            for (int t = 0; t < sms; ++t) {
+                long long g = groups * t / sms;
+                const long long g1 = groups * (t + 1) / sms;
+                double c = 0.0;
+                while (g < g1) {
+                    const int run = (int)std::min<long long>(g1 - g, n16 - g % n16), pieces = (run + p.max16 - 1) / p.max16, n = (run + pieces - 1) / pieces;
+                    c += n_steps * n_ops * unit_clocks(n) + kPassClocks;
+                    g += n;
+                }
+                worst = std::max(worst, c);
+            }
+            p.clocks = kLaunchClocks - kPassClocks + worst;
+            if (p.clocks < best.clocks) best = p;
+        }
     }
     return best;
 }
 
-// Estimated duration (us) of the exact-expansion GEMM on B200, a fit to measurements at batch <= 64:
-// 11 + 0.75 * (K/2) per 64-column step of the busiest CTA, times the number of waves.
-double rabit_gemm_tc_estimate_us(const rabit_layer& L, int batch) {
-    const int sms = L.sm_count > 0 ? L.sm_count : 148;
-    const int tb = L.geom.K > 2 ? 128 : 256;
-    const int n_tiles = L.geom.n_rt * ((batch + tb - 1) / tb);
-    const int split = choose_split(n_tiles, L.geom.N, tb, sms);
-    const int n_steps = (L.geom.N + kStepCols - 1) / kStepCols;
-    const double waves = split > 1 ? 1.0 : (double)((n_tiles + sms - 1) / sms);
-    return waves * (11.0 + 0.375 * L.geom.K * (double)((n_steps + split - 1) / split));
+int sms_of(const rabit_layer& L) { return L.sm_count > 0 ? L.sm_count : 148; }
+
+Plan plan_for(const rabit_layer& L, bool deq, int batch) {
+    struct Entry { int n_rt, n_steps, K, deq, n16, sms; Plan plan; };
+    static thread_local std::vector<Entry> plans;     // a search costs tens of microseconds; a program calls few shapes
+    const int n16 = (batch + kGroupCols - 1) / kGroupCols, n_rt = L.geom.n_rt, n_steps = (L.geom.N + kStepCols - 1) / kStepCols, K = L.geom.K, sms = sms_of(L);
+    for (const Entry& e : plans)
+        if (e.n_rt == n_rt && e.n_steps == n_steps && e.K == K && e.deq == (int)deq && e.n16 == n16 && e.sms == sms) return e.plan;
+    if (plans.size() >= 256) plans.clear();
+    plans.push_back(Entry{n_rt, n_steps, K, (int)deq, n16, sms, make_plan(n_rt, n_steps, K, deq, n16, sms, L.device)});
+    return plans.back().plan;
 }
+
+}  // namespace
 
 bool rabit_gemm_tc_supports(const rabit_layer& L, int batch) {
-    return batch >= 1 && L.geom.K <= 3 && encode_tiled_fn() != nullptr;
+    return batch >= 1 && batch <= (1 << 24) && L.geom.K <= 3 && encode_tiled_fn() != nullptr;
 }
 
-template <int TB, int KP, bool DEQ>
-static cudaError_t launch_gemm(const rabit_layer& L, const void* x, void* y, int batch, cudaStream_t stream) {
-    EncodeTiledFn encode = encode_tiled_fn();
-    if (!encode) return cudaErrorNotSupported;
+// Estimated duration (us) of the exact-expansion GEMM on B200, at 1.9 GHz.
+double rabit_gemm_tc_estimate_us(const rabit_layer& L, int batch) { return plan_for(L, false, batch).clocks / 1900.0; }
+
+cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, int batch, cudaStream_t stream, bool dequantised) {
+    const RabitGeom& G = L.geom;
+    const Plan p = plan_for(L, dequantised, batch);
+    if (p.tasks < 1) return cudaErrorInvalidValue;
     CUtensorMap map;
-    const cuuint64_t dims[2] = {(cuuint64_t)L.geom.N, (cuuint64_t)batch};
-    const cuuint64_t strides[1] = {(cuuint64_t)L.geom.N * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kStepCols, (cuuint32_t)TB};
-    const cuuint32_t estr[2] = {1, 1};
-    if (encode(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(x), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
+    cudaError_t e = x_tensor_map(x, G.N, batch, p.box16, &map);
+    if (e != cudaSuccess) return e;
+    e = prepare_kernel(G.K, dequantised, L.device);
+    if (e != cudaSuccess) return e;
 
     GemmParams P;
-    P.G = L.geom;
     P.bits = reinterpret_cast<const unsigned char*>(L.d_bits);
     P.g = (const __half*)L.d_g;
     P.h = (const __half*)L.d_h;
     P.y = (__half*)y;
     P.status = L.d_status;
+    P.M = G.M; P.N = G.N; P.Mp = G.Mp; P.n_ct = G.n_ct;
     P.batch = batch;
-    P.n_bt = (batch + TB - 1) / TB;
-    const int n_tiles = L.geom.n_rt * P.n_bt;
-    static bool attr_done[64] = {false};                                          // function attributes are per device
-    const int dev_slot = L.device >= 0 && L.device < 64 ? L.device : 0;
-    const size_t smem = sizeof(Smem<TB, KP, DEQ ? 1 : KP>) + 1024;               // slack for the 1024-byte alignment of the stages
-    if (!attr_done[dev_slot] || dev_slot != L.device) {
-        cudaError_t e = cudaFuncSetAttribute(rabit_gemm_tc_kernel<TB, KP, DEQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_done[dev_slot] = true;
-    }
-    const int sms = L.sm_count > 0 ? L.sm_count : 148;
-    const bool ring_holds_exchange = sizeof(InStage<TB, KP>) * GemmCfg<TB, KP, DEQ ? 1 : KP>::kStages >= (size_t)kTileM * TB * 4;   // the receive buffer lives in the input ring
+    P.n16 = (batch + kGroupCols - 1) / kGroupCols;
+    P.n_tasks = p.tasks;
+    P.chunks = p.chunks; P.chunk16 = p.chunk16;
+    P.n_groups = (long long)G.n_rt * P.n16;
+    P.max16 = p.max16;
+    P.split = p.split;
+    P.stages = p.stages; P.stage_bytes = p.stage_bytes; P.w_stages = p.w_stages;
+    P.box16 = p.box16;
+    P.n_acc = p.n_acc;
+    P.units = p.units; P.a_col = p.n_acc * p.max16 * kGroupCols;
 
-    static bool limits_done[64] = {false};
-    if (!limits_done[dev_slot]) {                                            // how many clusters of each size fit at once (asked once per kernel)
-        for (int lg = 1; lg <= 3; ++lg) {
-            cudaLaunchConfig_t q = {};
-            q.gridDim = dim3((unsigned int)((sms / (1 << lg)) * (1 << lg)));
-            q.blockDim = dim3(kThreads);
-            q.dynamicSmemBytes = smem;
-            cudaLaunchAttribute qa[1];
-            qa[0].id = cudaLaunchAttributeClusterDimension;
-            qa[0].val.clusterDim.x = 1u << lg;
-            qa[0].val.clusterDim.y = 1;
-            qa[0].val.clusterDim.z = 1;
-            q.attrs = qa;
-            q.numAttrs = 1;
-            int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, rabit_gemm_tc_kernel<TB, KP, DEQ>, &q) == cudaSuccess && n > 0) g_cluster_limit[lg] = n;
-            else cudaGetLastError();
-        }
-        limits_done[dev_slot] = true;
-    }
-
-    // One launch over tiles [lo, hi).  Few tiles: the CTAs of a cluster share each tile's contraction (see choose_split).
-    auto launch_range = [&](int lo, int hi) -> cudaError_t {
-        GemmParams Q = P;
-        Q.tile_lo = lo;
-        Q.tile_hi = hi;
-        const int count = hi - lo;
-        int grid = sms < count ? sms : count;
-        int split = ring_holds_exchange ? choose_split(count, L.geom.N, TB, sms) : 1;
-        Q.split = split;
-        if (split > 1) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3((unsigned int)(count * split));
-            cfg.blockDim = dim3(kThreads);
-            cfg.dynamicSmemBytes = smem;
-            cfg.stream = stream;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = (unsigned int)split;
-            attr[0].val.clusterDim.y = 1;
-            attr[0].val.clusterDim.z = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            if (cudaLaunchKernelEx(&cfg, rabit_gemm_tc_kernel<TB, KP, DEQ>, Q, map) == cudaSuccess) return cudaSuccess;
-            cudaGetLastError();                                    // clusters of this size cannot be placed here: one CTA per tile instead
-            Q.split = 1;
-        }
-        rabit_gemm_tc_kernel<TB, KP, DEQ><<<grid, kThreads, smem, stream>>>(Q, map);
-        return cudaGetLastError();
-    };
-    // A few tiles beyond whole waves would cost a whole wave of their own: they go to a second, split launch.
-    const int whole = (n_tiles / sms) * sms, rest = n_tiles - whole;
-    if (whole > 0 && rest > 0 && ring_holds_exchange && choose_split(rest, L.geom.N, TB, sms) >= 2) {
-        cudaError_t e = launch_range(0, whole);
-        if (e != cudaSuccess) return e;
-        return launch_range(whole, n_tiles);
-    }
-    return launch_range(0, n_tiles);
-}
-
-cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, int batch, cudaStream_t stream, bool dequantised) {
-    if (dequantised)                                                                 // one accumulator: the widest batch tile for every K
-        return L.geom.K > 2 ? launch_gemm<256, 3, true>(L, x, y, batch, stream) : launch_gemm<256, 2, true>(L, x, y, batch, stream);
-    if (L.geom.K > 2) return launch_gemm<128, 3, false>(L, x, y, batch, stream);   // three accumulators of 128 columns
-    // Always the widest batch tile: a tcgen05.mma of M = 128 takes about 128 clocks whatever its N (measured),
-    // so narrower tiles would not shorten a step, they would only expand the signs more often.
-    return launch_gemm<256, 2, false>(L, x, y, batch, stream);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned int)(p.tasks * p.split));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = p.smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned int)p.split;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = p.split > 1 ? 2 : 1;
+    void* args[2] = {&P, &map};
+    return cudaLaunchKernelExC(&cfg, kernel_for(G.K, dequantised), args);
 }
