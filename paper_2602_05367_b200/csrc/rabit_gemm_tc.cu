@@ -664,9 +664,13 @@ bool fill_resources(Plan& p, int K, int n_ops, int steps) {
     return true;
 }
 
-// Clocks of a (step, path) unit: four MMAs of n16 groups of batch columns, or the expansion of its two sign tiles (measured
-// 270 to 290 per unit and SM up to 128 columns: about 165 clocks of integer issue, the rest hand-over).
-double unit_clocks(int n16) { return std::max(32.0 * n16 + 40.0, 280.0); }
+// Clocks of a (step, path) unit: four MMAs of the pass's batch columns, or the expansion of its two sign tiles (measured 270 to
+// 290 per unit and SM: about 165 clocks of integer issue, the rest hand-over; more if a group has only one unit's room
+// in tensor memory and has to wait for its MMAs).
+double unit_clocks(int n16, const Plan& p, int n_ops) {
+    const bool two_each = p.units >= 2 * (n_ops == 3 ? 3 : 4);
+    return std::max(32.0 * n16 + 40.0, two_each ? 280.0 : n_ops == 3 ? 410.0 : 320.0);
+}
 
 const void* kernel_for(int K, bool deq) {
     if (K == 1) return deq ? (const void*)rabit_gemm_tc_kernel<1, true> : (const void*)rabit_gemm_tc_kernel<1, false>;
@@ -726,7 +730,7 @@ Plan make_plan(int n_rt, int n_steps, int K, bool deq, int n16, int sms, int dev
                 if (prepare_kernel(K, deq, device) != cudaSuccess || resident_clusters(kernel_for(K, deq), split, p.smem, sms) < p.tasks) continue;
             }
             const double rounds = (double)((ctas + sms - 1) / sms);
-            p.clocks = kLaunchClocks + (split > 1 ? kExchangeClocks : 0.0) + rounds * ((n_steps + split - 1) / split) * n_ops * unit_clocks(p.chunk16) +
+            p.clocks = kLaunchClocks + (split > 1 ? kExchangeClocks : 0.0) + rounds * ((n_steps + split - 1) / split) * n_ops * unit_clocks(p.chunk16, p, n_ops) +
                        (rounds - 1.0) * kPassClocks;
             if (p.clocks < best.clocks) best = p;
         }
@@ -753,7 +757,7 @@ Plan make_plan(int n_rt, int n_steps, int K, bool deq, int n16, int sms, int dev
                 double c = 0.0;
                 while (g < g1) {
                     const int run = (int)std::min<long long>(g1 - g, n16 - g % n16), pieces = (run + p.max16 - 1) / p.max16, n = (run + pieces - 1) / pieces;
-                    c += n_steps * n_ops * unit_clocks(n) + kPassClocks;
+                    c += n_steps * n_ops * unit_clocks(n, p, n_ops) + kPassClocks;
                     g += n;
                 }
                 worst = std::max(worst, c);
