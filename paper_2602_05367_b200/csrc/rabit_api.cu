@@ -59,28 +59,28 @@ extern "C" int rabit_pack(const uint32_t* planes, const uint16_t* g, const uint1
     if (attr.type != cudaMemoryTypeDevice && attr.type != cudaMemoryTypeManaged)
         return rabit_fail(RABIT_INVALID_ARG, "rabit_pack: dev_buf is not device memory");
 
-    std::vector<uint8_t> image;
+    std::vector<uint8_t> tail;
     try {
-        image.resize(hdr.total_bytes);
+        if (!rabit_build_meta(g, h, K, M, N, &G, &hdr, &tail))
+            return rabit_fail(RABIT_UNSUPPORTED_SHAPE, "rabit_pack: unsupported shape K=%d M=%d N=%d (need 1<=K<=3, M>=1, N%%32==0)", K, M, N);
     } catch (const std::bad_alloc&) {
-        return rabit_fail(RABIT_INVALID_ARG, "rabit_pack: out of host memory for the staging image");
+        return rabit_fail(RABIT_INVALID_ARG, "rabit_pack: out of host memory");
     }
-    int rc = rabit_pack_host(planes, g, h, K, M, N, image.data(), image.size());
-    if (rc != RABIT_OK) return rc;
+    // Only the canonical planes and the scales cross to the device (a quarter of the image); both arrangements of the signs
+    // are made there.  The planes wait in the section of the sign tiles, which is written last.  (Packing on the host and
+    // uploading the image took 3.3 ms for 4096 x 4096, this 0.3 ms.)
     cudaStream_t st = (cudaStream_t)stream;
-    RABIT_CUDA_TRY(cudaMemcpyAsync(dev_buf, image.data(), hdr.total_bytes, cudaMemcpyHostToDevice, st));
+    char* base = (char*)dev_buf;
+    RABIT_CUDA_TRY(cudaMemcpyAsync(base + hdr.off_bits, planes, (size_t)K * M * (N / 32) * 4, cudaMemcpyHostToDevice, st));
+    RABIT_CUDA_TRY(cudaMemcpyAsync(base + hdr.off_g, tail.data(), tail.size(), cudaMemcpyHostToDevice, st));
+    cudaError_t e = rabit_launch_pack_planes(G, hdr, base, (const uint32_t*)(base + hdr.off_bits), st);
+    if (e != cudaSuccess) return rabit_fail(RABIT_CUDA_ERROR, "rabit_pack: launch failed: %s", cudaGetErrorString(e));
+    RABIT_CUDA_TRY(cudaMemsetAsync(base + hdr.off_acc, 0, (size_t)(hdr.total_bytes - hdr.off_acc), st));
     RABIT_CUDA_TRY(cudaStreamSynchronize(st));
 
     rabit_layer* L = new (std::nothrow) rabit_layer;
     if (!L) return rabit_fail(RABIT_INVALID_ARG, "rabit_pack: out of host memory");
-    RabitHeader packed_hdr;
-    std::memcpy(&packed_hdr, image.data(), sizeof(packed_hdr));
-    RabitGeom packed_geom;
-    if (!rabit_geom_from_header(packed_hdr, &packed_geom)) {
-        delete L;
-        return rabit_fail(RABIT_INVALID_ARG, "rabit_pack: internal error, packed header unreadable");
-    }
-    bind_layer(L, packed_geom, packed_hdr, dev_buf, attr.device);
+    bind_layer(L, G, hdr, dev_buf, attr.device);
     *out = L;
     return RABIT_OK;
 }
@@ -115,19 +115,13 @@ extern "C" int rabit_derive_pack(const float* W_dev, const uint16_t* g, const ui
         return rabit_fail(RABIT_INVALID_ARG, "rabit_derive_pack: W overlaps dev_buf");
     cudaStream_t st = (cudaStream_t)stream;
     char* base = (char*)dev_buf;
-    // scales from the host (a few KB); the header travels as a parameter of the second kernel
+    // scales from the host (a few KB); the header travels as a parameter of the kernel
     RABIT_CUDA_TRY(cudaMemcpyAsync(base + hdr.off_g, tail.data(), tail.size(), cudaMemcpyHostToDevice, st));
-    cudaError_t e = rabit_launch_derive(G, W_dev, (const uint16_t*)(base + hdr.off_g), (const uint16_t*)(base + hdr.off_h),
-                                        (uint4*)(base + hdr.off_bits), st);
-    // the second kernel also puts the exchange buffer (all-ones words) and the flags (zero) into their resting state
-    if (e == cudaSuccess)
-        e = rabit_launch_tiles_to_lut(G, (const uint4*)(base + hdr.off_bits), (unsigned char*)(base + hdr.off_lut),
-                                      base + hdr.off_partial, (size_t)(hdr.off_flags - hdr.off_partial),
-                                      base + hdr.off_flags, (size_t)(hdr.off_lut - hdr.off_flags), &hdr, base, st);
+    cudaError_t e = rabit_launch_derive(G, hdr, base, W_dev, st);
     if (e != cudaSuccess) return rabit_fail(RABIT_CUDA_ERROR, "rabit_derive_pack: launch failed: %s", cudaGetErrorString(e));
-    // The accumulate words are cleared AFTER the kernels on purpose: the decode kernels start copying weights before
+    // The accumulate words are cleared AFTER the kernel on purpose: the decode kernels start copying weights before
     // they wait for the previous kernel in the stream (weights normally never depend on it).  A fill between the
-    // kernels that write this layer's weights and its first use is an ordinary stream dependency, which such a
+    // kernel that writes this layer's weights and its first use is an ordinary stream dependency, which such a
     // kernel cannot overtake.
     RABIT_CUDA_TRY(cudaMemsetAsync(base + hdr.off_acc, 0, (size_t)(hdr.total_bytes - hdr.off_acc), st));
     // No synchronisation: copies from pageable host memory return once the source has been staged, so the
