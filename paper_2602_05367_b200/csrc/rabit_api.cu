@@ -310,11 +310,11 @@ extern "C" size_t rabit_stage_bytes(const rabit_layer* layer, int batch) {
     return rabit_align256((size_t)batch * layer->geom.N * 2) + rabit_align256((size_t)batch * layer->geom.M * 2);
 }
 
-// Device address under which the GPU can store straight into a host buffer of `bytes` bytes (page-locked,
-// mapped memory, 16-byte aligned), or nullptr if the buffer is ordinary pageable memory.
-static void* mapped_output_alias(void* host_ptr, size_t bytes) {
+// Device address under which the GPU can reach a host buffer of `bytes` bytes directly (page-locked, mapped memory,
+// 16-byte aligned), or nullptr if the buffer is ordinary pageable memory.
+static void* mapped_alias(const void* host_ptr, size_t bytes) {
     cudaPointerAttributes first, last;
-    if (cudaPointerGetAttributes(&first, host_ptr) != cudaSuccess || cudaPointerGetAttributes(&last, (char*)host_ptr + bytes - 1) != cudaSuccess) {
+    if (cudaPointerGetAttributes(&first, host_ptr) != cudaSuccess || cudaPointerGetAttributes(&last, (const char*)host_ptr + bytes - 1) != cudaSuccess) {
         cudaGetLastError();                                              // not an error of the caller: fall back to a copy
         return nullptr;
     }
@@ -323,6 +323,10 @@ static void* mapped_output_alias(void* host_ptr, size_t bytes) {
     if (((uintptr_t)first.devicePointer & 15u) != 0) return nullptr;
     return first.devicePointer;
 }
+
+// Inputs up to this size come from page-locked memory by a kernel (rabit_fetch.cu), larger ones by the copy engine, whose
+// hand-over is then the smaller part (16 GB/s over the bus here: 256 KB take 16 us either way).
+static const size_t kFetchBytes = 256 * 1024;
 
 extern "C" int rabit_linear_host(const rabit_layer* layer, const void* x_host, void* y_host, int batch,
                                  void* dev_stage, size_t dev_stage_bytes, void* stream) {
@@ -338,10 +342,13 @@ extern "C" int rabit_linear_host(const rabit_layer* layer, const void* x_host, v
     char* dx = (char*)dev_stage;
     char* dy = dx + rabit_align256(xb);
     cudaStream_t st = (cudaStream_t)stream;
-    RABIT_CUDA_TRY(cudaMemcpyAsync(dx, x_host, xb, cudaMemcpyHostToDevice, st));
+    const void* mapped = xb <= kFetchBytes ? mapped_alias(x_host, xb) : nullptr;
+    void* dxv = dx;
+    if (mapped) RABIT_CUDA_TRY(rabit_launch_fetch(&mapped, &dxv, &xb, 1, st));
+    else RABIT_CUDA_TRY(cudaMemcpyAsync(dx, x_host, xb, cudaMemcpyHostToDevice, st));
     // A decode-sized result goes straight to mapped host memory from the kernel's last stores (a few KB; the
     // copy engine's latency for so small a copy is longer than the kernel); anything else through the stage.
-    void* direct = batch <= RABIT_MAX_GEMV_BATCH ? mapped_output_alias(y_host, yb) : nullptr;
+    void* direct = batch <= RABIT_MAX_GEMV_BATCH ? mapped_alias(y_host, yb) : nullptr;
     int rc = rabit_linear(layer, dx, direct ? direct : dy, batch, stream);
     if (rc != RABIT_OK) return rc;
     if (!direct) RABIT_CUDA_TRY(cudaMemcpyAsync(y_host, dy, yb, cudaMemcpyDeviceToHost, st));
@@ -374,21 +381,32 @@ extern "C" int rabit_linear_group_host(const rabit_layer* const* layers, const v
     char* cur = (char*)dev_stage;
     const void* dx[8];
     void* dy[8];
+    const void* fetch_src[8];
+    void* fetch_dst[8];
+    size_t fetch_bytes[8];
+    int n_fetch = 0;
     for (int l = 0; l < n_layers; ++l) {
         const size_t xb = (size_t)batch * layers[l]->geom.N * 2;
         dx[l] = nullptr;
         for (int m = 0; m < l; ++m)                                      // the same host input (and width) again: reuse its copy
             if (xs_host[m] == xs_host[l] && layers[m]->geom.N == layers[l]->geom.N) { dx[l] = dx[m]; break; }
         if (!dx[l]) {
-            RABIT_CUDA_TRY(cudaMemcpyAsync(cur, xs_host[l], xb, cudaMemcpyHostToDevice, st));
+            const void* mapped = xb <= kFetchBytes ? mapped_alias(xs_host[l], xb) : nullptr;
+            if (mapped) {
+                fetch_src[n_fetch] = mapped; fetch_dst[n_fetch] = cur; fetch_bytes[n_fetch] = xb;
+                ++n_fetch;
+            } else {
+                RABIT_CUDA_TRY(cudaMemcpyAsync(cur, xs_host[l], xb, cudaMemcpyHostToDevice, st));
+            }
             dx[l] = cur;
             cur += rabit_align256(xb);
         }
     }
+    if (n_fetch > 0) RABIT_CUDA_TRY(rabit_launch_fetch(fetch_src, fetch_dst, fetch_bytes, n_fetch, st));
     bool staged[8];
     for (int l = 0; l < n_layers; ++l) {                                 // decode-sized results: straight to mapped host memory (see rabit_linear_host)
         const size_t yb = (size_t)batch * layers[l]->geom.M * 2;
-        void* direct = batch <= RABIT_MAX_GEMV_BATCH ? mapped_output_alias(ys_host[l], yb) : nullptr;
+        void* direct = batch <= RABIT_MAX_GEMV_BATCH ? mapped_alias(ys_host[l], yb) : nullptr;
         staged[l] = direct == nullptr;
         dy[l] = direct ? direct : cur;
         cur += rabit_align256(yb);

@@ -54,6 +54,9 @@ bool rabit_build_meta(const uint16_t* g, const uint16_t* h, int K, int M, int N,
 cudaError_t rabit_launch_derive(const RabitGeom& G, const RabitHeader& hdr, char* base, const float* W, cudaStream_t stream);
 cudaError_t rabit_launch_pack_planes(const RabitGeom& G, const RabitHeader& hdr, char* base, const uint32_t* planes, cudaStream_t stream);
 
+// up to 8 copies from device-visible host memory to the device by a kernel (rabit_fetch.cu); sizes are multiples of 16 bytes
+cudaError_t rabit_launch_fetch(const void* const* src, void* const* dst, const size_t* bytes, int n, cudaStream_t stream);
+
 // kernel launchers; each enqueues on `stream` and returns a cudaError_t from the launch
 cudaError_t rabit_launch_plain(const rabit_layer& L, const void* x, void* y, int batch, cudaStream_t stream);
 cudaError_t rabit_launch_gemv_mma(const rabit_layer& L, const void* x, void* y, int batch, cudaStream_t stream);
