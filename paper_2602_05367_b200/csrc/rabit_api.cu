@@ -262,9 +262,14 @@ extern "C" int rabit_linear_group(const rabit_layer* const* layers, const void* 
         }
     }
     {
-        bool f16 = true;                                         // 3..16 rows: every layer takes the f16 tensor-core GEMV, launch by launch
-        for (int l = 0; l < n_layers && f16; ++l) f16 = layers[l]->variant == 0 && rabit_gemv_f16_supports(*layers[l], batch);
-        if (f16) {
+        bool f16 = batch <= RABIT_MAX_GEMV_BATCH;                // 3..16 rows: the f16 tensor-core GEMV
+        for (int l = 0; l < n_layers && f16; ++l) f16 = (layers[l]->variant == 0 || layers[l]->variant == 6) && rabit_gemv_f16_supports(*layers[l], batch);
+        if (f16 && !rabit_gemv_lut_supports(*layers[0], batch) && rabit_gemv_f16_group_supports(layers, n_layers, batch)) {
+            cudaError_t e = rabit_launch_gemv_f16_group(layers, n_layers, xs, ys, batch, st);
+            if (e != cudaSuccess) return rabit_fail(RABIT_CUDA_ERROR, "rabit_linear_group: launch failed: %s", cudaGetErrorString(e));
+            return RABIT_OK;
+        }
+        if (f16) {                                               // unlike path counts, or one layer twice: launch by launch
             for (int l = 0; l < n_layers; ++l) {
                 int rc = rabit_linear(layers[l], xs[l], ys[l], batch, stream);
                 if (rc != RABIT_OK) return rc;

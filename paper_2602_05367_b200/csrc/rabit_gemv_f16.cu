@@ -23,22 +23,25 @@
 //     b0 = x[n = gq][cols 0,2]           b1 = x[n = gq][cols 1,3]         (one 8-byte load per lane and k-step, two permutes)
 // and the accumulator lane holds rows gq, gq + 8 of the block and batch rows 2tq, 2tq + 1.
 //
-// Work split.  The layer is n_rt row tiles x n_cs slices of 256 columns; in that order the (row tile, slice) pairs are cut
-// into one contiguous range per SM and every SM's range into two parts, by a cost model on the host (plan_ranges).  One
-// CTA of 16 warps per SM; its two groups of 8 warps each take one part and share nothing but the SM (own barrier, own
-// shared memory): while one group adds up a segment and waits for its atomics, the other computes.  The part of a range
-// inside one row tile is a segment.  Warp w of a group works on path w % K and shares the column tiles of the segment
-// with the other warps of that path.  A warp streams its tiles through a ring of its own in shared memory with
-// asynchronous 16-byte copies (one per lane and tile, each lane reads back only what it copied itself, so no barrier is
-// involved), kRing - 1 tiles ahead: with 16 warps per SM that keeps about 56 KB per SM in flight, which is what the HBM
-// latency needs (with the tiles prefetched into registers, two to four per warp, the kernel ran at the speed of its
-// memory latency, 1.1 to 1.7 TB/s).  At the end of a segment every warp writes its accumulators to its own slot of shared
-// memory, the group adds the slots path by path in a fixed order (deterministic) and applies g_k to each path's sum, and
-// every output of the segment goes, as in the table-driven kernel, into the row's 64-bit accumulate word with one
-// integer atomic (fixed-point grid of the packer, arrival count in bits 55..62, bit 63 = non-finite); the thread whose
-// add completes a row (the count reaches the number of segments of that row tile) rounds it to fp16, stores y and clears
-// the word.  A contribution that covers s slices is shifted by s * 2^fix_bits, so the total shift is the same
-// n_cs * 2^fix_bits for every split.  Nothing waits for another CTA or for the other group.
+// Work split.  The layer is n_rt row tiles x n_cs slices of 256 columns.  Every row tile is cut into m equal units and a CTA
+// (16 warps, one CTA per SM) takes j consecutive units (split_layer on the host chooses m and j by a cost model).  The part
+// of a CTA's range inside one row tile is a segment.  Warp w works on path w % K and shares the column tiles of the segment
+// with the other warps of that path.  A warp streams its tiles through a ring of its own in shared memory with asynchronous
+// 16-byte copies (one per lane and tile, each lane reads back only what it copied itself, so no barrier is involved),
+// kRing - 1 tiles ahead: with 16 warps per SM that keeps about 56 KB per SM in flight, which is what the HBM latency needs
+// (with the tiles prefetched into registers, two to four per warp, the kernel ran at the speed of its memory latency, 1.1
+// to 1.7 TB/s).  At the end of a segment every warp writes its accumulators to its own slot of shared memory and the CTA adds
+// the slots path by path in a fixed order (deterministic), applying g_k to each path's sum.  A segment that is a whole row
+// tile stores y.  Otherwise every output goes, as in the table-driven kernel, into the row's 64-bit accumulate word with one
+// integer atomic (fixed-point grid of the packer, arrival count in bits 55..62, bit 63 = non-finite); the thread whose add
+// completes a row (the count reaches the number of segments of that row tile) rounds it to fp16, stores y and clears the
+// word.  A contribution that covers s slices is shifted by s * 2^fix_bits, so the total shift is the same n_cs * 2^fix_bits
+// for every split.  Nothing waits for another CTA.
+//
+// What bounds it (B200, clocks per 512-byte tile and SM): 75 at up to eight batch rows and 105 at sixteen in the steady state,
+// of which the loads of x and h are 10 %; the rest is 16 or 32 MMAs of about 2 clocks and 128 half-rate integer operations,
+// which hardly overlap.  Segment ends are what a split can save: an arrival count found by searching a table of range
+// bounds in constant memory, cold in every launch, cost 1 us at each, publishing 16 rows from every SM 2 to 3 us.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -49,17 +52,15 @@
 
 namespace {
 
-constexpr int kWarps = 8;                              // warps of a group
-constexpr int kGroupThreads = kWarps * 32;
-constexpr int kGroups = 2;                             // independent groups of a CTA (one CTA per SM)
-constexpr int kThreads = kGroups * kGroupThreads;
+constexpr int kWarps = 16;
+constexpr int kThreads = kWarps * 32;
 constexpr int kRing = 8;                               // sign tiles a warp keeps in flight or in use (a power of two)
 constexpr long long kMaxPairs = 1LL << 30;
-constexpr int kMaxRanges = kGroups * 160;              // one range per group, up to 160 SMs
+constexpr int kMaxGroup = 8;
 constexpr int kSlotStride = 128 + 4;                  // floats per batch row of a slot: the pad spreads a warp's store over all banks
 constexpr unsigned long long kSumMask = (1ULL << 55) - 1;
 
-struct F16Params {
+struct F16Layer {
     const uint4* tiles;
     const __half* g;
     const __half* h;
@@ -67,20 +68,31 @@ struct F16Params {
     __half* y;
     unsigned long long* acc;        // [16][Mp], all zero between calls
     unsigned int* status;           // RABIT_CHECKED builds: set to 2 when an index check fails (the access is skipped)
-    int K, M, N, Mp, n_rt, n_ct, n_cs;
-    int batch;
-    int n_pairs;                    // n_rt * n_cs (row tile, slice) pairs; group q of CTA c owns pairs [bound[2c + q], bound[2c + q + 1])
+    int M, N, Mp, n_rt, n_ct, n_cs;
     int fix_bits;
     float inv_unit, unit, limit;
-    uint32_t two, two_pow_8;        // 2 and 256: multipliers the compiler cannot fold into shifts
-    int bound[kMaxRanges + 1];      // ascending; bound[2 * grid] = n_pairs
+    int cta0;                       // the layer's first CTA
+    int m, j;                       // units per row tile, units per CTA
+    int pad_;
 };
+static_assert(sizeof(F16Layer) % 4 == 0 && sizeof(F16Layer) <= 128, "F16Layer is copied to shared memory by one warp, a word per lane");
+struct F16Params {
+    int n_layers, K, batch;
+    uint32_t two, two_pow_8;        // 2 and 256: multipliers the compiler cannot fold into shifts
+    F16Layer layer[kMaxGroup];
+};
+
+// First pair of a unit: unit q of row tile t starts at slice q n_cs / m of it.  (Host and device.)
+__host__ __device__ __forceinline__ int unit_start(int unit, int m, int n_cs) {
+    const int t = unit / m;
+    return t * n_cs + (int)((long long)(unit - t * m) * n_cs / m);
+}
 
 // Checked build (-DRABIT_CHECKED, python paper_2602_05367_b200/build.py --checked): every index that addresses global or
 // shared memory is compared with its range first; a violation is recorded in the layer's status word and the access is
 // skipped (nothing traps).  In the ordinary build the checks compile to nothing.
 #ifdef RABIT_CHECKED
-#define RABIT_IN_RANGE(cond) ((cond) ? true : (atomicExch(P.status, 2u), false))
+#define RABIT_IN_RANGE(cond) ((cond) ? true : (atomicExch(L.status, 2u), false))
 #else
 #define RABIT_IN_RANGE(cond) true
 #endif
@@ -116,10 +128,6 @@ template <int N>
 __device__ __forceinline__ void copy_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
-// barrier of one group (ids 1 and 2; 0 is left to __syncthreads)
-__device__ __forceinline__ void group_sync(int group) {
-    asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(kGroupThreads) : "memory");
-}
 __device__ __forceinline__ uint4 lds_128(uint32_t addr) {
     uint4 v;
     asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
@@ -141,71 +149,70 @@ __device__ __forceinline__ float path_sums(const float* col, const __half (&g)[R
     return v;
 }
 
-// The range that holds pair u: the last r with bound[r] <= u (empty ranges have bound[r] == bound[r + 1] and lose to
-// the non-empty one that follows them).
-__device__ __forceinline__ int owner_of(const F16Params& P, int u, int n_ranges) {
-    int lo = 0, hi = n_ranges - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (P.bound[mid] <= u) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
 // NH = halves of the batch (8 rows each) a pass carries.
 template <int NH>
 __global__ void __launch_bounds__(kThreads, 1)
 rabit_gemv_f16_kernel(const __grid_constant__ F16Params P) {
-    extern __shared__ __align__(16) float smem_f[];                      // per group: [kWarps][NH * 8][kSlotStride] partial outputs, then the warps' rings
-    constexpr int kGroupFloats = kWarps * NH * 8 * kSlotStride + kWarps * kRing * 128;
-    const int group = threadIdx.x / kGroupThreads;                       // the two groups share nothing but the SM
-    const int tid = threadIdx.x % kGroupThreads, lane = tid & 31, warp = tid >> 5;
+    extern __shared__ __align__(16) float smem_f[];                      // [kWarps][NH * 8][kSlotStride] partial outputs, then the warps' rings
+    [[maybe_unused]] constexpr int kFloats = kWarps * NH * 8 * kSlotStride + kWarps * kRing * 128;
+    __shared__ F16Layer layer_copy;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int gq = lane >> 2, tq = lane & 3;
-    float* slots = smem_f + (size_t)group * kGroupFloats;
+    float* slots = smem_f;
     // the lane's 16 bytes of ring slot 0 of its warp; slot r is r * 512 bytes further
     const uint32_t ring = (uint32_t)__cvta_generic_to_shared(slots) + (uint32_t)(kWarps * NH * 8 * kSlotStride * sizeof(float)) +
                           (uint32_t)((warp * kRing * 32 + lane) * 16);
 
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     bool waited = false;
+    // the launch parameters sit in constant memory, cold in every launch: copied once, before the dependency wait
+    if (warp == 0) {
+        int li = 0;
+        while (li + 1 < P.n_layers && (int)blockIdx.x >= P.layer[li + 1].cta0) ++li;
+        if (lane < (int)(sizeof(F16Layer) / 4)) reinterpret_cast<uint32_t*>(&layer_copy)[lane] = reinterpret_cast<const uint32_t*>(&P.layer[li])[lane];
+    }
+    __syncthreads();
+    const F16Layer& L = layer_copy;
+    const __half *const h_base = L.h, *const x_base = L.x;               // (what the loop needs of the layer, in registers)
+    const int n_ct = L.n_ct, n_cs = L.n_cs;
 
-    // every warp works on ONE path: path k = warp % K, and the column tiles of a segment are dealt out among the group's
-    // warps of that path (K = 3: three, three and two warps)
+    // every warp works on ONE path: path k = warp % K, and the column tiles of a segment are dealt out among the
+    // warps of that path (K = 3: six, five and five warps)
     const int k = warp % P.K;
     const int n_same = (kWarps - k + P.K - 1) / P.K, j0 = warp / P.K;
-    const int hk = k * P.N + 4 * tq;                                      // element offsets (K * N and 16 * N fit 31 bits: N <= 65280)
+    const int hk = k * L.N + 4 * tq;                                      // element offsets (K * N and 16 * N fit 31 bits: N <= 65280)
     int xb[NH];
 #pragma unroll
     for (int hf = 0; hf < NH; ++hf)                                      // lanes beyond the batch read its last row; their columns are never stored
-        xb[hf] = min(8 * hf + gq, P.batch - 1) * P.N + 4 * tq;
+        xb[hf] = min(8 * hf + gq, P.batch - 1) * L.N + 4 * tq;
 
     // A segment: row tile rt, column tiles [ct0, c1) of which this warp takes every n_same-th, starting at ct0.
     struct Segment {
         int rt, n_slices, c1, ct0, n_my;
         const uint4* wsrc;                                               // the warp's first tile (this lane's 16 bytes)
     };
-    const int n_ranges = kGroups * gridDim.x;
-    int u = P.bound[kGroups * blockIdx.x + group];
-    const int u_end = P.bound[kGroups * blockIdx.x + group + 1];
+    const int c_rel = (int)blockIdx.x - L.cta0, n_units = L.n_rt * L.m;
+    int u = unit_start(c_rel * L.j, L.m, n_cs);
+    const int u_end = unit_start(min(n_units, (c_rel + 1) * L.j), L.m, n_cs);
     auto next_segment = [&]() {                                          // the segment that starts at pair u; advances u
         Segment sg;
-        sg.rt = u / P.n_cs;
-        const int s0 = u - sg.rt * P.n_cs;
-        const int s1 = min(P.n_cs, s0 + (u_end - u));
+        sg.rt = u / n_cs;
+        const int s0 = u - sg.rt * n_cs;
+        const int s1 = min(n_cs, s0 + (u_end - u));
         u += s1 - s0;
         sg.n_slices = s1 - s0;
-        sg.c1 = min(P.n_ct, s1 * 8);                                     // a slice is eight column tiles
+        sg.c1 = min(n_ct, s1 * 8);                                     // a slice is eight column tiles
         sg.ct0 = s0 * 8 + j0;
         sg.n_my = sg.ct0 < sg.c1 ? (sg.c1 - sg.ct0 + n_same - 1) / n_same : 0;
-        sg.wsrc = P.tiles + (size_t)(sg.rt * P.K + k) * P.n_ct * 32 + sg.ct0 * 32 + lane;
+        sg.wsrc = L.tiles + (size_t)(sg.rt * P.K + k) * n_ct * 32 + sg.ct0 * 32 + lane;
         return sg;
     };
     auto prefill = [&](const Segment& sg) {                              // the first kRing - 1 tiles of the warp; weights never depend on the stream's past
 #pragma unroll
         for (int i = 0; i < kRing - 1; ++i)
             copy_async_16(ring + i * 512, sg.wsrc + (size_t)i * n_same * 32,
-                          i < sg.n_my && RABIT_IN_RANGE(sg.wsrc + (size_t)i * n_same * 32 >= P.tiles &&
-                                                        sg.wsrc + (size_t)i * n_same * 32 < P.tiles + (size_t)P.n_rt * P.K * P.n_ct * 32));
+                          i < sg.n_my && RABIT_IN_RANGE(sg.wsrc + (size_t)i * n_same * 32 >= L.tiles &&
+                                                        sg.wsrc + (size_t)i * n_same * 32 < L.tiles + (size_t)L.n_rt * P.K * n_ct * 32));
     };
     bool more = u < u_end;
     Segment sg;
@@ -227,13 +234,17 @@ rabit_gemv_f16_kernel(const __grid_constant__ F16Params P) {
         // input scales and activations of the lane's four columns of k-step kh of column tile ct, as loaded (columns 0,1 | 2,3)
         auto fetch_hx = [&](int ct, int kh, uint2& fh, uint2 (&fx)[NH]) {
             const int off = ct * 32 + 16 * kh;
-            if (!RABIT_IN_RANGE(off >= 0 && hk + off + 4 <= P.K * P.N)) return;
-            fh = __ldg(reinterpret_cast<const uint2*>(P.h + hk + off));
+            if (!RABIT_IN_RANGE(off >= 0 && hk + off + 4 <= P.K * L.N)) return;
+            fh = __ldg(reinterpret_cast<const uint2*>(h_base + hk + off));
 #pragma unroll
             for (int hf = 0; hf < NH; ++hf)
-                if (RABIT_IN_RANGE(xb[hf] + off + 4 <= P.batch * P.N)) fx[hf] = __ldcg(reinterpret_cast<const uint2*>(P.x + xb[hf] + off));
+                if (RABIT_IN_RANGE(xb[hf] + off + 4 <= P.batch * L.N)) fx[hf] = __ldcg(reinterpret_cast<const uint2*>(x_base + xb[hf] + off));
         };
 
+        __half gk[RABIT_MAX_K];                                           // output scales of the thread's row (the same row for all its outputs), loaded long before they are used
+#pragma unroll
+        for (int kk = 0; kk < RABIT_MAX_K; ++kk)
+            gk[kk] = kk < P.K ? L.g[(size_t)kk * L.Mp + rt * RABIT_TILE_ROWS + (tid & 127)] : __half();
         // weights kRing - 1 tiles ahead (HBM latency), scales and activations one tile ahead, k-step by k-step in place
         if (!waited) {
             asm volatile("griddepcontrol.wait;" ::: "memory");            // x, y and the accumulate words only after this
@@ -241,17 +252,17 @@ rabit_gemv_f16_kernel(const __grid_constant__ F16Params P) {
         }
         uint2 fh[2], fx[2][NH];
 #pragma unroll
-        for (int kh = 0; kh < 2; ++kh) fetch_hx(min(ct0, P.n_ct - 1), kh, fh[kh], fx[kh]);
+        for (int kh = 0; kh < 2; ++kh) fetch_hx(min(ct0, n_ct - 1), kh, fh[kh], fx[kh]);
         for (int i = 0; i < n_my; ++i) {
             {
                 const int ct = ct0 + i * n_same;
                 const int ia = i + kRing - 1;                            // the tile that takes the slot freed in the last round
                 copy_async_16(ring + (ia & (kRing - 1)) * 512, wsrc + (size_t)ia * n_same * 32,
-                              ia < n_my && RABIT_IN_RANGE(wsrc + (size_t)ia * n_same * 32 >= P.tiles &&
-                                                          wsrc + (size_t)ia * n_same * 32 < P.tiles + (size_t)P.n_rt * P.K * P.n_ct * 32));
+                              ia < n_my && RABIT_IN_RANGE(wsrc + (size_t)ia * n_same * 32 >= L.tiles &&
+                                                          wsrc + (size_t)ia * n_same * 32 < L.tiles + (size_t)L.n_rt * P.K * n_ct * 32));
                 copy_async_wait<kRing - 1>();                            // tile i has landed (one group per tile, also for the tiles that do not exist)
                 const uint4 wv = lds_128(ring + (i & (kRing - 1)) * 512);
-                const int ct_next = min(ct + n_same, P.n_ct - 1);        // beyond the segment: a valid address, never used
+                const int ct_next = min(ct + n_same, n_ct - 1);        // beyond the segment: a valid address, never used
                 const uint32_t w[4] = {wv.x, wv.y, wv.z, wv.w};
 #pragma unroll
                 for (int kh = 0; kh < 2; ++kh) {
@@ -287,14 +298,10 @@ rabit_gemv_f16_kernel(const __grid_constant__ F16Params P) {
             sg = next_segment();
             prefill(sg);
         }
-        constexpr int kPer = NH * 8 * 128 / kGroupThreads;                    // outputs per thread (4 or 8)
-        __half gk[RABIT_MAX_K];                                           // output scales of the thread's row (the same row for all its outputs), loaded early
-#pragma unroll
-        for (int kk = 0; kk < RABIT_MAX_K; ++kk)
-            gk[kk] = kk < P.K ? P.g[(size_t)kk * P.Mp + rt * RABIT_TILE_ROWS + (tid & 127)] : __half();
+        constexpr int kPer = NH * 8 * 128 / kThreads;                         // outputs per thread (2 or 4)
         // ---- the warp's partial outputs -> its slot; slot layout [batch row][row of the tile]
         float* mine = slots + (size_t)warp * (NH * 8 * kSlotStride);
-        const bool slot_ok = RABIT_IN_RANGE(mine + (NH * 8 - 1) * kSlotStride + 127 < smem_f + kGroups * kGroupFloats);
+        const bool slot_ok = RABIT_IN_RANGE(mine + (NH * 8 - 1) * kSlotStride + 127 < smem_f + kFloats);
 #pragma unroll
         for (int p = 0; p < 8; ++p)
 #pragma unroll
@@ -306,51 +313,52 @@ rabit_gemv_f16_kernel(const __grid_constant__ F16Params P) {
                 mine[(b) * kSlotStride + row + 8] = acc[p][hf][2];
                 mine[(b + 1) * kSlotStride + row + 8] = acc[p][hf][3];
             }
-        group_sync(group);
+        __syncthreads();
         // ---- fixed-order sum over the warps, then one atomic per output of the segment
-        int arrivals = 0;                                                // segments of this row tile: the non-empty ranges that touch it
-        for (int r = owner_of(P, rt * P.n_cs, n_ranges), r1 = owner_of(P, (rt + 1) * P.n_cs - 1, n_ranges); r <= r1; ++r)
-            arrivals += P.bound[r] < P.bound[r + 1] ? 1 : 0;
-        // (thread t owns row t & 127 of the tile and the batch rows (t >> 7) + 2 i; rows beyond the batch are computed from
+        const int arrivals = (rt * L.m + L.m - 1) / L.j - rt * L.m / L.j + 1;    // segments of this row tile: the CTAs whose units touch it
+        // (thread t owns row t & 127 of the tile and the batch rows (t >> 7) + 4 i; rows beyond the batch are computed from
         // whatever their MMA columns held and dropped)
         unsigned long long old[kPer], add[kPer];
         bool bad[kPer];
 #pragma unroll
         for (int i = 0; i < kPer; ++i) {
-            const int o = tid + i * kGroupThreads, b = o >> 7, rl = o & 127;
+            const int o = tid + i * kThreads, b = o >> 7, rl = o & 127;
             // sum_k g_k * (sum over the warps of path k), in a fixed order
             const float* col = slots + b * kSlotStride + rl;
             const float v = P.K == 2 ? path_sums<2, NH>(col, gk) : P.K == 3 ? path_sums<3, NH>(col, gk) : path_sums<1, NH>(col, gk);
-            const float scaled = v * P.inv_unit;
-            bad[i] = !(fabsf(scaled) < P.limit * (float)n_slices);       // inf or NaN: finite inputs cannot get here
+            const float scaled = v * L.inv_unit;
+            bad[i] = !(fabsf(scaled) < L.limit * (float)n_slices);       // inf or NaN: finite inputs cannot get here
             const long long q = bad[i] ? 0LL : __float2ll_rn(scaled);
-            add[i] = (unsigned long long)(q + ((long long)n_slices << P.fix_bits)) + (1ULL << 55);
+            add[i] = (unsigned long long)(q + ((long long)n_slices << L.fix_bits)) + (1ULL << 55);
+            const int row = rt * RABIT_TILE_ROWS + rl;
+            if (arrivals == 1 && b < P.batch && row < L.M)               // a whole row tile: nobody else contributes
+                L.y[(size_t)b * L.M + row] = bad[i] ? __ushort_as_half((unsigned short)0x7FFF) : __float2half_rn(v);
         }
         // all atomics of the thread back to back: nothing between them that could wait for an answer
 #pragma unroll
         for (int i = 0; i < kPer; ++i) {
-            const int o = tid + i * kGroupThreads, b = o >> 7, rl = o & 127;
+            const int o = tid + i * kThreads, b = o >> 7, rl = o & 127;
             old[i] = 0ULL;
-            if (b >= P.batch) continue;
-            unsigned long long* word = P.acc + (size_t)b * P.Mp + rt * RABIT_TILE_ROWS + rl;
-            if (!RABIT_IN_RANGE(rt * RABIT_TILE_ROWS + rl < P.Mp && b < RABIT_LUT_MAX_BATCH)) continue;
+            if (b >= P.batch || arrivals == 1) continue;
+            unsigned long long* word = L.acc + (size_t)b * L.Mp + rt * RABIT_TILE_ROWS + rl;
+            if (!RABIT_IN_RANGE(rt * RABIT_TILE_ROWS + rl < L.Mp && b < RABIT_LUT_MAX_BATCH)) continue;
             if (bad[i]) atomicOr(word, 1ULL << 63);                      // sticky: the add below never carries into bit 63
             old[i] = atomicAdd(word, add[i]);
         }
 #pragma unroll
         for (int i = 0; i < kPer; ++i) {
-            const int o = tid + i * kGroupThreads, b = o >> 7, rl = o & 127;
-            if (b >= P.batch) continue;
+            const int o = tid + i * kThreads, b = o >> 7, rl = o & 127;
+            if (b >= P.batch || arrivals == 1) continue;
             if ((int)((old[i] >> 55) & 0xFFu) != arrivals - 1) continue;  // other segments of the row tile are still to come
             const unsigned long long sum = (old[i] & kSumMask) + (add[i] & kSumMask);
-            const long long total = (long long)sum - ((long long)P.n_cs << P.fix_bits);
+            const long long total = (long long)sum - ((long long)n_cs << L.fix_bits);
             const bool poisoned = bad[i] || (old[i] >> 63) != 0;
-            const float v = poisoned ? __int_as_float(0x7FC00000) : __ll2float_rn(total) * P.unit;
+            const float v = poisoned ? __int_as_float(0x7FC00000) : __ll2float_rn(total) * L.unit;
             const int row = rt * RABIT_TILE_ROWS + rl;
-            if (row < P.M) P.y[(size_t)b * P.M + row] = __float2half_rn(v);
-            P.acc[(size_t)b * P.Mp + row] = 0ULL;                         // resting state for the next call
+            if (row < L.M) L.y[(size_t)b * L.M + row] = __float2half_rn(v);
+            L.acc[(size_t)b * L.Mp + row] = 0ULL;                         // resting state for the next call
         }
-        group_sync(group);                                               // the slots are free for the next segment
+        __syncthreads();                                               // the slots are free for the next segment
     }
     if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -358,7 +366,7 @@ rabit_gemv_f16_kernel(const __grid_constant__ F16Params P) {
 template <int NH>
 cudaError_t launch(const F16Params& P, int grid, int device, cudaStream_t stream) {
     static bool attr_done[64] = {false};
-    const size_t smem = (size_t)kGroups * ((size_t)kWarps * NH * 8 * kSlotStride * sizeof(float) + (size_t)kWarps * kRing * 512);
+    const size_t smem = (size_t)kWarps * NH * 8 * kSlotStride * sizeof(float) + (size_t)kWarps * kRing * 512;
     const int slot = device >= 0 && device < 64 ? device : 0;
     if (!attr_done[slot] || slot != device) {
         cudaError_t e = cudaFuncSetAttribute(rabit_gemv_f16_kernel<NH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -378,104 +386,113 @@ cudaError_t launch(const F16Params& P, int grid, int device, cudaStream_t stream
     return cudaLaunchKernelEx(&cfg, rabit_gemv_f16_kernel<NH>, P);
 }
 
-}  // namespace
+struct Split {
+    int m, j, n_cta;
+    double us;                                                           // estimate
+};
 
-namespace {
-
-// Cuts the n_rt * n_cs (row tile, slice) pairs, in that order, into one contiguous range per SM and every SM's range into
-// two parts, one per group of its CTA.  A group's cost is its pairs plus `seg` for every segment after its first (a part
-// that crosses a row-tile boundary adds up and publishes twice, and while it does so its SM runs at half strength; the last
-// segment end is the same for everybody); an SM's cost is that of its slower group under the best cut between the two
-// parts, which is often the row-tile boundary itself.  The SM ranges are grown greedily under a cost limit and the
-// smallest limit that needs no more than `sms` ranges is found by bisection, so SMs whose range holds a boundary get
-// fewer pairs.  (Equal ranges cut in the middle, the previous form, left such SMs 30-40 % late; equal-cost parts
-// handed to independent CTAs, two per SM wherever the hardware put them, gave SMs unequal sums.)
-// bound[] receives the starts of the 2 * grid parts (bound[2 * grid] = n_pairs); returns grid.  Plans are cached per thread.
-int plan_ranges(int n_rt, int n_cs, int K, int NH, int sms, int* bound) {
-    struct Plan { int n_rt, n_cs, K, NH, sms, grid; int bound[kMaxRanges + 1]; };
-    static thread_local std::vector<Plan> plans;
-    for (const Plan& pl : plans)
-        if (pl.n_rt == n_rt && pl.n_cs == n_cs && pl.K == K && pl.NH == NH && pl.sms == sms) {
-            std::memcpy(bound, pl.bound, sizeof(pl.bound));
-            return pl.grid;
+// Cuts the n_rt * n_cs (row tile, slice) pairs into at most `ctas` ranges: every row tile into m equal units, j consecutive units
+// per CTA, for the m with the smallest estimate.  m = 1 is whole row tiles (no atomics), m = ctas / n_rt equal parts of
+// one, larger m ranges that cross row tiles.  The estimate, from timelines on B200: a tile takes 78 (up to eight batch rows)
+// or 108 clocks, a segment end inside a range 1.5 us, publishing parts of row tiles 0.6 us plus 128 * batch words per part
+// at 80 words per clock over the whole GPU.
+Split split_layer(int n_rt, int n_cs, int K, int batch, int ctas) {
+    const double pair_us = 8.0 * K * (batch > 8 ? 108.0 : 78.0) / 1900.0;
+    Split best = {1, 1, 0, 1e300};
+    for (int m = 1; m <= n_cs; ++m) {
+        const long long units = (long long)n_rt * m;
+        const int j = (int)((units + ctas - 1) / ctas), n = (int)((units + j - 1) / j);
+        // ranges repeat after lcm(m, j) units, so the first few CTAs show the worst one
+        double worst = 0.0;
+        long long parts = 0;                                             // segments that are not whole row tiles
+        const int look = std::min(n, m + 1);
+        for (int c = 0; c < look; ++c) {
+            const long long a = unit_start(c * j, m, n_cs), b = unit_start((int)std::min<long long>(units, (long long)(c + 1) * j), m, n_cs);
+            const long long segments = (b - 1) / n_cs - a / n_cs + 1;
+            const int cut = (a % n_cs != 0) + (b % n_cs != 0);
+            parts += segments == 1 && cut == 2 ? 1 : cut;
+            worst = std::max(worst, (double)(b - a) * pair_us + 1.5 * (double)(segments - 1));
         }
-    const long long n_pairs = (long long)n_rt * n_cs;
-    const int max_grid = (int)std::min<long long>(std::min(sms, kMaxRanges / kGroups), n_pairs);
-    // fitted to timelines on B200: a group works through a tile of a pair (8 K tiles) in about 0.068 us (NH = 1) or 0.085 us
-    // (NH = 2), a segment end takes it 3 to 3.5 us
-    const double seg = (NH == 1 ? 3.0 : 3.5) / (8.0 * K * (NH == 1 ? 0.068 : 0.085));
-    auto part_cost = [&](long long a, long long b) {                     // pairs [a, b) as one group's part
-        if (b <= a) return 0.0;
-        const long long segments = (b - 1) / n_cs - a / n_cs + 1;
-        return (double)(b - a) + seg * (double)(segments - 1);
-    };
-    auto best_cut = [&](long long a, long long b, double* cost) {        // the cut of [a, b) that makes the slower group fastest
-        long long best = b;
-        double best_cost = part_cost(a, b);
-        for (long long m = a + 1; m < b; ++m) {
-            const double c = std::max(part_cost(a, m), part_cost(m, b));
-            if (c < best_cost) { best_cost = c; best = m; }
-        }
-        *cost = best_cost;
-        return best;
-    };
-    auto cut_all = [&](double limit, int* out) {                         // greedy SM ranges under the limit; returns their number
-        int n = 0;
-        long long a = 0;
-        while (a < n_pairs) {
-            long long lo = a + 1, hi = std::min<long long>(n_pairs, a + 4 * (long long)limit + 8);   // largest b with cost <= limit
-            while (lo < hi) {
-                const long long mid = (lo + hi + 1) / 2;
-                double c;
-                best_cut(a, mid, &c);
-                if (c <= limit) lo = mid; else hi = mid - 1;
-            }
-            if (out && n < max_grid) {
-                double c;
-                out[kGroups * n] = (int)a;
-                out[kGroups * n + 1] = (int)best_cut(a, lo, &c);
-            }
-            ++n;
-            if (n > max_grid && !out) return n;
-            a = lo;
-        }
-        return n;
-    };
-    double lo = 1.0, hi = (double)n_pairs + seg * (n_rt + 1) + 1.0;
-    if (n_pairs <= max_grid) {
-        lo = hi = 0.5;                                                   // fewer pairs than SMs: one pair, one group per SM (a group alone on its SM is faster than two)
-    } else if (cut_all(lo, nullptr) > max_grid) {
-        for (int it = 0; it < 40; ++it) {
-            const double mid = 0.5 * (lo + hi);
-            if (cut_all(mid, nullptr) <= max_grid) hi = mid; else lo = mid;
-        }
-    } else {
-        hi = lo;
+        const double us = worst + (parts ? 0.6 + (double)parts * n / look * 128.0 * batch / 80.0 / 1900.0 : 0.0);
+        if (us < best.us) best = Split{m, j, n, us};
+        if (units >= 64LL * ctas) break;                                 // finer cuts change nothing any more
     }
-    int tmp[kMaxRanges + 2];
-    const int grid = cut_all(hi, tmp);
-    for (int r = 0; r <= kMaxRanges; ++r) bound[r] = r < kGroups * grid ? tmp[r] : (int)n_pairs;
+    return best;
+}
+
+// A launch's split.  CTAs in proportion to the pairs, at least one per layer; then one at a time from what is left, or from
+// the layer that would finish first, to the one that would finish last while that helps.  Remembered per thread by shape
+// (a decoder calls the same few groups over and over).
+struct GroupPlan {
+    int n, K, batch, sms, shape[kMaxGroup][2];
+    Split split[kMaxGroup];
+};
+GroupPlan plan_group(int n, const int (*shape)[2], int K, int batch, int sms) {
+    static thread_local std::vector<GroupPlan> plans;
+    for (const GroupPlan& pl : plans)
+        if (pl.n == n && pl.K == K && pl.batch == batch && pl.sms == sms && std::memcmp(pl.shape, shape, sizeof(int) * 2 * n) == 0) return pl;
+    GroupPlan pl;
+    std::memset(&pl, 0, sizeof(pl));
+    pl.n = n; pl.K = K; pl.batch = batch; pl.sms = sms;
+    std::memcpy(pl.shape, shape, sizeof(int) * 2 * n);
+    const int ctas = std::max(sms, n);
+    long long total = 0;
+    for (int l = 0; l < n; ++l) total += (long long)shape[l][0] * shape[l][1];
+    int give[kMaxGroup], given = 0;
+    for (int l = 0; l < n; ++l) {
+        give[l] = (int)std::max<long long>(1, (long long)ctas * shape[l][0] * shape[l][1] / total);
+        given += give[l];
+    }
+    while (given > ctas) {                                               // (many tiny layers beside a large one)
+        int big = 0;
+        for (int l = 1; l < n; ++l) if (give[l] > give[big]) big = l;
+        --give[big]; --given;
+    }
+    auto cut = [&](int l, int c) { return split_layer(shape[l][0], shape[l][1], K, batch, c); };
+    for (int l = 0; l < n; ++l) pl.split[l] = cut(l, n == 1 ? ctas : give[l]);
+    for (int iter = 0; iter < 24 && n > 1; ++iter) {
+        int hi = 0, lo = -1;
+        for (int l = 1; l < n; ++l) if (pl.split[l].us > pl.split[hi].us) hi = l;
+        bool better = false;
+        for (int take = 1; take <= ctas - given && !better; ++take) {    // the smallest number of spare CTAs that helps the slowest layer
+            const Split up = cut(hi, give[hi] + take);
+            if (up.us < pl.split[hi].us - 1e-9) { give[hi] += take; given += take; pl.split[hi] = up; better = true; }
+        }
+        for (int l = 0; l < n && !better; ++l)
+            if (l != hi && give[l] > 1 && (lo < 0 || pl.split[l].us < pl.split[lo].us)) lo = l;
+        if (!better && lo >= 0) {
+            const Split up = cut(hi, give[hi] + 1), down = cut(lo, give[lo] - 1);
+            if (std::max(up.us, down.us) < pl.split[hi].us - 1e-9) {
+                give[hi] += 1; give[lo] -= 1;
+                pl.split[hi] = up; pl.split[lo] = down;
+                better = true;
+            }
+        }
+        if (!better) break;
+    }
     if (plans.size() >= 256) plans.clear();
-    plans.emplace_back();
-    Plan& pl = plans.back();
-    pl.n_rt = n_rt; pl.n_cs = n_cs; pl.K = K; pl.NH = NH; pl.sms = sms; pl.grid = grid;
-    std::memcpy(pl.bound, bound, sizeof(pl.bound));
-    return grid;
+    plans.push_back(pl);
+    return pl;
 }
 
 }  // namespace
 
-// Host-only view of the work split (for tests): the starts of the 2 * grid group parts of a K-path layer of M x N at
-// `batch` rows on `sms` SMs; bound_out receives 2 * grid + 1 values, the last being the number of pairs.
+// Host-only view of the work split (for tests): two entries per CTA, the start of its range and its end (a range is not divided
+// any further: the second part is empty), for a K-path layer of M x N at `batch` rows on `sms` SMs; bound_out receives
+// 2 * grid + 1 values, the last being the number of pairs.
 int rabit_gemv_f16_plan(int K, int M, int N, int batch, int sms, int* bound_out, int max_out) {
     if (K < 1 || K > RABIT_MAX_K || M < 1 || N < 32 || (N % 32) != 0 || batch < 1 || batch > RABIT_MAX_GEMV_BATCH || sms < 1) return -1;
     const long long n_rt = ((long long)M + RABIT_TILE_ROWS - 1) / RABIT_TILE_ROWS, n_cs = ((long long)N + RABIT_LUT_COLS - 1) / RABIT_LUT_COLS;
     if (n_cs > RABIT_LUT_MAX_SLICES || n_rt * n_cs >= kMaxPairs) return -1;
-    int bound[kMaxRanges + 1];
-    const int grid = plan_ranges((int)n_rt, (int)n_cs, K, batch > 8 ? 2 : 1, sms, bound);
-    if (max_out < kGroups * grid + 1) return -1;
-    for (int r = 0; r <= kGroups * grid; ++r) bound_out[r] = bound[r];
-    return grid;
+    const int shape[1][2] = {{(int)n_rt, (int)n_cs}};
+    const Split sp = plan_group(1, shape, K, batch, sms).split[0];
+    if (max_out < 2 * sp.n_cta + 1) return -1;
+    for (int c = 0; c < sp.n_cta; ++c) {
+        bound_out[2 * c] = unit_start(c * sp.j, sp.m, (int)n_cs);
+        bound_out[2 * c + 1] = unit_start((int)std::min(n_rt * sp.m, (long long)(c + 1) * sp.j), sp.m, (int)n_cs);
+    }
+    bound_out[2 * sp.n_cta] = (int)(n_rt * n_cs);
+    return sp.n_cta;
 }
 
 bool rabit_gemv_f16_supports(const rabit_layer& L, int batch) {
@@ -485,28 +502,55 @@ bool rabit_gemv_f16_supports(const rabit_layer& L, int batch) {
     return (long long)L.geom.n_rt * L.geom.n_cs < kMaxPairs;
 }
 
-// One launch, 1..16 batch rows (x: [batch][N], y: [batch][M]).
-cudaError_t rabit_launch_gemv_f16(const rabit_layer& L, const void* x, void* y, int batch, cudaStream_t stream) {
-    if (!rabit_gemv_f16_supports(L, batch)) return cudaErrorInvalidValue;
-    const RabitGeom& G = L.geom;
+bool rabit_gemv_f16_group_supports(const rabit_layer* const* layers, int n_layers, int batch) {
+    if (n_layers < 1 || n_layers > kMaxGroup) return false;
+    for (int l = 0; l < n_layers; ++l) {
+        if (!rabit_gemv_f16_supports(*layers[l], batch) || layers[l]->geom.K != layers[0]->geom.K) return false;
+        for (int m = 0; m < l; ++m)
+            if (layers[m] == layers[l]) return false;                    // one layer twice would share its accumulate words
+    }
+    return true;
+}
+
+// One launch for n_layers independent layers of equal K, 1..16 batch rows (x_l: [batch][N_l], y_l: [batch][M_l]).
+cudaError_t rabit_launch_gemv_f16_group(const rabit_layer* const* layers, int n_layers, const void* const* xs, void* const* ys, int batch, cudaStream_t stream) {
+    if (!rabit_gemv_f16_group_supports(layers, n_layers, batch)) return cudaErrorInvalidValue;
+    const int K = layers[0]->geom.K, sms = layers[0]->sm_count > 0 ? layers[0]->sm_count : 148;
+    int shape[kMaxGroup][2];
+    for (int l = 0; l < n_layers; ++l) { shape[l][0] = layers[l]->geom.n_rt; shape[l][1] = layers[l]->geom.n_cs; }
+    const GroupPlan pl = plan_group(n_layers, shape, K, batch, sms);
     F16Params P;
-    P.tiles = L.d_bits;
-    P.g = (const __half*)L.d_g;
-    P.h = (const __half*)L.d_h;
-    P.x = (const __half*)x;
-    P.y = (__half*)y;
-    P.acc = L.d_acc;
-    P.status = L.d_status;
-    P.K = G.K; P.M = G.M; P.N = G.N; P.Mp = G.Mp; P.n_rt = G.n_rt; P.n_ct = G.n_ct; P.n_cs = G.n_cs;
+    P.n_layers = n_layers;
+    P.K = K;
     P.batch = batch;
-    P.fix_bits = G.fix_bits;
-    P.unit = ldexpf(1.f, G.unit_exp);
-    P.inv_unit = ldexpf(1.f, -G.unit_exp);
-    P.limit = ldexpf(1.f, G.fix_bits);
     P.two = 2u;
     P.two_pow_8 = 256u;
-    P.n_pairs = G.n_rt * G.n_cs;
-    const int sms = L.sm_count > 0 ? L.sm_count : 148;
-    const int grid = plan_ranges(G.n_rt, G.n_cs, G.K, batch > 8 ? 2 : 1, sms, P.bound);   // one CTA (two groups of eight warps) per SM
-    return batch <= 8 ? launch<1>(P, grid, L.device, stream) : launch<2>(P, grid, L.device, stream);
+    int at = 0;
+    for (int l = 0; l < n_layers; ++l) {
+        const rabit_layer& Ly = *layers[l];
+        const RabitGeom& G = Ly.geom;
+        F16Layer& D = P.layer[l];
+        D.tiles = Ly.d_bits;
+        D.g = (const __half*)Ly.d_g;
+        D.h = (const __half*)Ly.d_h;
+        D.x = (const __half*)xs[l];
+        D.y = (__half*)ys[l];
+        D.acc = Ly.d_acc;
+        D.status = Ly.d_status;
+        D.M = G.M; D.N = G.N; D.Mp = G.Mp; D.n_rt = G.n_rt; D.n_ct = G.n_ct; D.n_cs = G.n_cs;
+        D.fix_bits = G.fix_bits;
+        D.unit = ldexpf(1.f, G.unit_exp);
+        D.inv_unit = ldexpf(1.f, -G.unit_exp);
+        D.limit = ldexpf(1.f, G.fix_bits);
+        D.cta0 = at; D.m = pl.split[l].m; D.j = pl.split[l].j;
+        D.pad_ = 0;
+        at += pl.split[l].n_cta;
+    }
+    for (int l = n_layers; l < kMaxGroup; ++l) P.layer[l] = P.layer[0];
+    return batch <= 8 ? launch<1>(P, at, layers[0]->device, stream) : launch<2>(P, at, layers[0]->device, stream);
+}
+
+cudaError_t rabit_launch_gemv_f16(const rabit_layer& L, const void* x, void* y, int batch, cudaStream_t stream) {
+    const rabit_layer* one = &L;
+    return rabit_launch_gemv_f16_group(&one, 1, &x, &y, batch, stream);
 }
