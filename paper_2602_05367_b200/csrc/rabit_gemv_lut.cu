@@ -52,14 +52,20 @@ constexpr int kMaxGroup = 8;
 constexpr unsigned long long kSumMask = (1ULL << 55) - 1;
 
 // Tables: one 64 KB table serves two paths, entry e of (path k, byte group) at  e * 256 + (k & 1) * 128 + group * 4
-// of table k >> 1.  The tables start on a 64 KB boundary of the CTA's shared-memory window, so that a table address
-// is  base | byte << 8 | bank offset  and ONE byte permute builds it whole (no add): see the look-up loop.
+// of table k >> 1.  The kernel has no static shared memory, so its dynamic part starts at kSmemBase, right behind what the
+// system reserves (checked on the host), and a look-up address is  byte << 8 | bank offset,  which ONE byte permute builds,
+// plus a constant that fits the load's immediate.  (Starting the tables on a 64 KB boundary instead costs 63 KB of slack and
+// sixteen registers for the table base.)
+constexpr int kSmemBase = 1024;
 template <int K, int NB>
 struct Tab {
     static constexpr int kTables = (K + 1) / 2;                       // per batch row
     static constexpr int kBytes = kTables * 65536;                    // per batch row
-    static constexpr int kSmem = 65536 + NB * kBytes;                 // alignment slack + tables
-    __host__ __device__ static constexpr int offset(int k, int b) { return b * kBytes + (k >> 1) * 65536 + (k & 1) * 128; }
+    static constexpr int kTail = 256;                                 // behind the tables: the layer's descriptor and the CTA's range
+    // Never so little that two CTAs share an SM: with 64 KB each the hardware put two CTAs of one launch on one SM wherever the
+    // previous launch left room first, and a 4096 x 4096 layer went from 3.2 to 4.4 us.
+    static constexpr int kSmem = NB * kBytes + kTail > 116 * 1024 ? NB * kBytes + kTail : 116 * 1024;
+    __host__ __device__ static constexpr int offset(int k, int b) { return kSmemBase + b * kBytes + (k >> 1) * 65536 + (k & 1) * 128; }
 };
 
 template <int I, int N, typename F>
@@ -168,13 +174,12 @@ template <int K>
 struct Blk {
     uint4 v[2 * K];                  // one lane's 32 bytes per path: (path k, half hf) at v[2k + hf]
 };
+// half hf (byte groups 16 hf .. of the rotated order) of block bb of the range, every path
 template <int K>
-__device__ __forceinline__ Blk<K> load_blk(const uint4* range_base, int bb, int lane) {
-    Blk<K> r;
+__device__ __forceinline__ void load_half(Blk<K>& r, int hf, const uint4* range_base, int bb, int lane) {
     const uint4* p = range_base + (size_t)bb * (K * RABIT_LUT_PART_BYTES / 16) + lane;
 #pragma unroll
-    for (int i = 0; i < 2 * K; ++i) r.v[i] = ldg_stream(p + i * 32);
-    return r;
+    for (int k = 0; k < K; ++k) r.v[2 * k + hf] = ldg_stream(p + (2 * k + hf) * 32);
 }
 
 // What a lane still owes for the last block it accumulated: the answer of its atomic add is looked at
@@ -206,7 +211,7 @@ template <int K, int NB>
 __global__ void __launch_bounds__(kThreads, 1)
 rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
     using T = Tab<K, NB>;
-    extern __shared__ __align__(1024) unsigned char smem[];             // slack up to a 64 KB boundary, then the tables
+    extern __shared__ __align__(1024) unsigned char smem[];             // the tables, then what the CTA needs of the launch parameters
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
 #ifdef RABIT_TRACE
@@ -218,8 +223,8 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
     // The launch parameters live in constant memory, which is cold in every new launch: a first touch of one of its
     // lines costs a trip to L2.  Everything the CTA needs later is therefore copied to shared memory now, before the
     // dependency wait, so that none of those trips lands between the arrival of x and the end of the kernel.
-    __shared__ LutLayer layer_copy;
-    __shared__ CtaRange range_copy;
+    LutLayer& layer_copy = *reinterpret_cast<LutLayer*>(smem + NB * T::kBytes);
+    CtaRange& range_copy = *reinterpret_cast<CtaRange*>(smem + NB * T::kBytes + 128);
     if (warp == 0) {
         const CtaRange r0 = P.range[blockIdx.x];
         const uint32_t* src = reinterpret_cast<const uint32_t*>(&P.layer[r0.layer]);
@@ -238,21 +243,19 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
     Blk<K> cur;                                          // this warp's current block
 #pragma unroll
     for (int i = 0; i < 2 * K; ++i) cur.v[i] = make_uint4(0u, 0u, 0u, 0u);
-    if (n_mine > 0) cur = load_blk<K>(range_base, warp, lane);
+    if (n_mine > 0) {
+        load_half<K>(cur, 0, range_base, warp, lane);
+        load_half<K>(cur, 1, range_base, warp, lane);
+    }
 
-    const uint32_t tab0 = (smem_u32(smem) + 65535u) & ~65535u;
-    // c[j][h]: bytes 0, 1 = bank offsets (4 * group) of the groups this lane visits in steps 4j + 2h and 4j + 2h + 1,
-    // bytes 2, 3 = the upper half of the table base.  A permute of (weight word, c) then yields a complete address.
-    uint32_t c[8][2];
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-            c[j][h] = (uint32_t)((((4 * j + 2 * h) + lane) & 31) * 4) | (uint32_t)((((4 * j + 2 * h + 1) + lane) & 31) * 4) << 8 | (tab0 & 0xFFFF0000u);
+    const uint32_t tab0 = smem_u32(smem);                // == kSmemBase
+    // byte q of `bank0 + 0x10101010 * j`, modulo 128: bank offset (4 * group) of the group this lane visits in step 4j + q.  A
+    // permute of (weight word, that) yields byte << 8 | bank offset (its upper bytes copy a sign bit that is always clear).
+    const uint32_t bank0 = (uint32_t)((lane * 4) & 127) | (uint32_t)((lane * 4 + 4) & 127) << 8 | (uint32_t)((lane * 4 + 8) & 127) << 16 | (uint32_t)((lane * 4 + 12) & 127) << 24;
     int cs = R.b0 / L.n_rb;
     int seg_rb0 = R.b0 - cs * L.n_rb;                    // row block of the first block of the current segment
     int seg_begin = 0, seg_end = min(n_blocks, L.n_rb - seg_rb0);       // blocks [seg_begin, seg_end) of the range use slice cs
-    constexpr int kPairs = (8 * K + kWarps - 1) / kWarps;                // (path, upper index bits) pairs a warp builds
+    constexpr int kPairs = (8 * K + kWarps - 1) / kWarps;                // (path, upper three index bits) pairs a warp builds, 32 entries each
     uint4 hq[kPairs], xq[NB];
     auto load_h = [&](int slice) {                                      // static data: may be read before the dependency wait
 #pragma unroll
@@ -302,7 +305,7 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
                 const uint32_t dst = tab0 + b * T::kBytes + (k >> 1) * 65536 + (ehi * 32) * 256 + (k & 1) * 128 + lane * 4;
 #pragma unroll
                 for (int e = 0; e < 32; ++e)
-                    if (RABIT_IN_RANGE(dst + e * 256 >= tab0 && dst + e * 256 + 4 <= tab0 + (uint32_t)(NB * T::kBytes) && dst + e * 256 + 4 <= smem_u32(smem) + (uint32_t)T::kSmem))
+                    if (RABIT_IN_RANGE(dst + e * 256 >= tab0 && dst + e * 256 + 4 <= tab0 + (uint32_t)(NB * T::kBytes)))
                         sts_f32(dst + e * 256, v[e]);
             }
         }
@@ -362,10 +365,8 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
             graw[k] = 0;
             if (RABIT_IN_RANGE(row >= 0 && row < Mp)) graw[k] = ldg_u16_early(g_base + (size_t)k * Mp + row);
         }
-        const int bb_next = i + 1 < n_mine ? bb + kWarps : bb;
-        Blk<K> nxt = cur;
-        if (RABIT_IN_RANGE(bb_next >= 0 && bb_next < n_blocks && (long long)R.b0 + bb_next < (long long)L.n_cs * L.n_rb))
-            nxt = load_blk<K>(range_base, bb_next, lane);   // (the last iteration re-reads its own block: in bounds, unused)
+        const int bb_next = i + 1 < n_mine ? bb + kWarps : bb;           // (the last iteration re-reads its own block: in bounds, unused)
+        const bool next_ok = RABIT_IN_RANGE(bb_next >= 0 && bb_next < n_blocks && (long long)R.b0 + bb_next < (long long)L.n_cs * L.n_rb);
         if (owe) {
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
@@ -391,19 +392,22 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
         for (int b = 0; b < NB; ++b)
 #pragma unroll
             for (int k = 0; k < K; ++k) acc[b][k][0] = acc[b][k][1] = 0.f;
+        // (the next block's weights are loaded into the registers that the look-ups have freed, half by half: half a block,
+        // some 1200 clocks, ahead of their use)
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
+        for (int j = 0; j < 8; ++j) {
+            const uint32_t bank = (bank0 + 0x10101010u * (uint32_t)j) & 0x7F7F7F7Fu;
             static_for<0, K>([&](auto kc) {
                 constexpr int k = decltype(kc)::value;
                 const uint4 part = cur.v[2 * k + (j >> 2)];
                 const uint32_t w = (j & 3) == 0 ? part.x : (j & 3) == 1 ? part.y : (j & 3) == 2 ? part.z : part.w;
-                // address = table base | sign byte << 8 | bank offset, all from one permute
-                const uint32_t a0 = prmt(w, c[j][0], 0x7604), a1 = prmt(w, c[j][0], 0x7615);
-                const uint32_t a2 = prmt(w, c[j][1], 0x7624), a3 = prmt(w, c[j][1], 0x7635);
+                // sign byte << 8 | bank offset, from one permute
+                const uint32_t a0 = prmt(w, bank, 0xCC04), a1 = prmt(w, bank, 0xCC15);
+                const uint32_t a2 = prmt(w, bank, 0xCC26), a3 = prmt(w, bank, 0xCC37);
 #ifdef RABIT_CHECKED
                 {
-                    const uint32_t lo = tab0, hi = tab0 + 65536u - 128u;     // with the path offset added: inside table k >> 1
-                    if (!RABIT_IN_RANGE(a0 >= lo && a0 < hi && a1 >= lo && a1 < hi && a2 >= lo && a2 < hi && a3 >= lo && a3 < hi)) return;
+                    const uint32_t hi = 65536u - 128u;                   // with the path offset added: inside table k >> 1
+                    if (!RABIT_IN_RANGE(a0 < hi && a1 < hi && a2 < hi && a3 < hi)) return;
                 }
 #endif
                 static_for<0, NB>([&](auto bc) {
@@ -414,6 +418,9 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
                     acc[b][k][1] += lds_f32<T::offset(k, b)>(a3);
                 });
             });
+            if (j == 3 && next_ok) load_half<K>(cur, 0, range_base, bb_next, lane);
+            if (j == 7 && next_ok) load_half<K>(cur, 1, range_base, bb_next, lane);
+        }
 #ifdef RABIT_TRACE
         if (i == 0) RABIT_STAMP(7);                                     // first block's look-ups issued
         if (i < 11 && use_here_u64(__float_as_uint(acc[0][0][0] + acc[0][0][1] + acc[0][K - 1][0] + acc[0][K - 1][1])) != 0x13572468u) RABIT_STAMP(10 + 5 * i);   // look-ups answered
@@ -442,9 +449,6 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
             pd[b].bad = bad;
         }
         owe = true;
-#pragma unroll
-        for (int t = 0; t < 2 * K; ++t) cur.v[t] = nxt.v[t];             // the next block's weights have arrived by now
-        cur.v[0].x = (unsigned int)use_here_u64(cur.v[0].x);
     }
     if (owe) {
 #pragma unroll
@@ -541,8 +545,19 @@ cudaError_t launch_k(int K, int batch, const LutParams& P, int grid, int device,
 
 int rabit_gemv_lut_max_rows() { return 2; }
 
+// whether dynamic shared memory starts where the look-up addresses assume it
+static bool smem_base_ok(int device) {
+    static signed char known[64] = {0};                                  // 0 not asked yet, 1 yes, -1 no
+    signed char* k = device >= 0 && device < 64 ? &known[device] : nullptr;
+    if (k && *k) return *k > 0;
+    int reserved = -1;
+    const bool ok = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, device) == cudaSuccess && reserved == kSmemBase;
+    if (k) *k = ok ? 1 : -1;
+    return ok;
+}
+
 bool rabit_gemv_lut_supports(const rabit_layer& L, int batch) {
-    if (batch < 1 || batch > 2) return false;
+    if (batch < 1 || batch > 2 || !smem_base_ok(L.device)) return false;
     if (L.geom.K == 3 && batch > 1) return false;                        // four 64 KB tables do not fit into shared memory
     if (L.geom.n_cs > RABIT_LUT_MAX_SLICES) return false;
     return (long long)L.geom.n_cs * L.geom.n_rb < (1LL << 30) && L.d_lut != nullptr && L.d_acc != nullptr;
