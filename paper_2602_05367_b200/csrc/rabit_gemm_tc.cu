@@ -15,7 +15,7 @@
 // elected lane of a uniform loop): from a divergent single thread an MMA costs 90 to 125 clocks of issue whatever its N.
 //
 // Warps of a CTA:
-//   0      producer: per 64-column step the x rows by TMA (128-byte swizzle) into one ring, per eight steps the packed sign
+//   0      producer: per one to four 64-column steps the x rows by TMA (128-byte swizzle) into one ring, per eight steps the packed sign
 //          tiles and the h slices of every path by bulk copies into another; the first weights set off before the
 //          dependency wait.  (Few, large copies: with one per step and path, and x in boxes of 16 rows, this warp was
 //          what the CTA waited for: 28672 x 8192 at batch 512 390 us with boxes of 16 rows, 350 with two boxes a step.)
@@ -41,6 +41,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <cstddef>
 #include <type_traits>
 #include <vector>
 
@@ -75,7 +76,7 @@ struct GemmParams {
     long long n_groups;                     // row tiles * n16
     int max16;                              // most groups one pass can accumulate
     int split;                              // CTAs (one cluster) that share the contraction of a task: 1, 2, 4 or 8
-    int stages, stage_bytes;                // x ring (stage_bytes: one stage)
+    int stages, stage_bytes, x_steps;       // x ring: bytes and steps of one stage
     int w_stages;                           // weight ring, behind the x ring: per stage the sign tiles [K][8][512], then h [K][256]
     int box16;                              // groups of 16 batch columns per TMA box
     int n_acc;                              // accumulators (and issuing warps)
@@ -113,12 +114,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
                  : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {   // never blocks
-    uint32_t ok;
-    asm volatile("{ .reg .pred p; mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0;
-}
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
     if (mbar_try_wait(bar, parity)) return;
     const long long t0 = clock64();
@@ -133,6 +128,20 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                  ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+                 ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(bar) : "memory");
+}
+__device__ __forceinline__ uint4 lds_v4(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ uint2 lds_v2(uint32_t addr) {
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
+    return v;
 }
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
@@ -257,7 +266,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
     if (tid == 0) {
         for (int s = 0; s < stages; ++s) {
             mbar_init(smem_u32(&S.full[s]), 1);
-            mbar_init(smem_u32(&S.empty[s]), n_ops);
+            mbar_init(smem_u32(&S.empty[s]), P.n_acc);
         }
         for (int s = 0; s < w_stages; ++s) {
             mbar_init(smem_u32(&S.w_full[s]), 1);
@@ -325,23 +334,27 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
     if (warp == 0) {
         // ===================================== producer =====================================
         const bool elected = elect_one();
-        int it = 0, w_at = 0;                                    // steps and weight stages begun, over all passes
+        int it = 0, w_at = 0;                                    // x and weight stages begun, over all passes
         Walk at{0};
         PassWalker w(P, task);
         Pass ps;
         while (w.next(P, ps)) {
             const int boxes = (ps.n + P.box16 - 1) / P.box16;
-            for (int s = s_lo; s < s_hi; ++s, ++it) {
-                if ((s - s_lo) % kWSteps == 0) {
+            const uint32_t box_bytes = (uint32_t)(P.box16 * (kGroupCols * kStepCols * 2) * P.x_steps), tx = boxes * box_bytes;   // (what lies outside x arrives as zeros)
+            for (int s = s_lo; s < s_hi; s += P.x_steps, ++it) {
+                if ((s - s_lo) % kWSteps == 0) {                 // (x_steps divides kWSteps)
                     ++w_at;                                      // two stages behind the ring's depth: never held up by the stage in use
                     while (feed.more && feed.issued < w_at + w_stages - 2) feed_next(elected);
                 }
                 const uint32_t bar = smem_u32(&S.full[at.slot]), dst = smem_u32(ring + at.slot * stage_bytes);
                 if (it >= stages) mbar_wait(smem_u32(&S.empty[at.slot]), at.lap ^ 1u, abort_flag);
                 if (elected) {
-                    mbar_expect_tx(bar, (uint32_t)(boxes * P.box16 * (kGroupCols * kStepCols * 2)));
-                    for (int c = 0; c < boxes; ++c)
-                        tma_load_2d(dst + c * P.box16 * (kGroupCols * kStepCols * 2), &x_map, s * kStepCols, (ps.c16 + c * P.box16) * kGroupCols, bar);
+                    mbar_expect_tx(bar, tx);
+                    if (P.x_steps > 1) {
+                        tma_load_3d(dst, &x_map, 0, ps.c16 * kGroupCols, s, bar);
+                    } else {
+                        for (int c = 0; c < boxes; ++c) tma_load_2d(dst + c * box_bytes, &x_map, s * kStepCols, (ps.c16 + c * P.box16) * kGroupCols, bar);
+                    }
                 }
                 __syncwarp();
                 at.step(1, stages);
@@ -355,46 +368,48 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
             constexpr int m = decltype(acc)::value;
             const int n_acc = P.n_acc;
             const bool elected = elect_one();
-            int pass_i = 0, u = m, u_end = 0;
-            Walk uw{m}, xw{n_ops == 1 ? m : 0};                  // units and x stages of this accumulator
-            const int x_stride = n_ops == 1 ? n_acc : 1;
+            int pass_i = 0;
+            Walk uw{m}, xw{0};                                   // units of this accumulator, x stages
+            const int u_stride = n_ops == 1 ? n_acc : 1;         // steps from one of its units to the next
             const uint32_t full0 = smem_u32(&S.full[0]), empty0 = smem_u32(&S.empty[0]), a_ready0 = smem_u32(&S.a_ready[0]), a_empty0 = smem_u32(&S.a_empty[0]);
             const uint64_t bdesc0 = umma_desc(smem_u32(ring));
             const uint32_t a0 = tmem_base + (uint32_t)P.a_col, d = tmem_base + (uint32_t)(m * P.max16 * kGroupCols);
+            const uint32_t step_bytes = (uint32_t)stage_bytes / (uint32_t)P.x_steps;
+            int steps_before = 0;                                // of earlier passes
             PassWalker w(P, task);
             Pass ps;
             while (w.next(P, ps)) {
                 const uint32_t idesc = __shfl_sync(0xFFFFFFFFu, umma_idesc(ps.n * kGroupCols), 0);
                 if (pass_i > 0) mbar_wait(smem_u32(&S.acc_empty), (pass_i - 1) & 1, abort_flag);   // epilogue has drained the accumulators
                 ++pass_i;
-                const int u_short = (n_ct & 1) && s_hi == n_steps ? u_end + (s_hi - s_lo - 1) * n_ops : 0x7FFFFFFF;   // units from here on hold one column tile
-                u_end += (s_hi - s_lo) * n_ops;
                 uint32_t accumulate = 0u;
-                bool ready = mbar_test(a_ready0 + uw.slot * 8, uw.lap), x_ready = mbar_test(full0 + xw.slot * 8, xw.lap);
-                for (; u < u_end; u += n_acc) {
-                    const int us = uw.slot, slot = xw.slot;
-                    if (!x_ready) mbar_wait(full0 + slot * 8, xw.lap, abort_flag);
-                    if (!ready) mbar_wait(a_ready0 + us * 8, uw.lap, abort_flag);
-                    fence_after();
-                    uw.step(n_acc, units);
-                    xw.step(x_stride, stages);
-                    ready = mbar_test(a_ready0 + uw.slot * 8, uw.lap);                             // asked early, used next time round
-                    x_ready = mbar_test(full0 + xw.slot * 8, xw.lap);
-                    const uint64_t bdesc = bdesc0 + (uint64_t)((slot * stage_bytes) >> 4);
-                    const uint32_t a = a0 + us * kUnitCols;
-                    if (elected) {
-                        umma_f16_ts(d, a, bdesc, idesc, accumulate);
-                        umma_f16_ts(d, a + 8, bdesc + 2, idesc, 1u);
-                        if (u < u_short) {
-                            umma_f16_ts(d, a + 16, bdesc + 4, idesc, 1u);
-                            umma_f16_ts(d, a + 24, bdesc + 6, idesc, 1u);
+                for (int s = s_lo; s < s_hi; s += P.x_steps) {
+                    const int n_here = min(P.x_steps, s_hi - s);
+                    mbar_wait(full0 + xw.slot * 8, xw.lap, abort_flag);
+                    const uint64_t bdesc = bdesc0 + (uint64_t)((xw.slot * stage_bytes) >> 4);
+                    for (int si = n_ops == 1 && n_acc > 1 ? (m ^ (steps_before + s - s_lo)) & 1 : 0; si < n_here; si += u_stride) {
+                        mbar_wait(a_ready0 + uw.slot * 8, uw.lap, abort_flag);
+                        fence_after();
+                        const uint64_t bd = bdesc + (uint64_t)((si * step_bytes) >> 4);
+                        const uint32_t a = a0 + uw.slot * kUnitCols;
+                        if (elected) {
+                            umma_f16_ts(d, a, bd, idesc, accumulate);
+                            umma_f16_ts(d, a + 8, bd + 2, idesc, 1u);
+                            if (2 * (s + si) + 1 < n_ct) {       // (the last step may hold one column tile)
+                                umma_f16_ts(d, a + 16, bd + 4, idesc, 1u);
+                                umma_f16_ts(d, a + 24, bd + 6, idesc, 1u);
+                            }
+                            umma_commit(a_empty0 + uw.slot * 8);
                         }
-                        umma_commit(a_empty0 + us * 8);
-                        umma_commit(empty0 + slot * 8);
+                        accumulate = 1u;
+                        __syncwarp();
+                        uw.step(n_acc, units);
                     }
-                    accumulate = 1u;
+                    if (elected) umma_commit(empty0 + xw.slot * 8);
                     __syncwarp();
+                    xw.step(1, stages);
                 }
+                steps_before += s_hi - s_lo;
                 if (elected) umma_commit(smem_u32(&S.acc_ready));
                 __syncwarp();
             }
@@ -408,10 +423,21 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
         const int gq = lane >> 2, tq = lane & 3;
         const uint32_t lane_base = tmem_base + ((uint32_t)(32 * q) << 16);
         const int shift = 6 - 2 * q;                          // bit p of a byte to its top: a shift by 7 - p, this for p = 2q + 1 and one more for p = 2q
-        const uint32_t w_full0 = smem_u32(&S.w_full[0]), w_empty0 = smem_u32(&S.w_empty[0]), a_ready0 = smem_u32(&S.a_ready[0]), a_empty0 = smem_u32(&S.a_empty[0]);
-        const uint32_t a0 = lane_base + (uint32_t)P.a_col;
-        Walk uw{grp}, ww{0};
-        int pass_i = 0, u0 = 0, u = grp;                      // u: this group's next unit, counted over all passes
+        // Integer instructions take two issue clocks each and bound this loop (80 of them a unit and warp are the expansion
+        // itself), so everything around them is kept in few registers that only step: a group always has the same path, and
+        // its units alternate between the same one or two places in tensor memory.
+        const int path = grp % n_ops;
+        constexpr int kStepsOn = n_groups / n_ops;            // steps from one of the group's units to its next
+        const uint32_t dst0 = lane_base + (uint32_t)(P.a_col + grp * kUnitCols), dst_sum = 2 * dst0 + (units > n_groups ? n_groups * kUnitCols : 0);
+        const uint32_t bar0 = smem_u32(&S.a_empty[grp]), bar_sum = 2 * bar0 + (units > n_groups ? n_groups * 8u : 0u);
+        constexpr uint32_t kBack = (uint32_t)(offsetof(Control, a_empty) - offsetof(Control, a_ready));   // from a unit's a_empty barrier to its a_ready
+        const int lap_bit = units > n_groups ? 1 : 0;
+        const uint32_t w_full0 = smem_u32(&S.w_full[0]), w_empty0 = smem_u32(&S.w_empty[0]);
+        const uint32_t bits0 = smem_u32(w_ring) + lane * 16 + (DEQ ? 0 : path * kWTiles * RABIT_TILE_BYTES);
+        const uint32_t h0 = smem_u32(w_ring) + K * kWTiles * RABIT_TILE_BYTES + 8 * tq + (DEQ ? 0 : path * kWTiles * RABIT_TILE_COLS * 2);
+        uint32_t dst = dst0, bar = bar0, done = 0;            // done: the group's units so far
+        Walk ww{0};
+        int pass_i = 0, u0 = 0;
         PassWalker w(P, task);
         Pass ps;
         while (w.next(P, ps)) {
@@ -425,71 +451,68 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
                         for (int rh = 0; rh < 2; ++rh)
                             g_rows[k][pi][rh] = __half2half2(P.g[(size_t)k * P.Mp + ps.rt * kTileM + 32 * q + 16 * pi + gq + 8 * rh]);
             }
-            const int u_end = u0 + (s_hi - s_lo) * n_ops;
+            const int first = ((grp - u0 % n_groups + n_groups) % n_groups) / n_ops;   // the group's first step of the pass, and of each of its weight stages
             for (int j = 0; j < n_w && grp < n_groups; ++j) {
-              const unsigned char* w_stage = w_ring + ww.slot * (K * kWBytes) + lane * 16;
-              const unsigned char* h_stage = w_ring + ww.slot * (K * kWBytes) + K * kWTiles * RABIT_TILE_BYTES + 8 * tq;
-              const int uj = u0 + j * kWSteps * n_ops, uj_end = min(uj + kWSteps * n_ops, u_end);
-              mbar_wait(w_full0 + ww.slot * 8, ww.lap, abort_flag);
-              for (; u < uj_end; u += n_groups) {
-                const int sj = (u - uj) / n_ops, k = (u - uj) - sj * n_ops, us = uw.slot;
-                const unsigned char* bits = w_stage + sj * 2 * RABIT_TILE_BYTES;
-                const unsigned char* hs = h_stage + sj * kStepCols * 2;
-                if (u >= units) {
-                    mbar_wait(a_empty0 + us * 8, uw.lap ^ 1u, abort_flag);
+                const int step0 = s_lo + j * kWSteps, n_here = min(kWSteps, s_hi - step0), whole = min(n_here, n_ct / 2 - step0);   // steps with two column tiles
+                uint32_t bits = bits0 + ww.slot * (K * kWBytes) + first * (2 * RABIT_TILE_BYTES), hs = h0 + ww.slot * (K * kWBytes) + first * (kStepCols * 2);
+                mbar_wait(w_full0 + ww.slot * 8, ww.lap, abort_flag);
+                for (int sj = first; sj < n_here; sj += kStepsOn) {
+                    mbar_wait(bar, ((done >> lap_bit) & 1u) ^ 1u, abort_flag);             // (the first time round this is the barrier's previous phase: free)
                     fence_after();
-                }
-                const uint32_t dst = a0 + us * kUnitCols;
-                auto expand_tile = [&](int ct2) {
-                    uint32_t o[2][8];                                                      // [row block][16-column half, row half, column pair]
-                    // dequantised: sum_k +-g_k[row] h_k[col], accumulated from the last (smallest) path to the first with one
-                    // fused multiply-add per path
+                    auto expand_tile = [&](int ct2) {
+                        uint32_t o[2][8];                                                  // [row block][16-column half, row half, column pair]
+                        // dequantised: sum_k +-g_k[row] h_k[col], accumulated from the last (smallest) path to the first with one
+                        // fused multiply-add per path
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) o[0][i] = o[1][i] = 0u;
+                        for (int i = 0; i < 8; ++i) o[0][i] = o[1][i] = 0u;
 #pragma unroll
-                    for (int kk = DEQ ? K - 1 : 0; kk >= 0; --kk) {
-                        const int kp = DEQ ? kk : k;
-                        const uint4 wv = *reinterpret_cast<const uint4*>(bits + (kp * kWTiles + ct2) * RABIT_TILE_BYTES);
-                        const uint32_t word[4] = {wv.x, wv.y, wv.z, wv.w};
+                        for (int kk = DEQ ? K - 1 : 0; kk >= 0; --kk) {
+                            const uint4 wv = lds_v4(bits + (kk * kWTiles + ct2) * RABIT_TILE_BYTES);
+                            const uint32_t word[4] = {wv.x, wv.y, wv.z, wv.w};
 #pragma unroll
-                        for (int ah = 0; ah < 2; ++ah) {
-                            const uint2 hv = *reinterpret_cast<const uint2*>(hs + (kp * kWTiles * RABIT_TILE_COLS + 32 * ct2 + 16 * ah) * 2);
+                            for (int ah = 0; ah < 2; ++ah) {
+                                const uint2 hv = lds_v2(hs + (kk * kWTiles * RABIT_TILE_COLS + 32 * ct2 + 16 * ah) * 2);
 #pragma unroll
-                            for (int rh = 0; rh < 2; ++rh)
+                                for (int rh = 0; rh < 2; ++rh)
 #pragma unroll
-                                for (int pair = 0; pair < 2; ++pair) {
-                                    // bytes [0, c0, 0, c1]: bit p of the pair's columns at 8 + p and 24 + p
-                                    const uint32_t v = __byte_perm(word[2 * ah + rh], 0u, pair ? 0x3424 : 0x1404) << shift;
-                                    const uint32_t hp = pair ? hv.y : hv.x;
+                                    for (int pair = 0; pair < 2; ++pair) {
+                                        // bytes [0, c0, 0, c1]: bit p of the pair's columns at 8 + p and 24 + p
+                                        const uint32_t v = __byte_perm(word[2 * ah + rh], 0u, pair ? 0x3424 : 0x1404) << shift;
+                                        const uint32_t hp = pair ? hv.y : hv.x;
 #pragma unroll
-                                    for (int pi = 0; pi < 2; ++pi) {
-                                        const uint32_t m = ((pi ? v : v << 1) & 0x80008000u) ^ hp;
-                                        uint32_t& a = o[pi][4 * ah + 2 * rh + pair];
-                                        if (DEQ) {
-                                            const __half2 sum = __hfma2(g_rows[kk][pi][rh], *reinterpret_cast<const __half2*>(&m), *reinterpret_cast<const __half2*>(&a));
-                                            a = *reinterpret_cast<const uint32_t*>(&sum);
-                                        } else {
-                                            a = m;
+                                        for (int pi = 0; pi < 2; ++pi) {
+                                            const uint32_t m = ((pi ? v : v << 1) & 0x80008000u) ^ hp;
+                                            uint32_t& a = o[pi][4 * ah + 2 * rh + pair];
+                                            if (DEQ) {
+                                                const __half2 sum = __hfma2(g_rows[kk][pi][rh], *reinterpret_cast<const __half2*>(&m), *reinterpret_cast<const __half2*>(&a));
+                                                a = *reinterpret_cast<const uint32_t*>(&sum);
+                                            } else {
+                                                a = m;
+                                            }
                                         }
                                     }
-                                }
+                            }
                         }
-                    }
-                    tmem_st_16x256b_x2(dst + ct2 * 16, o[0]);
-                    tmem_st_16x256b_x2(dst + ct2 * 16 + (16u << 16), o[1]);
-                };
-                expand_tile(0);
-                if (2 * (s_lo + j * kWSteps + sj) + 1 < n_ct) expand_tile(1);
-                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                fence_before();
+                        tmem_st_16x256b_x2(dst + ct2 * 16, o[0]);
+                        tmem_st_16x256b_x2(dst + ct2 * 16 + (16u << 16), o[1]);
+                    };
+                    expand_tile(0);
+                    if (sj < whole) expand_tile(1);
+                    bits += kStepsOn * 2 * RABIT_TILE_BYTES;
+                    hs += kStepsOn * kStepCols * 2;
+                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                    fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar - kBack);
+                    dst = dst_sum - dst;
+                    bar = bar_sum - bar;
+                    ++done;
+                }
                 __syncwarp();
-                if (lane == 0) mbar_arrive(a_ready0 + us * 8);
-                uw.step(n_groups, units);
-              }
-              if (lane == 0) mbar_arrive(w_empty0 + ww.slot * 8);
-              ww.step(1, w_stages);
+                if (lane == 0) mbar_arrive(w_empty0 + ww.slot * 8);
+                ww.step(1, w_stages);
             }
-            u0 = u_end;
+            u0 += (s_hi - s_lo) * n_ops;
             if (split > 1) break;                              // the cluster's epilogue follows the role branches
             // ---- epilogue of this pass
             mbar_wait(smem_u32(&S.acc_ready), pass_i & 1, abort_flag);
@@ -613,24 +636,25 @@ EncodeTiledFn encode_tiled_fn() {
     return fn;
 }
 
-// Descriptor of x [batch][N] in boxes of 16 * box16 rows x 64 columns.  A pure function of its arguments; the last few are
+// Descriptor of x [batch][N] in boxes of 16 * box16 rows x 64 columns, or x_steps such boxes side by side.  A pure function of its arguments; the last few are
 // remembered per thread (encoding one costs about a microsecond of host time).
-cudaError_t x_tensor_map(const void* x, int N, int batch, int box16, CUtensorMap* out) {
-    struct Entry { const void* x; int N, batch, box16; CUtensorMap map; };
+cudaError_t x_tensor_map(const void* x, int N, int batch, int box16, int x_steps, CUtensorMap* out) {
+    struct Entry { const void* x; int N, batch, box16, x_steps; CUtensorMap map; };
     static thread_local Entry recent[8];
     static thread_local int next = 0;
     for (const Entry& e : recent)
-        if (e.x == x && e.N == N && e.batch == batch && e.box16 == box16) { *out = e.map; return cudaSuccess; }
+        if (e.x == x && e.N == N && e.batch == batch && e.box16 == box16 && e.x_steps == x_steps) { *out = e.map; return cudaSuccess; }
     EncodeTiledFn encode = encode_tiled_fn();
     if (!encode) return cudaErrorNotSupported;
-    const cuuint64_t dims[2] = {(cuuint64_t)N, (cuuint64_t)batch};
-    const cuuint64_t strides[1] = {(cuuint64_t)N * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kStepCols, (cuuint32_t)(box16 * kGroupCols)};
-    const cuuint32_t estr[2] = {1, 1};
-    if (encode(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(x), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+    // (with several steps per box N is a multiple of 64, so that no box reads beyond a row)
+    const cuuint64_t dims[3] = {(cuuint64_t)(x_steps > 1 ? kStepCols : N), (cuuint64_t)batch, (cuuint64_t)(N / kStepCols)};
+    const cuuint64_t strides[2] = {(cuuint64_t)N * 2, (cuuint64_t)kStepCols * 2};
+    const cuuint32_t box[3] = {(cuuint32_t)kStepCols, (cuuint32_t)(box16 * kGroupCols), (cuuint32_t)x_steps};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    if (encode(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, x_steps > 1 ? 3 : 2, const_cast<void*>(x), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
-    recent[next] = Entry{x, N, batch, box16, *out};
+    recent[next] = Entry{x, N, batch, box16, x_steps, *out};
     next = (next + 1) & 7;
     return cudaSuccess;
 }
@@ -639,24 +663,29 @@ cudaError_t x_tensor_map(const void* x, int N, int batch, int box16, CUtensorMap
 
 struct Plan {
     int chunks, chunk16, split, max16, tasks;        // chunks == 0: contiguous group ranges
-    int stages, stage_bytes, w_stages, box16, units, n_acc;
+    int stages, stage_bytes, x_steps, w_stages, box16, units, n_acc;
     size_t smem;
     double clocks;                                   // estimate
 };
 
 // Ring, tensor-memory and shared-memory figures of passes of up to max16 groups; false if they do not fit.  The units are a
-// multiple of the expander groups and of the accumulators (see Walk), the x stages of two for the same reason.
-bool fill_resources(Plan& p, int K, int n_ops, int steps) {
+// multiple of the expander groups and of the accumulators (see Walk).
+bool fill_resources(Plan& p, int K, int n_ops, int steps, bool one_box) {
     if (p.max16 * kGroupCols > 256) return false;
     const int turn = n_ops == 3 ? 3 : 4;
     auto free_units = [&](int n_acc) { return (512 - n_acc * p.max16 * kGroupCols) / kUnitCols; };
     p.n_acc = n_ops > 1 ? n_ops : steps >= 2 && free_units(2) >= turn ? 2 : 1;
     if (free_units(p.n_acc) < turn) return false;
     p.units = free_units(p.n_acc) >= 2 * turn ? 2 * turn : turn;
-    p.stage_bytes = (p.max16 + p.box16 - 1) / p.box16 * p.box16 * kGroupCols * kStepCols * 2;
+    const int step_bytes = (p.max16 + p.box16 - 1) / p.box16 * p.box16 * kGroupCols * kStepCols * 2;
     const int room = (226 - 1) * 1024 - kControlBytes;
-    p.stages = std::min(kMaxStages, (room - 3 * K * kWBytes) / p.stage_bytes / 2 * 2);
-    if (p.stages < 4) return false;
+    // as many steps per x stage (one copy of the producer, which needs some 600 clocks for each) as leave three stages
+    for (p.x_steps = one_box ? 4 : 1;; p.x_steps /= 2) {
+        p.stage_bytes = step_bytes * p.x_steps;
+        p.stages = std::min(kMaxStages, (room - 3 * K * kWBytes) / p.stage_bytes);
+        if (p.stages >= (p.x_steps > 1 ? 3 : 4)) break;
+        if (p.x_steps == 1) return false;
+    }
     p.w_stages = std::min(kMaxWStages, (room - p.stages * p.stage_bytes) / (K * kWBytes));
     // Never so little that two CTAs could share an SM: each takes all of its tensor memory, and of two clusters waiting
     // crosswise for each other's neither would ever get it.
@@ -710,7 +739,7 @@ constexpr double kPassClocks = 3000.0;               // pipeline fill and epilog
 constexpr double kLaunchClocks = 5000.0;             // launch, first loads, last epilogue
 constexpr double kExchangeClocks = 1500.0;           // cluster barriers and exchange of a split task
 
-Plan make_plan(int n_rt, int n_steps, int K, bool deq, int n16, int sms, int device) {
+Plan make_plan(int n_rt, int n_steps, int K, bool deq, int n16, int sms, int device, bool wide_x) {
     const int n_ops = deq ? 1 : K;
     Plan best = {};
     best.clocks = 1e300;
@@ -719,7 +748,7 @@ Plan make_plan(int n_rt, int n_steps, int K, bool deq, int n16, int sms, int dev
         Plan p = {};
         p.max16 = p.chunk16 = p.box16 = (n16 + chunks - 1) / chunks;
         p.chunks = (n16 + p.chunk16 - 1) / p.chunk16;
-        if (p.chunks != chunks || !fill_resources(p, K, n_ops, n_steps / 8)) continue;
+        if (p.chunks != chunks || !fill_resources(p, K, n_ops, n_steps / 8, wide_x)) continue;
         for (int split = 1; split <= 8; split *= 2) {
             p.split = split;
             p.tasks = n_rt * chunks;
@@ -747,9 +776,9 @@ Plan make_plan(int n_rt, int n_steps, int K, bool deq, int n16, int sms, int dev
             // most passes of a range are cut to this size: two boxes of it make one step
             const int run = std::min(per_sm, n16), pieces = (run + p.max16 - 1) / p.max16;
             p.box16 = ((run + pieces - 1) / pieces + 1) / 2;
-            if (fill_resources(p, K, n_ops, n_steps)) break;
+            if (fill_resources(p, K, n_ops, n_steps, false)) break;
         }
-        if (fill_resources(p, K, n_ops, n_steps)) {
+        if (fill_resources(p, K, n_ops, n_steps, false)) {
             double worst = 0.0;
             for (int t = 0; t < sms; ++t) {
                 long long g = groups * t / sms;
@@ -772,13 +801,13 @@ Plan make_plan(int n_rt, int n_steps, int K, bool deq, int n16, int sms, int dev
 int sms_of(const rabit_layer& L) { return L.sm_count > 0 ? L.sm_count : 148; }
 
 Plan plan_for(const rabit_layer& L, bool deq, int batch) {
-    struct Entry { int n_rt, n_steps, K, deq, n16, sms; Plan plan; };
+    struct Entry { int n_rt, n_ct, K, deq, n16, sms; Plan plan; };
     static thread_local std::vector<Entry> plans;     // a search costs tens of microseconds; a program calls few shapes
-    const int n16 = (batch + kGroupCols - 1) / kGroupCols, n_rt = L.geom.n_rt, n_steps = (L.geom.N + kStepCols - 1) / kStepCols, K = L.geom.K, sms = sms_of(L);
+    const int n16 = (batch + kGroupCols - 1) / kGroupCols, n_rt = L.geom.n_rt, n_ct = L.geom.n_ct, K = L.geom.K, sms = sms_of(L);
     for (const Entry& e : plans)
-        if (e.n_rt == n_rt && e.n_steps == n_steps && e.K == K && e.deq == (int)deq && e.n16 == n16 && e.sms == sms) return e.plan;
+        if (e.n_rt == n_rt && e.n_ct == n_ct && e.K == K && e.deq == (int)deq && e.n16 == n16 && e.sms == sms) return e.plan;
     if (plans.size() >= 256) plans.clear();
-    plans.push_back(Entry{n_rt, n_steps, K, (int)deq, n16, sms, make_plan(n_rt, n_steps, K, deq, n16, sms, L.device)});
+    plans.push_back(Entry{n_rt, n_ct, K, (int)deq, n16, sms, make_plan(n_rt, (n_ct + 1) / 2, K, deq, n16, sms, L.device, n_ct % 2 == 0)});
     return plans.back().plan;
 }
 
@@ -796,7 +825,7 @@ cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, i
     const Plan p = plan_for(L, dequantised, batch);
     if (p.tasks < 1) return cudaErrorInvalidValue;
     CUtensorMap map;
-    cudaError_t e = x_tensor_map(x, G.N, batch, p.box16, &map);
+    cudaError_t e = x_tensor_map(x, G.N, batch, p.box16, p.x_steps, &map);
     if (e != cudaSuccess) return e;
     e = prepare_kernel(G.K, dequantised, L.device);
     if (e != cudaSuccess) return e;
@@ -815,7 +844,7 @@ cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, i
     P.n_groups = (long long)G.n_rt * P.n16;
     P.max16 = p.max16;
     P.split = p.split;
-    P.stages = p.stages; P.stage_bytes = p.stage_bytes; P.w_stages = p.w_stages;
+    P.stages = p.stages; P.stage_bytes = p.stage_bytes; P.x_steps = p.x_steps; P.w_stages = p.w_stages;
     P.box16 = p.box16;
     P.n_acc = p.n_acc;
     P.units = p.units; P.a_col = p.n_acc * p.max16 * kGroupCols;
