@@ -468,7 +468,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
 #pragma unroll
                         for (int kk = DEQ ? K - 1 : 0; kk >= 0; --kk) {
                             const uint4 wv = lds_v4(bits + (kk * kWTiles + ct2) * RABIT_TILE_BYTES);
-                            const uint32_t word[4] = {wv.x, wv.y, wv.z, wv.w};
+                            const uint32_t word[4] = {wv.x << shift, wv.y << shift, wv.z << shift, wv.w << shift};
 #pragma unroll
                             for (int ah = 0; ah < 2; ++ah) {
                                 const uint2 hv = lds_v2(hs + (kk * kWTiles * RABIT_TILE_COLS + 32 * ct2 + 16 * ah) * 2);
@@ -476,19 +476,19 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
                                 for (int rh = 0; rh < 2; ++rh)
 #pragma unroll
                                     for (int pair = 0; pair < 2; ++pair) {
-                                        // bytes [0, c0, 0, c1]: bit p of the pair's columns at 8 + p and 24 + p
-                                        const uint32_t v = __byte_perm(word[2 * ah + rh], 0u, pair ? 0x3424 : 0x1404) << shift;
+                                        // bytes [0, c0, 0, c1]: row block 2q + 1's bits at 15 and 31, row block 2q's one below
+                                        const uint32_t v = __byte_perm(word[2 * ah + rh], 0u, pair ? 0x3424 : 0x1404);
                                         const uint32_t hp = pair ? hv.y : hv.x;
+                                        // bit 14 alone is the fp16 number 2: h - 2 h or h - 0 h, exact, and a floating operation costs half an integer one
+                                        const uint32_t two = v & 0x40004000u, odd = (v & 0x80008000u) ^ hp;
+                                        const __half2 h2 = *reinterpret_cast<const __half2*>(&hp);
+                                        const __half2 even2 = __hfma2(*reinterpret_cast<const __half2*>(&two), __hneg2(h2), h2);
 #pragma unroll
                                         for (int pi = 0; pi < 2; ++pi) {
-                                            const uint32_t m = ((pi ? v : v << 1) & 0x80008000u) ^ hp;
+                                            const __half2 m = pi ? *reinterpret_cast<const __half2*>(&odd) : even2;
                                             uint32_t& a = o[pi][4 * ah + 2 * rh + pair];
-                                            if (DEQ) {
-                                                const __half2 sum = __hfma2(g_rows[kk][pi][rh], *reinterpret_cast<const __half2*>(&m), *reinterpret_cast<const __half2*>(&a));
-                                                a = *reinterpret_cast<const uint32_t*>(&sum);
-                                            } else {
-                                                a = m;
-                                            }
+                                            const __half2 r = DEQ ? __hfma2(g_rows[DEQ ? kk : 0][pi][rh], m, *reinterpret_cast<const __half2*>(&a)) : m;
+                                            a = *reinterpret_cast<const uint32_t*>(&r);
                                         }
                                     }
                             }
