@@ -76,6 +76,7 @@ struct GemmParams {
     long long n_groups;                     // row tiles * n16
     int max16;                              // most groups one pass can accumulate
     int split;                              // CTAs (one cluster) that share the contraction of a task: 1, 2, 4 or 8
+    int recv_off;                           // receive buffer of a split task, from the control block
     int stages, stage_bytes, x_steps;       // x ring: bytes and steps of one stage
     int w_stages;                           // weight ring, behind the x ring: per stage the sign tiles [K][8][512], then h [K][256]
     int box16;                              // groups of 16 batch columns per TMA box
@@ -214,25 +215,26 @@ struct Pass {
     int rt, c16, n;                         // row tile, first group, groups
 };
 struct PassWalker {
-    long long g, g1;
+    int rt, c16, left;                      // where the next pass starts, groups left in the task
     __device__ PassWalker(const GemmParams& P, int task) {
         if (P.chunks > 0) {
-            const int rt = task / P.chunks, c = (task - rt * P.chunks) * P.chunk16;
-            g = (long long)rt * P.n16 + c;
-            g1 = g + min(P.chunk16, P.n16 - c);
+            rt = task / P.chunks;
+            c16 = (task - rt * P.chunks) * P.chunk16;
+            left = min(P.chunk16, P.n16 - c16);
         } else {
-            g = P.n_groups * task / P.n_tasks;
-            g1 = P.n_groups * (task + 1) / P.n_tasks;
+            const long long g = P.n_groups * task / P.n_tasks;
+            rt = (int)(g / P.n16);
+            c16 = (int)(g - (long long)rt * P.n16);
+            left = (int)(P.n_groups * (task + 1) / P.n_tasks - g);
         }
     }
     __device__ bool next(const GemmParams& P, Pass& ps) {
-        if (g >= g1) return false;
-        ps.rt = (int)(g / P.n16);
-        ps.c16 = (int)(g - (long long)ps.rt * P.n16);
-        const int run = (int)min(g1 - g, (long long)(P.n16 - ps.c16));
-        const int pieces = (run + P.max16 - 1) / P.max16;
-        ps.n = (run + pieces - 1) / pieces;
-        g += ps.n;
+        if (left <= 0) return false;
+        const int run = min(left, P.n16 - c16), pieces = run <= P.max16 ? 1 : (run + P.max16 - 1) / P.max16;
+        ps = Pass{rt, c16, pieces == 1 ? run : (run + pieces - 1) / pieces};
+        left -= ps.n;
+        c16 += ps.n;
+        if (c16 == P.n16) { c16 = 0; ++rt; }
         return true;
     }
 };
@@ -245,12 +247,20 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
     // the swizzled x tiles need 1024-byte alignment; the launch reserves the slack
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     Control& S = *reinterpret_cast<Control*>(smem);
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
+    // The launch parameters sit in constant memory, cold in every launch (a first touch is a trip to L2, several in a row
+    // between the dependency wait and the first MMA): touched here once.  So is the tensor map.  (A copy of them in shared
+    // memory is no better: the values are then not uniform to the compiler, and the issuers' loops grow by 15 %.)
+    if (tid < (int)(sizeof(GemmParams) / 4)) {
+        const uint32_t word = reinterpret_cast<const uint32_t*>(&P)[tid];
+        asm volatile("" ::"r"(word));
+    }
+    if (tid == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&x_map) : "memory");
     unsigned char* ring = smem + kControlBytes;
     unsigned char* w_ring = ring + P.stages * P.stage_bytes;
-    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
     constexpr int n_ops = DEQ ? 1 : K;                            // operand units (and accumulators) per step
     constexpr int n_groups = n_ops == 3 ? 3 : 4;                  // expander groups at work
-    const int stages = P.stages, w_stages = P.w_stages, units = P.units;
+    const int stages = P.stages, w_stages = P.w_stages, units = P.units, x_steps = P.x_steps, n_acc = P.n_acc;
     const int stage_bytes = P.stage_bytes, n_ct = P.n_ct;
     const int n_steps = (P.N + kStepCols - 1) / kStepCols;        // N % 32 == 0: the last step may hold one column tile only
     volatile int* abort_flag = &S.abort_flag;
@@ -282,6 +292,21 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    if (split > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // (awaited before the exchange: every CTA of the cluster runs)
+    const PassWalker first_pass(P, task);
+    // Output scales of the row whose accumulators this thread reads: loaded when a pass begins, converted (which waits for
+    // them) when it ends.
+    unsigned short graw[K];
+    auto load_scales = [&](int rt) {
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(graw[k]) : "l"(P.g + (size_t)k * P.Mp + rt * kTileM + (warp & 3) * 32 + lane));
+    };
+    auto scale = [&](int k) {
+        unsigned short r;
+        asm volatile("mov.b16 %0, %1;" : "=h"(r) : "h"(graw[k]));
+        return __half2float(__ushort_as_half(r));
+    };
 
     const int n_w = (s_hi - s_lo + kWSteps - 1) / kWSteps;        // weight stages of a pass
     // weight stage j of a pass over row tile rt into slot `slot` (these do not depend on the stream's past)
@@ -304,7 +329,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
         Walk at;
         bool more;
     };
-    WeightFeed feed{PassWalker(P, task), Pass{}, 0, 0, Walk{0}, false};
+    WeightFeed feed{first_pass, Pass{}, 0, 0, Walk{0}, false};
     auto feed_next = [&](bool elected) {
         if (feed.issued >= w_stages) mbar_wait(smem_u32(&S.w_empty[feed.at.slot]), feed.at.lap ^ 1u, abort_flag);
         if (elected) load_weights(feed.ps.rt, feed.j, feed.at.slot);
@@ -336,12 +361,12 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
         const bool elected = elect_one();
         int it = 0, w_at = 0;                                    // x and weight stages begun, over all passes
         Walk at{0};
-        PassWalker w(P, task);
+        PassWalker w = first_pass;
         Pass ps;
         while (w.next(P, ps)) {
             const int boxes = (ps.n + P.box16 - 1) / P.box16;
-            const uint32_t box_bytes = (uint32_t)(P.box16 * (kGroupCols * kStepCols * 2) * P.x_steps), tx = boxes * box_bytes;   // (what lies outside x arrives as zeros)
-            for (int s = s_lo; s < s_hi; s += P.x_steps, ++it) {
+            const uint32_t box_bytes = (uint32_t)(P.box16 * (kGroupCols * kStepCols * 2) * x_steps), tx = boxes * box_bytes;   // (what lies outside x arrives as zeros)
+            for (int s = s_lo; s < s_hi; s += x_steps, ++it) {
                 if ((s - s_lo) % kWSteps == 0) {                 // (x_steps divides kWSteps)
                     ++w_at;                                      // two stages behind the ring's depth: never held up by the stage in use
                     while (feed.more && feed.issued < w_at + w_stages - 2) feed_next(elected);
@@ -350,7 +375,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
                 if (it >= stages) mbar_wait(smem_u32(&S.empty[at.slot]), at.lap ^ 1u, abort_flag);
                 if (elected) {
                     mbar_expect_tx(bar, tx);
-                    if (P.x_steps > 1) {
+                    if (x_steps > 1) {
                         tma_load_3d(dst, &x_map, 0, ps.c16 * kGroupCols, s, bar);
                     } else {
                         for (int c = 0; c < boxes; ++c) tma_load_2d(dst + c * box_bytes, &x_map, s * kStepCols, (ps.c16 + c * P.box16) * kGroupCols, bar);
@@ -366,7 +391,6 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
         // issues: see the header.)
         auto issue_units = [&](auto acc) {
             constexpr int m = decltype(acc)::value;
-            const int n_acc = P.n_acc;
             const bool elected = elect_one();
             int pass_i = 0;
             Walk uw{m}, xw{0};                                   // units of this accumulator, x stages
@@ -374,17 +398,17 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
             const uint32_t full0 = smem_u32(&S.full[0]), empty0 = smem_u32(&S.empty[0]), a_ready0 = smem_u32(&S.a_ready[0]), a_empty0 = smem_u32(&S.a_empty[0]);
             const uint64_t bdesc0 = umma_desc(smem_u32(ring));
             const uint32_t a0 = tmem_base + (uint32_t)P.a_col, d = tmem_base + (uint32_t)(m * P.max16 * kGroupCols);
-            const uint32_t step_bytes = (uint32_t)stage_bytes / (uint32_t)P.x_steps;
+            const uint32_t step_bytes = (uint32_t)stage_bytes / (uint32_t)x_steps;
             int steps_before = 0;                                // of earlier passes
-            PassWalker w(P, task);
+            PassWalker w = first_pass;
             Pass ps;
             while (w.next(P, ps)) {
                 const uint32_t idesc = __shfl_sync(0xFFFFFFFFu, umma_idesc(ps.n * kGroupCols), 0);
                 if (pass_i > 0) mbar_wait(smem_u32(&S.acc_empty), (pass_i - 1) & 1, abort_flag);   // epilogue has drained the accumulators
                 ++pass_i;
                 uint32_t accumulate = 0u;
-                for (int s = s_lo; s < s_hi; s += P.x_steps) {
-                    const int n_here = min(P.x_steps, s_hi - s);
+                for (int s = s_lo; s < s_hi; s += x_steps) {
+                    const int n_here = min(x_steps, s_hi - s);
                     mbar_wait(full0 + xw.slot * 8, xw.lap, abort_flag);
                     const uint64_t bdesc = bdesc0 + (uint64_t)((xw.slot * stage_bytes) >> 4);
                     for (int si = n_ops == 1 && n_acc > 1 ? (m ^ (steps_before + s - s_lo)) & 1 : 0; si < n_here; si += u_stride) {
@@ -415,8 +439,8 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
             }
         };
         if (warp == 1) issue_units(std::integral_constant<int, 0>{});
-        else if (warp == 2 && P.n_acc > 1) issue_units(std::integral_constant<int, 1>{});
-        else if (warp == 3 && P.n_acc > 2) issue_units(std::integral_constant<int, 2>{});
+        else if (warp == 2 && n_acc > 1) issue_units(std::integral_constant<int, 1>{});
+        else if (warp == 3 && n_acc > 2) issue_units(std::integral_constant<int, 2>{});
     } else if (warp >= 4) {
         // ============================ expanders, then epilogue ============================
         const int grp = (warp - 4) >> 2, q = warp & 3;        // tensor-memory lanes this warp may touch: 32q .. 32q + 31
@@ -438,7 +462,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
         uint32_t dst = dst0, bar = bar0, done = 0;            // done: the group's units so far
         Walk ww{0};
         int pass_i = 0, u0 = 0;
-        PassWalker w(P, task);
+        PassWalker w = first_pass;
         Pass ps;
         while (w.next(P, ps)) {
             __half2 g_rows[DEQ ? K : 1][2][2];                 // DEQ: output scales of this thread's rows (row block, row half), both halves alike
@@ -451,6 +475,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
                         for (int rh = 0; rh < 2; ++rh)
                             g_rows[k][pi][rh] = __half2half2(P.g[(size_t)k * P.Mp + ps.rt * kTileM + 32 * q + 16 * pi + gq + 8 * rh]);
             }
+            load_scales(ps.rt);
             const int first = ((grp - u0 % n_groups + n_groups) % n_groups) / n_ops;   // the group's first step of the pass, and of each of its weight stages
             for (int j = 0; j < n_w && grp < n_groups; ++j) {
                 const int step0 = s_lo + j * kWSteps, n_here = min(kWSteps, s_hi - step0), whole = min(n_here, n_ct / 2 - step0);   // steps with two column tiles
@@ -519,9 +544,6 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
             ++pass_i;
             fence_after();
             const int row = ps.rt * kTileM + q * 32 + lane;
-            float gk[K];
-#pragma unroll
-            for (int k = 0; k < K; ++k) gk[k] = __half2float(P.g[(size_t)k * P.Mp + row]);
 #pragma unroll 1
             for (int c = grp; c < ps.n; c += kExpandGroups) {
                 float v[16];
@@ -529,11 +551,11 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
                 for (int i = 0; i < 16; ++i) v[i] = 0.f;
 #pragma unroll
                 for (int m = 0; m < (n_ops == 1 ? 2 : n_ops); ++m) {
-                    if (n_ops == 1 && m >= P.n_acc) break;
+                    if (n_ops == 1 && m >= n_acc) break;
                     uint32_t d[16];
                     tmem_ld16(lane_base + (uint32_t)((m * P.max16 + c) * kGroupCols), d);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    const float gm = DEQ ? 1.f : gk[n_ops == 1 ? 0 : m];
+                    const float gm = DEQ ? 1.f : scale(n_ops == 1 ? 0 : m);
 #pragma unroll
                     for (int i = 0; i < 16; ++i) v[i] = fmaf(gm, __uint_as_float(d[i]), v[i]);
                 }
@@ -554,10 +576,9 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
     if (split > 1) {
         // ---- epilogue of a split task.  Every CTA of the cluster holds a partial result in tensor memory.  Group c of 16
         //      batch columns is finished by CTA c % split: all CTAs send it that group's columns (already scaled by g_k and
-        //      summed over the paths) into its receive buffer recv[its c / split][source rank][column][row] (the input ring's
-        //      memory: nothing uses it once every CTA's MMAs have retired, which the first cluster barrier
-        //      establishes).  After the second barrier each CTA adds what it received in rank order and stores fp16.
-        PassWalker w(P, task);
+        //      summed over the paths) into its receive buffer recv[its c / split][source rank][column][row], behind the rings.
+        //      After the cluster barrier each CTA adds what it received in rank order and stores fp16.
+        PassWalker w = first_pass;
         Pass ps;
         w.next(P, ps);
         if (warp >= 4) {
@@ -565,14 +586,10 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
             fence_after();
         }
         __syncwarp();
-        cluster_sync_all();
-        float* recv = reinterpret_cast<float*>(ring);
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        float* recv = reinterpret_cast<float*>(smem + P.recv_off);
         if (warp >= 4) {
             const int grp = (warp - 4) >> 2, q = warp & 3, r_in = q * 32 + lane;
-            const int row = ps.rt * kTileM + r_in;
-            float gk[K];
-#pragma unroll
-            for (int k = 0; k < K; ++k) gk[k] = __half2float(P.g[(size_t)k * P.Mp + row]);
 #pragma unroll 1
             for (int c = grp; c < ps.n; c += kExpandGroups) {
                 float v[16];
@@ -580,11 +597,11 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
                 for (int i = 0; i < 16; ++i) v[i] = 0.f;
 #pragma unroll
                 for (int m = 0; m < (n_ops == 1 ? 2 : n_ops); ++m) {
-                    if (n_ops == 1 && m >= P.n_acc) break;
+                    if (n_ops == 1 && m >= n_acc) break;
                     uint32_t d[16];
                     tmem_ld16(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)((m * P.max16 + c) * kGroupCols), d);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    const float gm = DEQ ? 1.f : gk[n_ops == 1 ? 0 : m];
+                    const float gm = DEQ ? 1.f : scale(n_ops == 1 ? 0 : m);
 #pragma unroll
                     for (int i = 0; i < 16; ++i) v[i] = fmaf(gm, __uint_as_float(d[i]), v[i]);
                 }
@@ -663,7 +680,7 @@ cudaError_t x_tensor_map(const void* x, int N, int batch, int box16, int x_steps
 
 struct Plan {
     int chunks, chunk16, split, max16, tasks;        // chunks == 0: contiguous group ranges
-    int stages, stage_bytes, x_steps, w_stages, box16, units, n_acc;
+    int stages, stage_bytes, x_steps, w_stages, box16, units, n_acc, recv_off;
     size_t smem;
     double clocks;                                   // estimate
 };
@@ -671,6 +688,7 @@ struct Plan {
 // Ring, tensor-memory and shared-memory figures of passes of up to max16 groups; false if they do not fit.  The units are a
 // multiple of the expander groups and of the accumulators (see Walk).
 bool fill_resources(Plan& p, int K, int n_ops, int steps, bool one_box) {
+    const int recv_bytes = p.split > 1 ? (p.chunk16 + p.split - 1) / p.split * p.split * kGroupCols * kTileM * 4 : 0;
     if (p.max16 * kGroupCols > 256) return false;
     const int turn = n_ops == 3 ? 3 : 4;
     auto free_units = [&](int n_acc) { return (512 - n_acc * p.max16 * kGroupCols) / kUnitCols; };
@@ -678,27 +696,28 @@ bool fill_resources(Plan& p, int K, int n_ops, int steps, bool one_box) {
     if (free_units(p.n_acc) < turn) return false;
     p.units = free_units(p.n_acc) >= 2 * turn ? 2 * turn : turn;
     const int step_bytes = (p.max16 + p.box16 - 1) / p.box16 * p.box16 * kGroupCols * kStepCols * 2;
-    const int room = (226 - 1) * 1024 - kControlBytes;
+    const int room = (226 - 1) * 1024 - kControlBytes - recv_bytes;
     // as many steps per x stage (one copy of the producer, which needs some 600 clocks for each) as leave three stages
     for (p.x_steps = one_box ? 4 : 1;; p.x_steps /= 2) {
         p.stage_bytes = step_bytes * p.x_steps;
-        p.stages = std::min(kMaxStages, (room - 3 * K * kWBytes) / p.stage_bytes);
+        p.stages = std::max(0, std::min(kMaxStages, (room - 3 * K * kWBytes) / p.stage_bytes));
         if (p.stages >= (p.x_steps > 1 ? 3 : 4)) break;
         if (p.x_steps == 1) return false;
     }
     p.w_stages = std::min(kMaxWStages, (room - p.stages * p.stage_bytes) / (K * kWBytes));
     // Never so little that two CTAs could share an SM: each takes all of its tensor memory, and of two clusters waiting
     // crosswise for each other's neither would ever get it.
-    p.smem = std::max<size_t>(1024 + kControlBytes + (size_t)p.stages * p.stage_bytes + (size_t)p.w_stages * K * kWBytes, 152 * 1024);
+    p.recv_off = kControlBytes + p.stages * p.stage_bytes + p.w_stages * K * kWBytes;
+    p.smem = std::max<size_t>(1024 + (size_t)p.recv_off + recv_bytes, 152 * 1024);
     return true;
 }
 
-// Clocks of a (step, path) unit: four MMAs of the pass's batch columns, or the expansion of its two sign tiles (measured 270 to
-// 290 per unit and SM: about 165 clocks of integer issue, the rest hand-over; more if a group has only one unit's room
-// in tensor memory and has to wait for its MMAs).
+// Clocks of a (step, path) unit, fitted on B200: four MMAs of the pass's batch columns, or the expansion of its two sign tiles
+// (about 130 clocks of integer issue and 50 around them; more if a group has only one unit's room in tensor memory and has
+// to wait for its MMAs).
 double unit_clocks(int n16, const Plan& p, int n_ops) {
     const bool two_each = p.units >= 2 * (n_ops == 3 ? 3 : 4);
-    return std::max(32.0 * n16 + 40.0, two_each ? 280.0 : n_ops == 3 ? 410.0 : 320.0);
+    return std::max(32.0 * n16 + 52.0, two_each ? 180.0 + 8.0 * n16 : n_ops == 3 ? 345.0 : 300.0);
 }
 
 const void* kernel_for(int K, bool deq) {
@@ -748,16 +767,14 @@ Plan make_plan(int n_rt, int n_steps, int K, bool deq, int n16, int sms, int dev
         Plan p = {};
         p.max16 = p.chunk16 = p.box16 = (n16 + chunks - 1) / chunks;
         p.chunks = (n16 + p.chunk16 - 1) / p.chunk16;
-        if (p.chunks != chunks || !fill_resources(p, K, n_ops, n_steps / 8, wide_x)) continue;
+        if (p.chunks != chunks) continue;
         for (int split = 1; split <= 8; split *= 2) {
             p.split = split;
             p.tasks = n_rt * chunks;
             const long long ctas = (long long)p.tasks * split;
-            if (split > 1) {
-                if (n_steps / split < 4 || ctas > sms) continue;
-                if ((size_t)((p.chunk16 + split - 1) / split * split) * kGroupCols * kTileM * 4 > (size_t)p.stages * p.stage_bytes + (size_t)p.w_stages * K * kWBytes) continue;
-                if (prepare_kernel(K, deq, device) != cudaSuccess || resident_clusters(kernel_for(K, deq), split, p.smem, sms) < p.tasks) continue;
-            }
+            if (split > 1 && (n_steps / split < 4 || ctas > sms)) continue;
+            if (!fill_resources(p, K, n_ops, n_steps / split, wide_x)) continue;
+            if (split > 1 && (prepare_kernel(K, deq, device) != cudaSuccess || resident_clusters(kernel_for(K, deq), split, p.smem, sms) < p.tasks)) continue;
             const double rounds = (double)((ctas + sms - 1) / sms);
             p.clocks = kLaunchClocks + (split > 1 ? kExchangeClocks : 0.0) + rounds * ((n_steps + split - 1) / split) * n_ops * unit_clocks(p.chunk16, p, n_ops) +
                        (rounds - 1.0) * kPassClocks;
@@ -844,6 +861,7 @@ cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, i
     P.n_groups = (long long)G.n_rt * P.n16;
     P.max16 = p.max16;
     P.split = p.split;
+    P.recv_off = p.recv_off;
     P.stages = p.stages; P.stage_bytes = p.stage_bytes; P.x_steps = p.x_steps; P.w_stages = p.w_stages;
     P.box16 = p.box16;
     P.n_acc = p.n_acc;
