@@ -54,6 +54,7 @@ constexpr int kStepCols = 64;               // input columns per pipeline step (
 constexpr int kGroupCols = 16;              // batch columns come in groups of 16 (MMA N granularity)
 constexpr int kUnitCols = kStepCols / 2;    // tensor-memory columns of one expanded unit (128 rows x 64 columns of fp16)
 constexpr int kMaxStages = 8, kMaxUnits = 8;
+constexpr int kSliceSteps = RABIT_LUT_COLS / kStepCols;   // steps of a 256-column slice
 constexpr int kWSteps = 8;                  // steps per stage of the weight ring
 constexpr int kWTiles = 2 * kWSteps, kWBytes = kWTiles * (RABIT_TILE_BYTES + RABIT_TILE_COLS * 2);   // per path
 constexpr int kMaxWStages = 4;
@@ -61,6 +62,7 @@ constexpr int kExpandGroups = 4;            // of four warps each
 constexpr int kExpandWarps = 4 * kExpandGroups;
 constexpr int kThreads = (4 + kExpandWarps) * 32;
 constexpr long long kWaitLimitCycles = 1LL << 31;
+constexpr unsigned long long kSumMask = (1ULL << 55) - 1;
 
 struct GemmParams {
     const unsigned char* bits;
@@ -73,7 +75,11 @@ struct GemmParams {
     int n16;                                // groups of 16 batch columns
     int n_tasks;                            // tasks of the grid: one per CTA, or one per cluster if split > 1
     int chunks, chunk16;                    // > 0: a task is (row tile, chunk of chunk16 groups); 0: a contiguous range of groups
-    long long n_groups;                     // row tiles * n16
+    long long n_groups;                     // row tiles * n16 (stream: row tiles * n_cs)
+    int stream, n_cs;                       // stream: a task is a contiguous range of (row tile, slice) pairs, all of at most 16 batch columns
+    unsigned long long* acc;                // stream: accumulate words [16][Mp], all zero between calls, and their grid
+    int fix_bits;
+    float inv_unit, unit, limit;
     int max16;                              // most groups one pass can accumulate
     int split;                              // CTAs (one cluster) that share the contraction of a task: 1, 2, 4 or 8
     int recv_off;                           // receive buffer of a split task, from the control block
@@ -182,6 +188,10 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
                    "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
                  : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
+}
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all() {
@@ -213,25 +223,39 @@ struct Walk {
 // A task's passes: runs of groups inside one row tile, at most max16 groups each, cut evenly.
 struct Pass {
     int rt, c16, n;                         // row tile, first group, groups
+    int s_lo, s_hi;                         // steps
 };
 struct PassWalker {
-    int rt, c16, left;                      // where the next pass starts, groups left in the task
-    __device__ PassWalker(const GemmParams& P, int task) {
+    int rt, c16, left;                      // where the next pass starts, groups left in the task (stream: slice and slices)
+    int s_lo, s_hi;
+    // rank: which part of the steps (split contraction)
+    __device__ PassWalker(const GemmParams& P, int task, int rank, int n_steps) {
+        s_lo = (int)((long long)n_steps * rank / P.split);
+        s_hi = (int)((long long)n_steps * (rank + 1) / P.split);
         if (P.chunks > 0) {
             rt = task / P.chunks;
             c16 = (task - rt * P.chunks) * P.chunk16;
             left = min(P.chunk16, P.n16 - c16);
         } else {
+            const int per_rt = P.stream ? P.n_cs : P.n16;
             const long long g = P.n_groups * task / P.n_tasks;
-            rt = (int)(g / P.n16);
-            c16 = (int)(g - (long long)rt * P.n16);
+            rt = (int)(g / per_rt);
+            c16 = (int)(g - (long long)rt * per_rt);
             left = (int)(P.n_groups * (task + 1) / P.n_tasks - g);
         }
     }
     __device__ bool next(const GemmParams& P, Pass& ps) {
         if (left <= 0) return false;
+        if (P.stream) {
+            const int run = min(left, P.n_cs - c16);
+            ps = Pass{rt, 0, 1, c16 * kSliceSteps, min((c16 + run) * kSliceSteps, s_hi)};
+            left -= run;
+            c16 = 0;
+            ++rt;
+            return true;
+        }
         const int run = min(left, P.n16 - c16), pieces = run <= P.max16 ? 1 : (run + P.max16 - 1) / P.max16;
-        ps = Pass{rt, c16, pieces == 1 ? run : (run + pieces - 1) / pieces};
+        ps = Pass{rt, c16, pieces == 1 ? run : (run + pieces - 1) / pieces, s_lo, s_hi};
         left -= ps.n;
         c16 += ps.n;
         if (c16 == P.n16) { c16 = 0; ++rt; }
@@ -270,8 +294,6 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
     uint32_t crank = 0;
     if (split > 1) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
     const int task = split > 1 ? (int)blockIdx.x / split : (int)blockIdx.x;
-    const int s_lo = __shfl_sync(0xFFFFFFFFu, (int)((long long)n_steps * crank / split), 0);
-    const int s_hi = __shfl_sync(0xFFFFFFFFu, (int)((long long)n_steps * (crank + 1) / split), 0);
 
     if (tid == 0) {
         for (int s = 0; s < stages; ++s) {
@@ -293,7 +315,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
     }
     __syncthreads();
     if (split > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // (awaited before the exchange: every CTA of the cluster runs)
-    const PassWalker first_pass(P, task);
+    const PassWalker first_pass(P, task, (int)crank, n_steps);
     // Output scales of the row whose accumulators this thread reads: loaded when a pass begins, converted (which waits for
     // them) when it ends.
     unsigned short graw[K];
@@ -308,10 +330,10 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
         return __half2float(__ushort_as_half(r));
     };
 
-    const int n_w = (s_hi - s_lo + kWSteps - 1) / kWSteps;        // weight stages of a pass
-    // weight stage j of a pass over row tile rt into slot `slot` (these do not depend on the stream's past)
-    auto load_weights = [&](int rt, int j, int slot) {
-        const int ct0 = 2 * (s_lo + kWSteps * j), cts = min(kWTiles, min(2 * s_hi, n_ct) - ct0);
+    auto weight_stages = [](const Pass& ps) { return (ps.s_hi - ps.s_lo + kWSteps - 1) / kWSteps; };
+    // weight stage j of a pass into slot `slot` (these do not depend on the stream's past)
+    auto load_weights = [&](const Pass& ps, int j, int slot) {
+        const int rt = ps.rt, ct0 = 2 * (ps.s_lo + kWSteps * j), cts = min(kWTiles, min(2 * ps.s_hi, n_ct) - ct0);
         const uint32_t bar = smem_u32(&S.w_full[slot]), dst = smem_u32(w_ring + slot * (K * kWBytes));
         mbar_expect_tx(bar, (uint32_t)(K * cts * (RABIT_TILE_BYTES + RABIT_TILE_COLS * 2)));
 #pragma unroll
@@ -332,11 +354,11 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
     WeightFeed feed{first_pass, Pass{}, 0, 0, Walk{0}, false};
     auto feed_next = [&](bool elected) {
         if (feed.issued >= w_stages) mbar_wait(smem_u32(&S.w_empty[feed.at.slot]), feed.at.lap ^ 1u, abort_flag);
-        if (elected) load_weights(feed.ps.rt, feed.j, feed.at.slot);
+        if (elected) load_weights(feed.ps, feed.j, feed.at.slot);
         __syncwarp();
         ++feed.issued;
         feed.at.step(1, w_stages);
-        if (++feed.j == n_w) { feed.j = 0; feed.more = feed.w.next(P, feed.ps); }
+        if (++feed.j == weight_stages(feed.ps)) { feed.j = 0; feed.more = feed.w.next(P, feed.ps); }
     };
     if (warp == 0) {
         const bool elected = elect_one();
@@ -366,8 +388,8 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
         while (w.next(P, ps)) {
             const int boxes = (ps.n + P.box16 - 1) / P.box16;
             const uint32_t box_bytes = (uint32_t)(P.box16 * (kGroupCols * kStepCols * 2) * x_steps), tx = boxes * box_bytes;   // (what lies outside x arrives as zeros)
-            for (int s = s_lo; s < s_hi; s += x_steps, ++it) {
-                if ((s - s_lo) % kWSteps == 0) {                 // (x_steps divides kWSteps)
+            for (int s = ps.s_lo; s < ps.s_hi; s += x_steps, ++it) {
+                if ((s - ps.s_lo) % kWSteps == 0) {                 // (x_steps divides kWSteps)
                     ++w_at;                                      // two stages behind the ring's depth: never held up by the stage in use
                     while (feed.more && feed.issued < w_at + w_stages - 2) feed_next(elected);
                 }
@@ -407,22 +429,46 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
                 if (pass_i > 0) mbar_wait(smem_u32(&S.acc_empty), (pass_i - 1) & 1, abort_flag);   // epilogue has drained the accumulators
                 ++pass_i;
                 uint32_t accumulate = 0u;
+                const int s_lo = __shfl_sync(0xFFFFFFFFu, ps.s_lo, 0), s_hi = __shfl_sync(0xFFFFFFFFu, ps.s_hi, 0);
                 for (int s = s_lo; s < s_hi; s += x_steps) {
                     const int n_here = min(x_steps, s_hi - s);
                     mbar_wait(full0 + xw.slot * 8, xw.lap, abort_flag);
                     const uint64_t bdesc = bdesc0 + (uint64_t)((xw.slot * stage_bytes) >> 4);
-                    for (int si = n_ops == 1 && n_acc > 1 ? (m ^ (steps_before + s - s_lo)) & 1 : 0; si < n_here; si += u_stride) {
+                    int si = n_ops == 1 && n_acc > 1 ? (m ^ (steps_before + s - s_lo)) & 1 : 0;
+                    auto issue = [&](uint32_t a, int step, bool first) {
+                        const uint64_t bd = bdesc + (uint64_t)((step * step_bytes) >> 4);
+                        umma_f16_ts(d, a, bd, idesc, first ? accumulate : 1u);
+                        umma_f16_ts(d, a + 8, bd + 2, idesc, 1u);
+                        if (2 * (s + step) + 1 < n_ct) {         // (the last step may hold one column tile)
+                            umma_f16_ts(d, a + 16, bd + 4, idesc, 1u);
+                            umma_f16_ts(d, a + 24, bd + 6, idesc, 1u);
+                        }
+                    };
+                    // with two paths two units at a time: their waits overlap (one at a time the two issuers were what layers with
+                    // few batch columns waited for; with one or three paths this measured slower)
+                    for (; n_ops == 2 && si + u_stride < n_here; si += 2 * u_stride) {
+                        Walk second = uw;
+                        second.step(n_acc, units);
+                        const bool r1 = mbar_try_wait(a_ready0 + uw.slot * 8, uw.lap), r2 = mbar_try_wait(a_ready0 + second.slot * 8, second.lap);
+                        if (!r1) mbar_wait(a_ready0 + uw.slot * 8, uw.lap, abort_flag);
+                        if (!r2) mbar_wait(a_ready0 + second.slot * 8, second.lap, abort_flag);
+                        fence_after();
+                        if (elected) {
+                            issue(a0 + uw.slot * kUnitCols, si, true);
+                            umma_commit(a_empty0 + uw.slot * 8);
+                            issue(a0 + second.slot * kUnitCols, si + u_stride, false);
+                            umma_commit(a_empty0 + second.slot * 8);
+                        }
+                        accumulate = 1u;
+                        __syncwarp();
+                        uw = second;
+                        uw.step(n_acc, units);
+                    }
+                    for (; si < n_here; si += u_stride) {
                         mbar_wait(a_ready0 + uw.slot * 8, uw.lap, abort_flag);
                         fence_after();
-                        const uint64_t bd = bdesc + (uint64_t)((si * step_bytes) >> 4);
-                        const uint32_t a = a0 + uw.slot * kUnitCols;
                         if (elected) {
-                            umma_f16_ts(d, a, bd, idesc, accumulate);
-                            umma_f16_ts(d, a + 8, bd + 2, idesc, 1u);
-                            if (2 * (s + si) + 1 < n_ct) {       // (the last step may hold one column tile)
-                                umma_f16_ts(d, a + 16, bd + 4, idesc, 1u);
-                                umma_f16_ts(d, a + 24, bd + 6, idesc, 1u);
-                            }
+                            issue(a0 + uw.slot * kUnitCols, si, true);
                             umma_commit(a_empty0 + uw.slot * 8);
                         }
                         accumulate = 1u;
@@ -477,8 +523,8 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
             }
             load_scales(ps.rt);
             const int first = ((grp - u0 % n_groups + n_groups) % n_groups) / n_ops;   // the group's first step of the pass, and of each of its weight stages
-            for (int j = 0; j < n_w && grp < n_groups; ++j) {
-                const int step0 = s_lo + j * kWSteps, n_here = min(kWSteps, s_hi - step0), whole = min(n_here, n_ct / 2 - step0);   // steps with two column tiles
+            for (int j = 0; j < weight_stages(ps) && grp < n_groups; ++j) {
+                const int step0 = ps.s_lo + j * kWSteps, n_here = min(kWSteps, ps.s_hi - step0), whole = min(n_here, n_ct / 2 - step0);   // steps with two column tiles
                 uint32_t bits = bits0 + ww.slot * (K * kWBytes) + first * (2 * RABIT_TILE_BYTES), hs = h0 + ww.slot * (K * kWBytes) + first * (kStepCols * 2);
                 mbar_wait(w_full0 + ww.slot * 8, ww.lap, abort_flag);
                 for (int sj = first; sj < n_here; sj += kStepsOn) {
@@ -537,13 +583,71 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
                 if (lane == 0) mbar_arrive(w_empty0 + ww.slot * 8);
                 ww.step(1, w_stages);
             }
-            u0 += (s_hi - s_lo) * n_ops;
+            u0 += (ps.s_hi - ps.s_lo) * n_ops;
             if (split > 1) break;                              // the cluster's epilogue follows the role branches
             // ---- epilogue of this pass
             mbar_wait(smem_u32(&S.acc_ready), pass_i & 1, abort_flag);
             ++pass_i;
             fence_after();
             const int row = ps.rt * kTileM + q * 32 + lane;
+            if (P.stream) {
+                // Up to 16 batch columns, four per group.  A segment that is a whole row tile is stored; otherwise every output goes
+                // into its 64-bit accumulate word with one integer atomic (as in rabit_gemv_f16.cu: fixed-point grid of the packer,
+                // a segment of s slices shifted by s * 2^fix_bits, arrivals in bits 55..62, bit 63 = non-finite), and the thread
+                // whose add completes a word rounds it to fp16, stores y and clears it.
+                float v[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int m = 0; m < (n_ops == 1 ? 2 : n_ops); ++m) {
+                    if (n_ops == 1 && m >= n_acc) break;
+                    uint32_t d[4];
+                    tmem_ld4(lane_base + (uint32_t)(m * P.max16 * kGroupCols + 4 * grp), d);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    const float gm = DEQ ? 1.f : scale(n_ops == 1 ? 0 : m);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) v[i] = fmaf(gm, __uint_as_float(d[i]), v[i]);
+                }
+                fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&S.acc_empty));
+                const int n_here = P.batch - 4 * grp;            // batch columns of this group, if positive
+                const int n_slices = (ps.s_hi - ps.s_lo + kSliceSteps - 1) / kSliceSteps;
+                if (n_slices == P.n_cs) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (i < n_here && row < P.M) P.y[(size_t)(4 * grp + i) * P.M + row] = __float2half_rn(v[i]);
+                    continue;
+                }
+                unsigned long long* word = P.acc + (size_t)(4 * grp) * P.Mp + row;
+                unsigned long long old[4], add[4];
+                uint32_t bad = 0u;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float scaled = v[i] * P.inv_unit;
+                    if (!(fabsf(scaled) < P.limit * (float)n_slices)) bad |= 1u << i;             // inf or NaN: finite inputs cannot get here
+                    const long long qv = (bad >> i) & 1u ? 0LL : __float2ll_rn(scaled);
+                    add[i] = (unsigned long long)(qv + ((long long)n_slices << P.fix_bits)) + (1ULL << 55);
+                }
+                // all atomics of the thread back to back: nothing between them that could wait for an answer
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    old[i] = 0ULL;
+                    if (i >= n_here) continue;
+                    if ((bad >> i) & 1u) atomicOr(word + (size_t)i * P.Mp, 1ULL << 63);           // sticky: the add below never carries into bit 63
+                    old[i] = atomicAdd(word + (size_t)i * P.Mp, add[i]);
+                }
+                const long long first = (long long)ps.rt * P.n_cs, last = first + P.n_cs - 1;     // segments of this row tile: the tasks that touch it
+                const int arrivals = (int)(((last + 1) * P.n_tasks - 1) / P.n_groups) - (int)(((first + 1) * P.n_tasks - 1) / P.n_groups) + 1;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (i >= n_here || (int)((old[i] >> 55) & 0xFFu) != arrivals - 1) continue;   // other segments are still to come
+                    const unsigned long long sum = (old[i] & kSumMask) + (add[i] & kSumMask);
+                    const long long total = (long long)sum - ((long long)P.n_cs << P.fix_bits);
+                    const bool poisoned = ((bad >> i) & 1u) || (old[i] >> 63) != 0;
+                    if (row < P.M) P.y[(size_t)(4 * grp + i) * P.M + row] = poisoned ? __ushort_as_half((unsigned short)0x7FFF) : __float2half_rn(__ll2float_rn(total) * P.unit);
+                    word[(size_t)i * P.Mp] = 0ULL;               // resting state for the next call
+                }
+                continue;
+            }
 #pragma unroll 1
             for (int c = grp; c < ps.n; c += kExpandGroups) {
                 float v[16];
@@ -680,6 +784,7 @@ cudaError_t x_tensor_map(const void* x, int N, int batch, int box16, int x_steps
 
 struct Plan {
     int chunks, chunk16, split, max16, tasks;        // chunks == 0: contiguous group ranges
+    int stream;                                      // contiguous ranges of (row tile, slice) pairs
     int stages, stage_bytes, x_steps, w_stages, box16, units, n_acc, recv_off;
     size_t smem;
     double clocks;                                   // estimate
@@ -692,7 +797,8 @@ bool fill_resources(Plan& p, int K, int n_ops, int steps, bool one_box) {
     if (p.max16 * kGroupCols > 256) return false;
     const int turn = n_ops == 3 ? 3 : 4;
     auto free_units = [&](int n_acc) { return (512 - n_acc * p.max16 * kGroupCols) / kUnitCols; };
-    p.n_acc = n_ops > 1 ? n_ops : steps >= 2 && free_units(2) >= turn ? 2 : 1;
+    // (one path: a second accumulator needs a step for each in every pass; a stream's shortest one is the last slice)
+    p.n_acc = n_ops > 1 ? n_ops : (p.stream ? steps % kSliceSteps != 1 : steps >= 2) && free_units(2) >= turn ? 2 : 1;
     if (free_units(p.n_acc) < turn) return false;
     p.units = free_units(p.n_acc) >= 2 * turn ? 2 * turn : turn;
     const int step_bytes = (p.max16 + p.box16 - 1) / p.box16 * p.box16 * kGroupCols * kStepCols * 2;
@@ -755,10 +861,12 @@ int resident_clusters(const void* kernel, int split, size_t smem, int sms) {
 }
 
 constexpr double kPassClocks = 3000.0;               // pipeline fill and epilogue of a pass that nothing overlaps
-constexpr double kLaunchClocks = 5000.0;             // launch, first loads, last epilogue
-constexpr double kExchangeClocks = 1500.0;           // cluster barriers and exchange of a split task
+constexpr double kLaunchClocks = 8000.0;             // launch, first loads, last epilogue
+constexpr double kExchangeClocks = 2500.0;           // exchange of a split task
+constexpr double kPublishClocks = 1500.0;            // atomics of a part of a row tile, besides their throughput
 
-Plan make_plan(int n_rt, int n_steps, int K, bool deq, int n16, int sms, int device, bool wide_x) {
+Plan make_plan(int n_rt, int n_steps, int K, bool deq, int batch, int sms, int device, bool wide_x) {
+    const int n16 = (batch + kGroupCols - 1) / kGroupCols;
     const int n_ops = deq ? 1 : K;
     Plan best = {};
     best.clocks = 1e300;
@@ -781,6 +889,30 @@ Plan make_plan(int n_rt, int n_steps, int K, bool deq, int n16, int sms, int dev
             if (p.clocks < best.clocks) best = p;
         }
         if (p.chunk16 <= 4) break;                   // narrower passes cost as much as these
+    }
+    // (c) up to 16 columns: contiguous ranges of (row tile, slice) pairs, met in the accumulate words
+    const int n_cs = (n_steps + kSliceSteps - 1) / kSliceSteps;
+    if (n16 == 1 && n_cs <= RABIT_LUT_MAX_SLICES) {
+        Plan p = {};
+        p.stream = p.split = p.max16 = p.box16 = 1;
+        const long long pairs = (long long)n_rt * n_cs;
+        auto consider = [&](long long tasks) {
+            p.tasks = (int)tasks;
+            long long worst = 0, parts = 0;                                   // in clocks; segments that are not whole row tiles
+            const double pair = kSliceSteps * n_ops * unit_clocks(1, p, n_ops);
+            for (long long t = 0; t < tasks; ++t) {
+                const long long a = pairs * t / tasks, b = pairs * (t + 1) / tasks, segments = (b - 1) / n_cs - a / n_cs + 1;
+                const int cut = (a % n_cs != 0) + (b % n_cs != 0);
+                parts += segments == 1 && cut == 2 ? 1 : cut;
+                worst = std::max(worst, (long long)((b - a) * pair + (segments - 1) * kPassClocks));
+            }
+            p.clocks = kLaunchClocks + worst + (parts > 0 ? kPublishClocks + parts * 128.0 * batch / 80.0 : 0.0);
+            if (p.clocks < best.clocks) best = p;
+        };
+        if (fill_resources(p, K, n_ops, n_steps, wide_x)) {
+            for (long long m = 1; m <= n_cs && n_rt * m <= sms; ++m) consider(n_rt * m);      // equal parts of a row tile
+            consider(std::min<long long>(sms, pairs));
+        }
     }
     // (b) contiguous ranges of groups, one per SM: no last wave
     const long long groups = (long long)n_rt * n16;
@@ -824,7 +956,7 @@ Plan plan_for(const rabit_layer& L, bool deq, int batch) {
     for (const Entry& e : plans)
         if (e.n_rt == n_rt && e.n_ct == n_ct && e.K == K && e.deq == (int)deq && e.n16 == n16 && e.sms == sms) return e.plan;
     if (plans.size() >= 256) plans.clear();
-    plans.push_back(Entry{n_rt, n_ct, K, (int)deq, n16, sms, make_plan(n_rt, (n_ct + 1) / 2, K, deq, n16, sms, L.device, n_ct % 2 == 0)});
+    plans.push_back(Entry{n_rt, n_ct, K, (int)deq, n16, sms, make_plan(n_rt, (n_ct + 1) / 2, K, deq, n16 * kGroupCols, sms, L.device, n_ct % 2 == 0)});
     return plans.back().plan;
 }
 
@@ -858,7 +990,11 @@ cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, i
     P.n16 = (batch + kGroupCols - 1) / kGroupCols;
     P.n_tasks = p.tasks;
     P.chunks = p.chunks; P.chunk16 = p.chunk16;
-    P.n_groups = (long long)G.n_rt * P.n16;
+    P.n_groups = (long long)G.n_rt * (p.stream ? G.n_cs : P.n16);
+    P.stream = p.stream; P.n_cs = G.n_cs;
+    P.acc = L.d_acc;
+    P.fix_bits = G.fix_bits;
+    P.unit = ldexpf(1.f, G.unit_exp); P.inv_unit = ldexpf(1.f, -G.unit_exp); P.limit = ldexpf(1.f, G.fix_bits);
     P.max16 = p.max16;
     P.split = p.split;
     P.recv_off = p.recv_off;
