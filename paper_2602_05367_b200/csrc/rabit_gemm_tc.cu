@@ -75,7 +75,7 @@ struct GemmParams {
     int n16;                                // groups of 16 batch columns
     int n_tasks;                            // tasks of the grid: one per CTA, or one per cluster if split > 1
     int chunks, chunk16;                    // > 0: a task is (row tile, chunk of chunk16 groups); 0: a contiguous range of groups
-    long long n_groups;                     // row tiles * n16 (stream: row tiles * n_cs)
+    int n_groups, quot, rem;                // row tiles * n16 (stream: row tiles * n_cs); that by n_tasks
     int stream, n_cs;                       // stream: a task is a contiguous range of (row tile, slice) pairs, all of at most 16 batch columns
     unsigned long long* acc;                // stream: accumulate words [16][Mp], all zero between calls, and their grid
     int fix_bits;
@@ -237,11 +237,11 @@ struct PassWalker {
             c16 = (task - rt * P.chunks) * P.chunk16;
             left = min(P.chunk16, P.n16 - c16);
         } else {
-            const int per_rt = P.stream ? P.n_cs : P.n16;
-            const long long g = P.n_groups * task / P.n_tasks;
-            rt = (int)(g / per_rt);
-            c16 = (int)(g - (long long)rt * per_rt);
-            left = (int)(P.n_groups * (task + 1) / P.n_tasks - g);
+            // floor(n_groups * task / n_tasks), from quotient and remainder of n_groups: no 64-bit division
+            const int per_rt = P.stream ? P.n_cs : P.n16, g = P.quot * task + P.rem * task / P.n_tasks;
+            rt = g / per_rt;
+            c16 = g - rt * per_rt;
+            left = P.quot * (task + 1) + P.rem * (task + 1) / P.n_tasks - g;
         }
     }
     __device__ bool next(const GemmParams& P, Pass& ps) {
@@ -273,13 +273,14 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
     Control& S = *reinterpret_cast<Control*>(smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
     // The launch parameters sit in constant memory, cold in every launch (a first touch is a trip to L2, several in a row
-    // between the dependency wait and the first MMA): touched here once.  So is the tensor map.  (A copy of them in shared
-    // memory is no better: the values are then not uniform to the compiler, and the issuers' loops grow by 15 %.)
-    if (tid < (int)(sizeof(GemmParams) / 4)) {
-        const uint32_t word = reinterpret_cast<const uint32_t*>(&P)[tid];
+    // between the dependency wait and the first MMA): touched here once, a 64-byte line per warp.  So is the tensor map.  (A
+    // copy of them in shared memory is no better: the values are then not uniform to the compiler, and the issuers' loops
+    // grow by 15 %.)
+    if (warp < (int)((sizeof(GemmParams) + 63) / 64)) {
+        const uint32_t word = reinterpret_cast<const uint32_t*>(&P)[warp * 16];
         asm volatile("" ::"r"(word));
     }
-    if (tid == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&x_map) : "memory");
+    if (warp == kThreads / 32 - 1 && lane == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&x_map) : "memory");
     unsigned char* ring = smem + kControlBytes;
     unsigned char* w_ring = ring + P.stages * P.stage_bytes;
     constexpr int n_ops = DEQ ? 1 : K;                            // operand units (and accumulators) per step
@@ -295,22 +296,15 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
     if (split > 1) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
     const int task = split > 1 ? (int)blockIdx.x / split : (int)blockIdx.x;
 
-    if (tid == 0) {
-        for (int s = 0; s < stages; ++s) {
-            mbar_init(smem_u32(&S.full[s]), 1);
-            mbar_init(smem_u32(&S.empty[s]), P.n_acc);
+    if (warp == 1) {                                              // (all of them, whatever the rings use: a lane each)
+        if (lane < kMaxStages) { mbar_init(smem_u32(&S.full[lane]), 1); mbar_init(smem_u32(&S.empty[lane]), n_acc); }
+        if (lane < kMaxWStages) { mbar_init(smem_u32(&S.w_full[lane]), 1); mbar_init(smem_u32(&S.w_empty[lane]), 4 * n_groups); }
+        if (lane < kMaxUnits) { mbar_init(smem_u32(&S.a_ready[lane]), 4); mbar_init(smem_u32(&S.a_empty[lane]), 1); }
+        if (lane == 0) {
+            mbar_init(smem_u32(&S.acc_ready), n_acc);
+            mbar_init(smem_u32(&S.acc_empty), kExpandWarps);
+            S.abort_flag = 0;
         }
-        for (int s = 0; s < w_stages; ++s) {
-            mbar_init(smem_u32(&S.w_full[s]), 1);
-            mbar_init(smem_u32(&S.w_empty[s]), 4 * n_groups);
-        }
-        for (int u = 0; u < units; ++u) {
-            mbar_init(smem_u32(&S.a_ready[u]), 4);
-            mbar_init(smem_u32(&S.a_empty[u]), 1);
-        }
-        mbar_init(smem_u32(&S.acc_ready), P.n_acc);
-        mbar_init(smem_u32(&S.acc_empty), kExpandWarps);
-        S.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -892,7 +886,7 @@ Plan make_plan(int n_rt, int n_steps, int K, bool deq, int batch, int sms, int d
     }
     // (c) up to 16 columns: contiguous ranges of (row tile, slice) pairs, met in the accumulate words
     const int n_cs = (n_steps + kSliceSteps - 1) / kSliceSteps;
-    if (n16 == 1 && n_cs <= RABIT_LUT_MAX_SLICES) {
+    if (n16 == 1 && n_cs <= RABIT_LUT_MAX_SLICES && (long long)n_rt * n_cs < (1LL << 30)) {
         Plan p = {};
         p.stream = p.split = p.max16 = p.box16 = 1;
         const long long pairs = (long long)n_rt * n_cs;
@@ -916,7 +910,7 @@ Plan make_plan(int n_rt, int n_steps, int K, bool deq, int batch, int sms, int d
     }
     // (b) contiguous ranges of groups, one per SM: no last wave
     const long long groups = (long long)n_rt * n16;
-    if (groups >= 2LL * sms) {
+    if (groups >= 2LL * sms && groups < (1LL << 30)) {
         Plan p = {};
         p.split = 1;
         p.tasks = sms;
@@ -990,7 +984,8 @@ cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, i
     P.n16 = (batch + kGroupCols - 1) / kGroupCols;
     P.n_tasks = p.tasks;
     P.chunks = p.chunks; P.chunk16 = p.chunk16;
-    P.n_groups = (long long)G.n_rt * (p.stream ? G.n_cs : P.n16);
+    P.n_groups = (int)std::min<long long>(0x7FFFFFFF, (long long)G.n_rt * (p.stream ? G.n_cs : P.n16));   // (only read where it fits)
+    P.quot = P.n_groups / P.n_tasks; P.rem = P.n_groups % P.n_tasks;
     P.stream = p.stream; P.n_cs = G.n_cs;
     P.acc = L.d_acc;
     P.fix_bits = G.fix_bits;
