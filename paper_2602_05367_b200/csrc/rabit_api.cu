@@ -1,4 +1,5 @@
 // C ABI of the library: argument checks, pack/upload, dispatch, error strings.
+#include <algorithm>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -138,6 +139,11 @@ static bool ranges_overlap(const void* a, size_t an, const void* b, size_t bn) {
     return a0 < b0 + bn && b0 < a0 + an;
 }
 
+// Rows up to which the f16 GEMV is the faster of the two tensor-core kernels: its MMAs carry eight rows, a second set for 9 to
+// 16 makes it slower than the GEMM, which costs the same from 1 to 16 (B200, us at 8 / 9 / 16 rows against the GEMM:
+// 4096 x 4096 6.8 / 8.4 / 8.9 against 7.8, 14336 x 4096 13 / 18.3 / 20.6 against 16.0, 28672 x 8192 38 / 54 / 55 against 44).
+static const int kF16Rows = 8;
+
 extern "C" int rabit_linear(const rabit_layer* layer, const void* x, void* y, int batch, void* stream) {
     rabit_clear_error();
     if (!layer) return rabit_fail(RABIT_INVALID_ARG, "rabit_linear: layer is NULL");
@@ -210,10 +216,10 @@ extern "C" int rabit_linear(const rabit_layer* layer, const void* x, void* y, in
                                           batch - b0 >= rows ? rows : batch - b0, st);
             break;
         }
-        case 6:                             // beyond 16 rows the GEMM: one launch of it beats two passes on every shape measured
-            if (!rabit_gemv_f16_supports(*layer, batch < RABIT_MAX_GEMV_BATCH ? batch : RABIT_MAX_GEMV_BATCH))   // (14336 x 4096 at batch 32: 24 us against 39)
+        case 6:                             // beyond eight rows the GEMM (see kF16Rows)
+            if (!rabit_gemv_f16_supports(*layer, batch < RABIT_MAX_GEMV_BATCH ? batch : RABIT_MAX_GEMV_BATCH))
                 return rabit_fail(RABIT_INVALID_ARG, "rabit_linear: f16 tensor-core GEMV cannot run this layer");
-            e = batch <= RABIT_MAX_GEMV_BATCH ? rabit_launch_gemv_f16(*layer, x, y, batch, st) : rabit_launch_gemm_tc(*layer, x, y, batch, st);
+            e = batch <= kF16Rows || !rabit_gemm_tc_supports(*layer, batch) ? rabit_launch_gemv_f16(*layer, x, y, batch, st) : rabit_launch_gemm_tc(*layer, x, y, batch, st);
             break;
         default:
             e = rabit_launch_plain(*layer, x, y, batch, st);
@@ -264,7 +270,18 @@ extern "C" int rabit_linear_group(const rabit_layer* const* layers, const void* 
     {
         bool f16 = batch <= RABIT_MAX_GEMV_BATCH;                // 3..16 rows: the f16 tensor-core GEMV
         for (int l = 0; l < n_layers && f16; ++l) f16 = (layers[l]->variant == 0 || layers[l]->variant == 6) && rabit_gemv_f16_supports(*layers[l], batch);
-        if (f16 && !rabit_gemv_lut_supports(*layers[0], batch) && rabit_gemv_f16_group_supports(layers, n_layers, batch)) {
+        // beyond eight rows the GEMM, up to four layers a launch
+        bool gemm = f16 && batch > kF16Rows;
+        for (int l = 0; l < n_layers && gemm; l += rabit_gemm_tc_max_group())
+            gemm = rabit_gemm_tc_group_supports(layers + l, std::min(rabit_gemm_tc_max_group(), n_layers - l), batch);
+        if (gemm) {
+            cudaError_t e = cudaSuccess;
+            for (int l = 0; l < n_layers && e == cudaSuccess; l += rabit_gemm_tc_max_group())
+                e = rabit_launch_gemm_tc_group(layers + l, std::min(rabit_gemm_tc_max_group(), n_layers - l), xs + l, ys + l, batch, st);
+            if (e != cudaSuccess) return rabit_fail(RABIT_CUDA_ERROR, "rabit_linear_group: launch failed: %s", cudaGetErrorString(e));
+            return RABIT_OK;
+        }
+        if (f16 && batch <= kF16Rows && !rabit_gemv_lut_supports(*layers[0], batch) && rabit_gemv_f16_group_supports(layers, n_layers, batch)) {
             cudaError_t e = rabit_launch_gemv_f16_group(layers, n_layers, xs, ys, batch, st);
             if (e != cudaSuccess) return rabit_fail(RABIT_CUDA_ERROR, "rabit_linear_group: launch failed: %s", cudaGetErrorString(e));
             return RABIT_OK;

@@ -64,22 +64,29 @@ constexpr int kThreads = (4 + kExpandWarps) * 32;
 constexpr long long kWaitLimitCycles = 1LL << 31;
 constexpr unsigned long long kSumMask = (1ULL << 55) - 1;
 
-struct GemmParams {
+constexpr int kMaxGroup = 4;                // layers of a grouped launch
+
+struct GemmLayer {
     const unsigned char* bits;
     const __half* g;
     const __half* h;
     __half* y;
     unsigned int* status;
-    int M, N, Mp, n_ct;
+    unsigned long long* acc;                // stream: accumulate words [16][Mp], all zero between calls, and their grid
+    int M, N, Mp, n_rt, n_ct, n_cs;
+    int fix_bits;
+    float inv_unit, unit, limit;
+    int pair0;                              // grouped launch: (row tile, slice) pairs of the layers before this one
+};
+template <int NL>
+struct GemmParams {
+    int n_layers;
     int batch;
     int n16;                                // groups of 16 batch columns
     int n_tasks;                            // tasks of the grid: one per CTA, or one per cluster if split > 1
     int chunks, chunk16;                    // > 0: a task is (row tile, chunk of chunk16 groups); 0: a contiguous range of groups
-    int n_groups, quot, rem;                // row tiles * n16 (stream: row tiles * n_cs); that by n_tasks
-    int stream, n_cs;                       // stream: a task is a contiguous range of (row tile, slice) pairs, all of at most 16 batch columns
-    unsigned long long* acc;                // stream: accumulate words [16][Mp], all zero between calls, and their grid
-    int fix_bits;
-    float inv_unit, unit, limit;
+    int n_groups, quot, rem;                // row tiles * n16 (stream: row tiles * n_cs, over all layers); that by n_tasks
+    int stream;                             // a task is a contiguous range of (row tile, slice) pairs, all of at most 16 batch columns
     int max16;                              // most groups one pass can accumulate
     int split;                              // CTAs (one cluster) that share the contraction of a task: 1, 2, 4 or 8
     int recv_off;                           // receive buffer of a split task, from the control block
@@ -88,6 +95,11 @@ struct GemmParams {
     int box16;                              // groups of 16 batch columns per TMA box
     int n_acc;                              // accumulators (and issuing warps)
     int units, a_col;                       // expanded-unit ring in tensor memory: unit u % units at columns a_col + 32 * that
+    GemmLayer L[NL];
+};
+template <int NL>
+struct alignas(64) XMaps {
+    CUtensorMap map[NL];
 };
 
 struct Control {                            // ahead of the ring in shared memory
@@ -222,40 +234,51 @@ struct Walk {
 
 // A task's passes: runs of groups inside one row tile, at most max16 groups each, cut evenly.
 struct Pass {
-    int rt, c16, n;                         // row tile, first group, groups
+    int l, rt, c16, n;                      // layer, row tile, first group, groups
     int s_lo, s_hi;                         // steps
 };
+template <int NL>
 struct PassWalker {
-    int rt, c16, left;                      // where the next pass starts, groups left in the task (stream: slice and slices)
+    int l, rt, c16, left;                   // where the next pass starts, groups left in the task (stream: slice and slices)
     int s_lo, s_hi;
     // rank: which part of the steps (split contraction)
-    __device__ PassWalker(const GemmParams& P, int task, int rank, int n_steps) {
-        s_lo = (int)((long long)n_steps * rank / P.split);
-        s_hi = (int)((long long)n_steps * (rank + 1) / P.split);
-        if (P.chunks > 0) {
+    __device__ PassWalker(const GemmParams<NL>& P, int task, int rank) {
+        l = 0;
+        if (NL == 1) {
+            const int n_steps = (P.L[0].N + kStepCols - 1) / kStepCols;   // N % 32 == 0: the last step may hold one column tile only
+            s_lo = (int)((long long)n_steps * rank / P.split);
+            s_hi = (int)((long long)n_steps * (rank + 1) / P.split);
+        }
+        if (NL == 1 && P.chunks > 0) {
             rt = task / P.chunks;
             c16 = (task - rt * P.chunks) * P.chunk16;
             left = min(P.chunk16, P.n16 - c16);
         } else {
             // floor(n_groups * task / n_tasks), from quotient and remainder of n_groups: no 64-bit division
-            const int per_rt = P.stream ? P.n_cs : P.n16, g = P.quot * task + P.rem * task / P.n_tasks;
+            int g = P.quot * task + P.rem * task / P.n_tasks;
+            left = P.quot * (task + 1) + P.rem * (task + 1) / P.n_tasks - g;
+            if (NL > 1) {
+                while (l + 1 < P.n_layers && g >= P.L[l + 1].pair0) ++l;
+                g -= P.L[l].pair0;
+            }
+            const int per_rt = NL > 1 || P.stream ? P.L[l].n_cs : P.n16;
             rt = g / per_rt;
             c16 = g - rt * per_rt;
-            left = P.quot * (task + 1) + P.rem * (task + 1) / P.n_tasks - g;
         }
     }
-    __device__ bool next(const GemmParams& P, Pass& ps) {
+    __device__ bool next(const GemmParams<NL>& P, Pass& ps) {
         if (left <= 0) return false;
-        if (P.stream) {
-            const int run = min(left, P.n_cs - c16);
-            ps = Pass{rt, 0, 1, c16 * kSliceSteps, min((c16 + run) * kSliceSteps, s_hi)};
+        if (NL > 1 || P.stream) {
+            const int n_cs = P.L[l].n_cs, run = min(left, n_cs - c16);
+            ps = Pass{l, rt, 0, 1, c16 * kSliceSteps, min((c16 + run) * kSliceSteps, NL > 1 ? (P.L[l].n_ct + 1) / 2 : s_hi)};
             left -= run;
             c16 = 0;
             ++rt;
+            if (NL > 1 && rt == P.L[l].n_rt) { rt = 0; ++l; }             // (a task that ends here never looks at the layer again)
             return true;
         }
         const int run = min(left, P.n16 - c16), pieces = run <= P.max16 ? 1 : (run + P.max16 - 1) / P.max16;
-        ps = Pass{rt, c16, pieces == 1 ? run : (run + pieces - 1) / pieces, s_lo, s_hi};
+        ps = Pass{0, rt, c16, pieces == 1 ? run : (run + pieces - 1) / pieces, s_lo, s_hi};
         left -= ps.n;
         c16 += ps.n;
         if (c16 == P.n16) { c16 = 0; ++rt; }
@@ -263,10 +286,11 @@ struct PassWalker {
     }
 };
 
-// K paths; DEQ: see above.
-template <int K, bool DEQ>
+// K paths; DEQ: see above.  NL > 1: up to NL layers of at most 16 batch columns in one launch (stream tasks; each layer has
+// its own x, of which the layers may share one).
+template <int K, bool DEQ, int NL>
 __global__ void __launch_bounds__(kThreads, 1)
-rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant__ CUtensorMap x_map) {
+rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_constant__ XMaps<NL> x_maps) {
     extern __shared__ unsigned char smem_raw[];
     // the swizzled x tiles need 1024-byte alignment; the launch reserves the slack
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -276,22 +300,22 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
     // between the dependency wait and the first MMA): touched here once, a 64-byte line per warp.  So is the tensor map.  (A
     // copy of them in shared memory is no better: the values are then not uniform to the compiler, and the issuers' loops
     // grow by 15 %.)
-    if (warp < (int)((sizeof(GemmParams) + 63) / 64)) {
+    if (warp < (int)((sizeof(GemmParams<NL>) + 63) / 64)) {
         const uint32_t word = reinterpret_cast<const uint32_t*>(&P)[warp * 16];
         asm volatile("" ::"r"(word));
     }
-    if (warp == kThreads / 32 - 1 && lane == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&x_map) : "memory");
+    if (warp == kThreads / 32 - 1 && lane < (NL == 1 ? 1 : P.n_layers)) asm volatile("prefetch.tensormap [%0];" ::"l"(&x_maps.map[NL == 1 ? 0 : lane]) : "memory");
+    auto layer = [&](const Pass& ps) -> const GemmLayer& { return P.L[NL == 1 ? 0 : ps.l]; };
     unsigned char* ring = smem + kControlBytes;
     unsigned char* w_ring = ring + P.stages * P.stage_bytes;
     constexpr int n_ops = DEQ ? 1 : K;                            // operand units (and accumulators) per step
     constexpr int n_groups = n_ops == 3 ? 3 : 4;                  // expander groups at work
     const int stages = P.stages, w_stages = P.w_stages, units = P.units, x_steps = P.x_steps, n_acc = P.n_acc;
-    const int stage_bytes = P.stage_bytes, n_ct = P.n_ct;
-    const int n_steps = (P.N + kStepCols - 1) / kStepCols;        // N % 32 == 0: the last step may hold one column tile only
+    const int stage_bytes = P.stage_bytes;
     volatile int* abort_flag = &S.abort_flag;
     // Split contraction: the CTAs of a cluster work on the same task, rank r taking the r-th part of the steps; their
     // partial results meet through distributed shared memory at the end (such a task is one pass).
-    const int split = P.split;
+    const int split = NL == 1 ? P.split : 1;
     uint32_t crank = 0;
     if (split > 1) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
     const int task = split > 1 ? (int)blockIdx.x / split : (int)blockIdx.x;
@@ -309,14 +333,14 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
     }
     __syncthreads();
     if (split > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // (awaited before the exchange: every CTA of the cluster runs)
-    const PassWalker first_pass(P, task, (int)crank, n_steps);
+    const PassWalker<NL> first_pass(P, task, (int)crank);
     // Output scales of the row whose accumulators this thread reads: loaded when a pass begins, converted (which waits for
     // them) when it ends.
     unsigned short graw[K];
-    auto load_scales = [&](int rt) {
+    auto load_scales = [&](const Pass& ps) {
 #pragma unroll
         for (int k = 0; k < K; ++k)
-            asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(graw[k]) : "l"(P.g + (size_t)k * P.Mp + rt * kTileM + (warp & 3) * 32 + lane));
+            asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(graw[k]) : "l"(layer(ps).g + (size_t)k * layer(ps).Mp + ps.rt * kTileM + (warp & 3) * 32 + lane));
     };
     auto scale = [&](int k) {
         unsigned short r;
@@ -327,19 +351,20 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
     auto weight_stages = [](const Pass& ps) { return (ps.s_hi - ps.s_lo + kWSteps - 1) / kWSteps; };
     // weight stage j of a pass into slot `slot` (these do not depend on the stream's past)
     auto load_weights = [&](const Pass& ps, int j, int slot) {
-        const int rt = ps.rt, ct0 = 2 * (ps.s_lo + kWSteps * j), cts = min(kWTiles, min(2 * ps.s_hi, n_ct) - ct0);
+        const GemmLayer& L = layer(ps);
+        const int rt = ps.rt, n_ct = L.n_ct, ct0 = 2 * (ps.s_lo + kWSteps * j), cts = min(kWTiles, min(2 * ps.s_hi, n_ct) - ct0);
         const uint32_t bar = smem_u32(&S.w_full[slot]), dst = smem_u32(w_ring + slot * (K * kWBytes));
         mbar_expect_tx(bar, (uint32_t)(K * cts * (RABIT_TILE_BYTES + RABIT_TILE_COLS * 2)));
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            bulk_g2s(dst + k * kWTiles * RABIT_TILE_BYTES, P.bits + (((size_t)rt * K + k) * n_ct + ct0) * RABIT_TILE_BYTES, cts * RABIT_TILE_BYTES, bar);
-            bulk_g2s(dst + K * kWTiles * RABIT_TILE_BYTES + k * kWTiles * RABIT_TILE_COLS * 2, P.h + (size_t)k * P.N + (size_t)ct0 * RABIT_TILE_COLS,
+            bulk_g2s(dst + k * kWTiles * RABIT_TILE_BYTES, L.bits + (((size_t)rt * K + k) * n_ct + ct0) * RABIT_TILE_BYTES, cts * RABIT_TILE_BYTES, bar);
+            bulk_g2s(dst + K * kWTiles * RABIT_TILE_BYTES + k * kWTiles * RABIT_TILE_COLS * 2, L.h + (size_t)k * L.N + (size_t)ct0 * RABIT_TILE_COLS,
                      cts * RABIT_TILE_COLS * 2, bar);
         }
     };
     // the weight stages of all passes in order; `next` starts one if its slot is free or becomes free
     struct WeightFeed {
-        PassWalker w;
+        PassWalker<NL> w;
         Pass ps;
         int j, issued;
         Walk at;
@@ -377,7 +402,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
         const bool elected = elect_one();
         int it = 0, w_at = 0;                                    // x and weight stages begun, over all passes
         Walk at{0};
-        PassWalker w = first_pass;
+        PassWalker<NL> w = first_pass;
         Pass ps;
         while (w.next(P, ps)) {
             const int boxes = (ps.n + P.box16 - 1) / P.box16;
@@ -392,9 +417,9 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
                 if (elected) {
                     mbar_expect_tx(bar, tx);
                     if (x_steps > 1) {
-                        tma_load_3d(dst, &x_map, 0, ps.c16 * kGroupCols, s, bar);
+                        tma_load_3d(dst, &x_maps.map[NL == 1 ? 0 : ps.l], 0, ps.c16 * kGroupCols, s, bar);
                     } else {
-                        for (int c = 0; c < boxes; ++c) tma_load_2d(dst + c * box_bytes, &x_map, s * kStepCols, (ps.c16 + c * P.box16) * kGroupCols, bar);
+                        for (int c = 0; c < boxes; ++c) tma_load_2d(dst + c * box_bytes, &x_maps.map[NL == 1 ? 0 : ps.l], s * kStepCols, (ps.c16 + c * P.box16) * kGroupCols, bar);
                     }
                 }
                 __syncwarp();
@@ -416,7 +441,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
             const uint32_t a0 = tmem_base + (uint32_t)P.a_col, d = tmem_base + (uint32_t)(m * P.max16 * kGroupCols);
             const uint32_t step_bytes = (uint32_t)stage_bytes / (uint32_t)x_steps;
             int steps_before = 0;                                // of earlier passes
-            PassWalker w = first_pass;
+            PassWalker<NL> w = first_pass;
             Pass ps;
             while (w.next(P, ps)) {
                 const uint32_t idesc = __shfl_sync(0xFFFFFFFFu, umma_idesc(ps.n * kGroupCols), 0);
@@ -424,6 +449,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
                 ++pass_i;
                 uint32_t accumulate = 0u;
                 const int s_lo = __shfl_sync(0xFFFFFFFFu, ps.s_lo, 0), s_hi = __shfl_sync(0xFFFFFFFFu, ps.s_hi, 0);
+                const int n_ct = NL == 1 ? P.L[0].n_ct : __shfl_sync(0xFFFFFFFFu, P.L[ps.l].n_ct, 0);
                 for (int s = s_lo; s < s_hi; s += x_steps) {
                     const int n_here = min(x_steps, s_hi - s);
                     mbar_wait(full0 + xw.slot * 8, xw.lap, abort_flag);
@@ -502,9 +528,11 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
         uint32_t dst = dst0, bar = bar0, done = 0;            // done: the group's units so far
         Walk ww{0};
         int pass_i = 0, u0 = 0;
-        PassWalker w = first_pass;
+        PassWalker<NL> w = first_pass;
         Pass ps;
         while (w.next(P, ps)) {
+            const GemmLayer& L = layer(ps);
+            const int n_ct = L.n_ct;
             __half2 g_rows[DEQ ? K : 1][2][2];                 // DEQ: output scales of this thread's rows (row block, row half), both halves alike
             if (DEQ) {
 #pragma unroll
@@ -513,9 +541,9 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
                     for (int pi = 0; pi < 2; ++pi)
 #pragma unroll
                         for (int rh = 0; rh < 2; ++rh)
-                            g_rows[k][pi][rh] = __half2half2(P.g[(size_t)k * P.Mp + ps.rt * kTileM + 32 * q + 16 * pi + gq + 8 * rh]);
+                            g_rows[k][pi][rh] = __half2half2(L.g[(size_t)k * L.Mp + ps.rt * kTileM + 32 * q + 16 * pi + gq + 8 * rh]);
             }
-            load_scales(ps.rt);
+            load_scales(ps);
             const int first = ((grp - u0 % n_groups + n_groups) % n_groups) / n_ops;   // the group's first step of the pass, and of each of its weight stages
             for (int j = 0; j < weight_stages(ps) && grp < n_groups; ++j) {
                 const int step0 = ps.s_lo + j * kWSteps, n_here = min(kWSteps, ps.s_hi - step0), whole = min(n_here, n_ct / 2 - step0);   // steps with two column tiles
@@ -584,7 +612,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
             ++pass_i;
             fence_after();
             const int row = ps.rt * kTileM + q * 32 + lane;
-            if (P.stream) {
+            if (NL > 1 || P.stream) {
                 // Up to 16 batch columns, four per group.  A segment that is a whole row tile is stored; otherwise every output goes
                 // into its 64-bit accumulate word with one integer atomic (as in rabit_gemv_f16.cu: fixed-point grid of the packer,
                 // a segment of s slices shifted by s * 2^fix_bits, arrivals in bits 55..62, bit 63 = non-finite), and the thread
@@ -605,45 +633,45 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
                 if (lane == 0) mbar_arrive(smem_u32(&S.acc_empty));
                 const int n_here = P.batch - 4 * grp;            // batch columns of this group, if positive
                 const int n_slices = (ps.s_hi - ps.s_lo + kSliceSteps - 1) / kSliceSteps;
-                if (n_slices == P.n_cs) {
+                if (n_slices == L.n_cs) {
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
-                        if (i < n_here && row < P.M) P.y[(size_t)(4 * grp + i) * P.M + row] = __float2half_rn(v[i]);
+                        if (i < n_here && row < L.M) L.y[(size_t)(4 * grp + i) * L.M + row] = __float2half_rn(v[i]);
                     continue;
                 }
-                unsigned long long* word = P.acc + (size_t)(4 * grp) * P.Mp + row;
+                unsigned long long* word = L.acc + (size_t)(4 * grp) * L.Mp + row;
                 unsigned long long old[4], add[4];
                 uint32_t bad = 0u;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const float scaled = v[i] * P.inv_unit;
-                    if (!(fabsf(scaled) < P.limit * (float)n_slices)) bad |= 1u << i;             // inf or NaN: finite inputs cannot get here
+                    const float scaled = v[i] * L.inv_unit;
+                    if (!(fabsf(scaled) < L.limit * (float)n_slices)) bad |= 1u << i;             // inf or NaN: finite inputs cannot get here
                     const long long qv = (bad >> i) & 1u ? 0LL : __float2ll_rn(scaled);
-                    add[i] = (unsigned long long)(qv + ((long long)n_slices << P.fix_bits)) + (1ULL << 55);
+                    add[i] = (unsigned long long)(qv + ((long long)n_slices << L.fix_bits)) + (1ULL << 55);
                 }
                 // all atomics of the thread back to back: nothing between them that could wait for an answer
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     old[i] = 0ULL;
                     if (i >= n_here) continue;
-                    if ((bad >> i) & 1u) atomicOr(word + (size_t)i * P.Mp, 1ULL << 63);           // sticky: the add below never carries into bit 63
-                    old[i] = atomicAdd(word + (size_t)i * P.Mp, add[i]);
+                    if ((bad >> i) & 1u) atomicOr(word + (size_t)i * L.Mp, 1ULL << 63);           // sticky: the add below never carries into bit 63
+                    old[i] = atomicAdd(word + (size_t)i * L.Mp, add[i]);
                 }
-                const long long first = (long long)ps.rt * P.n_cs, last = first + P.n_cs - 1;     // segments of this row tile: the tasks that touch it
+                const long long first = (NL == 1 ? 0LL : (long long)L.pair0) + (long long)ps.rt * L.n_cs, last = first + L.n_cs - 1;     // segments of this row tile: the tasks that touch it
                 const int arrivals = (int)(((last + 1) * P.n_tasks - 1) / P.n_groups) - (int)(((first + 1) * P.n_tasks - 1) / P.n_groups) + 1;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     if (i >= n_here || (int)((old[i] >> 55) & 0xFFu) != arrivals - 1) continue;   // other segments are still to come
                     const unsigned long long sum = (old[i] & kSumMask) + (add[i] & kSumMask);
-                    const long long total = (long long)sum - ((long long)P.n_cs << P.fix_bits);
+                    const long long total = (long long)sum - ((long long)L.n_cs << L.fix_bits);
                     const bool poisoned = ((bad >> i) & 1u) || (old[i] >> 63) != 0;
-                    if (row < P.M) P.y[(size_t)(4 * grp + i) * P.M + row] = poisoned ? __ushort_as_half((unsigned short)0x7FFF) : __float2half_rn(__ll2float_rn(total) * P.unit);
-                    word[(size_t)i * P.Mp] = 0ULL;               // resting state for the next call
+                    if (row < L.M) L.y[(size_t)(4 * grp + i) * L.M + row] = poisoned ? __ushort_as_half((unsigned short)0x7FFF) : __float2half_rn(__ll2float_rn(total) * L.unit);
+                    word[(size_t)i * L.Mp] = 0ULL;               // resting state for the next call
                 }
                 continue;
             }
 #pragma unroll 1
-            for (int c = grp; c < ps.n; c += kExpandGroups) {
+            for (int c = grp; NL == 1 && c < ps.n; c += kExpandGroups) {
                 float v[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) v[i] = 0.f;
@@ -658,11 +686,11 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
                     for (int i = 0; i < 16; ++i) v[i] = fmaf(gm, __uint_as_float(d[i]), v[i]);
                 }
                 const int b0 = (ps.c16 + c) * kGroupCols;
-                __half* yp = P.y + (size_t)b0 * P.M + row;
-                if (row < P.M) {
+                __half* yp = L.y + (size_t)b0 * L.M + row;
+                if (row < L.M) {
 #pragma unroll
                     for (int i = 0; i < 16; ++i)
-                        if (b0 + i < P.batch) yp[(size_t)i * P.M] = __float2half_rn(v[i]);
+                        if (b0 + i < P.batch) yp[(size_t)i * L.M] = __float2half_rn(v[i]);
                 }
             }
             fence_before();
@@ -676,7 +704,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
         //      batch columns is finished by CTA c % split: all CTAs send it that group's columns (already scaled by g_k and
         //      summed over the paths) into its receive buffer recv[its c / split][source rank][column][row], behind the rings.
         //      After the cluster barrier each CTA adds what it received in rank order and stores fp16.
-        PassWalker w = first_pass;
+        PassWalker<NL> w = first_pass;
         Pass ps;
         w.next(P, ps);
         if (warp >= 4) {
@@ -721,7 +749,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
                     float sum = 0.f;
                     for (int r = 0; r < split; ++r) sum += src[(size_t)r * kGroupCols * kTileM];
                     const int b = (ps.c16 + c) * kGroupCols + i;
-                    if (b < P.batch && row < P.M) P.y[(size_t)b * P.M + row] = __float2half_rn(sum);
+                    if (b < P.batch && row < P.L[0].M) P.L[0].y[(size_t)b * P.L[0].M + row] = __float2half_rn(sum);
                 }
         }
     }
@@ -733,7 +761,8 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams P, const __grid_constant
     if (warp == 1) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
     }
-    if (tid == 0 && *abort_flag) atomicExch(P.status, 1u);
+    if (tid == 0 && *abort_flag)
+        for (int l = 0; l < (NL == 1 ? 1 : P.n_layers); ++l) atomicExch(P.L[l].status, 1u);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -820,18 +849,20 @@ double unit_clocks(int n16, const Plan& p, int n_ops) {
     return std::max(32.0 * n16 + 52.0, two_each ? 180.0 + 8.0 * n16 : n_ops == 3 ? 345.0 : 300.0);
 }
 
-const void* kernel_for(int K, bool deq) {
-    if (K == 1) return deq ? (const void*)rabit_gemm_tc_kernel<1, true> : (const void*)rabit_gemm_tc_kernel<1, false>;
-    if (K == 2) return deq ? (const void*)rabit_gemm_tc_kernel<2, true> : (const void*)rabit_gemm_tc_kernel<2, false>;
-    return deq ? (const void*)rabit_gemm_tc_kernel<3, true> : (const void*)rabit_gemm_tc_kernel<3, false>;
+// (group: the form for several layers)
+const void* kernel_for(int K, bool deq, bool group = false) {
+    if (group) return K == 1 ? (const void*)rabit_gemm_tc_kernel<1, false, kMaxGroup> : K == 2 ? (const void*)rabit_gemm_tc_kernel<2, false, kMaxGroup> : (const void*)rabit_gemm_tc_kernel<3, false, kMaxGroup>;
+    if (K == 1) return deq ? (const void*)rabit_gemm_tc_kernel<1, true, 1> : (const void*)rabit_gemm_tc_kernel<1, false, 1>;
+    if (K == 2) return deq ? (const void*)rabit_gemm_tc_kernel<2, true, 1> : (const void*)rabit_gemm_tc_kernel<2, false, 1>;
+    return deq ? (const void*)rabit_gemm_tc_kernel<3, true, 1> : (const void*)rabit_gemm_tc_kernel<3, false, 1>;
 }
 
 // Function attributes are per device.
-cudaError_t prepare_kernel(int K, bool deq, int device) {
-    static bool done[64][6] = {};
-    const int slot = device >= 0 && device < 64 ? device : 0, inst = 2 * (K - 1) + (deq ? 1 : 0);
+cudaError_t prepare_kernel(int K, bool deq, int device, bool group = false) {
+    static bool done[64][9] = {};
+    const int slot = device >= 0 && device < 64 ? device : 0, inst = 3 * (K - 1) + (group ? 2 : deq ? 1 : 0);
     if (done[slot][inst] && slot == device) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(kernel_for(K, deq), cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(kernel_for(K, deq, group), cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
     if (e == cudaSuccess) done[slot][inst] = true;
     return e;
 }
@@ -859,9 +890,59 @@ constexpr double kLaunchClocks = 8000.0;             // launch, first loads, las
 constexpr double kExchangeClocks = 2500.0;           // exchange of a split task
 constexpr double kPublishClocks = 1500.0;            // atomics of a part of a row tile, besides their throughput
 
+// Up to 16 batch columns: contiguous ranges of the layers' (row tile, slice) pairs, met in the accumulate words.  tasks = 0 if
+// they cannot be.  (Against tasks over clusters or one per row tile: 4096 x 4096 8.6 -> 7.8 us, with one path 7.2 -> 6.5,
+// 4096 x 14336 16.5 -> 15.8, 28672 x 8192 55 -> 44; nowhere slower, so such calls look no further.)
+Plan stream_plan(int n_layers, const int* n_rt, const int* n_ct, int K, bool deq, int batch, int sms) {
+    Plan best = {};
+    Plan p = {};
+    p.stream = p.split = p.max16 = p.box16 = 1;
+    const int n_ops = deq ? 1 : K;
+    long long pairs = 0, row_tiles = 0;
+    int most_cs = 0, tail = 2;                            // tail: steps of a last slice, 1 if any layer's has just one
+    bool wide_x = true;
+    for (int l = 0; l < n_layers; ++l) {
+        const int steps = (n_ct[l] + 1) / 2, n_cs = (steps + kSliceSteps - 1) / kSliceSteps;
+        pairs += (long long)n_rt[l] * n_cs;
+        row_tiles += n_rt[l];
+        most_cs = std::max(most_cs, n_cs);
+        if (steps % kSliceSteps == 1) tail = 1;
+        wide_x = wide_x && n_ct[l] % 2 == 0;
+    }
+    if (most_cs > RABIT_LUT_MAX_SLICES || pairs >= (1LL << 30) || !fill_resources(p, K, n_ops, tail, wide_x)) return best;
+    best.clocks = 1e300;
+    const double pair = kSliceSteps * n_ops * unit_clocks(1, p, n_ops);
+    auto consider = [&](long long tasks) {
+        p.tasks = (int)tasks;
+        double worst = 0.0;
+        long long parts = 0, base = 0, t = 0;             // segments that are not whole row tiles
+        int l = 0;
+        double c = 0.0;
+        for (long long at = 0; at < pairs;) {             // segment by segment
+            const int n_cs = ((n_ct[l] + 1) / 2 + kSliceSteps - 1) / kSliceSteps;
+            const long long t_end = pairs * (t + 1) / tasks, tile_end = at + n_cs - (at - base) % n_cs, end = std::min(t_end, tile_end);
+            c += (double)(end - at) * pair + (c > 0.0 ? kPassClocks : 0.0);
+            parts += end - at < n_cs;
+            at = end;
+            if (at == base + (long long)n_rt[l] * n_cs && l + 1 < n_layers) { base = at; ++l; }
+            if (at == t_end) { worst = std::max(worst, c); c = 0.0; ++t; }
+        }
+        p.clocks = kLaunchClocks + worst + (parts > 0 ? kPublishClocks + parts * 128.0 * batch / 80.0 : 0.0);
+        if (p.clocks < best.clocks) best = p;
+    };
+    for (long long m = 1; m <= most_cs && row_tiles * m <= sms; ++m) consider(row_tiles * m);   // equal parts of a row tile (or nearly)
+    consider(std::min<long long>(sms, pairs));
+    return best;
+}
+
 Plan make_plan(int n_rt, int n_steps, int K, bool deq, int batch, int sms, int device, bool wide_x) {
     const int n16 = (batch + kGroupCols - 1) / kGroupCols;
     const int n_ops = deq ? 1 : K;
+    if (n16 == 1) {
+        const int n_ct = wide_x ? 2 * n_steps : 2 * n_steps - 1;
+        const Plan p = stream_plan(1, &n_rt, &n_ct, K, deq, batch, sms);
+        if (p.tasks > 0) return p;
+    }
     Plan best = {};
     best.clocks = 1e300;
     // (a) uniform tasks: every row tile in `chunks` chunks, the contraction of a task over `split` CTAs
@@ -883,30 +964,6 @@ Plan make_plan(int n_rt, int n_steps, int K, bool deq, int batch, int sms, int d
             if (p.clocks < best.clocks) best = p;
         }
         if (p.chunk16 <= 4) break;                   // narrower passes cost as much as these
-    }
-    // (c) up to 16 columns: contiguous ranges of (row tile, slice) pairs, met in the accumulate words
-    const int n_cs = (n_steps + kSliceSteps - 1) / kSliceSteps;
-    if (n16 == 1 && n_cs <= RABIT_LUT_MAX_SLICES && (long long)n_rt * n_cs < (1LL << 30)) {
-        Plan p = {};
-        p.stream = p.split = p.max16 = p.box16 = 1;
-        const long long pairs = (long long)n_rt * n_cs;
-        auto consider = [&](long long tasks) {
-            p.tasks = (int)tasks;
-            long long worst = 0, parts = 0;                                   // in clocks; segments that are not whole row tiles
-            const double pair = kSliceSteps * n_ops * unit_clocks(1, p, n_ops);
-            for (long long t = 0; t < tasks; ++t) {
-                const long long a = pairs * t / tasks, b = pairs * (t + 1) / tasks, segments = (b - 1) / n_cs - a / n_cs + 1;
-                const int cut = (a % n_cs != 0) + (b % n_cs != 0);
-                parts += segments == 1 && cut == 2 ? 1 : cut;
-                worst = std::max(worst, (long long)((b - a) * pair + (segments - 1) * kPassClocks));
-            }
-            p.clocks = kLaunchClocks + worst + (parts > 0 ? kPublishClocks + parts * 128.0 * batch / 80.0 : 0.0);
-            if (p.clocks < best.clocks) best = p;
-        };
-        if (fill_resources(p, K, n_ops, n_steps, wide_x)) {
-            for (long long m = 1; m <= n_cs && n_rt * m <= sms; ++m) consider(n_rt * m);      // equal parts of a row tile
-            consider(std::min<long long>(sms, pairs));
-        }
     }
     // (b) contiguous ranges of groups, one per SM: no last wave
     const long long groups = (long long)n_rt * n16;
@@ -943,18 +1000,113 @@ Plan make_plan(int n_rt, int n_steps, int K, bool deq, int batch, int sms, int d
 
 int sms_of(const rabit_layer& L) { return L.sm_count > 0 ? L.sm_count : 148; }
 
-Plan plan_for(const rabit_layer& L, bool deq, int batch) {
-    struct Entry { int n_rt, n_ct, K, deq, n16, sms; Plan plan; };
+// The plan of a layer, or of several in one launch.
+Plan plan_for(const rabit_layer* const* layers, int n_layers, bool deq, int batch) {
+    struct Entry { int n, n_rt[kMaxGroup], n_ct[kMaxGroup], K, deq, n16, sms; Plan plan; };
     static thread_local std::vector<Entry> plans;     // a search costs tens of microseconds; a program calls few shapes
-    const int n16 = (batch + kGroupCols - 1) / kGroupCols, n_rt = L.geom.n_rt, n_ct = L.geom.n_ct, K = L.geom.K, sms = sms_of(L);
-    for (const Entry& e : plans)
-        if (e.n_rt == n_rt && e.n_ct == n_ct && e.K == K && e.deq == (int)deq && e.n16 == n16 && e.sms == sms) return e.plan;
+    const int n16 = (batch + kGroupCols - 1) / kGroupCols, K = layers[0]->geom.K, sms = sms_of(*layers[0]);
+    for (const Entry& e : plans) {
+        bool same = e.n == n_layers && e.K == K && e.deq == (int)deq && e.n16 == n16 && e.sms == sms;
+        for (int l = 0; l < n_layers && same; ++l) same = e.n_rt[l] == layers[l]->geom.n_rt && e.n_ct[l] == layers[l]->geom.n_ct;
+        if (same) return e.plan;
+    }
+    Entry e = {};
+    e.n = n_layers; e.K = K; e.deq = (int)deq; e.n16 = n16; e.sms = sms;
+    for (int l = 0; l < n_layers; ++l) { e.n_rt[l] = layers[l]->geom.n_rt; e.n_ct[l] = layers[l]->geom.n_ct; }
+    e.plan = n_layers > 1 ? stream_plan(n_layers, e.n_rt, e.n_ct, K, deq, n16 * kGroupCols, sms)
+                          : make_plan(e.n_rt[0], (e.n_ct[0] + 1) / 2, K, deq, n16 * kGroupCols, sms, layers[0]->device, e.n_ct[0] % 2 == 0);
     if (plans.size() >= 256) plans.clear();
-    plans.push_back(Entry{n_rt, n_ct, K, (int)deq, n16, sms, make_plan(n_rt, (n_ct + 1) / 2, K, deq, n16 * kGroupCols, sms, L.device, n_ct % 2 == 0)});
+    plans.push_back(e);
     return plans.back().plan;
+}
+Plan plan_for(const rabit_layer& L, bool deq, int batch) {
+    const rabit_layer* one = &L;
+    return plan_for(&one, 1, deq, batch);
+}
+
+void fill_layer(GemmLayer& D, const rabit_layer& L, void* y, int pair0) {
+    const RabitGeom& G = L.geom;
+    D.bits = reinterpret_cast<const unsigned char*>(L.d_bits);
+    D.g = (const __half*)L.d_g;
+    D.h = (const __half*)L.d_h;
+    D.y = (__half*)y;
+    D.status = L.d_status;
+    D.acc = L.d_acc;
+    D.M = G.M; D.N = G.N; D.Mp = G.Mp; D.n_rt = G.n_rt; D.n_ct = G.n_ct; D.n_cs = G.n_cs;
+    D.fix_bits = G.fix_bits;
+    D.unit = ldexpf(1.f, G.unit_exp); D.inv_unit = ldexpf(1.f, -G.unit_exp); D.limit = ldexpf(1.f, G.fix_bits);
+    D.pair0 = pair0;
+}
+template <int NL>
+void fill_common(GemmParams<NL>& P, const Plan& p, int n_layers, int batch, long long n_groups) {
+    P.n_layers = n_layers;
+    P.batch = batch;
+    P.n16 = (batch + kGroupCols - 1) / kGroupCols;
+    P.n_tasks = p.tasks;
+    P.chunks = p.chunks; P.chunk16 = p.chunk16;
+    P.n_groups = (int)std::min<long long>(0x7FFFFFFF, n_groups);          // (only read where it fits)
+    P.quot = P.n_groups / P.n_tasks; P.rem = P.n_groups % P.n_tasks;
+    P.stream = p.stream;
+    P.max16 = p.max16;
+    P.split = p.split;
+    P.recv_off = p.recv_off;
+    P.stages = p.stages; P.stage_bytes = p.stage_bytes; P.x_steps = p.x_steps; P.w_stages = p.w_stages;
+    P.box16 = p.box16;
+    P.n_acc = p.n_acc;
+    P.units = p.units; P.a_col = p.n_acc * p.max16 * kGroupCols;
 }
 
 }  // namespace
+
+int rabit_gemm_tc_max_group() { return kMaxGroup; }
+
+// One launch for several layers of at most 16 batch rows: equal path counts, no layer twice (it would share its accumulate words).
+bool rabit_gemm_tc_group_supports(const rabit_layer* const* layers, int n_layers, int batch) {
+    if (n_layers < 1 || n_layers > kMaxGroup || batch < 1 || batch > kGroupCols) return false;
+    long long pairs = 0;
+    for (int l = 0; l < n_layers; ++l) {
+        const rabit_layer& L = *layers[l];
+        if (!rabit_gemm_tc_supports(L, batch) || L.geom.K != layers[0]->geom.K || L.geom.n_cs > RABIT_LUT_MAX_SLICES) return false;
+        pairs += (long long)L.geom.n_rt * L.geom.n_cs;
+        for (int m = 0; m < l; ++m)
+            if (layers[m] == &L) return false;
+    }
+    return pairs < (1LL << 30);
+}
+
+cudaError_t rabit_launch_gemm_tc_group(const rabit_layer* const* layers, int n_layers, const void* const* xs, void* const* ys, int batch, cudaStream_t stream) {
+    if (n_layers == 1) return rabit_launch_gemm_tc(*layers[0], xs[0], ys[0], batch, stream);
+    if (!rabit_gemm_tc_group_supports(layers, n_layers, batch)) return cudaErrorInvalidValue;
+    const int K = layers[0]->geom.K, device = layers[0]->device;
+    const Plan p = plan_for(layers, n_layers, false, batch);
+    if (p.tasks < 1) return cudaErrorInvalidValue;
+    GemmParams<kMaxGroup> P;
+    XMaps<kMaxGroup> maps;
+    int pairs = 0;
+    for (int l = 0; l < kMaxGroup; ++l) {
+        if (l >= n_layers) { P.L[l] = P.L[0]; maps.map[l] = maps.map[0]; continue; }
+        const RabitGeom& G = layers[l]->geom;
+        cudaError_t e = x_tensor_map(xs[l], G.N, batch, 1, p.x_steps, &maps.map[l]);
+        if (e != cudaSuccess) return e;
+        fill_layer(P.L[l], *layers[l], ys[l], pairs);
+        pairs += G.n_rt * G.n_cs;
+    }
+    fill_common(P, p, n_layers, batch, pairs);
+    cudaError_t e = prepare_kernel(K, false, device, true);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned int)p.tasks);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = p.smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    void* args[2] = {&P, &maps};
+    return cudaLaunchKernelExC(&cfg, kernel_for(K, false, true), args);
+}
 
 bool rabit_gemm_tc_supports(const rabit_layer& L, int batch) {
     return batch >= 1 && batch <= (1 << 24) && L.geom.K <= 3 && encode_tiled_fn() != nullptr;
@@ -967,36 +1119,15 @@ cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, i
     const RabitGeom& G = L.geom;
     const Plan p = plan_for(L, dequantised, batch);
     if (p.tasks < 1) return cudaErrorInvalidValue;
-    CUtensorMap map;
-    cudaError_t e = x_tensor_map(x, G.N, batch, p.box16, p.x_steps, &map);
+    XMaps<1> maps;
+    cudaError_t e = x_tensor_map(x, G.N, batch, p.box16, p.x_steps, &maps.map[0]);
     if (e != cudaSuccess) return e;
     e = prepare_kernel(G.K, dequantised, L.device);
     if (e != cudaSuccess) return e;
 
-    GemmParams P;
-    P.bits = reinterpret_cast<const unsigned char*>(L.d_bits);
-    P.g = (const __half*)L.d_g;
-    P.h = (const __half*)L.d_h;
-    P.y = (__half*)y;
-    P.status = L.d_status;
-    P.M = G.M; P.N = G.N; P.Mp = G.Mp; P.n_ct = G.n_ct;
-    P.batch = batch;
-    P.n16 = (batch + kGroupCols - 1) / kGroupCols;
-    P.n_tasks = p.tasks;
-    P.chunks = p.chunks; P.chunk16 = p.chunk16;
-    P.n_groups = (int)std::min<long long>(0x7FFFFFFF, (long long)G.n_rt * (p.stream ? G.n_cs : P.n16));   // (only read where it fits)
-    P.quot = P.n_groups / P.n_tasks; P.rem = P.n_groups % P.n_tasks;
-    P.stream = p.stream; P.n_cs = G.n_cs;
-    P.acc = L.d_acc;
-    P.fix_bits = G.fix_bits;
-    P.unit = ldexpf(1.f, G.unit_exp); P.inv_unit = ldexpf(1.f, -G.unit_exp); P.limit = ldexpf(1.f, G.fix_bits);
-    P.max16 = p.max16;
-    P.split = p.split;
-    P.recv_off = p.recv_off;
-    P.stages = p.stages; P.stage_bytes = p.stage_bytes; P.x_steps = p.x_steps; P.w_stages = p.w_stages;
-    P.box16 = p.box16;
-    P.n_acc = p.n_acc;
-    P.units = p.units; P.a_col = p.n_acc * p.max16 * kGroupCols;
+    GemmParams<1> P;
+    fill_layer(P.L[0], L, y, 0);
+    fill_common(P, p, 1, batch, (long long)G.n_rt * (p.stream ? G.n_cs : (batch + kGroupCols - 1) / kGroupCols));
 
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned int)(p.tasks * p.split));
@@ -1012,6 +1143,6 @@ cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, i
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = p.split > 1 ? 2 : 1;
-    void* args[2] = {&P, &map};
+    void* args[2] = {&P, &maps};
     return cudaLaunchKernelExC(&cfg, kernel_for(G.K, dequantised), args);
 }

@@ -88,6 +88,9 @@ cudaError_t rabit_launch_gemv_lut_group(const rabit_layer* const* layers, int n_
                                         int batch, cudaStream_t stream, unsigned long long* const* acc_override, unsigned int* status_override);
 cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, int batch, cudaStream_t stream, bool dequantised = false);
 bool rabit_gemm_tc_supports(const rabit_layer& L, int batch);
+int rabit_gemm_tc_max_group();
+bool rabit_gemm_tc_group_supports(const rabit_layer* const* layers, int n_layers, int batch);
+cudaError_t rabit_launch_gemm_tc_group(const rabit_layer* const* layers, int n_layers, const void* const* xs, void* const* ys, int batch, cudaStream_t stream);
 double rabit_gemm_tc_estimate_us(const rabit_layer& L, int batch);
 
 #endif  // RABIT_INTERNAL_H_
