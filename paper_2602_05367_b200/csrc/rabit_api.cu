@@ -167,7 +167,7 @@ extern "C" int rabit_linear(const rabit_layer* layer, const void* x, void* y, in
         const double packed_mb = (double)G.K * G.Mp * G.N / 8.0e6;
         if (rabit_gemv_lut_supports(*layer, batch)) {
             variant = 5;
-        } else if (batch <= RABIT_MAX_GEMV_BATCH && rabit_gemv_f16_supports(*layer, RABIT_MAX_GEMV_BATCH)) {
+        } else if (batch <= RABIT_MAX_GEMV_BATCH && rabit_gemv_f16_supports(*layer, kF16Rows)) {
             variant = 6;                    // 3..16 rows: one pass over the weights with the batch in the MMA's N dimension
         } else if (batch <= 4 && packed_mb <= 8.0 && rabit_gemv_lut_supports(*layer, 1)) {
             variant = 5;                    // two passes of the table-driven kernel
@@ -217,9 +217,9 @@ extern "C" int rabit_linear(const rabit_layer* layer, const void* x, void* y, in
             break;
         }
         case 6:                             // beyond eight rows the GEMM (see kF16Rows)
-            if (!rabit_gemv_f16_supports(*layer, batch < RABIT_MAX_GEMV_BATCH ? batch : RABIT_MAX_GEMV_BATCH))
+            if (!rabit_gemv_f16_supports(*layer, std::min(batch, kF16Rows)) || (batch > kF16Rows && !rabit_gemm_tc_supports(*layer, batch)))
                 return rabit_fail(RABIT_INVALID_ARG, "rabit_linear: f16 tensor-core GEMV cannot run this layer");
-            e = batch <= kF16Rows || !rabit_gemm_tc_supports(*layer, batch) ? rabit_launch_gemv_f16(*layer, x, y, batch, st) : rabit_launch_gemm_tc(*layer, x, y, batch, st);
+            e = batch <= kF16Rows ? rabit_launch_gemv_f16(*layer, x, y, batch, st) : rabit_launch_gemm_tc(*layer, x, y, batch, st);
             break;
         default:
             e = rabit_launch_plain(*layer, x, y, batch, st);
@@ -269,7 +269,7 @@ extern "C" int rabit_linear_group(const rabit_layer* const* layers, const void* 
     }
     {
         bool f16 = batch <= RABIT_MAX_GEMV_BATCH;                // 3..16 rows: the f16 tensor-core GEMV
-        for (int l = 0; l < n_layers && f16; ++l) f16 = (layers[l]->variant == 0 || layers[l]->variant == 6) && rabit_gemv_f16_supports(*layers[l], batch);
+        for (int l = 0; l < n_layers && f16; ++l) f16 = (layers[l]->variant == 0 || layers[l]->variant == 6) && rabit_gemv_f16_supports(*layers[l], std::min(batch, kF16Rows));
         // beyond eight rows the GEMM, up to four layers a launch
         bool gemm = f16 && batch > kF16Rows;
         for (int l = 0; l < n_layers && gemm; l += rabit_gemm_tc_max_group())

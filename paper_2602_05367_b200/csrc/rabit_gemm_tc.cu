@@ -64,6 +64,8 @@ constexpr int kThreads = (4 + kExpandWarps) * 32;
 constexpr long long kWaitLimitCycles = 1LL << 31;
 constexpr unsigned long long kSumMask = (1ULL << 55) - 1;
 
+constexpr int kMaxTasks = 512;
+constexpr long long kMaxPairs = 1LL << 23; // (row tile, slice) pairs of a stream launch
 constexpr int kMaxGroup = 4;                // layers of a grouped launch
 
 struct GemmLayer {
@@ -657,8 +659,9 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                     if ((bad >> i) & 1u) atomicOr(word + (size_t)i * L.Mp, 1ULL << 63);           // sticky: the add below never carries into bit 63
                     old[i] = atomicAdd(word + (size_t)i * L.Mp, add[i]);
                 }
-                const long long first = (NL == 1 ? 0LL : (long long)L.pair0) + (long long)ps.rt * L.n_cs, last = first + L.n_cs - 1;     // segments of this row tile: the tasks that touch it
-                const int arrivals = (int)(((last + 1) * P.n_tasks - 1) / P.n_groups) - (int)(((first + 1) * P.n_tasks - 1) / P.n_groups) + 1;
+                // segments of this row tile: the tasks that touch it (pairs < kMaxPairs and tasks <= kMaxTasks: 32 bits hold the products)
+                const uint32_t first = (uint32_t)((NL == 1 ? 0 : L.pair0) + ps.rt * L.n_cs), past = first + (uint32_t)L.n_cs, tasks = (uint32_t)P.n_tasks;
+                const int arrivals = (int)((past * tasks - 1u) / (uint32_t)P.n_groups) - (int)(((first + 1u) * tasks - 1u) / (uint32_t)P.n_groups) + 1;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     if (i >= n_here || (int)((old[i] >> 55) & 0xFFu) != arrivals - 1) continue;   // other segments are still to come
@@ -670,27 +673,29 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                 }
                 continue;
             }
+            if constexpr (NL == 1) {
 #pragma unroll 1
-            for (int c = grp; NL == 1 && c < ps.n; c += kExpandGroups) {
-                float v[16];
+                for (int c = grp; c < ps.n; c += kExpandGroups) {
+                    float v[16];
 #pragma unroll
-                for (int i = 0; i < 16; ++i) v[i] = 0.f;
+                    for (int i = 0; i < 16; ++i) v[i] = 0.f;
 #pragma unroll
-                for (int m = 0; m < (n_ops == 1 ? 2 : n_ops); ++m) {
-                    if (n_ops == 1 && m >= n_acc) break;
-                    uint32_t d[16];
-                    tmem_ld16(lane_base + (uint32_t)((m * P.max16 + c) * kGroupCols), d);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    const float gm = DEQ ? 1.f : scale(n_ops == 1 ? 0 : m);
+                    for (int m = 0; m < (n_ops == 1 ? 2 : n_ops); ++m) {
+                        if (n_ops == 1 && m >= n_acc) break;
+                        uint32_t d[16];
+                        tmem_ld16(lane_base + (uint32_t)((m * P.max16 + c) * kGroupCols), d);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                        const float gm = DEQ ? 1.f : scale(n_ops == 1 ? 0 : m);
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) v[i] = fmaf(gm, __uint_as_float(d[i]), v[i]);
-                }
-                const int b0 = (ps.c16 + c) * kGroupCols;
-                __half* yp = L.y + (size_t)b0 * L.M + row;
-                if (row < L.M) {
+                        for (int i = 0; i < 16; ++i) v[i] = fmaf(gm, __uint_as_float(d[i]), v[i]);
+                    }
+                    const int b0 = (ps.c16 + c) * kGroupCols;
+                    __half* yp = L.y + (size_t)b0 * L.M + row;
+                    if (row < L.M) {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        if (b0 + i < P.batch) yp[(size_t)i * L.M] = __float2half_rn(v[i]);
+                        for (int i = 0; i < 16; ++i)
+                            if (b0 + i < P.batch) yp[(size_t)i * L.M] = __float2half_rn(v[i]);
+                    }
                 }
             }
             fence_before();
@@ -909,7 +914,7 @@ Plan stream_plan(int n_layers, const int* n_rt, const int* n_ct, int K, bool deq
         if (steps % kSliceSteps == 1) tail = 1;
         wide_x = wide_x && n_ct[l] % 2 == 0;
     }
-    if (most_cs > RABIT_LUT_MAX_SLICES || pairs >= (1LL << 30) || !fill_resources(p, K, n_ops, tail, wide_x)) return best;
+    if (most_cs > RABIT_LUT_MAX_SLICES || pairs >= kMaxPairs || sms > kMaxTasks || !fill_resources(p, K, n_ops, tail, wide_x)) return best;
     best.clocks = 1e300;
     const double pair = kSliceSteps * n_ops * unit_clocks(1, p, n_ops);
     auto consider = [&](long long tasks) {
@@ -1071,7 +1076,7 @@ bool rabit_gemm_tc_group_supports(const rabit_layer* const* layers, int n_layers
         for (int m = 0; m < l; ++m)
             if (layers[m] == &L) return false;
     }
-    return pairs < (1LL << 30);
+    return pairs < kMaxPairs && sms_of(*layers[0]) <= kMaxTasks;
 }
 
 cudaError_t rabit_launch_gemm_tc_group(const rabit_layer* const* layers, int n_layers, const void* const* xs, void* const* ys, int batch, cudaStream_t stream) {
