@@ -30,7 +30,7 @@
 //          store.
 //
 // Work.  One CTA per SM.  An output tile is 128 weight rows x N batch columns, N a multiple of 16 chosen for the call.
-// make_plan() picks between: whole tiles; tiles whose contraction is split over a cluster of 2, 4 or 8 CTAs that add their partial
+// make_plan() picks between: whole tiles; tiles whose contraction is split over a cluster of 2 to 8 CTAs that add their partial
 // results through distributed shared memory (fixed order, no atomics); and, for long batches, contiguous ranges of
 // 16-column groups in (row tile, group) order, one per SM, so that no last wave is left over.
 //
@@ -90,7 +90,7 @@ struct GemmParams {
     int n_groups, quot, rem;                // row tiles * n16 (stream: row tiles * n_cs, over all layers); that by n_tasks
     int stream;                             // a task is a contiguous range of (row tile, slice) pairs, all of at most 16 batch columns
     int max16;                              // most groups one pass can accumulate
-    int split;                              // CTAs (one cluster) that share the contraction of a task: 1, 2, 4 or 8
+    int split;                              // CTAs (one cluster) that share the contraction of a task, up to 8
     int recv_off;                           // receive buffer of a split task, from the control block
     int stages, stage_bytes, x_steps;       // x ring: bytes and steps of one stage
     int w_stages;                           // weight ring, behind the x ring: per stage the sign tiles [K][8][512], then h [K][256]
@@ -956,7 +956,7 @@ Plan make_plan(int n_rt, int n_steps, int K, bool deq, int batch, int sms, int d
         p.max16 = p.chunk16 = p.box16 = (n16 + chunks - 1) / chunks;
         p.chunks = (n16 + p.chunk16 - 1) / p.chunk16;
         if (p.chunks != chunks) continue;
-        for (int split = 1; split <= 8; split *= 2) {
+        for (int split = 1; split <= 8; ++split) {
             p.split = split;
             p.tasks = n_rt * chunks;
             const long long ctas = (long long)p.tasks * split;
