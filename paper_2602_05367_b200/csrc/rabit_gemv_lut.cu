@@ -365,8 +365,8 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
             graw[k] = 0;
             if (RABIT_IN_RANGE(row >= 0 && row < Mp)) graw[k] = ldg_u16_early(g_base + (size_t)k * Mp + row);
         }
-        const int bb_next = i + 1 < n_mine ? bb + kWarps : bb;           // (the last iteration re-reads its own block: in bounds, unused)
-        const bool next_ok = RABIT_IN_RANGE(bb_next >= 0 && bb_next < n_blocks && (long long)R.b0 + bb_next < (long long)L.n_cs * L.n_rb);
+        const int bb_next = bb + kWarps;
+        const bool next_ok = i + 1 < n_mine && RABIT_IN_RANGE(bb_next >= 0 && bb_next < n_blocks && (long long)R.b0 + bb_next < (long long)L.n_cs * L.n_rb);
         if (owe) {
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
