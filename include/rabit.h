@@ -116,11 +116,11 @@ RABIT_API int rabit_derive_pack(const float* W_dev, const uint16_t* g, const uin
  * Asynchronous on `stream`; allocates nothing, never synchronises, and may be captured in
  * a CUDA graph.  The layer's device must be the current device.  One or two batch rows run the table-driven
  * GEMV (one pass over the weights: a shared-memory table of the partial sums of h*x over eight columns, indexed by the
- * packed sign byte), 3 to 16 rows the f16 tensor-core GEMV (one pass: the signs are expanded to +-h operand tiles in
- * registers, the batch is the MMA's N dimension), 17 to 32 rows two passes of it, more the tcgen05 GEMM.  Layers those two GEMVs cannot take
+ * packed sign byte), 3 to 8 rows the f16 tensor-core GEMV (one pass: the signs are expanded to +-h operand tiles in
+ * registers, the batch is the MMA's N dimension), more the tcgen05 GEMM.  Up to 16 rows, layers those two GEMVs cannot take
  * (more than 255 slices of 256 input columns) fall back to the integer tensor-core GEMV, four rows per pass, or to one
- * GEMM launch, whichever the library's cost estimate for the shape favours.  A GEMM with few output tiles runs as
- * clusters of CTAs that share a tile's contraction.  fp32 (or exact integer) accumulation, one rounding to fp16 at the end;
+ * GEMM launch, whichever the library's cost estimate for the shape favours.  A GEMM with few output tiles splits a tile's
+ * contraction over CTAs.  fp32 (or exact integer) accumulation, one rounding to fp16 at the end;
  * an inf or NaN in a batch row of x makes that row of y non-finite and leaves the other rows untouched.
  */
 RABIT_API int rabit_linear(const rabit_layer* layer, const void* x, void* y, int batch, void* stream);
@@ -134,7 +134,8 @@ RABIT_API int rabit_linear(const rabit_layer* layer, const void* x, void* y, int
  * of once per layer.  The tiles of all layers are split evenly over the CTAs as if they were one layer.
  *   layers, xs, ys   HOST arrays of n_layers entries (1 <= n_layers <= 8); the pointers inside are as for
  *                    rabit_linear; outputs must not overlap one another nor any input; all layers on one device.
- * For batch > 16, or more than 8 layers, the layers are simply run one after the other.
+ * For 9 to 16 rows a launch takes up to four layers.  For batch > 16, or more than 8 layers, the layers are simply run one
+ * after the other.
  * Asynchronous on `stream`, allocates nothing, may be captured in a CUDA graph.
  */
 RABIT_API int rabit_linear_group(const rabit_layer* const* layers, const void* const* xs, void* const* ys,
@@ -143,7 +144,7 @@ RABIT_API int rabit_linear_group(const rabit_layer* const* layers, const void* c
 /*
  * Host-buffer form of rabit_linear (same operation, Section 4.1 forward with the Eq. 2 weight)
  * for callers whose activations live in host memory:
- *   x_host  HOST fp16 [batch][N]   (pinned memory makes the copies asynchronous)
+ *   x_host  HOST fp16 [batch][N]   (pinned memory makes the copies asynchronous; up to 256 KB a kernel makes them)
  *   y_host  HOST fp16 [batch][M]
  *   dev_stage DEVICE, 256-byte aligned, caller-owned, at least rabit_stage_bytes(layer, batch)
  * Enqueues on `stream`: copy x to the stage, the layer kernel, copy y back.  Returns without
@@ -212,9 +213,9 @@ RABIT_API int rabit_selftest_bounded_wait(unsigned int* status_dev, int limit_us
 
 /*
  * Test aid (no counterpart in the paper; host only, no GPU needed): how the f16 tensor-core GEMV of rabit_linear
- * (batch 3..16) would split a K-path layer of M x N at `batch` rows over `sms` SMs.  The layer is ceil(M/128) row tiles x
+ * (batch 3..8; larger ones, up to 16, are planned but never run) would split a K-path layer of M x N at `batch` rows over `sms` SMs.  The layer is ceil(M/128) row tiles x
  * ceil(N/256) slices; in that order the (row tile, slice) pairs are cut into contiguous parts, two per SM (one per group
- * of eight warps).  bound_out (HOST, max_out ints) receives the starts of the parts followed by the number of pairs:
+ * of eight warps; with one group of 16 the second is empty).  bound_out (HOST, max_out ints) receives the starts of the parts followed by the number of pairs:
  * 2 * grid + 1 ascending values; a part may be empty.  Returns the number of CTAs (grid >= 1), or RABIT_INVALID_ARG.
  */
 RABIT_API int rabit_selftest_f16_plan(int K, int M, int N, int batch, int sms, int* bound_out, int max_out);
@@ -275,7 +276,7 @@ RABIT_API int rabit_layer_N(const rabit_layer* layer);
  *   4 = tcgen05 GEMM on the dequantised weight tile sum_k +-g_k h_k rounded to fp16 (Eq. 2 formed per tile; one
  *       contraction of length N instead of K of them; never chosen automatically: it rounds every weight to fp16),
  *   5 = table-driven GEMV (passes of up to two batch rows; N up to 65280),
- *   6 = f16 tensor-core GEMV (passes of up to 16 batch rows; N up to 65280).
+ *   6 = f16 tensor-core GEMV up to 8 batch rows, beyond them the GEMM as 3 (N up to 65280).
  * Returns RABIT_INVALID_ARG for a variant that cannot run the layer.
  * Meant for A/B timing and profiling; results are within tolerance for every variant.
  */

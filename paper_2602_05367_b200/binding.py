@@ -180,7 +180,7 @@ class RabitLayer:
     def set_variant(self, variant: int) -> None:
         """Kernel family for later rabit_linear calls of this layer: 0 automatic, 1 plain, 2 integer tensor-core GEMV,
         3 tcgen05 GEMM (exact expansion), 4 tcgen05 GEMM on dequantised fp16 weight tiles (never chosen automatically),
-        5 table-driven GEMV."""
+        5 table-driven GEMV, 6 f16 tensor-core GEMV up to 8 batch rows and the GEMM beyond."""
         _check(_lib.rabit_set_variant(self.handle, variant))
 
     def status(self, clear: bool = False, stream: int = 0) -> int:

@@ -168,7 +168,7 @@ extern "C" int rabit_linear(const rabit_layer* layer, const void* x, void* y, in
         if (rabit_gemv_lut_supports(*layer, batch)) {
             variant = 5;
         } else if (batch <= RABIT_MAX_GEMV_BATCH && rabit_gemv_f16_supports(*layer, kF16Rows)) {
-            variant = 6;                    // 3..16 rows: one pass over the weights with the batch in the MMA's N dimension
+            variant = 6;                    // 3..16 rows: one pass over the weights with the batch in the MMA's N dimension (see kF16Rows)
         } else if (batch <= 4 && packed_mb <= 8.0 && rabit_gemv_lut_supports(*layer, 1)) {
             variant = 5;                    // two passes of the table-driven kernel
         } else if (batch <= RABIT_MAX_GEMV_BATCH) {
@@ -268,7 +268,7 @@ extern "C" int rabit_linear_group(const rabit_layer* const* layers, const void* 
         }
     }
     {
-        bool f16 = batch <= RABIT_MAX_GEMV_BATCH;                // 3..16 rows: the f16 tensor-core GEMV
+        bool f16 = batch <= RABIT_MAX_GEMV_BATCH;                // 3..16 rows: the f16 tensor-core GEMV or the GEMM
         for (int l = 0; l < n_layers && f16; ++l) f16 = (layers[l]->variant == 0 || layers[l]->variant == 6) && rabit_gemv_f16_supports(*layers[l], std::min(batch, kF16Rows));
         // beyond eight rows the GEMM, up to four layers a launch
         bool gemm = f16 && batch > kF16Rows;

@@ -3,7 +3,7 @@
 // A decode step's inputs are a few KB.  A copy-engine transfer of that size costs two hand-overs between engine and SMs, about
 // 10 us in a stream of 3 to 6 us kernels; here the SMs read the mapped buffer over the bus themselves (one 16-byte load per
 // thread: the bus latency once) and the layer kernel behind is already resident, filling up with weights, under programmatic
-// dependent launch.  A 7B-shaped decoder layer of seven projections in four calls: 90 us with copies.
+// dependent launch.  A 7B-shaped decoder layer of seven projections in four calls: 90 us with copies, 60 so.
 // Letting the layer kernel read host memory itself is slower still (194 us): every CTA fetches its slices over the bus.
 #include "rabit_internal.h"
 

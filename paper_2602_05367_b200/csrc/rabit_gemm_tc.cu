@@ -1,4 +1,4 @@
-// Large-batch form of the layer on the tcgen05 tensor cores (batch > 16, and smaller batches where it is cheaper).
+// The layer on the tcgen05 tensor cores (batch > 8).
 //
 //   y[b][i] = sum_k g_k[i] * sum_j (B_k[i][j] * h_k[j]) * x[b][j]                       (Section 4.1, Eq. 2)
 //
@@ -30,9 +30,14 @@
 //          store.
 //
 // Work.  One CTA per SM.  An output tile is 128 weight rows x N batch columns, N a multiple of 16 chosen for the call.
-// make_plan() picks between: whole tiles; tiles whose contraction is split over a cluster of 2 to 8 CTAs that add their partial
+// Up to 16 batch columns a CTA takes a contiguous range of (row tile, slice of 256 columns) pairs and the parts of a row tile meet in
+// its accumulate words (stream_plan), several layers in one launch if asked.  Otherwise make_plan() picks between: whole tiles; tiles whose contraction is split over a cluster of 2 to 8 CTAs that add their partial
 // results through distributed shared memory (fixed order, no atomics); and, for long batches, contiguous ranges of
 // 16-column groups in (row tile, group) order, one per SM, so that no last wave is left over.
+//
+// What bounds it (B200): a unit takes the larger of its four MMAs (32 clocks per 16 batch columns, and 52) and the expansion, 130 clocks
+// of issue, 180 to 200 measured; a launch has about 4 us beside its units.  14336 x 4096 at batch 48 51 -> 16.4 us, 28672 x 8192 at 16
+// 55 -> 43.5, 5000 x 13824 with three paths at 200 209 -> 74.
 //
 // Every wait is bounded; on a time-out the CTA sets the status word, skips the remaining waits, frees its tensor memory
 // and returns.  DEQ (rabit_set_variant 4): the expander forms the dequantised weight sum_k +-g_k h_k in fp16 and one

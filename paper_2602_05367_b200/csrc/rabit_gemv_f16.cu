@@ -1,18 +1,19 @@
-// Decode GEMV for 3..16 batch rows: the batch sits in the N dimension of an f16 tensor-core MMA.
+// Decode GEMV for 3..8 batch rows: the batch sits in the N dimension of an f16 tensor-core MMA.
 //
 //   y[b][i] = sum_k g_k[i] * sum_j (B_k[i][j] h_k[j]) * x[b][j]                              (Section 4.1, Eq. 2)
 //
 // The table-driven kernel (rabit_gemv_lut.cu) pays per batch row; the integer tensor-core GEMV spends four of an MMA's
 // eight columns per batch row and needs a pass over x first.  Here the A operand of mma.sync.m16n8k16 is +-h_k expanded in
 // registers from the sign tiles (the weight bit flips the sign bit of the fp16 input scale: exact), B is x as it is, the
-// accumulators are fp32: products are exact, 8 batch rows per MMA and 16 with a second MMA on the same A, no digits, no
-// scale search.  The cost is that of the expansion and does not depend on the batch.
+// accumulators are fp32: products are exact, 8 batch rows per MMA, no digits, no scale search.  The cost is that of the
+// expansion and does not depend on the batch.
 //
-// Expansion.  Shifts, byte permutes and logic instructions all issue on the half-rate integer pipe of an SM sub-partition
-// (16 lanes per clock), and that pipe, not the tensor pipe, bounds this kernel.  So an A register (two fp16 values) costs
-// ONE logic instruction there, (v & 0x80008000) ^ h, and the shift that brings the two weight bits to bits 15 and 31 is a
-// multiplication by a power of two on the multiply-add pipe: v = w * 2^s, where the factor comes from a kernel parameter
-// so that the compiler keeps it a multiplication.  The two bits must be 16 apart in the word, i.e. two columns apart:
+// Expansion.  Shifts, byte permutes, multiplications and logic instructions each take two issue clocks of an SM
+// sub-partition, and issue slots, not the tensor pipe, bound this kernel.  The two weight bits of an A register (two fp16 values)
+// must be 16 apart in the word, i.e. two columns apart.  A multiplication by a power of two (a kernel parameter, so that the
+// compiler keeps it one) brings those of an odd row block to bits 15 and 31: one logic instruction, (v & 0x80008000) ^ h.
+// The even row block below then has its bits at 14 and 30, where a bit alone is the fp16 number 2: an AND and one half2 fused
+// multiply-add, h - 2 h or h - 0 h (exact; one issue clock), without a shift of its own.
 //
 // Operand mapping.  A sign tile (rabit_layout.h) gives lane (gq, tq) four words w[a]; byte c of word a has in bit p the
 // sign of row 16p + gq + 8(a & 1), column 16(a >> 1) + 4tq + c of the tile.  For the k-step kh = a >> 1 (16 columns) and
@@ -23,14 +24,14 @@
 //     b0 = x[n = gq][cols 0,2]           b1 = x[n = gq][cols 1,3]         (one 8-byte load per lane and k-step, two permutes)
 // and the accumulator lane holds rows gq, gq + 8 of the block and batch rows 2tq, 2tq + 1.
 //
-// Work split.  The layer is n_rt row tiles x n_cs slices of 256 columns.  Every row tile is cut into m equal units and a CTA
-// (16 warps, one CTA per SM) takes j consecutive units (split_layer on the host chooses m and j by a cost model).  The part
-// of a CTA's range inside one row tile is a segment.  Warp w works on path w % K and shares the column tiles of the segment
+// Work split.  The launch's layers are n_rt row tiles x n_cs slices of 256 columns each; the host cuts these pairs, in that
+// order, into contiguous ranges, one per SM, worked through by one group of 16 warps or cut once more for two groups of 8
+// (struct Planner).  The part of a range inside one row tile is a segment.  Warp w of a group works on path w % K and shares the column tiles of the segment
 // with the other warps of that path.  A warp streams its tiles through a ring of its own in shared memory with asynchronous
 // 16-byte copies (one per lane and tile, each lane reads back only what it copied itself, so no barrier is involved),
 // kRing - 1 tiles ahead: with 16 warps per SM that keeps about 56 KB per SM in flight, which is what the HBM latency needs
 // (with the tiles prefetched into registers, two to four per warp, the kernel ran at the speed of its memory latency, 1.1
-// to 1.7 TB/s).  At the end of a segment every warp writes its accumulators to its own slot of shared memory and the CTA adds
+// to 1.7 TB/s).  At the end of a segment every warp writes its accumulators to its own slot of shared memory and the group adds
 // the slots path by path in a fixed order (deterministic), applying g_k to each path's sum.  A segment that is a whole row
 // tile stores y.  Otherwise every output goes, as in the table-driven kernel, into the row's 64-bit accumulate word with one
 // integer atomic (fixed-point grid of the packer, arrival count in bits 55..62, bit 63 = non-finite); the thread whose add
@@ -38,10 +39,10 @@
 // word.  A contribution that covers s slices is shifted by s * 2^fix_bits, so the total shift is the same n_cs * 2^fix_bits
 // for every split.  Nothing waits for another CTA.
 //
-// What bounds it (B200, clocks per 512-byte tile and SM): 75 at up to eight batch rows and 105 at sixteen in the steady state,
-// of which the loads of x and h are 10 %; the rest is 16 or 32 MMAs of about 2 clocks and 128 half-rate integer operations,
-// which hardly overlap.  Segment ends are what a split can save: an arrival count found by searching a table of range
-// bounds in constant memory, cold in every launch, cost 1 us at each, publishing 16 rows from every SM 2 to 3 us.
+// What bounds it (B200, clocks per 512-byte tile and SM): about 70 in the steady state, of which the loads of x and h are 10 %;
+// the rest is 16 MMAs of about 2 clocks and the expansion, which hardly overlap.  Segment ends are what a split can save: an
+// arrival count found by searching a table of range bounds in constant memory, cold in every launch, cost 1 us at each (it
+// now comes with the range).  4096 x 14336 at 5 rows 13.1 -> 11.3 us, 4096 x 4096 at 8 7.1 -> 5.9, 28672 x 8192 at 8 37.9 -> 37.6.
 #include <cuda_fp16.h>
 
 #include <algorithm>

@@ -1,5 +1,5 @@
 // Decode GEMV on the integer tensor-core path (1, 2 or 4 batch rows per launch; the dispatcher uses it for batches
-// 3..16, the table-driven kernel of rabit_gemv_lut.cu takes batches 1..2).
+// 3..8 and the GEMM beyond, the table-driven kernel of rabit_gemv_lut.cu takes batches 1..2).
 //
 //   y[b][i] = sum_k g_k[i] * sum_j B_k[i][j] * t_k[b][j],   t_k[b][j] = h_k[j] * x[b][j]     (Section 4.1, Eq. 2)
 //

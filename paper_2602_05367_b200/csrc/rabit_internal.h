@@ -72,7 +72,7 @@ unsigned int* rabit_static_scratch_status(int device);   // rabit_noalloc.cu; nu
 // when tracing is off, the buffer is full or the library was built without RABIT_TRACE.
 unsigned long long* rabit_trace_slot(int ctas);
 
-// f16 tensor-core GEMV for 3..16 batch rows (rabit_gemv_f16.cu)
+// f16 tensor-core GEMV for up to 8 batch rows (rabit_gemv_f16.cu)
 cudaError_t rabit_launch_gemv_f16(const rabit_layer& L, const void* x, void* y, int batch, cudaStream_t stream);
 bool rabit_gemv_f16_supports(const rabit_layer& L, int batch);
 bool rabit_gemv_f16_group_supports(const rabit_layer* const* layers, int n_layers, int batch);

@@ -6,7 +6,7 @@
 //   header | sign tiles | g fp16 [K][Mp] | h fp16 [K][N] | fp32 partial scratch | flags + status |
 //   look-up blocks | u64 accumulate words
 //
-// (1) Sign tiles (tensor-core kernels: the f16 and integer-MMA GEMVs of batches 3..16 and the tcgen05 GEMM).
+// (1) Sign tiles (tensor-core kernels: the f16 and integer-MMA GEMVs and the tcgen05 GEMM).
 // The sign bits of each path are cut into tiles of 128 output rows x 32 input columns.
 // One tile is 512 bytes = 32 lanes x 16 bytes, so a warp reads a tile with one 128-bit
 // access per lane.  The eight bits of every byte belong to eight different 16-row blocks of
