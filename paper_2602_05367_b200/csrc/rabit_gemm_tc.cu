@@ -37,7 +37,7 @@
 //
 // What bounds it (B200): a unit takes the larger of its four MMAs (32 clocks per 16 batch columns, and 52) and the expansion, 130 clocks
 // of issue, 180 to 200 measured; a launch has about 4 us beside its units.  14336 x 4096 at batch 48 51 -> 16.4 us, 28672 x 8192 at 16
-// 55 -> 43.5, 5000 x 13824 with three paths at 200 209 -> 74.
+// 55 -> 43.5, 5000 x 13824 with three paths at 200 209 -> 68.
 //
 // Every wait is bounded; on a time-out the CTA sets the status word, skips the remaining waits, frees its tensor memory
 // and returns.  DEQ (rabit_set_variant 4): the expander forms the dequantised weight sum_k +-g_k h_k in fp16 and one
@@ -101,6 +101,7 @@ struct GemmParams {
     int w_stages;                           // weight ring, behind the x ring: per stage the sign tiles [K][8][512], then h [K][256]
     int box16;                              // groups of 16 batch columns per TMA box
     int n_acc;                              // accumulators (and issuing warps)
+    int paths;                              // path-major tasks: how many
     int units, a_col;                       // expanded-unit ring in tensor memory: unit u % units at columns a_col + 32 * that
     GemmLayer L[NL];
 };
@@ -211,6 +212,11 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+                   "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
+}
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all() {
@@ -243,11 +249,13 @@ struct Walk {
 struct Pass {
     int l, rt, c16, n;                      // layer, row tile, first group, groups
     int s_lo, s_hi;                         // steps
+    int path;                               // path-major tasks: of this pass
 };
-template <int NL>
+template <int NL, bool SEQ>
 struct PassWalker {
     int l, rt, c16, left;                   // where the next pass starts, groups left in the task (stream: slice and slices)
     int s_lo, s_hi;
+    int path = 0;
     // rank: which part of the steps (split contraction)
     __device__ PassWalker(const GemmParams<NL>& P, int task, int rank) {
         l = 0;
@@ -277,7 +285,7 @@ struct PassWalker {
         if (left <= 0) return false;
         if (NL > 1 || P.stream) {
             const int n_cs = P.L[l].n_cs, run = min(left, n_cs - c16);
-            ps = Pass{l, rt, 0, 1, c16 * kSliceSteps, min((c16 + run) * kSliceSteps, NL > 1 ? (P.L[l].n_ct + 1) / 2 : s_hi)};
+            ps = Pass{l, rt, 0, 1, c16 * kSliceSteps, min((c16 + run) * kSliceSteps, NL > 1 ? (P.L[l].n_ct + 1) / 2 : s_hi), 0};
             left -= run;
             c16 = 0;
             ++rt;
@@ -285,7 +293,11 @@ struct PassWalker {
             return true;
         }
         const int run = min(left, P.n16 - c16), pieces = run <= P.max16 ? 1 : (run + P.max16 - 1) / P.max16;
-        ps = Pass{0, rt, c16, pieces == 1 ? run : (run + pieces - 1) / pieces, s_lo, s_hi};
+        ps = Pass{0, rt, c16, pieces == 1 ? run : (run + pieces - 1) / pieces, s_lo, s_hi, path};
+        if (SEQ) {                                                       // (such a task is one chunk: all its passes are the same but for the path)
+            if (++path < P.paths) return true;
+            path = 0;
+        }
         left -= ps.n;
         c16 += ps.n;
         if (c16 == P.n16) { c16 = 0; ++rt; }
@@ -294,8 +306,11 @@ struct PassWalker {
 };
 
 // K paths; DEQ: see above.  NL > 1: up to NL layers of at most 16 batch columns in one launch (stream tasks; each layer has
-// its own x, of which the layers may share one).
-template <int K, bool DEQ, int NL>
+// its own x, of which the layers may share one).  SEQ (an instance with K = 1): path-major, for three paths.  Three accumulators
+// leave room for 8 groups of columns at most, so wider batches expanded every tile two or three times; here a task
+// is a pass per path on one accumulator, the sum of the scaled passes stays in tensor memory beside it, and up to 13 groups fit
+// (5000 x 13824 at batch 200: each tile expanded once instead of three times).
+template <int K, bool DEQ, int NL, bool SEQ>
 __global__ void __launch_bounds__(kThreads, 1)
 rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_constant__ XMaps<NL> x_maps) {
     extern __shared__ unsigned char smem_raw[];
@@ -316,7 +331,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
     unsigned char* ring = smem + kControlBytes;
     unsigned char* w_ring = ring + P.stages * P.stage_bytes;
     constexpr int n_ops = DEQ ? 1 : K;                            // operand units (and accumulators) per step
-    constexpr int n_groups = n_ops == 3 ? 3 : 4;                  // expander groups at work
+    constexpr int n_groups = n_ops == 3 || SEQ ? 3 : 4;                  // expander groups at work
     const int stages = P.stages, w_stages = P.w_stages, units = P.units, x_steps = P.x_steps, n_acc = P.n_acc;
     const int stage_bytes = P.stage_bytes;
     volatile int* abort_flag = &S.abort_flag;
@@ -340,19 +355,28 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
     }
     __syncthreads();
     if (split > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // (awaited before the exchange: every CTA of the cluster runs)
-    const PassWalker<NL> first_pass(P, task, (int)crank);
+    const PassWalker<NL, SEQ> first_pass(P, task, (int)crank);
     // Output scales of the row whose accumulators this thread reads: loaded when a pass begins, converted (which waits for
     // them) when it ends.
     unsigned short graw[K];
     auto load_scales = [&](const Pass& ps) {
 #pragma unroll
         for (int k = 0; k < K; ++k)
-            asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(graw[k]) : "l"(layer(ps).g + (size_t)k * layer(ps).Mp + ps.rt * kTileM + (warp & 3) * 32 + lane));
+            asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(graw[k]) : "l"(layer(ps).g + (size_t)(SEQ ? ps.path : k) * layer(ps).Mp + ps.rt * kTileM + (warp & 3) * 32 + lane));
     };
     auto scale = [&](int k) {
         unsigned short r;
         asm volatile("mov.b16 %0, %1;" : "=h"(r) : "h"(graw[k]));
         return __half2float(__ushort_as_half(r));
+    };
+
+    // SEQ: sum of the scaled passes before the last, 16 columns of group c
+    [[maybe_unused]] auto path_sum = [&](int c, float (&v)[16]) {
+        uint32_t d[16];
+        tmem_ld16(__shfl_sync(0xFFFFFFFFu, S.tmem_base, 0) + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((P.max16 + c) * kGroupCols), d);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(d[i]);
     };
 
     auto weight_stages = [](const Pass& ps) { return (ps.s_hi - ps.s_lo + kWSteps - 1) / kWSteps; };
@@ -364,14 +388,14 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
         mbar_expect_tx(bar, (uint32_t)(K * cts * (RABIT_TILE_BYTES + RABIT_TILE_COLS * 2)));
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            bulk_g2s(dst + k * kWTiles * RABIT_TILE_BYTES, L.bits + (((size_t)rt * K + k) * n_ct + ct0) * RABIT_TILE_BYTES, cts * RABIT_TILE_BYTES, bar);
-            bulk_g2s(dst + K * kWTiles * RABIT_TILE_BYTES + k * kWTiles * RABIT_TILE_COLS * 2, L.h + (size_t)k * L.N + (size_t)ct0 * RABIT_TILE_COLS,
+            bulk_g2s(dst + k * kWTiles * RABIT_TILE_BYTES, L.bits + ((SEQ ? (size_t)rt * P.paths + ps.path : (size_t)rt * K + k) * n_ct + ct0) * RABIT_TILE_BYTES, cts * RABIT_TILE_BYTES, bar);
+            bulk_g2s(dst + K * kWTiles * RABIT_TILE_BYTES + k * kWTiles * RABIT_TILE_COLS * 2, L.h + (size_t)(SEQ ? ps.path : k) * L.N + (size_t)ct0 * RABIT_TILE_COLS,
                      cts * RABIT_TILE_COLS * 2, bar);
         }
     };
     // the weight stages of all passes in order; `next` starts one if its slot is free or becomes free
     struct WeightFeed {
-        PassWalker<NL> w;
+        PassWalker<NL, SEQ> w;
         Pass ps;
         int j, issued;
         Walk at;
@@ -409,7 +433,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
         const bool elected = elect_one();
         int it = 0, w_at = 0;                                    // x and weight stages begun, over all passes
         Walk at{0};
-        PassWalker<NL> w = first_pass;
+        PassWalker<NL, SEQ> w = first_pass;
         Pass ps;
         while (w.next(P, ps)) {
             const int boxes = (ps.n + P.box16 - 1) / P.box16;
@@ -448,7 +472,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
             const uint32_t a0 = tmem_base + (uint32_t)P.a_col, d = tmem_base + (uint32_t)(m * P.max16 * kGroupCols);
             const uint32_t step_bytes = (uint32_t)stage_bytes / (uint32_t)x_steps;
             int steps_before = 0;                                // of earlier passes
-            PassWalker<NL> w = first_pass;
+            PassWalker<NL, SEQ> w = first_pass;
             Pass ps;
             while (w.next(P, ps)) {
                 const uint32_t idesc = __shfl_sync(0xFFFFFFFFu, umma_idesc(ps.n * kGroupCols), 0);
@@ -535,7 +559,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
         uint32_t dst = dst0, bar = bar0, done = 0;            // done: the group's units so far
         Walk ww{0};
         int pass_i = 0, u0 = 0;
-        PassWalker<NL> w = first_pass;
+        PassWalker<NL, SEQ> w = first_pass;
         Pass ps;
         while (w.next(P, ps)) {
             const GemmLayer& L = layer(ps);
@@ -551,12 +575,13 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                             g_rows[k][pi][rh] = __half2half2(L.g[(size_t)k * L.Mp + ps.rt * kTileM + 32 * q + 16 * pi + gq + 8 * rh]);
             }
             load_scales(ps);
-            const int first = ((grp - u0 % n_groups + n_groups) % n_groups) / n_ops;   // the group's first step of the pass, and of each of its weight stages
+            int first = ((grp - u0 % n_groups + n_groups) % n_groups) / n_ops;   // the group's first step of the pass, and (unless its stride does not divide them) of each weight stage
             for (int j = 0; j < weight_stages(ps) && grp < n_groups; ++j) {
                 const int step0 = ps.s_lo + j * kWSteps, n_here = min(kWSteps, ps.s_hi - step0), whole = min(n_here, n_ct / 2 - step0);   // steps with two column tiles
                 uint32_t bits = bits0 + ww.slot * (K * kWBytes) + first * (2 * RABIT_TILE_BYTES), hs = h0 + ww.slot * (K * kWBytes) + first * (kStepCols * 2);
                 mbar_wait(w_full0 + ww.slot * 8, ww.lap, abort_flag);
-                for (int sj = first; sj < n_here; sj += kStepsOn) {
+                int sj = first;
+                for (; sj < n_here; sj += kStepsOn) {
                     mbar_wait(bar, ((done >> lap_bit) & 1u) ^ 1u, abort_flag);             // (the first time round this is the barrier's previous phase: free)
                     fence_after();
                     auto expand_tile = [&](int ct2) {
@@ -608,12 +633,13 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                     bar = bar_sum - bar;
                     ++done;
                 }
+                if (kWSteps % kStepsOn != 0) first = sj - n_here;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(w_empty0 + ww.slot * 8);
                 ww.step(1, w_stages);
             }
             u0 += (ps.s_hi - ps.s_lo) * n_ops;
-            if (split > 1) break;                              // the cluster's epilogue follows the role branches
+            if (split > 1 && (!SEQ || ps.path == P.paths - 1)) break;   // the cluster's epilogue follows the role branches
             // ---- epilogue of this pass
             mbar_wait(smem_u32(&S.acc_ready), pass_i & 1, abort_flag);
             ++pass_i;
@@ -678,12 +704,35 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                 }
                 continue;
             }
+            if constexpr (SEQ) {
+                if (ps.path < P.paths - 1) {
+                    // a path that is not the last: its scaled result joins the sum beside the accumulator
+#pragma unroll 1
+                    for (int c = grp; c < ps.n; c += kExpandGroups) {
+                        const uint32_t acc = lane_base + (uint32_t)(c * kGroupCols), sum = acc + (uint32_t)(P.max16 * kGroupCols);
+                        uint32_t d[16], t[16];
+                        tmem_ld16(acc, d);
+                        if (ps.path > 0) tmem_ld16(sum, t);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                        const float g = scale(0);
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) t[i] = __float_as_uint(fmaf(g, __uint_as_float(d[i]), ps.path > 0 ? __uint_as_float(t[i]) : 0.f));
+                        tmem_st16(sum, t);
+                    }
+                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                    fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&S.acc_empty));
+                    continue;
+                }
+            }
             if constexpr (NL == 1) {
 #pragma unroll 1
                 for (int c = grp; c < ps.n; c += kExpandGroups) {
                     float v[16];
 #pragma unroll
                     for (int i = 0; i < 16; ++i) v[i] = 0.f;
+                    if constexpr (SEQ) path_sum(c, v);
 #pragma unroll
                     for (int m = 0; m < (n_ops == 1 ? 2 : n_ops); ++m) {
                         if (n_ops == 1 && m >= n_acc) break;
@@ -714,15 +763,16 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
         //      batch columns is finished by CTA c % split: all CTAs send it that group's columns (already scaled by g_k and
         //      summed over the paths) into its receive buffer recv[its c / split][source rank][column][row], behind the rings.
         //      After the cluster barrier each CTA adds what it received in rank order and stores fp16.
-        PassWalker<NL> w = first_pass;
+        PassWalker<NL, SEQ> w = first_pass;
         Pass ps;
         w.next(P, ps);
         if (warp >= 4) {
-            mbar_wait(smem_u32(&S.acc_ready), 0, abort_flag);
+            mbar_wait(smem_u32(&S.acc_ready), SEQ ? (P.paths - 1) & 1 : 0, abort_flag);
             fence_after();
         }
         __syncwarp();
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (SEQ) cluster_sync_all();                           // the receive buffer lies in the rings: every CTA's are done with
         float* recv = reinterpret_cast<float*>(smem + P.recv_off);
         if (warp >= 4) {
             const int grp = (warp - 4) >> 2, q = warp & 3, r_in = q * 32 + lane;
@@ -731,6 +781,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                 float v[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) v[i] = 0.f;
+                if constexpr (SEQ) path_sum(c, v);
 #pragma unroll
                 for (int m = 0; m < (n_ops == 1 ? 2 : n_ops); ++m) {
                     if (n_ops == 1 && m >= n_acc) break;
@@ -818,6 +869,7 @@ cudaError_t x_tensor_map(const void* x, int N, int batch, int box16, int x_steps
 struct Plan {
     int chunks, chunk16, split, max16, tasks;        // chunks == 0: contiguous group ranges
     int stream;                                      // contiguous ranges of (row tile, slice) pairs
+    int seq;                                         // path-major
     int stages, stage_bytes, x_steps, w_stages, box16, units, n_acc, recv_off;
     size_t smem;
     double clocks;                                   // estimate
@@ -828,14 +880,14 @@ struct Plan {
 bool fill_resources(Plan& p, int K, int n_ops, int steps, bool one_box) {
     const int recv_bytes = p.split > 1 ? (p.chunk16 + p.split - 1) / p.split * p.split * kGroupCols * kTileM * 4 : 0;
     if (p.max16 * kGroupCols > 256) return false;
-    const int turn = n_ops == 3 ? 3 : 4;
-    auto free_units = [&](int n_acc) { return (512 - n_acc * p.max16 * kGroupCols) / kUnitCols; };
+    const int turn = n_ops == 3 || p.seq ? 3 : 4;
+    auto free_units = [&](int n_acc) { return (512 - (n_acc + p.seq) * p.max16 * kGroupCols) / kUnitCols; };
     // (one path: a second accumulator needs a step for each in every pass; a stream's shortest one is the last slice)
-    p.n_acc = n_ops > 1 ? n_ops : (p.stream ? steps % kSliceSteps != 1 : steps >= 2) && free_units(2) >= turn ? 2 : 1;
+    p.n_acc = p.seq ? 1 : n_ops > 1 ? n_ops : (p.stream ? steps % kSliceSteps != 1 : steps >= 2) && free_units(2) >= turn ? 2 : 1;
     if (free_units(p.n_acc) < turn) return false;
     p.units = free_units(p.n_acc) >= 2 * turn ? 2 * turn : turn;
     const int step_bytes = (p.max16 + p.box16 - 1) / p.box16 * p.box16 * kGroupCols * kStepCols * 2;
-    const int room = (226 - 1) * 1024 - kControlBytes - recv_bytes;
+    const int room = (226 - 1) * 1024 - kControlBytes - (p.seq ? 0 : recv_bytes);
     // as many steps per x stage (one copy of the producer, which needs some 600 clocks for each) as leave three stages
     for (p.x_steps = one_box ? 4 : 1;; p.x_steps /= 2) {
         p.stage_bytes = step_bytes * p.x_steps;
@@ -847,32 +899,41 @@ bool fill_resources(Plan& p, int K, int n_ops, int steps, bool one_box) {
     // Never so little that two CTAs could share an SM: each takes all of its tensor memory, and of two clusters waiting
     // crosswise for each other's neither would ever get it.
     p.recv_off = kControlBytes + p.stages * p.stage_bytes + p.w_stages * K * kWBytes;
-    p.smem = std::max<size_t>(1024 + (size_t)p.recv_off + recv_bytes, 152 * 1024);
-    return true;
+    size_t used = (size_t)p.recv_off;
+    if (p.seq) {                                             // the receive buffer takes the rings' place
+        p.recv_off = kControlBytes;
+        used = std::max<size_t>(used, kControlBytes + recv_bytes);
+    } else {
+        used += recv_bytes;
+    }
+    p.smem = std::max<size_t>(1024 + used, 152 * 1024);
+    return p.smem <= 226 * 1024;
 }
 
 // Clocks of a (step, path) unit, fitted on B200: four MMAs of the pass's batch columns, or the expansion of its two sign tiles
 // (about 130 clocks of integer issue and 50 around them; more if a group has only one unit's room in tensor memory and has
-// to wait for its MMAs).
+// to wait for its MMAs).  Path-major: one warp issues everything and is the bound up to 16 groups (390 clocks at 7 groups, 510 at 13),
+// so that it pays only where the others expand a tile several times: 5000 x 13824 at batch 130 / 200 71 -> 56 / 75 -> 68 us.
 double unit_clocks(int n16, const Plan& p, int n_ops) {
-    const bool two_each = p.units >= 2 * (n_ops == 3 ? 3 : 4);
-    return std::max(32.0 * n16 + 52.0, two_each ? 180.0 + 8.0 * n16 : n_ops == 3 ? 345.0 : 300.0);
+    if (p.seq) return 250.0 + 20.0 * n16;
+    return std::max(32.0 * n16 + 52.0, p.units >= 2 * (n_ops == 3 ? 3 : 4) ? 180.0 + 8.0 * n16 : n_ops == 3 ? 345.0 : 300.0);
 }
 
 // (group: the form for several layers)
-const void* kernel_for(int K, bool deq, bool group = false) {
-    if (group) return K == 1 ? (const void*)rabit_gemm_tc_kernel<1, false, kMaxGroup> : K == 2 ? (const void*)rabit_gemm_tc_kernel<2, false, kMaxGroup> : (const void*)rabit_gemm_tc_kernel<3, false, kMaxGroup>;
-    if (K == 1) return deq ? (const void*)rabit_gemm_tc_kernel<1, true, 1> : (const void*)rabit_gemm_tc_kernel<1, false, 1>;
-    if (K == 2) return deq ? (const void*)rabit_gemm_tc_kernel<2, true, 1> : (const void*)rabit_gemm_tc_kernel<2, false, 1>;
-    return deq ? (const void*)rabit_gemm_tc_kernel<3, true, 1> : (const void*)rabit_gemm_tc_kernel<3, false, 1>;
+const void* kernel_for(int K, bool deq, bool group = false, bool seq = false) {
+    if (seq) return (const void*)rabit_gemm_tc_kernel<1, false, 1, true>;
+    if (group) return K == 1 ? (const void*)rabit_gemm_tc_kernel<1, false, kMaxGroup, false> : K == 2 ? (const void*)rabit_gemm_tc_kernel<2, false, kMaxGroup, false> : (const void*)rabit_gemm_tc_kernel<3, false, kMaxGroup, false>;
+    if (K == 1) return deq ? (const void*)rabit_gemm_tc_kernel<1, true, 1, false> : (const void*)rabit_gemm_tc_kernel<1, false, 1, false>;
+    if (K == 2) return deq ? (const void*)rabit_gemm_tc_kernel<2, true, 1, false> : (const void*)rabit_gemm_tc_kernel<2, false, 1, false>;
+    return deq ? (const void*)rabit_gemm_tc_kernel<3, true, 1, false> : (const void*)rabit_gemm_tc_kernel<3, false, 1, false>;
 }
 
 // Function attributes are per device.
-cudaError_t prepare_kernel(int K, bool deq, int device, bool group = false) {
-    static bool done[64][9] = {};
-    const int slot = device >= 0 && device < 64 ? device : 0, inst = 3 * (K - 1) + (group ? 2 : deq ? 1 : 0);
+cudaError_t prepare_kernel(int K, bool deq, int device, bool group = false, bool seq = false) {
+    static bool done[64][10] = {};
+    const int slot = device >= 0 && device < 64 ? device : 0, inst = seq ? 9 : 3 * (K - 1) + (group ? 2 : deq ? 1 : 0);
     if (done[slot][inst] && slot == device) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(kernel_for(K, deq, group), cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(kernel_for(K, deq, group, seq), cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
     if (e == cudaSuccess) done[slot][inst] = true;
     return e;
 }
@@ -961,18 +1022,20 @@ Plan make_plan(int n_rt, int n_steps, int K, bool deq, int batch, int sms, int d
         p.max16 = p.chunk16 = p.box16 = (n16 + chunks - 1) / chunks;
         p.chunks = (n16 + p.chunk16 - 1) / p.chunk16;
         if (p.chunks != chunks) continue;
-        for (int split = 1; split <= 8; ++split) {
-            p.split = split;
-            p.tasks = n_rt * chunks;
-            const long long ctas = (long long)p.tasks * split;
-            if (split > 1 && (n_steps / split < 4 || ctas > sms)) continue;
-            if (!fill_resources(p, K, n_ops, n_steps / split, wide_x)) continue;
-            if (split > 1 && (prepare_kernel(K, deq, device) != cudaSuccess || resident_clusters(kernel_for(K, deq), split, p.smem, sms) < p.tasks)) continue;
-            const double rounds = (double)((ctas + sms - 1) / sms);
-            p.clocks = kLaunchClocks + (split > 1 ? kExchangeClocks : 0.0) + rounds * ((n_steps + split - 1) / split) * n_ops * unit_clocks(p.chunk16, p, n_ops) +
-                       (rounds - 1.0) * kPassClocks;
-            if (p.clocks < best.clocks) best = p;
-        }
+        for (int seq = 0; seq <= (K == 3 && !deq ? 1 : 0); ++seq)
+            for (int split = 1; split <= 8; ++split) {
+                p.split = split;
+                p.seq = seq;
+                p.tasks = n_rt * chunks;
+                const long long ctas = (long long)p.tasks * split;
+                if (split > 1 && (n_steps / split < 4 || ctas > sms)) continue;
+                if (!fill_resources(p, seq ? 1 : K, seq ? 1 : n_ops, n_steps / split, wide_x)) continue;
+                if (split > 1 && (prepare_kernel(K, deq, device, false, seq != 0) != cudaSuccess || resident_clusters(kernel_for(K, deq, false, seq != 0), split, p.smem, sms) < p.tasks)) continue;
+                const double rounds = (double)((ctas + sms - 1) / sms);
+                p.clocks = kLaunchClocks + (split > 1 ? kExchangeClocks * (1 + seq) : 0.0) + rounds * ((n_steps + split - 1) / split) * n_ops * unit_clocks(p.chunk16, p, seq ? 1 : n_ops) +
+                           (rounds * (seq ? K : 1) - 1.0) * kPassClocks;
+                if (p.clocks < best.clocks) best = p;
+            }
         if (p.chunk16 <= 4) break;                   // narrower passes cost as much as these
     }
     // (b) contiguous ranges of groups, one per SM: no last wave
@@ -1063,7 +1126,7 @@ void fill_common(GemmParams<NL>& P, const Plan& p, int n_layers, int batch, long
     P.stages = p.stages; P.stage_bytes = p.stage_bytes; P.x_steps = p.x_steps; P.w_stages = p.w_stages;
     P.box16 = p.box16;
     P.n_acc = p.n_acc;
-    P.units = p.units; P.a_col = p.n_acc * p.max16 * kGroupCols;
+    P.units = p.units; P.a_col = (p.n_acc + p.seq) * p.max16 * kGroupCols;
 }
 
 }  // namespace
@@ -1091,6 +1154,7 @@ cudaError_t rabit_launch_gemm_tc_group(const rabit_layer* const* layers, int n_l
     const Plan p = plan_for(layers, n_layers, false, batch);
     if (p.tasks < 1) return cudaErrorInvalidValue;
     GemmParams<kMaxGroup> P;
+    P.paths = K;
     XMaps<kMaxGroup> maps;
     int pairs = 0;
     for (int l = 0; l < kMaxGroup; ++l) {
@@ -1132,10 +1196,11 @@ cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, i
     XMaps<1> maps;
     cudaError_t e = x_tensor_map(x, G.N, batch, p.box16, p.x_steps, &maps.map[0]);
     if (e != cudaSuccess) return e;
-    e = prepare_kernel(G.K, dequantised, L.device);
+    e = prepare_kernel(G.K, dequantised, L.device, false, p.seq != 0);
     if (e != cudaSuccess) return e;
 
     GemmParams<1> P;
+    P.paths = G.K;
     fill_layer(P.L[0], L, y, 0);
     fill_common(P, p, 1, batch, (long long)G.n_rt * (p.stream ? G.n_cs : (batch + kGroupCols - 1) / kGroupCols));
 
@@ -1154,5 +1219,5 @@ cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, i
     cfg.attrs = attr;
     cfg.numAttrs = p.split > 1 ? 2 : 1;
     void* args[2] = {&P, &maps};
-    return cudaLaunchKernelExC(&cfg, kernel_for(G.K, dequantised), args);
+    return cudaLaunchKernelExC(&cfg, kernel_for(G.K, dequantised, false, p.seq != 0), args);
 }

@@ -16,6 +16,8 @@ pytestmark = pytest.mark.gpu
     (1, 1000, 8224, 10),                     # and that step a single column tile
     # the contraction over clusters of 3, 5, 7 and 8 CTAs
     (3, 5000, 832, 24), (2, 3200, 2080, 33), (1, 2600, 2048, 40), (2, 160, 4096, 17),
+    # three paths one after the other on one accumulator, the contraction whole and over a cluster; one column more and it is not
+    (3, 13000, 2080, 208), (3, 2500, 8192, 200), (3, 13000, 2080, 209),
     # several 16-column groups per pass, ranges of groups, boxes of one and more steps
     (2, 3000, 160, 200), (2, 20000, 128, 300), (1, 300, 4096, 65),
 ])
