@@ -362,7 +362,7 @@ def bench_rabit(args) -> dict:
                "h2d_bytes_per_step": int(sum(2 * batch * shapes[grp[0]].N for grp in GROUPS) if grouped else sum(2 * batch * sh.N for sh in shapes)),
                "d2h_bytes_per_step": int(sum(2 * batch * sh.M for sh in shapes)),
                "steps": e2e_steps, "note": ("rabit_linear_group_host (prepared calls) per group of projections (a shared input is copied once)" if grouped else
-                        "rabit_linear_host per projection") + ": pinned host x -> device stage by copy, kernel, y stored by the kernel straight into pinned (mapped) host memory, host synchronises after every step"}
+                        "rabit_linear_host per projection") + ": pinned host x -> device stage by a kernel that reads it over the bus, kernel, y stored by the kernel straight into pinned (mapped) host memory, host synchronises after every step"}
 
     read_peak = measure_stream_read(device, stream) if (rank == 0 and not args.no_extras) else None
     peak = peaks["hbm_gbs"]
