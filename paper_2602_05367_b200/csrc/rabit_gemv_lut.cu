@@ -23,8 +23,8 @@
 //     prefetch in L2);
 //   * after the wait: x of the slice is read, the table is built (lane = byte group, warp = path x upper
 //     three index bits; 32 entries each by doubling), and the warps take the blocks round-robin, lane =
-//     row.  A lane holds its 16*K weight words in registers (128-bit streaming loads; the next block's come half by half into the
-//     registers the look-ups have freed, and none after a warp's last block: reloading it there, unused, cost a 7B decoder
+//     row.  A lane holds its 16*K weight words in registers (128-bit streaming loads; the next block's come into the
+//     registers behind the look-ups, and none after a warp's last block: reloading it there, unused, cost a 7B decoder
 //     layer 22.0 instead of 21.3 us; two blocks ahead 23.1, rings filled by bulk copies 22.8 to 24.5), walks the 32 byte groups of
 //     its row in an order rotated by its lane index (so the 32 look-ups of a warp step hit 32 banks), and
 //     ends with  p = sum_k g_k[row] * s_k;
@@ -392,8 +392,9 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
         for (int b = 0; b < NB; ++b)
 #pragma unroll
             for (int k = 0; k < K; ++k) acc[b][k][0] = acc[b][k][1] = 0.f;
-        // (the next block's weights are loaded into the registers that the look-ups have freed, half by half: half a block,
-        // some 1200 clocks, ahead of their use)
+        // (the next block's weights are loaded into the registers that the look-ups have used up, all together behind the last of
+        // them: the other warps' look-ups cover the wait.  Half by half, each as soon as its registers are free, is no faster with one batch
+        // row and slower with two: 28672 x 8192 23.9 against 22.9 us)
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const uint32_t bank = (bank0 + 0x10101010u * (uint32_t)j) & 0x7F7F7F7Fu;
@@ -418,8 +419,7 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
                     acc[b][k][1] += lds_f32<T::offset(k, b)>(a3);
                 });
             });
-            if (j == 3 && next_ok) load_half<K>(cur, 0, range_base, bb_next, lane);
-            if (j == 7 && next_ok) load_half<K>(cur, 1, range_base, bb_next, lane);
+            if (j == 7 && next_ok) { load_half<K>(cur, 0, range_base, bb_next, lane); load_half<K>(cur, 1, range_base, bb_next, lane); }
         }
 #ifdef RABIT_TRACE
         if (i == 0) RABIT_STAMP(7);                                     // first block's look-ups issued
