@@ -199,7 +199,8 @@ RABIT_API int rabit_linear_static_scratch(const rabit_layer* layer, const void* 
  * A grouped launch records a run-out wait in the status word of every layer of the group.
  * This call synchronises `stream`, reads the layer's word and the word of the built-in scratch array of
  * rabit_linear_static_scratch, and returns RABIT_OK or RABIT_DEVICE_FAULT.  With `clear` non-zero it also puts the
- * words and the layer's exchange buffer back into their resting state; do that before the layer is used again.
+ * words and the layer's reduction scratch (exchange buffer and accumulate words) back into their resting state; do that,
+ * for every layer of the call, before the layer is used again.
  */
 RABIT_API int rabit_layer_status(const rabit_layer* layer, int clear, void* stream);
 

@@ -454,9 +454,10 @@ extern "C" int rabit_layer_status(const rabit_layer* layer, int clear, void* str
     if (word != 0 || word_static != 0) {
         if (clear) {
             // a contributor that gave up may still have published a partial sum after its finisher restored the resting
-            // state: put the whole exchange buffer back, not just the word
+            // state, and one whose index check failed has left words incomplete: put all of the scratch back, not just the status word
             const size_t partial_bytes = (size_t)((const char*)layer->d_flags - (const char*)layer->d_partial);
             RABIT_CUDA_TRY(cudaMemsetAsync(layer->d_partial, 0xFF, partial_bytes, st));
+            RABIT_CUDA_TRY(cudaMemsetAsync(layer->d_acc, 0, (size_t)(layer->dev_base + layer->dev_bytes - (const char*)layer->d_acc), st));
             RABIT_CUDA_TRY(cudaMemsetAsync(layer->d_status, 0, 4, st));
             if (d_static) RABIT_CUDA_TRY(cudaMemsetAsync(d_static, 0, 4, st));
             RABIT_CUDA_TRY(cudaStreamSynchronize(st));
