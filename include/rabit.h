@@ -190,12 +190,15 @@ RABIT_API int rabit_linear_host(const rabit_layer* layer, const void* x_host, vo
 RABIT_API int rabit_linear_static_scratch(const rabit_layer* layer, const void* x, void* y, int batch, void* stream);
 
 /*
- * Health of a layer's kernels.  Every wait inside the kernels is bounded (about one second); a wait that
- * runs out makes the kernel set a status word, skip its remaining waits and return, so the context stays
- * usable but the outputs of that call are invalid.  (Only the tensor-core kernels wait for anything: the GEMV for
- * bulk copies and for the partial sums of CTAs with a lower index - it assumes that the CTAs of a grid no larger
- * than the device holds at once all become resident while it waits, which another tenant on the GPU can delay
- * beyond the limit - and the GEMM for its copy and tensor-memory barriers.  The table-driven GEMV never waits.)
+ * Health of a layer's kernels.  Every wait for a copy, an MMA or another CTA's partial sum is bounded (about one second); a wait
+ * that runs out makes the kernel skip its remaining waits, start no further copy, wait (again with that limit) for the copies
+ * and MMAs under way, set a status word and return, so the context stays usable but the outputs of that call are invalid.
+ * (Only two kernels wait for such things: the integer tensor-core GEMV for bulk copies and for the partial sums of CTAs with a
+ * lower index - it assumes that the CTAs of a grid no larger than the device holds at once all become resident while it
+ * waits, which another tenant on the GPU can delay beyond the limit - and the GEMM for its copy and tensor-memory
+ * barriers.  What has no bounded form: barriers among the threads of a CTA or of a cluster, which end because every
+ * thread reaches them after bounded waits, and the GEMM's allocation of tensor memory, which waits for whoever holds
+ * it on that SM.)
  * A grouped launch records a run-out wait in the status word of every layer of the group.
  * This call synchronises `stream`, reads the layer's word and the word of the built-in scratch array of
  * rabit_linear_static_scratch, and returns RABIT_OK or RABIT_DEVICE_FAULT.  With `clear` non-zero it also puts the
@@ -211,6 +214,15 @@ RABIT_API int rabit_layer_status(const rabit_layer* layer, int clear, void* stre
  * is a DEVICE word owned by the caller (4 bytes, 4-byte aligned); it holds 1 afterwards.
  */
 RABIT_API int rabit_selftest_bounded_wait(unsigned int* status_dev, int limit_us, void* stream);
+
+/*
+ * Test aid (no counterpart in the paper): makes a bounded wait of the layer's kernels run out.  From the next call on, the tcgen05
+ * GEMM's producer waits, before it starts the copy of activation stage `stage` (counted per CTA from 0), for a barrier that
+ * nothing ever signals; after the limit of about a second the kernel ends as described at rabit_layer_status.  CTAs with
+ * fewer stages are not affected.  A negative `stage` ends it.  Only a library built with -DRABIT_CHECKED does this; in the
+ * ordinary build the call returns RABIT_UNSUPPORTED_SHAPE.
+ */
+RABIT_API int rabit_selftest_withhold(rabit_layer* layer, int stage);
 
 /*
  * Test aid (no counterpart in the paper; host only, no GPU needed): how the f16 tensor-core GEMV of rabit_linear

@@ -25,6 +25,7 @@ static void bind_layer(rabit_layer* L, const RabitGeom& G, const RabitHeader& hd
     L->geom = G;
     L->device = device;
     L->variant = 0;
+    L->withhold = -1;
     L->sm_count = 0;
     cudaDeviceGetAttribute(&L->sm_count, cudaDevAttrMultiProcessorCount, device);
     L->dev_base = (char*)dev_buf;

@@ -39,8 +39,12 @@
 // of issue, 180 to 200 measured; a launch has about 4 us beside its units.  14336 x 4096 at batch 48 51 -> 16.4 us, 28672 x 8192 at 16
 // 55 -> 43.5, 5000 x 13824 with three paths at 200 209 -> 68.
 //
-// Every wait is bounded; on a time-out the CTA sets the status word, skips the remaining waits, frees its tensor memory
-// and returns.  DEQ (rabit_set_variant 4): the expander forms the dequantised weight sum_k +-g_k h_k in fp16 and one
+// Every wait on a barrier of shared memory is bounded.  On a time-out the CTA skips its remaining waits and the producer starts no
+// further copy; the other roles run on (an MMA on the wrong operand is harmless, and taking the accumulate words through their
+// full count leaves them at rest).  Copies and MMAs under way are awaited, again with a limit, before the tensor memory is freed,
+// the status word is set and the CTA returns.  (tcgen05.alloc and the cluster barriers have no bounded form.  The first ends because no two
+// CTAs that hold tensor memory share an SM, see fill_resources; the second because every thread reaches them after bounded
+// waits.)  DEQ (rabit_set_variant 4): the expander forms the dequantised weight sum_k +-g_k h_k in fp16 and one
 // contraction serves all paths (a K-th of the tensor work, one fp16 rounding per partial product and weight).
 #include <cuda.h>
 #include <cuda_fp16.h>
@@ -103,6 +107,9 @@ struct GemmParams {
     int n_acc;                              // accumulators (and issuing warps)
     int paths;                              // path-major tasks: how many
     int units, a_col;                       // expanded-unit ring in tensor memory: unit u % units at columns a_col + 32 * that
+#ifdef RABIT_CHECKED
+    int withhold;                           // x stage before which the producer waits for a barrier that nobody signals; -1: none
+#endif
     GemmLayer L[NL];
 };
 template <int NL>
@@ -119,8 +126,13 @@ struct Control {                            // ahead of the ring in shared memor
     unsigned long long a_empty[kMaxUnits];  // MMAs that read the unit retired
     unsigned long long acc_ready;           // all MMAs of the pass retired
     unsigned long long acc_empty;           // epilogue has read the accumulators
+    unsigned long long drained[3];          // after a time-out: everything this accumulator's warp issued has retired
+#ifdef RABIT_CHECKED
+    unsigned long long never;               // nothing arrives here (rabit_selftest_withhold)
+#endif
     uint32_t tmem_base;
     int abort_flag;
+    int x_begun, w_begun;                   // stages the producer started copies for
 };
 constexpr int kControlBytes = 1024;
 static_assert(sizeof(Control) <= kControlBytes, "control block");
@@ -141,11 +153,24 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
                  : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
+// Bounded wait: gives up after kWaitLimitCycles or once another thread of the CTA did.  Who gives up sets the flag before it goes
+// on, so whoever sees an arrival of such a thread sees the flag too: the producer looks at it between a wait and a copy.
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
     if (mbar_try_wait(bar, parity)) return;
     const long long t0 = clock64();
     while (!mbar_try_wait(bar, parity)) {
-        if (*abort_flag || clock64() - t0 > kWaitLimitCycles) { *abort_flag = 1; return; }
+        if (*abort_flag || clock64() - t0 > kWaitLimitCycles) {
+            *abort_flag = 1;
+            return;
+        }
+    }
+}
+// The copies of the first `begun` stages of a ring have landed (or the limit from t0 is over).
+__device__ __forceinline__ void drain_ring(const unsigned long long* bars, int stages, int begun, long long t0) {
+    for (int s = 0; s < stages && s < begun; ++s) {
+        const uint32_t last_lap = (uint32_t)((begun - 1 - s) / stages);
+        while (!mbar_try_wait((uint32_t)__cvta_generic_to_shared(&bars[s]), last_lap & 1u))
+            if (clock64() - t0 > kWaitLimitCycles) return;
     }
 }
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
@@ -350,6 +375,9 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
             mbar_init(smem_u32(&S.acc_ready), n_acc);
             mbar_init(smem_u32(&S.acc_empty), kExpandWarps);
             S.abort_flag = 0;
+#ifdef RABIT_CHECKED
+            mbar_init(smem_u32(&S.never), 1);
+#endif
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -397,14 +425,21 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
     struct WeightFeed {
         PassWalker<NL, SEQ> w;
         Pass ps;
-        int j, issued;
+        int j, issued, begun;                                    // begun: copies this lane started
         Walk at;
         bool more;
     };
-    WeightFeed feed{first_pass, Pass{}, 0, 0, Walk{0}, false};
+    WeightFeed feed{first_pass, Pass{}, 0, 0, 0, Walk{0}, false};
     auto feed_next = [&](bool elected) {
-        if (feed.issued >= w_stages) mbar_wait(smem_u32(&S.w_empty[feed.at.slot]), feed.at.lap ^ 1u, abort_flag);
-        if (elected) load_weights(feed.ps, feed.j, feed.at.slot);
+        bool go = elected;
+        if (feed.issued >= w_stages) {                           // (a slot's first copy needs no wait, and is safe whatever happened elsewhere)
+            mbar_wait(smem_u32(&S.w_empty[feed.at.slot]), feed.at.lap ^ 1u, abort_flag);
+            go = elected && !*abort_flag;
+        }
+        if (go) {
+            load_weights(feed.ps, feed.j, feed.at.slot);
+            ++feed.begun;
+        }
         __syncwarp();
         ++feed.issued;
         feed.at.step(1, w_stages);
@@ -431,7 +466,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
     if (warp == 0) {
         // ===================================== producer =====================================
         const bool elected = elect_one();
-        int it = 0, w_at = 0;                                    // x and weight stages begun, over all passes
+        int it = 0, w_at = 0, x_begun = 0;                       // x and weight stages over all passes; copies of x this lane started
         Walk at{0};
         PassWalker<NL, SEQ> w = first_pass;
         Pass ps;
@@ -444,8 +479,16 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                     while (feed.more && feed.issued < w_at + w_stages - 2) feed_next(elected);
                 }
                 const uint32_t bar = smem_u32(&S.full[at.slot]), dst = smem_u32(ring + at.slot * stage_bytes);
-                if (it >= stages) mbar_wait(smem_u32(&S.empty[at.slot]), at.lap ^ 1u, abort_flag);
-                if (elected) {
+#ifdef RABIT_CHECKED
+                if (it == P.withhold) mbar_wait(smem_u32(&S.never), 0u, abort_flag);
+#endif
+                bool go = elected;
+                if (it >= stages) {
+                    mbar_wait(smem_u32(&S.empty[at.slot]), at.lap ^ 1u, abort_flag);
+                    go = elected && !*abort_flag;
+                }
+                if (go) {
+                    ++x_begun;
                     mbar_expect_tx(bar, tx);
                     if (x_steps > 1) {
                         tma_load_3d(dst, &x_maps.map[NL == 1 ? 0 : ps.l], 0, ps.c16 * kGroupCols, s, bar);
@@ -457,6 +500,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                 at.step(1, stages);
             }
         }
+        if (elected) { S.x_begun = x_begun; S.w_begun = feed.begun; }
     } else if (warp < 4) {
         // ===================================== MMA issuers =====================================
         // Warp 1 + m issues the units u = m, m + n_acc, ... into accumulator m.  (The whole warp walks the loop, one elected lane
@@ -819,11 +863,32 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
     fence_before();
     __syncthreads();
     fence_after();
-    if (warp == 1) {
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
+    auto free_tensor_memory = [&] { asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory"); };
+    const bool gave_up = *abort_flag != 0;                     // (the same for every thread: nobody sets it any more)
+    if (warp == 1 && !gave_up) free_tensor_memory();
+    if (gave_up) [[unlikely]] {
+        // Copies and MMAs under way must not outlive the shared and tensor memory they work on.  (All of it in one branch of its
+        // own: with the ordinary path running through it a launch took 0.1 us longer.)
+        if (tid < 3) mbar_init(smem_u32(&S.drained[tid]), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        __syncthreads();
+        const long long t0 = clock64();
+        if (warp >= 1 && warp <= 3) {                            // (an arrival once all that this lane issued has retired)
+            const uint32_t bar = smem_u32(&S.drained[warp - 1]);
+            if (elect_one()) umma_commit(bar);
+            __syncwarp();
+            while (!mbar_try_wait(bar, 0u) && clock64() - t0 <= kWaitLimitCycles) { }
+        } else if (tid == 0) {
+            drain_ring(S.full, stages, S.x_begun, t0);
+            drain_ring(S.w_full, w_stages, S.w_begun, t0);
+        }
+        fence_before();
+        __syncthreads();
+        fence_after();
+        if (warp == 1) free_tensor_memory();
+        if (tid == 0)
+            for (int l = 0; l < (NL == 1 ? 1 : P.n_layers); ++l) atomicExch(P.L[l].status, 1u);
     }
-    if (tid == 0 && *abort_flag)
-        for (int l = 0; l < (NL == 1 ? 1 : P.n_layers); ++l) atomicExch(P.L[l].status, 1u);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -1111,7 +1176,7 @@ void fill_layer(GemmLayer& D, const rabit_layer& L, void* y, int pair0) {
     D.pair0 = pair0;
 }
 template <int NL>
-void fill_common(GemmParams<NL>& P, const Plan& p, int n_layers, int batch, long long n_groups) {
+void fill_common(GemmParams<NL>& P, const Plan& p, int n_layers, int batch, long long n_groups, [[maybe_unused]] int withhold) {
     P.n_layers = n_layers;
     P.batch = batch;
     P.n16 = (batch + kGroupCols - 1) / kGroupCols;
@@ -1127,6 +1192,9 @@ void fill_common(GemmParams<NL>& P, const Plan& p, int n_layers, int batch, long
     P.box16 = p.box16;
     P.n_acc = p.n_acc;
     P.units = p.units; P.a_col = (p.n_acc + p.seq) * p.max16 * kGroupCols;
+#ifdef RABIT_CHECKED
+    P.withhold = withhold;
+#endif
 }
 
 }  // namespace
@@ -1165,7 +1233,7 @@ cudaError_t rabit_launch_gemm_tc_group(const rabit_layer* const* layers, int n_l
         fill_layer(P.L[l], *layers[l], ys[l], pairs);
         pairs += G.n_rt * G.n_cs;
     }
-    fill_common(P, p, n_layers, batch, pairs);
+    fill_common(P, p, n_layers, batch, pairs, layers[0]->withhold);
     cudaError_t e = prepare_kernel(K, false, device, true);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -1202,7 +1270,7 @@ cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, i
     GemmParams<1> P;
     P.paths = G.K;
     fill_layer(P.L[0], L, y, 0);
-    fill_common(P, p, 1, batch, (long long)G.n_rt * (p.stream ? G.n_cs : (batch + kGroupCols - 1) / kGroupCols));
+    fill_common(P, p, 1, batch, (long long)G.n_rt * (p.stream ? G.n_cs : (batch + kGroupCols - 1) / kGroupCols), L.withhold);
 
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned int)(p.tasks * p.split));

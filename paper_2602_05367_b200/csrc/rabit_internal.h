@@ -14,6 +14,7 @@ struct rabit_layer {
     int device;
     int variant;                 // 0 auto, 1 plain, 2 integer-MMA GEMV, 3 tcgen05 GEMM, 4 dequantised-tile GEMM, 5 table-driven GEMV, 6 f16 tensor-core GEMV
     int sm_count;
+    int withhold;                // RABIT_CHECKED builds: see rabit_selftest_withhold; -1 none
     char* dev_base;              // caller-owned packed image
     size_t dev_bytes;
     const uint4* d_bits;         // sign tiles

@@ -82,3 +82,15 @@ extern "C" int rabit_selftest_bounded_wait(unsigned int* status_dev, int limit_u
     if (word != 1u) return rabit_fail(RABIT_DEVICE_FAULT, "rabit_selftest_bounded_wait: the kernel returned without recording the time-out");
     return RABIT_OK;
 }
+
+extern "C" int rabit_selftest_withhold(rabit_layer* layer, int stage) {
+    rabit_clear_error();
+    if (!layer) return rabit_fail(RABIT_INVALID_ARG, "rabit_selftest_withhold: layer is NULL");
+#ifdef RABIT_CHECKED
+    layer->withhold = stage < 0 ? -1 : stage;
+    return RABIT_OK;
+#else
+    (void)stage;
+    return rabit_fail(RABIT_UNSUPPORTED_SHAPE, "rabit_selftest_withhold: this library was built without RABIT_CHECKED");
+#endif
+}

@@ -24,7 +24,8 @@ def test_small_shapes_pass_under_the_checked_build():
         build.build(checked=True)
     env = dict(os.environ, RABIT_LIBRARY=lib)
     cmd = [sys.executable, "-m", "pytest", "-x", "-q", "-m", "gpu", os.path.join(ROOT, "tests", "test_gpu_parity.py"),
-           os.path.join(ROOT, "tests", "test_gpu_group.py"), "-k", "small_shapes or structured or outlier or repeated or group"]
+           os.path.join(ROOT, "tests", "test_gpu_group.py"), os.path.join(ROOT, "tests", "test_gpu_failure.py"),
+           "-k", "small_shapes or structured or outlier or repeated or group or withheld"]
     proc = subprocess.run(cmd, cwd=ROOT, env=env, capture_output=True, text=True, timeout=1200)
     assert proc.returncode == 0, proc.stdout[-3000:] + proc.stderr[-2000:]
     assert " passed" in proc.stdout
