@@ -218,8 +218,9 @@ RABIT_API int rabit_selftest_bounded_wait(unsigned int* status_dev, int limit_us
 /*
  * Test aid (no counterpart in the paper): makes a bounded wait of the layer's kernels run out.  From the next call on, the tcgen05
  * GEMM's producer waits, before it starts the copy of activation stage `stage` (counted per CTA from 0), for a barrier that
- * nothing ever signals; after the limit of about a second the kernel ends as described at rabit_layer_status.  CTAs with
- * fewer stages are not affected.  A negative `stage` ends it.  Only a library built with -DRABIT_CHECKED does this; in the
+ * nothing ever signals; after the limit of about a second the kernel ends as described at rabit_layer_status.  The integer
+ * tensor-core GEMV does the same at stage `stage` of 16 sign tiles (from 8 on: the first eight copies wait for nothing).  CTAs
+ * with fewer stages are not affected.  A negative `stage` ends it.  Only a library built with -DRABIT_CHECKED does this; in the
  * ordinary build the call returns RABIT_UNSUPPORTED_SHAPE.
  */
 RABIT_API int rabit_selftest_withhold(rabit_layer* layer, int stage);

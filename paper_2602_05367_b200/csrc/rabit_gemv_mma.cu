@@ -40,8 +40,9 @@
 //     bounded, so that case ends as a recorded time-out with invalid outputs, not as a hang), waiting
 //     (bounded) while it still sees the sentinel,
 //     puts the sentinel back, adds in a fixed order (deterministic) and stores fp16.
-// Every wait in the kernel is bounded; a wait that runs out sets a status word and the
-// kernel drains and returns (results are then invalid, the context stays usable).
+// Every wait in the kernel is bounded; after one that ran out no further copy is started, those under way
+// are awaited (with the same limit), and the kernel sets a status word and returns (results are then
+// invalid, the context stays usable).
 #include <cuda_fp16.h>
 
 #include "rabit_internal.h"
@@ -110,6 +111,9 @@ struct GroupParams {
     int n_layers;
     unsigned int* status[kMaxGroup];   // the status word of every layer of the group: a wait that runs out is recorded in all of them
     int nb;                  // batch rows actually present (<= the kernel's NB); the others are neither read nor written
+#ifdef RABIT_CHECKED
+    int withhold;            // stage before which the builders wait for a barrier that nobody signals (rabit_selftest_withhold); -1: none
+#endif
     GemvParams layer[kMaxGroup];
 };
 
@@ -123,6 +127,9 @@ struct __align__(128) Smem {
     unsigned long long empty[Cfg<NB>::kRing];
     unsigned int xmax_bits[NB];
     int abort_flag;
+#ifdef RABIT_CHECKED
+    unsigned long long never;
+#endif
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -144,16 +151,18 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
                  : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
-// Bounded wait: gives up after kWaitLimitCycles or as soon as any thread of the CTA gave up.
-__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-    if (mbar_try_wait(bar, parity)) return;
+// Bounded wait; false if it gave up, after kWaitLimitCycles or because another thread of the CTA did.  Who is told false does not
+// pass on what he waited for: no arrival that lets a stage be refilled, no copy into it.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    if (mbar_try_wait(bar, parity)) return true;
     const long long t0 = clock64();
     unsigned int ns = 32;
     while (!mbar_try_wait(bar, parity)) {
-        if (*abort_flag || clock64() - t0 > kWaitLimitCycles) { *abort_flag = 1; return; }
+        if (*abort_flag || clock64() - t0 > kWaitLimitCycles) { *abort_flag = 1; return false; }
         __nanosleep(ns);                                   // a waiting warp must not eat the issue slots of the working ones
         if (ns < 256) ns *= 2;
     }
+    return true;
 }
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
@@ -262,6 +271,9 @@ rabit_gemv_mma_kernel(const __grid_constant__ GroupParams GP) {
         }
         for (int b = 0; b < NB; ++b) S.xmax_bits[b] = 0;
         S.abort_flag = 0;
+#ifdef RABIT_CHECKED
+        mbar_init(smem_u32(&S.never), 1);
+#endif
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -269,6 +281,7 @@ rabit_gemv_mma_kernel(const __grid_constant__ GroupParams GP) {
     // The layer this CTA works on (the loop body runs once; it is written as passes with a running stage
     // counter `it0`, so ring slots and barrier phases would simply continue if a CTA ever took several layers).
     int it0 = 0;
+    int begun = 0;                                       // copies the issuing thread started
     bool first_pass = true;
     for (int li = 0; li < GP.n_layers; ++li) {
     const GemvParams& P = GP.layer[li];
@@ -298,6 +311,7 @@ rabit_gemv_mma_kernel(const __grid_constant__ GroupParams GP) {
             bulk_g2s(smem_u32(&S.bits[slot][0][0]), P.bits + ((size_t)lo + (size_t)i * kStageTiles) * RABIT_TILE_BYTES,
                      tiles * RABIT_TILE_BYTES, bar);
         }
+        begun = prefetched;
     }
     // Conversion lanes: lane index bi = 0..63 of a warp pair takes tile bi >> 2 of a stage and columns
     // 8*(bi & 3) .. +7 of it.  The first kHeadStages stages are converted by the MMA warps (pair warp >> 1
@@ -401,15 +415,20 @@ rabit_gemv_mma_kernel(const __grid_constant__ GroupParams GP) {
         }
 
         const bool issuer = tid == kMmaThreads;          // one lane issues the copies
+        bool live = true;                                // until a wait for a slot gives up
         for (int i0 = kHeadStages; i0 < n_stages; i0 += kBuildAhead) {
 #pragma unroll
             for (int d = 0; d < kBuildAhead; ++d) {
                 const int i = i0 + d;
                 if (i >= n_stages) break;
                 const int slot = (it0 + i) % kRing;
+#ifdef RABIT_CHECKED
+                if (i == GP.withhold && !mbar_wait(smem_u32(&S.never), 0u, abort_flag)) live = false;
+#endif
                 if (i >= kRing) {
-                    mbar_wait(smem_u32(&S.empty[slot]), (((it0 + i) / kRing) - 1) & 1, abort_flag);
-                    if (issuer) {
+                    if (!mbar_wait(smem_u32(&S.empty[slot]), (((it0 + i) / kRing) - 1) & 1, abort_flag)) live = false;
+                    if (issuer && live) {
+                        begun = i + 1;
                         const int tiles = min(kStageTiles, n_tiles - i * kStageTiles);
                         const uint32_t bar = smem_u32(&S.full[slot]);
                         mbar_expect_tx(bar, tiles * RABIT_TILE_BYTES);
@@ -421,7 +440,7 @@ rabit_gemv_mma_kernel(const __grid_constant__ GroupParams GP) {
                 prefetch_h(d);
                 prefetch_x(d);
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&S.full[slot]));
+                if (lane == 0 && live) mbar_arrive(smem_u32(&S.full[slot]));
             }
         }
     } else {
@@ -558,7 +577,7 @@ rabit_gemv_mma_kernel(const __grid_constant__ GroupParams GP) {
         const int slot = (it0 + i) % kRing;
         const int rel0 = i * kStageTiles + w, rel1 = rel0 + kMmaWarps;
         if (rel0 >= n_tiles) break;
-        mbar_wait(smem_u32(&S.full[slot]), ((it0 + i) / kRing) & 1, abort_flag);
+        const bool landed = mbar_wait(smem_u32(&S.full[slot]), ((it0 + i) / kRing) & 1, abort_flag);
         if (NB <= 2 && rel1 < seg_end) {
             const uint4 wa = S.bits[slot][w][lane];
             const uint4 wb = S.bits[slot][w + kMmaWarps][lane];
@@ -585,7 +604,7 @@ rabit_gemv_mma_kernel(const __grid_constant__ GroupParams GP) {
             }
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&S.empty[slot]));
+        if (lane == 0 && landed) mbar_arrive(smem_u32(&S.empty[slot]));
     }
     while (true) {
         segment_flush();
@@ -673,11 +692,10 @@ rabit_gemv_mma_kernel(const __grid_constant__ GroupParams GP) {
     __syncthreads();                                                           // abort_flag of every warp is final
     if (*abort_flag && tid == kMmaThreads) {
         // make sure no bulk copy is still in flight towards this CTA's shared memory
-        for (int it = max(0, it0 - kRing); it < it0; ++it) {
-            const long long t0 = clock64();
+        const long long t0 = clock64();
+        for (int it = max(0, begun - kRing); it < begun; ++it)
             while (!mbar_try_wait(smem_u32(&S.full[it % kRing]), (it / kRing) & 1))
                 if (clock64() - t0 > kWaitLimitCycles) break;
-        }
         for (int l = 0; l < GP.n_layers; ++l) atomicExch(GP.status[l], 1u);
     }
 }
@@ -732,6 +750,9 @@ cudaError_t rabit_launch_gemv_mma_group(const rabit_layer* const* layers, int n_
     GP.n_layers = n_layers;
     for (int l = 0; l < kMaxGroup; ++l) GP.status[l] = layers[l < n_layers ? l : 0]->d_status;
     GP.nb = batch;
+#ifdef RABIT_CHECKED
+    GP.withhold = layers[0]->withhold;
+#endif
     long long total = 0;
     for (int l = 0; l < n_layers; ++l) {
         const rabit_layer& L = *layers[l];

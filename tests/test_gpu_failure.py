@@ -45,9 +45,10 @@ def test_clearing_the_status_restores_the_whole_scratch(batch):
     ([(2, 20000, 1024)], 300, 3, (3,)),                     # several passes of 16-column groups a CTA
     ([(3, 1000, 2048)], 100, 4, (1,)),                      # dequantised tiles
     ([(2, 700, 8192), (2, 2500, 4352)], 16, 0, (0, 1)),     # several layers in one launch
+    ([(3, 6400, 6400)], 4, 2, (8, 11)),                     # integer tensor-core GEMV: 12.7 stages of 16 tiles a CTA
 ])
 def test_withheld_copy_ends_as_a_recorded_time_out(shapes, batch, variant, stages):
-    """The GEMM's producer waits for a barrier that nothing signals: every role gives up, the launch ends, the status of every
+    """The producer of the GEMM (or of the integer tensor-core GEMV) waits for a barrier that nothing signals: every role gives up, the launch ends, the status of every
     layer of the call says so, and after a clear the same layers compute the right result.  (Only the checked build has the
     switch, tests/test_gpu_checked_build.py runs this under it; the ordinary library refuses the call.)"""
     import time
