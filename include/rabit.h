@@ -235,6 +235,22 @@ RABIT_API int rabit_selftest_withhold(rabit_layer* layer, int stage);
 RABIT_API int rabit_selftest_f16_plan(int K, int M, int N, int batch, int sms, int* bound_out, int max_out);
 
 /*
+ * Test aid (no counterpart in the paper; host only, no GPU needed): how the tcgen05 GEMM would split one layer, or up to four of at
+ * most 16 rows in one launch, over `sms` SMs.
+ *   M, N        HOST, n_layers entries (1..4): the layers' shapes; K paths each; dequantised: as variant 4 (one layer)
+ *   candidate   -1: the split that would run; 0, 1, ...: each of the others that are weighed against it up to 16 rows
+ *   head_out    HOST, 8 ints: tasks, CTAs per task (a cluster that shares the contraction), 1 if tasks are ranges of (row tile,
+ *               slice of 256 columns) pairs that meet in the accumulate words, 1 if the paths run one after the other, most 16-column
+ *               groups of a pass, tasks per row tile (0: contiguous ranges), stages of the x ring, accumulators
+ *   passes_out  HOST, 10 ints per pass: task, CTA of the task, layer, row tile, first 16-column group, groups, first step and the
+ *               step after the last, path (if one after the other), and, for ranges of pairs, the number of contributions
+ *               at which an accumulate word of that row tile counts as complete
+ * Returns the number of passes, or RABIT_INVALID_ARG.
+ */
+RABIT_API int rabit_selftest_gemm_plan(int n_layers, const int* M, const int* N, int K, int dequantised, int batch, int sms, int candidate,
+                             int* head_out, int* passes_out, int max_passes);
+
+/*
  * Measurement aid (no counterpart in the paper): one kernel that reads `bytes` bytes of device memory once with
  * 128-bit streaming loads and keeps nothing.  Timed by the caller with CUDA events over a buffer much larger than L2
  * it gives the read-only HBM bandwidth this GPU delivers to plain loads, the natural ceiling of the decode GEMV.

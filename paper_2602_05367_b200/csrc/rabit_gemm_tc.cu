@@ -282,7 +282,7 @@ struct PassWalker {
     int s_lo, s_hi;
     int path = 0;
     // rank: which part of the steps (split contraction)
-    __device__ PassWalker(const GemmParams<NL>& P, int task, int rank) {
+    __host__ __device__ PassWalker(const GemmParams<NL>& P, int task, int rank) {
         l = 0;
         if (NL == 1) {
             const int n_steps = (P.L[0].N + kStepCols - 1) / kStepCols;   // N % 32 == 0: the last step may hold one column tile only
@@ -306,7 +306,7 @@ struct PassWalker {
             c16 = g - rt * per_rt;
         }
     }
-    __device__ bool next(const GemmParams<NL>& P, Pass& ps) {
+    __host__ __device__ bool next(const GemmParams<NL>& P, Pass& ps) {
         if (left <= 0) return false;
         if (NL > 1 || P.stream) {
             const int n_cs = P.L[l].n_cs, run = min(left, n_cs - c16);
@@ -329,6 +329,12 @@ struct PassWalker {
         return true;
     }
 };
+
+// Segments of a row tile of stream tasks: the tasks that touch its n_cs pairs, the first of which is pair `first` of n_pairs.  No task
+// is empty.  (pairs < kMaxPairs and tasks <= kMaxTasks: 32 bits hold the products)
+__host__ __device__ __forceinline__ int segment_arrivals(uint32_t first, uint32_t n_cs, uint32_t tasks, uint32_t n_pairs) {
+    return (int)(((first + n_cs) * tasks - 1u) / n_pairs) - (int)(((first + 1u) * tasks - 1u) / n_pairs) + 1;
+}
 
 // K paths; DEQ: see above.  NL > 1: up to NL layers of at most 16 batch columns in one launch (stream tasks; each layer has
 // its own x, of which the layers may share one).  SEQ (an instance with K = 1): path-major, for three paths.  Three accumulators
@@ -734,9 +740,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                     if ((bad >> i) & 1u) atomicOr(word + (size_t)i * L.Mp, 1ULL << 63);           // sticky: the add below never carries into bit 63
                     old[i] = atomicAdd(word + (size_t)i * L.Mp, add[i]);
                 }
-                // segments of this row tile: the tasks that touch it (pairs < kMaxPairs and tasks <= kMaxTasks: 32 bits hold the products)
-                const uint32_t first = (uint32_t)((NL == 1 ? 0 : L.pair0) + ps.rt * L.n_cs), past = first + (uint32_t)L.n_cs, tasks = (uint32_t)P.n_tasks;
-                const int arrivals = (int)((past * tasks - 1u) / (uint32_t)P.n_groups) - (int)(((first + 1u) * tasks - 1u) / (uint32_t)P.n_groups) + 1;
+                const int arrivals = segment_arrivals((uint32_t)((NL == 1 ? 0 : L.pair0) + ps.rt * L.n_cs), (uint32_t)L.n_cs, (uint32_t)P.n_tasks, (uint32_t)P.n_groups);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     if (i >= n_here || (int)((old[i] >> 55) & 0xFFu) != arrivals - 1) continue;   // other segments are still to come
@@ -1026,10 +1030,19 @@ constexpr double kLaunchClocks = 8000.0;             // launch, first loads, las
 constexpr double kExchangeClocks = 2500.0;           // exchange of a split task
 constexpr double kPublishClocks = 1500.0;            // atomics of a part of a row tile, besides their throughput
 
+// Task counts worth an estimate: equal parts of every row tile (or nearly), and one task per SM.  Never more tasks than pairs: an
+// empty one would count among the arrivals of a row tile that it does not contribute to.  (Layers of unlike widths: parts for the
+// widest are more than the narrow ones have pairs.)
+template <typename F>
+void stream_task_counts(long long row_tiles, long long pairs, int most_cs, int sms, F&& consider) {
+    for (long long m = 1; m <= most_cs && row_tiles * m <= std::min<long long>(sms, pairs); ++m) consider(row_tiles * m);
+    consider(std::min<long long>(sms, pairs));
+}
+
 // Up to 16 batch columns: contiguous ranges of the layers' (row tile, slice) pairs, met in the accumulate words.  tasks = 0 if
-// they cannot be.  (Against tasks over clusters or one per row tile: 4096 x 4096 8.6 -> 7.8 us, with one path 7.2 -> 6.5,
+// they cannot be.  (candidate >= 0: that one of the task counts instead of the cheapest, for rabit_selftest_gemm_plan.)  (Against tasks over clusters or one per row tile: 4096 x 4096 8.6 -> 7.8 us, with one path 7.2 -> 6.5,
 // 4096 x 14336 16.5 -> 15.8, 28672 x 8192 55 -> 44; nowhere slower, so such calls look no further.)
-Plan stream_plan(int n_layers, const int* n_rt, const int* n_ct, int K, bool deq, int batch, int sms) {
+Plan stream_plan(int n_layers, const int* n_rt, const int* n_ct, int K, bool deq, int batch, int sms, int candidate = -1) {
     Plan best = {};
     Plan p = {};
     p.stream = p.split = p.max16 = p.box16 = 1;
@@ -1048,7 +1061,9 @@ Plan stream_plan(int n_layers, const int* n_rt, const int* n_ct, int K, bool deq
     if (most_cs > RABIT_LUT_MAX_SLICES || pairs >= kMaxPairs || sms > kMaxTasks || !fill_resources(p, K, n_ops, tail, wide_x)) return best;
     best.clocks = 1e300;
     const double pair = kSliceSteps * n_ops * unit_clocks(1, p, n_ops);
-    auto consider = [&](long long tasks) {
+    int considered = 0;
+    stream_task_counts(row_tiles, pairs, most_cs, sms, [&](long long tasks) {
+        if (candidate >= 0 && considered++ != candidate) return;
         p.tasks = (int)tasks;
         double worst = 0.0;
         long long parts = 0, base = 0, t = 0;             // segments that are not whole row tiles
@@ -1065,12 +1080,11 @@ Plan stream_plan(int n_layers, const int* n_rt, const int* n_ct, int K, bool deq
         }
         p.clocks = kLaunchClocks + worst + (parts > 0 ? kPublishClocks + parts * 128.0 * batch / 80.0 : 0.0);
         if (p.clocks < best.clocks) best = p;
-    };
-    for (long long m = 1; m <= most_cs && row_tiles * m <= sms; ++m) consider(row_tiles * m);   // equal parts of a row tile (or nearly)
-    consider(std::min<long long>(sms, pairs));
+    });
     return best;
 }
 
+// (device < 0: planned without a GPU, as if it placed every cluster that its SMs have room for)
 Plan make_plan(int n_rt, int n_steps, int K, bool deq, int batch, int sms, int device, bool wide_x) {
     const int n16 = (batch + kGroupCols - 1) / kGroupCols;
     const int n_ops = deq ? 1 : K;
@@ -1095,7 +1109,7 @@ Plan make_plan(int n_rt, int n_steps, int K, bool deq, int batch, int sms, int d
                 const long long ctas = (long long)p.tasks * split;
                 if (split > 1 && (n_steps / split < 4 || ctas > sms)) continue;
                 if (!fill_resources(p, seq ? 1 : K, seq ? 1 : n_ops, n_steps / split, wide_x)) continue;
-                if (split > 1 && (prepare_kernel(K, deq, device, false, seq != 0) != cudaSuccess || resident_clusters(kernel_for(K, deq, false, seq != 0), split, p.smem, sms) < p.tasks)) continue;
+                if (split > 1 && device >= 0 && (prepare_kernel(K, deq, device, false, seq != 0) != cudaSuccess || resident_clusters(kernel_for(K, deq, false, seq != 0), split, p.smem, sms) < p.tasks)) continue;
                 const double rounds = (double)((ctas + sms - 1) / sms);
                 p.clocks = kLaunchClocks + (split > 1 ? kExchangeClocks * (1 + seq) : 0.0) + rounds * ((n_steps + split - 1) / split) * n_ops * unit_clocks(p.chunk16, p, seq ? 1 : n_ops) +
                            (rounds * (seq ? K : 1) - 1.0) * kPassClocks;
@@ -1197,7 +1211,65 @@ void fill_common(GemmParams<NL>& P, const Plan& p, int n_layers, int batch, long
 #endif
 }
 
+// The passes of every task of a plan, kPassInts integers each; their number.
+constexpr int kPassInts = 10;
+template <int NL, bool SEQ>
+int list_passes(GemmParams<NL>& P, const Plan& p, int n_layers, const int (*shape)[2], int K, int batch, int* out, int max_passes) {
+    long long pairs = 0;
+    for (int l = 0; l < NL; ++l) {
+        GemmLayer& D = P.L[l];
+        const int k = l < n_layers ? l : 0;
+        D.N = shape[k][1];
+        D.n_rt = (shape[k][0] + kTileM - 1) / kTileM;
+        D.n_ct = D.N / RABIT_TILE_COLS;
+        D.n_cs = (D.N + RABIT_LUT_COLS - 1) / RABIT_LUT_COLS;
+        D.pair0 = (int)pairs;
+        if (l < n_layers) pairs += (long long)D.n_rt * D.n_cs;
+    }
+    P.paths = K;
+    fill_common(P, p, n_layers, batch, p.stream ? pairs : (long long)P.L[0].n_rt * ((batch + kGroupCols - 1) / kGroupCols), -1);
+    int n = 0;
+    for (int task = 0; task < p.tasks; ++task)
+        for (int rank = 0; rank < p.split; ++rank) {
+            PassWalker<NL, SEQ> w(P, task, rank);
+            Pass ps;
+            while (w.next(P, ps)) {
+                if (n == max_passes) return -1;
+                const GemmLayer& L = P.L[ps.l];
+                const int arrivals = p.stream ? segment_arrivals((uint32_t)(L.pair0 + ps.rt * L.n_cs), (uint32_t)L.n_cs, (uint32_t)P.n_tasks, (uint32_t)P.n_groups) : 0;
+                const int v[kPassInts] = {task, rank, ps.l, ps.rt, ps.c16, ps.n, ps.s_lo, ps.s_hi, ps.path, arrivals};
+                std::copy(v, v + kPassInts, out + (size_t)kPassInts * n++);
+            }
+        }
+    return n;
+}
+
 }  // namespace
+
+// Host-only view of the work split (see rabit_selftest_gemm_plan).
+int rabit_gemm_tc_plan(int n_layers, const int (*shape)[2], int K, bool deq, int batch, int sms, int candidate, int head[8], int* out, int max_passes) {
+    if (n_layers < 1 || n_layers > kMaxGroup || K < 1 || K > RABIT_MAX_K || batch < 1 || batch > (1 << 24) || sms < 1 || sms > kMaxTasks) return -1;
+    if (n_layers > 1 && (batch > kGroupCols || deq)) return -1;
+    int n_rt[kMaxGroup], n_ct[kMaxGroup];
+    for (int l = 0; l < n_layers; ++l) {
+        if (shape[l][0] < 1 || shape[l][1] < RABIT_TILE_COLS || shape[l][1] % RABIT_TILE_COLS != 0) return -1;
+        n_rt[l] = (shape[l][0] + kTileM - 1) / kTileM;
+        n_ct[l] = shape[l][1] / RABIT_TILE_COLS;
+    }
+    const int cols = (batch + kGroupCols - 1) / kGroupCols * kGroupCols;
+    if (candidate >= 0 && cols > kGroupCols) return -1;
+    const Plan p = candidate >= 0 || n_layers > 1 ? stream_plan(n_layers, n_rt, n_ct, K, deq, cols, sms, candidate)
+                                                  : make_plan(n_rt[0], (n_ct[0] + 1) / 2, K, deq, cols, sms, -1, n_ct[0] % 2 == 0);
+    if (p.tasks < 1) return -1;
+    const int h[8] = {p.tasks, p.split, p.stream, p.seq, p.max16, p.chunks, p.stages, p.n_acc};
+    std::copy(h, h + 8, head);
+    if (n_layers > 1) {
+        GemmParams<kMaxGroup> P = {};
+        return list_passes<kMaxGroup, false>(P, p, n_layers, shape, K, batch, out, max_passes);
+    }
+    GemmParams<1> P = {};
+    return p.seq ? list_passes<1, true>(P, p, 1, shape, K, batch, out, max_passes) : list_passes<1, false>(P, p, 1, shape, K, batch, out, max_passes);
+}
 
 int rabit_gemm_tc_max_group() { return kMaxGroup; }
 

@@ -56,6 +56,17 @@ extern "C" int rabit_selftest_f16_plan(int K, int M, int N, int batch, int sms, 
     return grid;
 }
 
+extern "C" int rabit_selftest_gemm_plan(int n_layers, const int* M, const int* N, int K, int dequantised, int batch, int sms, int candidate,
+                                        int* head_out, int* passes_out, int max_passes) {
+    rabit_clear_error();
+    if (!M || !N || !head_out || !passes_out) return rabit_fail(RABIT_INVALID_ARG, "rabit_selftest_gemm_plan: null pointer");
+    int shape[4][2] = {};
+    for (int l = 0; l < n_layers && l < 4; ++l) { shape[l][0] = M[l]; shape[l][1] = N[l]; }
+    const int n = rabit_gemm_tc_plan(n_layers, shape, K, dequantised != 0, batch, sms, candidate, head_out, passes_out, max_passes);
+    if (n < 0) return rabit_fail(RABIT_INVALID_ARG, "rabit_selftest_gemm_plan: unsupported shape, no such candidate or too small an output array");
+    return n;
+}
+
 extern "C" int rabit_selftest_stream_read(const void* src_dev, size_t bytes, unsigned int* sink_dev, void* stream) {
     rabit_clear_error();
     if (!src_dev || ((uintptr_t)src_dev & 15u)) return rabit_fail(RABIT_INVALID_ARG, "rabit_selftest_stream_read: src_dev must be a 16-byte aligned device pointer");

@@ -43,6 +43,7 @@ def test_clearing_the_status_restores_the_whole_scratch(batch):
     ([(2, 3000, 8192)], 48, 3, (0, 3)),                     # the contraction over clusters
     ([(3, 2500, 8192)], 200, 3, (2, 20)),                   # path after path, over clusters
     ([(2, 20000, 1024)], 300, 3, (3,)),                     # several passes of 16-column groups a CTA
+    ([(2, 20153, 992)], 46, 3, (5,)),                       # contiguous ranges of 16-column groups
     ([(3, 1000, 2048)], 100, 4, (1,)),                      # dequantised tiles
     ([(2, 700, 8192), (2, 2500, 4352)], 16, 0, (0, 1)),     # several layers in one launch
     ([(3, 6400, 6400)], 4, 2, (8, 11)),                     # integer tensor-core GEMV: 12.7 stages of 16 tiles a CTA
