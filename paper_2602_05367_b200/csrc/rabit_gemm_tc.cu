@@ -258,6 +258,20 @@ __device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
 
+// Checked build (-DRABIT_CHECKED, python paper_2602_05367_b200/build.py --checked): every index that addresses global, shared or
+// tensor memory is compared with its range first; a violation sets the status word to 2 and the access is skipped (never a
+// trap; roles that wait for a skipped one end by their time-out).  In the ordinary build the checks compile to nothing.
+#ifdef RABIT_CHECKED
+#define RABIT_IN_RANGE(cond) ((cond) ? true : (atomicExch(P.L[0].status, 2u), false))
+__device__ __forceinline__ uint32_t smem_bytes() {
+    uint32_t v;
+    asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(v));
+    return v;
+}
+#else
+#define RABIT_IN_RANGE(cond) true
+#endif
+
 // One role's walk through a ring: every `stride`-th slot, with the parity of the slot's current lap.  A ring is a multiple of
 // every stride in use, so a slot is met by the same warps in every lap and a warp that waits for a slot's barrier is
 // never two laps from it (the parity would not tell the two apart).
@@ -394,6 +408,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
     // them) when it ends.
     unsigned short graw[K];
     auto load_scales = [&](const Pass& ps) {
+        if (!RABIT_IN_RANGE(ps.rt >= 0 && ps.rt < layer(ps).n_rt && ps.path >= 0 && ps.path < P.paths)) return;
 #pragma unroll
         for (int k = 0; k < K; ++k)
             asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(graw[k]) : "l"(layer(ps).g + (size_t)(SEQ ? ps.path : k) * layer(ps).Mp + ps.rt * kTileM + (warp & 3) * 32 + lane));
@@ -419,6 +434,8 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
         const GemmLayer& L = layer(ps);
         const int rt = ps.rt, n_ct = L.n_ct, ct0 = 2 * (ps.s_lo + kWSteps * j), cts = min(kWTiles, min(2 * ps.s_hi, n_ct) - ct0);
         const uint32_t bar = smem_u32(&S.w_full[slot]), dst = smem_u32(w_ring + slot * (K * kWBytes));
+        if (!RABIT_IN_RANGE(rt >= 0 && rt < L.n_rt && ps.path >= 0 && ps.path < P.paths && ct0 >= 0 && cts > 0 && ct0 + cts <= n_ct && L.N == n_ct * RABIT_TILE_COLS && slot < w_stages &&
+                            dst + K * kWBytes <= smem_u32(smem_raw) + smem_bytes())) return;
         mbar_expect_tx(bar, (uint32_t)(K * cts * (RABIT_TILE_BYTES + RABIT_TILE_COLS * 2)));
 #pragma unroll
         for (int k = 0; k < K; ++k) {
@@ -493,7 +510,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                     mbar_wait(smem_u32(&S.empty[at.slot]), at.lap ^ 1u, abort_flag);
                     go = elected && !*abort_flag;
                 }
-                if (go) {
+                if (go && RABIT_IN_RANGE(at.slot < stages && tx <= (uint32_t)stage_bytes && dst + tx <= smem_u32(w_ring) && ps.c16 >= 0 && ps.c16 + ps.n <= P.n16)) {
                     ++x_begun;
                     mbar_expect_tx(bar, tx);
                     if (x_steps > 1) {
@@ -528,6 +545,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                 const uint32_t idesc = __shfl_sync(0xFFFFFFFFu, umma_idesc(ps.n * kGroupCols), 0);
                 if (pass_i > 0) mbar_wait(smem_u32(&S.acc_empty), (pass_i - 1) & 1, abort_flag);   // epilogue has drained the accumulators
                 ++pass_i;
+                if (!RABIT_IN_RANGE(ps.n >= 1 && ps.n <= P.max16 && (m + 1) * P.max16 * kGroupCols <= P.a_col && P.a_col + units * kUnitCols <= 512)) break;
                 uint32_t accumulate = 0u;
                 const int s_lo = __shfl_sync(0xFFFFFFFFu, ps.s_lo, 0), s_hi = __shfl_sync(0xFFFFFFFFu, ps.s_hi, 0);
                 const int n_ct = NL == 1 ? P.L[0].n_ct : __shfl_sync(0xFFFFFFFFu, P.L[ps.l].n_ct, 0);
@@ -634,6 +652,8 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                 for (; sj < n_here; sj += kStepsOn) {
                     mbar_wait(bar, ((done >> lap_bit) & 1u) ^ 1u, abort_flag);             // (the first time round this is the barrier's previous phase: free)
                     fence_after();
+                    if (!RABIT_IN_RANGE((dst & 0xFFFFu) - (tmem_base & 0xFFFFu) >= (uint32_t)P.a_col && (dst & 0xFFFFu) - (tmem_base & 0xFFFFu) + kUnitCols <= 512u && sj < kWSteps && ww.slot < w_stages &&
+                                        bar >= smem_u32(&S.a_empty[0]) && bar <= smem_u32(&S.a_empty[units - 1]))) break;
                     auto expand_tile = [&](int ct2) {
                         uint32_t o[2][8];                                                  // [row block][16-column half, row half, column pair]
                         // dequantised: sum_k +-g_k[row] h_k[col], accumulated from the last (smallest) path to the first with one
@@ -736,7 +756,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     old[i] = 0ULL;
-                    if (i >= n_here) continue;
+                    if (i >= n_here || !RABIT_IN_RANGE(row >= 0 && row < L.Mp && 4 * grp + i < RABIT_LUT_MAX_BATCH)) continue;
                     if ((bad >> i) & 1u) atomicOr(word + (size_t)i * L.Mp, 1ULL << 63);           // sticky: the add below never carries into bit 63
                     old[i] = atomicAdd(word + (size_t)i * L.Mp, add[i]);
                 }
@@ -840,6 +860,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
 #pragma unroll
                     for (int i = 0; i < 16; ++i) v[i] = fmaf(gm, __uint_as_float(d[i]), v[i]);
                 }
+                if (!RABIT_IN_RANGE((const unsigned char*)(recv + ((size_t)((c / split) * split + split) * kGroupCols) * kTileM) <= smem_raw + smem_bytes())) continue;
                 const uint32_t dst = cluster_map(smem_u32(recv + ((size_t)((c / split) * split + crank) * kGroupCols) * kTileM + r_in), (uint32_t)(c % split));
 #pragma unroll
                 for (int i = 0; i < 16; ++i) st_cluster_f32(dst + (uint32_t)(i * kTileM * 4), v[i]);

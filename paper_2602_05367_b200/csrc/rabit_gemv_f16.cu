@@ -260,7 +260,7 @@ rabit_gemv_f16_kernel(const __grid_constant__ F16Params P) {
         __half gk[RABIT_MAX_K];                                           // output scales of the thread's row (the same row for all its outputs), loaded long before they are used
 #pragma unroll
         for (int kk = 0; kk < RABIT_MAX_K; ++kk)
-            gk[kk] = kk < P.K ? L.g[(size_t)kk * L.Mp + rt * RABIT_TILE_ROWS + (tid & 127)] : __half();
+            gk[kk] = kk < P.K && RABIT_IN_RANGE(rt >= 0 && rt < L.n_rt) ? L.g[(size_t)kk * L.Mp + rt * RABIT_TILE_ROWS + (tid & 127)] : __half();
         // weights kRing - 1 tiles ahead (HBM latency), scales and activations one tile ahead, k-step by k-step in place
         if (!waited) {
             asm volatile("griddepcontrol.wait;" ::: "memory");            // x, y and the accumulate words only after this

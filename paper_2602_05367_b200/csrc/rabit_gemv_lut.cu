@@ -264,7 +264,7 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
             const int pi = warp + u * kWarps;
             const int col = slice * RABIT_LUT_COLS + 8 * lane;
             hq[u] = make_uint4(0u, 0u, 0u, 0u);
-            if (pi < 8 * K && col < L.N) hq[u] = __ldg(reinterpret_cast<const uint4*>(L.h + (size_t)(pi >> 3) * L.N + col));
+            if (pi < 8 * K && col < L.N && RABIT_IN_RANGE(slice >= 0 && slice < L.n_cs && col + 8 <= L.N)) hq[u] = __ldg(reinterpret_cast<const uint4*>(L.h + (size_t)(pi >> 3) * L.N + col));
         }
     };
     auto load_x = [&](int slice) {                                      // L2 (not L1): written by the previous kernel in the stream
@@ -272,7 +272,7 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
             xq[b] = make_uint4(0u, 0u, 0u, 0u);
-            if (col < L.N) xq[b] = __ldcg(reinterpret_cast<const uint4*>(L.x + (size_t)b * L.N + col));
+            if (col < L.N && RABIT_IN_RANGE(slice >= 0 && slice < L.n_cs && col + 8 <= L.N)) xq[b] = __ldcg(reinterpret_cast<const uint4*>(L.x + (size_t)b * L.N + col));
         }
     };
     // table of the slice whose h and x sit in hq / xq:  entry e of (path k, group) = sum_{bit<8} (e has bit ? -t : +t),  t = h * x

@@ -1,6 +1,6 @@
-"""The small-shape parity suite under the checked build of the library (-DRABIT_CHECKED): every index that addresses
-memory in the decode kernels (table-driven and f16 GEMV) is compared with its range first, a violation sets the layer's status word and
-skips the access.  This stands in for a memory checker: the suite must pass with a clear status word.  The checked library
+"""The small-shape parity suite and the edges of the work splits under the checked build of the library (-DRABIT_CHECKED): every
+index that addresses memory in the table-driven and f16 GEMVs and in the GEMM is compared with its range first, a violation sets the
+layer's status word and skips the access.  This stands in for a memory checker: the suite must pass with a clear status word.  The checked library
 is a separate file (librabit_checked.so) selected through RABIT_LIBRARY, so it runs in a child process."""
 import importlib.util
 import os
@@ -25,7 +25,8 @@ def test_small_shapes_pass_under_the_checked_build():
     env = dict(os.environ, RABIT_LIBRARY=lib)
     cmd = [sys.executable, "-m", "pytest", "-x", "-q", "-m", "gpu", os.path.join(ROOT, "tests", "test_gpu_parity.py"),
            os.path.join(ROOT, "tests", "test_gpu_group.py"), os.path.join(ROOT, "tests", "test_gpu_failure.py"),
-           "-k", "small_shapes or structured or outlier or repeated or group or withheld"]
+           os.path.join(ROOT, "tests", "test_gpu_gemm.py"), os.path.join(ROOT, "tests", "test_gpu_edges.py"),
+           "-k", "small_shapes or structured or outlier or repeated or group or withheld or gemm_shapes or small_batches or splits or dequantised"]
     proc = subprocess.run(cmd, cwd=ROOT, env=env, capture_output=True, text=True, timeout=1200)
     assert proc.returncode == 0, proc.stdout[-3000:] + proc.stderr[-2000:]
     assert " passed" in proc.stdout

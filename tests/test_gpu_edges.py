@@ -91,3 +91,45 @@ def test_page_locked_inputs_up_to_and_beyond_what_a_kernel_fetches(N, batch, off
     torch.cuda.synchronize()
     assert np.array_equal(y_host.numpy().view(np.uint16), want.cpu().numpy().view(np.uint16))
     layer.free()
+
+
+@pytest.mark.parametrize("K,M,N", [(1, 1, 32), (3, 129, 96), (2, 300, 672)])
+def test_packing_and_host_calls_write_nothing_outside_their_buffers(K, M, N):
+    """The kernels that the checked build leaves out (packing, derivation, fetching of inputs): image, stage and outputs lie between
+    guard bands that have to come back untouched."""
+    import ctypes
+    import torch
+    import paper_2602_05367_b200 as rabit
+    from paper_2602_05367_b200 import binding
+    lib, vp, band = binding.raw_lib(), ctypes.c_void_p, 4096
+    L = make_layer(M, N, K, key=(115, K, M, N))
+    g16, h16 = L.g.view(np.uint16), L.h.view(np.uint16)
+    nbytes = rabit.packed_bytes(K, M, N)
+    stream = vp(torch.cuda.current_stream().cuda_stream)
+
+    def guarded(n, dtype, device):
+        raw = torch.full((band + n + band,), 0xA5, dtype=torch.uint8, device=device)
+        if device == "cpu":
+            raw = raw.pin_memory()
+        return raw, raw[band:band + n].view(dtype), lambda: bool((raw[:band] == 0xA5).all()) and bool((raw[band + n:] == 0xA5).all())
+
+    W = torch.randn((M, N), device="cuda")
+    for derive in (False, True):
+        raw, image, intact = guarded(nbytes, torch.uint8, "cuda")
+        assert image.data_ptr() % 256 == 0
+        out = vp()
+        if derive:
+            rc = lib.rabit_derive_pack(vp(W.data_ptr()), g16.ctypes.data, h16.ctypes.data, K, M, N, vp(image.data_ptr()), nbytes, stream, ctypes.byref(out))
+        else:
+            rc = lib.rabit_pack(L.planes.ctypes.data, g16.ctypes.data, h16.ctypes.data, K, M, N, vp(image.data_ptr()), nbytes, stream, ctypes.byref(out))
+        assert rc == 0, rabit.last_error()
+        for batch in (1, 5):
+            need = lib.rabit_stage_bytes(out, batch)
+            stage_raw, stage, stage_intact = guarded(need, torch.uint8, "cuda")
+            x = torch.from_numpy(make_x(batch, N, key=(115, batch))).pin_memory()
+            y_raw, y, y_intact = guarded(batch * M * 2, torch.float16, "cpu")
+            assert lib.rabit_linear_host(out, vp(x.data_ptr()), vp(y.data_ptr()), batch, vp(stage.data_ptr()), need, stream) == 0, rabit.last_error()
+            torch.cuda.synchronize()
+            assert stage_intact() and y_intact() and np.isfinite(y.numpy().astype(np.float64)).all()
+        assert intact()
+        assert lib.rabit_free(out) == 0
