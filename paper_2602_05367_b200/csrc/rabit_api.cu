@@ -165,19 +165,18 @@ extern "C" int rabit_linear(const rabit_layer* layer, const void* x, void* y, in
 
     int variant = layer->variant;
     if (variant == 0) {
-        const double packed_mb = (double)G.K * G.Mp * G.N / 8.0e6;
         if (rabit_gemv_lut_supports(*layer, batch)) {
             variant = 5;
         } else if (batch <= RABIT_MAX_GEMV_BATCH && rabit_gemv_f16_supports(*layer, kF16Rows)) {
-            variant = 6;                    // 3..16 rows: one pass over the weights with the batch in the MMA's N dimension (see kF16Rows)
-        } else if (batch <= 4 && packed_mb <= 8.0 && rabit_gemv_lut_supports(*layer, 1)) {
-            variant = 5;                    // two passes of the table-driven kernel
+            variant = 6;                    // the f16 GEMV, beyond kF16Rows the GEMM (also two rows of three paths, whose tables do not fit)
         } else if (batch <= RABIT_MAX_GEMV_BATCH) {
             variant = rabit_gemv_mma_supports(*layer, batch) ? 2 : 1;
-            // From 5 batch rows on the integer-MMA GEMV makes two to four passes over the weights; the tensor-core GEMM,
-            // whose cost does not depend on the batch up to 256, is then often cheaper.  Both estimates are fits to
-            // measurements on B200 (us): a GEMV pass of four rows costs 10 + max(0, packed MB - 4) / 1.3.
+            // Layers of more than 255 slices, or beyond the f16 GEMV's 32-bit offsets.  From 5 batch rows on the integer-MMA GEMV
+            // makes two to four passes over the weights; the tensor-core GEMM, which costs the same from 1 to 16 rows, is then
+            // often cheaper.  Both estimates are fits to measurements on B200 (us): a GEMV pass of four rows costs
+            // 10 + max(0, packed MB - 4) / 1.3.
             if (variant == 2 && batch > 4 && rabit_gemm_tc_supports(*layer, batch)) {
+                const double packed_mb = (double)G.K * G.Mp * G.N / 8.0e6;
                 const double passes = (double)((batch + rabit_gemv_mma_max_rows() - 1) / rabit_gemv_mma_max_rows());
                 const double gemv_us = passes * (10.0 + (packed_mb > 4.0 ? (packed_mb - 4.0) / 1.3 : 0.0));
                 const double gemm_us = rabit_gemm_tc_estimate_us(*layer, batch);
