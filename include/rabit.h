@@ -78,14 +78,14 @@ RABIT_API int rabit_unpack_host(const void* image, size_t image_bytes,
                       uint32_t* planes_out, uint16_t* g_out, uint16_t* h_out);
 
 /*
- * Pack (as rabit_pack_host) and copy the image into caller-owned device memory, then create
- * the descriptor.
+ * Pack into caller-owned device memory (the same bytes as rabit_pack_host), then create the descriptor.  Only the canonical
+ * planes and the scales cross to the device; both arrangements of the signs are made there.
  *   dev_buf   DEVICE  256-byte aligned, dev_bytes >= rabit_packed_bytes(K,M,N); must stay
  *                     valid and unmodified by the caller until rabit_free.
- *   stream    the copy is enqueued on it and the call returns after it has completed.
+ *   stream    the copies and kernels are enqueued on it and the call returns after they have completed.
  *   out       receives the new descriptor.
  * dev_buf also holds the layer's reduction scratch, in its resting state: the fp32 exchange buffer of the tensor-core
- * GEMV is all-ones words (0xFFFFFFFF, "nothing published"), the 64-bit accumulate words of the table-driven and f16 GEMVs, the
+ * GEMV is all-ones words (0xFFFFFFFF, "nothing published"), the 64-bit accumulate words of the other GEMVs and the GEMM, the
  * reserved flags and the status word are zero.  Every call leaves it in that state, so calls on one layer must not
  * overlap in time (different layers may).  A caller that moves or restores an image must keep these values.
  */
@@ -227,8 +227,8 @@ RABIT_API int rabit_selftest_withhold(rabit_layer* layer, int stage);
 
 /*
  * Test aid (no counterpart in the paper; host only, no GPU needed): how the f16 tensor-core GEMV of rabit_linear
- * (batch 3..8; larger ones, up to 16, are planned but never run) would split a K-path layer of M x N at `batch` rows over `sms` SMs.  The layer is ceil(M/128) row tiles x
- * ceil(N/256) slices; in that order the (row tile, slice) pairs are cut into contiguous parts, two per SM (one per group
+ * (batch 3..8; larger ones, up to 16, are planned but never run) would split a K-path layer of M x N at `batch` rows over
+ * `sms` SMs.  The layer is ceil(M/128) row tiles x ceil(N/256) slices; in that order the (row tile, slice) pairs are cut into contiguous parts, two per SM (one per group
  * of eight warps; with one group of 16 the second is empty).  bound_out (HOST, max_out ints) receives the starts of the parts followed by the number of pairs:
  * 2 * grid + 1 ascending values; a part may be empty.  Returns the number of CTAs (grid >= 1), or RABIT_INVALID_ARG.
  */

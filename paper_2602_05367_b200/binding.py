@@ -213,7 +213,7 @@ class RabitLayer:
 
 
 def rabit_pack(planes, g, h, device="cuda:0", stream: Optional[int] = None) -> RabitLayer:
-    """Pack on the host, upload into a torch-allocated device buffer, return the layer."""
+    """Upload the planes and pack them on the device into a torch-allocated buffer; return the layer."""
     planes, g16, h16, K, M, N = _host_arrays(planes, g, h)
     nbytes = packed_bytes(K, M, N)
     if nbytes == 0:

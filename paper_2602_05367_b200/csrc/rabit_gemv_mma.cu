@@ -1,5 +1,6 @@
-// Decode GEMV on the integer tensor-core path (1, 2 or 4 batch rows per launch; the dispatcher uses it for batches
-// 3..8 and the GEMM beyond, the table-driven kernel of rabit_gemv_lut.cu takes batches 1..2).
+// Decode GEMV on the integer tensor-core path (1, 2 or 4 batch rows per launch).  The dispatcher uses it up to 16 rows for layers
+// that neither the table-driven nor the f16 GEMV takes (more than 255 slices of 256 columns); rabit_linear_static_scratch
+// always runs it.
 //
 //   y[b][i] = sum_k g_k[i] * sum_j B_k[i][j] * t_k[b][j],   t_k[b][j] = h_k[j] * x[b][j]     (Section 4.1, Eq. 2)
 //

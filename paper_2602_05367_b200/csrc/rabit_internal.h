@@ -24,7 +24,7 @@ struct rabit_layer {
     unsigned int* d_flags;       // u32 [n_rt*K + RABIT_MAX_GRID] reserved (stay zero; no kernel uses them), then one status word
     unsigned int* d_status;      // u32, non-zero once a kernel gave up on a bounded wait
     const unsigned char* d_lut;  // look-up blocks (table-driven GEMV)
-    unsigned long long* d_acc;   // u64 [RABIT_LUT_MAX_BATCH][Mp] accumulate words of the table-driven GEMV (zero between calls)
+    unsigned long long* d_acc;   // u64 [RABIT_LUT_MAX_BATCH][Mp] accumulate words of the decode GEMVs and the GEMM (zero between calls)
 };
 
 // error reporting (thread-local message); returns `code`

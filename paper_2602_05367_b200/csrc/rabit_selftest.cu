@@ -1,4 +1,4 @@
-// Self-test of the bounded-wait mechanism used by every kernel of the library: a wait that cannot
+// Self-tests and host-only views.  The bounded wait is the mechanism of every kernel that waits: a wait that cannot
 // succeed must end by itself, record that it did, and leave the context usable.
 #include "rabit_internal.h"
 

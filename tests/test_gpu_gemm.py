@@ -15,10 +15,10 @@ GEMM = 3    # variant number of the tcgen05 GEMM
     (2, 128, 64, 17),        # one tile, one step
     (2, 256, 256, 40),
     (1, 200, 96, 64),        # ragged M, a last step with a single column tile
-    (2, 1000, 1184, 300),    # several row tiles, two batch tiles with a ragged tail, N % 64 == 32
+    (2, 1000, 1184, 300),    # several row tiles, four chunks of batch columns with a ragged tail, N % 64 == 32
     (2, 384, 2048, 512),
     (2, 2500, 512, 257),
-    (3, 300, 352, 130),      # three paths: 128-wide batch tiles, two of them with a ragged tail
+    (3, 300, 352, 130),      # three paths: three chunks of batch columns, the last with a ragged tail
     (3, 128, 64, 17),
 ])
 @pytest.mark.parametrize("variant", [0, GEMM])
@@ -54,7 +54,7 @@ def test_gemm_structured_inputs():
 
 
 def test_three_paths_large_batch():
-    """K = 3 runs with three 128-column accumulators; automatic dispatch and the explicit variant agree with the oracle."""
+    """K = 3 runs with three accumulators; automatic dispatch and the explicit variant agree with the oracle."""
     L = make_layer(160, 256, 3, key=(63,))
     x = make_x(48, 256, key=(63,))
     check_against_oracle(L, x, run_layer(L, x, 0))
@@ -68,22 +68,22 @@ def test_three_paths_large_batch():
     (2, 1000, 1184, 16),
 ])
 def test_gemm_runs_small_batches_too(K, M, N, batch):
-    """The tensor-core GEMM forced onto decode-sized batches (its batch tile is then mostly zero fill)."""
+    """The tensor-core GEMM forced onto decode-sized batches (a pass of 16 columns, most of them zero fill)."""
     L = make_layer(M, N, K, key=(62, K, M, N))
     x = make_x(batch, N, key=(62, M, N, batch))
     y = run_layer(L, x, GEMM)
     check_against_oracle(L, x, y)
 
 
-@pytest.mark.parametrize("batch", [2, 3, 4, 8, 12, 16, 17, 32, 33])
+@pytest.mark.parametrize("batch", [2, 3, 4, 8, 9, 12, 16, 17, 32, 33])
 def test_dispatch_by_batch(batch):
-    """One or two rows take the table-driven GEMV, 3 to 32 the f16 tensor-core GEMV (passes of 16 rows), more the GEMM.
-    Whichever kernel runs, the result is within tolerance and is exactly what that kernel gives when forced."""
+    """One or two rows take the table-driven GEMV, 3 to 8 the f16 tensor-core GEMV, more the GEMM.  Whichever kernel runs, the
+    result is within tolerance and is exactly what that kernel gives when forced."""
     L = make_layer(14336, 512, 2, key=(63,))
     x = make_x(batch, 512, key=(63, batch))
     y_auto = run_layer(L, x, 0)
     check_against_oracle(L, x, y_auto)
-    expect = 5 if batch <= 2 else 6 if batch <= 32 else GEMM
+    expect = 5 if batch <= 2 else 6 if batch <= 8 else GEMM
     y_forced = run_layer(L, x, expect)
     assert np.array_equal(y_auto.view(np.uint16), y_forced.view(np.uint16))
 
@@ -114,15 +114,15 @@ def test_dequantised_tile_gemm(K, M, N, batch):
 
 
 @pytest.mark.parametrize("K,M,N,batch,variant", [
-    (2, 256, 4096, 64, GEMM),      # 2 tiles, 64 steps: eight CTAs share a tile (32-column slices)
-    (2, 256, 4096, 300, GEMM),     # two batch tiles, ragged
+    (2, 256, 4096, 64, GEMM),      # 2 row tiles, 64 steps: eight CTAs share each
+    (2, 256, 4096, 300, GEMM),     # five chunks of batch columns, ragged
     (2, 200, 4160, 40, DEQ),       # ragged rows, 65 steps split unevenly
-    (3, 256, 2048, 100, GEMM),     # three paths: 128-wide tiles, four CTAs per tile
-    (1, 384, 1024, 17, GEMM),      # two CTAs per tile
-    (2, 1024, 8192, 512, GEMM),    # the 70B k/v projection at batch 512: 16 tiles, eight CTAs each
-    (2, 19200, 1024, 20, GEMM),    # 150 tiles on 148 SMs: one whole wave, then the two tiles left over as a split launch
+    (3, 256, 2048, 100, GEMM),     # three paths, two chunks, eight CTAs each
+    (1, 384, 1024, 17, GEMM),      # 16 steps: one CTA per row tile
+    (2, 1024, 8192, 512, GEMM),    # the 70B k/v projection at batch 512: 32 tasks of four CTAs
+    (2, 19200, 1024, 20, GEMM),    # 150 row tiles on 148 SMs: contiguous ranges of 16-column groups
     (2, 19100, 1024, 20, DEQ),
-    (2, 11008, 1024, 40, GEMM),    # 86 tiles: more than half the SMs, one CTA per tile
+    (2, 11008, 1024, 40, GEMM),    # 86 row tiles: more than half the SMs, one CTA each
 ])
 def test_gemm_split_contraction_across_a_cluster(K, M, N, batch, variant):
     """Layers with few output tiles: the CTAs of a cluster split the contraction of a tile and add their partial

@@ -42,7 +42,7 @@ def test_batches(batch, variant):
 @pytest.mark.parametrize("K,M,N", [(2, 192, 896), (3, 300, 640), (1, 129, 288), (2, 1000, 4352), (2, 4096, 4096)])
 @pytest.mark.parametrize("batch", [3, 7, 8, 9, 16])
 def test_f16_tensor_core_gemv_batches(K, M, N, batch):
-    """The batch 3..16 kernel (batch in the MMA's N dimension) forced, every batch width class, ragged shapes, K = 1..3."""
+    """Variant 6 forced: the f16 GEMV up to 8 rows (batch in the MMA's N dimension), the GEMM at 9 to 16; ragged shapes, K = 1..3."""
     L = make_layer(M, N, K, key=(69, K, M, N))
     x = make_x(batch, N, key=(69, M, N, batch))
     y = run_layer(L, x, 6)
@@ -54,7 +54,7 @@ def test_f16_tensor_core_gemv_batches(K, M, N, batch):
 @pytest.mark.parametrize("batch", [1, 2, 5, 16])
 def test_widest_layer_of_the_accumulate_word_kernels(batch):
     """N = 65280 is 255 slices of 256 columns, the most the eight-bit arrival count of an accumulate word can take: the
-    table-driven kernel (batch 1, 2) and the f16 GEMV (5, 16) at that limit, where a row's word collects up to 255
+    table-driven kernel (batch 1, 2), the f16 GEMV (5) and the GEMM (16) at that limit, where a row's word collects up to 255
     contributions on a grid of 46 magnitude bits."""
     L = make_layer(200, 65280, 2, key=(70,))
     x = make_x(batch, 65280, key=(70, batch))

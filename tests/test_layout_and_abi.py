@@ -188,9 +188,13 @@ def test_every_declared_symbol_is_exported():
     (2, 14336, 4096, 16, 148), (2, 14336, 4096, 8, 148), (2, 4096, 4096, 16, 148), (2, 4096, 14336, 3, 148),
     (2, 28672, 8192, 16, 148), (2, 1024, 4096, 8, 148), (3, 11008, 4096, 16, 148), (1, 129, 288, 5, 148),
     (2, 200, 65280, 16, 148), (2, 128, 32, 3, 148), (2, 100000, 4096, 12, 148), (2, 4096, 11008, 16, 132), (2, 300, 640, 7, 4),
+    # what the kernel runs: 3 to 8 rows
+    (2, 4096, 4096, 8, 148), (2, 28672, 8192, 8, 148), (3, 11008, 4096, 7, 148), (2, 200, 65280, 8, 148), (2, 100000, 4096, 5, 148),
+    (2, 4096, 11008, 4, 132), (1, 1, 32, 3, 148), (3, 12000, 512, 6, 160), (1, 5000, 3200, 5, 1),
 ])
 def test_work_split_of_the_f16_gemv(K, M, N, batch, sms):
-    """Host logic of the batch 3..16 kernel: the (row tile, slice) pairs are cut into two contiguous parts per SM.  Whatever
+    """Host logic of the batch 3..8 kernel (the view also plans up to 16 rows, which the GEMM runs): the (row tile, slice) pairs are
+    cut into two contiguous parts per SM.  Whatever
     the cost model prefers, the parts must tile the pairs exactly, in order, on no more CTAs than SMs; no row tile may be
     touched by more parts than the eight-bit arrival count of an accumulate word can hold; and the split must be the
     same every time (the plan is cached)."""
