@@ -16,8 +16,10 @@ Prints one JSON line on rank 0.
 from __future__ import annotations
 
 import argparse
+import hashlib
 import json
 import os
+import re
 import subprocess
 import sys
 import threading
@@ -164,16 +166,26 @@ def load_peaks():
     return {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0, "source": "fallback"}
 
 
-def recorded_traffic(key: str):
+def kernel_digest(source: str) -> str:
+    """Digest of a kernel's source file (in the package's csrc) without comments and white space: the same for as long as the
+    code is the same."""
+    with open(os.path.join(ROOT, "paper_2602_05367_b200", "csrc", source)) as f:
+        code = re.sub(r"//[^\n]*|/\*.*?\*/", "", f.read(), flags=re.S)
+    return hashlib.sha256("".join(code.split()).encode()).hexdigest()[:16]
+
+
+def recorded_traffic(key: str, path: str = os.path.join(ROOT, "profiles", "gemv_lut_traffic.json")):
     """DRAM bytes per step from the ncu capture recorded in profiles/gemv_lut_traffic.json, or None when no capture of
-    this workload is on record there (the file names the command and the kernel source it was taken with)."""
-    path = os.path.join(ROOT, "profiles", "gemv_lut_traffic.json")
+    this workload is on record there, or one of another version of the kernel (the file names the command and the
+    digest of the source that it was taken with)."""
     try:
-        rec = json.load(open(path))
+        with open(path) as f:
+            entry = json.load(f).get(key)
     except (OSError, ValueError):
         return None
-    entry = rec.get(key)
-    return None if entry is None else entry.get("dram_bytes_per_step")
+    if entry is None or entry.get("kernel_digest") != kernel_digest("rabit_gemv_lut.cu"):
+        return None
+    return entry.get("dram_bytes_per_step")
 
 
 def time_replays(stream, graphs, repeats: int, warm: int = 1):
@@ -743,7 +755,7 @@ def bench_derive(args) -> dict:
         cases.append({"M": sh.M, "N": sh.N, "us": us, "gbs": nbytes / us / 1e3,
                       "roofline": {"bound": "hbm", "achieved": nbytes / us / 1e3, "peak": hbm_peak, "unit": "GB/s", "frac": nbytes / us / 1e3 / hbm_peak},
                       "note": "back-to-back asynchronous calls through the C ABI, CUDA events around all of them: includes the "
-                              "upload of the scales, the second kernel (look-up blocks, scratch fills, header) and the fill of the accumulate words"})
+                              "upload of the scales, the kernel (both arrangements of the signs, scratch fills, header) and the fill of the accumulate words"})
         del Ws
         torch.cuda.empty_cache()
     head = max(cases, key=lambda c: c["M"] * c["N"])
