@@ -132,7 +132,7 @@ struct Control {                            // ahead of the ring in shared memor
 #endif
     uint32_t tmem_base;
     int abort_flag;
-    int x_begun, w_begun;                   // stages the producer started copies for
+    int x_begun, w_begun;                   // stages the producer started copies for, once it has left its loop; -1 before
 };
 constexpr int kControlBytes = 1024;
 static_assert(sizeof(Control) <= kControlBytes, "control block");
@@ -153,16 +153,26 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
                  : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
-// Bounded wait: gives up after kWaitLimitCycles or once another thread of the CTA did.  Who gives up sets the flag before it goes
-// on, so whoever sees an arrival of such a thread sees the flag too: the producer looks at it between a wait and a copy.
-__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-    if (mbar_try_wait(bar, parity)) return;
+// Bounded wait; false if it gave up, after kWaitLimitCycles or once another thread of the CTA did.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    if (mbar_try_wait(bar, parity)) return true;
     const long long t0 = clock64();
     while (!mbar_try_wait(bar, parity)) {
         if (*abort_flag || clock64() - t0 > kWaitLimitCycles) {
             *abort_flag = 1;
-            return;
+            return false;
         }
+    }
+    return true;
+}
+// The same for a stage of a ring.  Who went on without it would free it while its copy may be under way, so he first lets the
+// producer leave its loop (with the same limit): that one has nothing but consumers to wait for and soon sees the flag, or is
+// done.  (This way a wait that succeeds costs what it did.  A look at the flag between the producer's wait and its copy, or a
+// condition of its own on the elected lane, cost wide passes of one path up to 14 %: 14336 x 4096 at batch 400 59 -> 67 us.)
+__device__ __forceinline__ void mbar_wait_stage(uint32_t bar, uint32_t parity, volatile int* abort_flag, const volatile int* producer_left) {
+    if (!mbar_wait(bar, parity, abort_flag)) {
+        const long long t0 = clock64();
+        while (*producer_left < 0 && clock64() - t0 <= kWaitLimitCycles) { }
     }
 }
 // The copies of the first `begun` stages of a ring have landed (or the limit from t0 is over).
@@ -395,6 +405,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
             mbar_init(smem_u32(&S.acc_ready), n_acc);
             mbar_init(smem_u32(&S.acc_empty), kExpandWarps);
             S.abort_flag = 0;
+            S.x_begun = -1;
 #ifdef RABIT_CHECKED
             mbar_init(smem_u32(&S.never), 1);
 #endif
@@ -448,30 +459,24 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
     struct WeightFeed {
         PassWalker<NL, SEQ> w;
         Pass ps;
-        int j, issued, begun;                                    // begun: copies this lane started
+        int j, issued;
         Walk at;
         bool more;
     };
-    WeightFeed feed{first_pass, Pass{}, 0, 0, 0, Walk{0}, false};
-    auto feed_next = [&](bool elected) {
-        bool go = elected;
-        if (feed.issued >= w_stages) {                           // (a slot's first copy needs no wait, and is safe whatever happened elsewhere)
-            mbar_wait(smem_u32(&S.w_empty[feed.at.slot]), feed.at.lap ^ 1u, abort_flag);
-            go = elected && !*abort_flag;
-        }
-        if (go) {
-            load_weights(feed.ps, feed.j, feed.at.slot);
-            ++feed.begun;
-        }
-        __syncwarp();
+    WeightFeed feed{first_pass, Pass{}, 0, 0, Walk{0}, false};
+    auto feed_next = [&](bool elected) {                         // false: gave up (lane by lane: nothing below may wait for the other lanes)
+        if (feed.issued >= w_stages && !mbar_wait(smem_u32(&S.w_empty[feed.at.slot]), feed.at.lap ^ 1u, abort_flag)) return false;
+        if (elected) load_weights(feed.ps, feed.j, feed.at.slot);
         ++feed.issued;
         feed.at.step(1, w_stages);
         if (++feed.j == weight_stages(feed.ps)) { feed.j = 0; feed.more = feed.w.next(P, feed.ps); }
+        return true;
     };
     if (warp == 0) {
         const bool elected = elect_one();
         feed.more = feed.w.next(P, feed.ps);
         while (feed.more && feed.issued < w_stages) feed_next(elected);
+        __syncwarp();
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // Tensor memory is taken only after the dependency wait: a CTA that held some while the kernel before it in the stream
@@ -489,29 +494,26 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
     if (warp == 0) {
         // ===================================== producer =====================================
         const bool elected = elect_one();
-        int it = 0, w_at = 0, x_begun = 0;                       // x and weight stages over all passes; copies of x this lane started
+        int it = 0, w_at = 0;                                    // x and weight stages begun, over all passes
+        bool go = true;
         Walk at{0};
         PassWalker<NL, SEQ> w = first_pass;
         Pass ps;
-        while (w.next(P, ps)) {
+        while (go && w.next(P, ps)) {
             const int boxes = (ps.n + P.box16 - 1) / P.box16;
             const uint32_t box_bytes = (uint32_t)(P.box16 * (kGroupCols * kStepCols * 2) * x_steps), tx = boxes * box_bytes;   // (what lies outside x arrives as zeros)
             for (int s = ps.s_lo; s < ps.s_hi; s += x_steps, ++it) {
                 if ((s - ps.s_lo) % kWSteps == 0) {                 // (x_steps divides kWSteps)
                     ++w_at;                                      // two stages behind the ring's depth: never held up by the stage in use
-                    while (feed.more && feed.issued < w_at + w_stages - 2) feed_next(elected);
+                    while (go && feed.more && feed.issued < w_at + w_stages - 2) go = feed_next(elected);
+                    if (!go) break;
                 }
                 const uint32_t bar = smem_u32(&S.full[at.slot]), dst = smem_u32(ring + at.slot * stage_bytes);
 #ifdef RABIT_CHECKED
-                if (it == P.withhold) mbar_wait(smem_u32(&S.never), 0u, abort_flag);
+                if (it == P.withhold && !mbar_wait(smem_u32(&S.never), 0u, abort_flag)) { go = false; break; }
 #endif
-                bool go = elected;
-                if (it >= stages) {
-                    mbar_wait(smem_u32(&S.empty[at.slot]), at.lap ^ 1u, abort_flag);
-                    go = elected && !*abort_flag;
-                }
-                if (go && RABIT_IN_RANGE(at.slot < stages && tx <= (uint32_t)stage_bytes && dst + tx <= smem_u32(w_ring) && ps.c16 >= 0 && ps.c16 + ps.n <= P.n16)) {
-                    ++x_begun;
+                if (it >= stages && !mbar_wait(smem_u32(&S.empty[at.slot]), at.lap ^ 1u, abort_flag)) { go = false; break; }
+                if (elected && RABIT_IN_RANGE(at.slot < stages && tx <= (uint32_t)stage_bytes && dst + tx <= smem_u32(w_ring) && ps.c16 >= 0 && ps.c16 + ps.n <= P.n16)) {
                     mbar_expect_tx(bar, tx);
                     if (x_steps > 1) {
                         tma_load_3d(dst, &x_maps.map[NL == 1 ? 0 : ps.l], 0, ps.c16 * kGroupCols, s, bar);
@@ -519,11 +521,14 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                         for (int c = 0; c < boxes; ++c) tma_load_2d(dst + c * box_bytes, &x_maps.map[NL == 1 ? 0 : ps.l], s * kStepCols, (ps.c16 + c * P.box16) * kGroupCols, bar);
                     }
                 }
-                __syncwarp();
                 at.step(1, stages);
             }
         }
-        if (elected) { S.x_begun = x_begun; S.w_begun = feed.begun; }
+        if (elected) {
+            S.w_begun = feed.issued;
+            *(volatile int*)&S.x_begun = it;
+        }
+        __syncwarp();
     } else if (warp < 4) {
         // ===================================== MMA issuers =====================================
         // Warp 1 + m issues the units u = m, m + n_acc, ... into accumulator m.  (The whole warp walks the loop, one elected lane
@@ -551,7 +556,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                 const int n_ct = NL == 1 ? P.L[0].n_ct : __shfl_sync(0xFFFFFFFFu, P.L[ps.l].n_ct, 0);
                 for (int s = s_lo; s < s_hi; s += x_steps) {
                     const int n_here = min(x_steps, s_hi - s);
-                    mbar_wait(full0 + xw.slot * 8, xw.lap, abort_flag);
+                    mbar_wait_stage(full0 + xw.slot * 8, xw.lap, abort_flag, &S.x_begun);
                     const uint64_t bdesc = bdesc0 + (uint64_t)((xw.slot * stage_bytes) >> 4);
                     int si = n_ops == 1 && n_acc > 1 ? (m ^ (steps_before + s - s_lo)) & 1 : 0;
                     auto issue = [&](uint32_t a, int step, bool first) {
@@ -647,7 +652,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
             for (int j = 0; j < weight_stages(ps) && grp < n_groups; ++j) {
                 const int step0 = ps.s_lo + j * kWSteps, n_here = min(kWSteps, ps.s_hi - step0), whole = min(n_here, n_ct / 2 - step0);   // steps with two column tiles
                 uint32_t bits = bits0 + ww.slot * (K * kWBytes) + first * (2 * RABIT_TILE_BYTES), hs = h0 + ww.slot * (K * kWBytes) + first * (kStepCols * 2);
-                mbar_wait(w_full0 + ww.slot * 8, ww.lap, abort_flag);
+                mbar_wait_stage(w_full0 + ww.slot * 8, ww.lap, abort_flag, &S.x_begun);
                 int sj = first;
                 for (; sj < n_here; sj += kStepsOn) {
                     mbar_wait(bar, ((done >> lap_bit) & 1u) ^ 1u, abort_flag);             // (the first time round this is the barrier's previous phase: free)
