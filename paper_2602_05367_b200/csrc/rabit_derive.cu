@@ -45,11 +45,13 @@ __device__ __forceinline__ int slice_byte(int K, int k, int rl, int group) {
 }
 
 // One CTA per (row tile, slice of 256 columns), one warp per column tile; lane (gq, tq) owns rows 16p + gq + 8 alo and columns
-// 16 ah + 4 tq + c, which are the 16 bytes per path it owns in the sign tile.  Bound: HBM (4 bytes read per weight).  The sign
-// bit of a residual is shifted into two words with one funnel shift each: in (c, p) order it is the tile's word (byte c,
-// bit p), in (p, c) order a row's nibble, of which two neighbouring lanes make a byte of the look-up blocks.  Five to seven
-// instructions per weight at K = 2, where a compare, a select and an OR per path and element took about 18, and a second
-// kernel of 17 us gathered the look-up blocks from the tiles.
+// 16 ah + 4 tq + c, which are the 16 bytes per path it owns in the sign tile.  The sign bit of a residual is shifted into two words
+// with one funnel shift each: in (c, p) order it is the tile's word (byte c, bit p), in (p, c) order a row's nibble, of which
+// two neighbouring lanes make a byte of the look-up blocks.  Bound: latency.  11008 x 4096 at K = 2 takes 47 to 48 us for a floor
+// of 32: 13.7 instructions per weight (loads, recurrence, both arrangements), issue slots 39 % and HBM 47 % busy, 15 warps per
+// SM mostly waiting for W, of which 128 registers a thread leave no more than a part ahead.
+// (Before: 43.9 us with a compare, a select and an OR per path and element, and 17 for a second kernel that gathered the
+// look-up blocks from the tiles.)
 template <int K>
 __global__ void __launch_bounds__(kWarps * 32, 2)
 rabit_derive_kernel(RabitGeom G, const float* __restrict__ W, const __half* __restrict__ g, const __half* __restrict__ h,

@@ -31,20 +31,24 @@
 //
 // Work.  One CTA per SM.  An output tile is 128 weight rows x N batch columns, N a multiple of 16 chosen for the call.
 // Up to 16 batch columns a CTA takes a contiguous range of (row tile, slice of 256 columns) pairs and the parts of a row tile meet in
-// its accumulate words (stream_plan), several layers in one launch if asked.  Otherwise make_plan() picks between: whole tiles; tiles whose contraction is split over a cluster of 2 to 8 CTAs that add their partial
-// results through distributed shared memory (fixed order, no atomics); and, for long batches, contiguous ranges of
-// 16-column groups in (row tile, group) order, one per SM, so that no last wave is left over.
+// its accumulate words (stream_plan), several layers in one launch if asked.  Otherwise make_plan() picks between: whole tiles;
+// tiles whose contraction is split over a cluster of 2 to 8 CTAs that add their partial results through distributed shared
+// memory (fixed order, no atomics); and, for long batches, contiguous ranges of 16-column groups in (row tile, group) order,
+// one per SM, so that no last wave is left over.
 //
-// What bounds it (B200): a unit takes the larger of its four MMAs (32 clocks per 16 batch columns, and 52) and the expansion, 130 clocks
-// of issue, 180 to 200 measured; a launch has about 4 us beside its units.  14336 x 4096 at batch 48 51 -> 16.4 us, 28672 x 8192 at 16
-// 55 -> 43.5, 5000 x 13824 with three paths at 200 209 -> 68.
+// What bounds it (B200): a unit takes the larger of its four MMAs (32 clocks per 16 batch columns, and 52) and the expansion,
+// 130 clocks of issue, 181 measured at 16 columns and 188 at 48 (ALU pipe 63 % and 55 % busy).  A launch has 4 to 5 us beside
+// its units: of a 4096 x 4096 launch at 16 rows, in clocks of a median CTA, 3300 from the end of the dependency wait to the first MMA (tensor memory 800,
+// first weights seen 1300, x 820, first unit 370) and 3000 from the last MMA to the exit (sums and the atomics' answers 2260,
+// teardown 700).  14336 x 4096 at batch 48 51 -> 16.3 us, 28672 x 8192 at 16 55 -> 43.5, 5000 x 13824 with three paths at 200 209 -> 80
+// under sustained load, when the power cap sets the clock (68 to 70 alone).
 //
 // Every wait on a barrier of shared memory is bounded.  On a time-out the CTA skips its remaining waits and the producer starts no
 // further copy; the other roles run on (an MMA on the wrong operand is harmless, and taking the accumulate words through their
 // full count leaves them at rest).  Copies and MMAs under way are awaited, again with a limit, before the tensor memory is freed,
-// the status word is set and the CTA returns.  (tcgen05.alloc and the cluster barriers have no bounded form.  The first ends because no two
-// CTAs that hold tensor memory share an SM, see fill_resources; the second because every thread reaches them after bounded
-// waits.)  DEQ (rabit_set_variant 4): the expander forms the dequantised weight sum_k +-g_k h_k in fp16 and one
+// the status word is set and the CTA returns.  (tcgen05.alloc and the cluster barriers have no bounded form.  The first ends
+// because no two CTAs of this kernel share an SM, see fill_resources, and waits for a foreign one's to leave; the second
+// because every thread reaches them after bounded waits.)  DEQ (rabit_set_variant 4): the expander forms the dequantised weight sum_k +-g_k h_k in fp16 and one
 // contraction serves all paths (a K-th of the tensor work, one fp16 rounding per partial product and weight).
 #include <cuda.h>
 #include <cuda_fp16.h>

@@ -9,8 +9,11 @@
 // built once per CTA in shared memory: one byte permute (the address), one shared-memory load and one
 // fp32 add per EIGHT weights.  The input scale h_k is applied once per table (t = h * x), the signed
 // accumulation is the sum of table entries in fp32 registers, and every weight bit is read once.
-// Measured on B200: the look-ups alone run at 81 clocks per 2 KB block per SM (the shared-memory pipe's
-// rate: 64 look-ups + 16 for the weights), 7.3 TB/s over 148 SMs, above what HBM delivers.
+// Measured on B200, clocks per 2 KB block and SM on a layer of 114688 x 8192: the look-ups alone 67 (64 conflict-free wavefronts of
+// the shared-memory pipe; 8.9 TB/s over 148 SMs, above what HBM delivers), the whole loop 118 with one batch row (5.1 TB/s)
+// and 187 with two (look-ups alone 146).  One row: without the loads of the next blocks 99, without the atomics 115.5,
+// without the look-ups 106: the loop waits for its weights, of which at most one block per warp (32 KB per SM) is under way.
+// Two rows: without the atomics 163, without the loads no faster: there the look-ups bound it.  (28672 x 8192: 15.0 and 22.9 us.)
 //
 // Work split.  The layer is a grid of blocks (32 rows x 256 columns x K paths, K KB each) stored
 // slice-major; CTA c owns a contiguous range of block positions (cut on the host so that all CTAs cost
@@ -470,8 +473,8 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
 struct Cost {
     long long block, table;
 };
-// SM clock cycles, from the phase stamps of the kernel on B200: a block of K paths (look-ups, loads, its atomic) and a
-// table (build plus the two barriers around it).
+// A block of K paths (look-ups, loads, its atomic) and a table (build plus the two barriers around it); only their ratio matters
+// for the cut.  (The block's figure is in clocks of an earlier loop: it takes 118 now.)
 // (the table figure is a fit: the split that minimises the measured step time charges a table about 26 blocks, far
 // more than its 430 cycles of stores, because a rebuild in mid-range also stops every warp at two barriers)
 // (two batch rows: a quarter less measured best, 22016 x 4096 11.5 -> 10.9 us, with one path 9.8 -> 9.3)
