@@ -145,7 +145,7 @@ static bool ranges_overlap(const void* a, size_t an, const void* b, size_t bn) {
 // 4096 x 4096 6.8 / 8.4 / 8.9 against 7.8, 14336 x 4096 13 / 18.3 / 20.6 against 16.0, 28672 x 8192 38 / 54 / 55 against 44).
 static const int kF16Rows = 8;
 
-extern "C" int rabit_linear(const rabit_layer* layer, const void* x, void* y, int batch, void* stream) {
+static int linear_call(const rabit_layer* layer, const void* x, void* y, int batch, void* stream) {
     rabit_clear_error();
     if (!layer) return rabit_fail(RABIT_INVALID_ARG, "rabit_linear: layer is NULL");
     if (!x || !y) return rabit_fail(RABIT_INVALID_ARG, "rabit_linear: null x or y");
@@ -229,8 +229,11 @@ extern "C" int rabit_linear(const rabit_layer* layer, const void* x, void* y, in
     return RABIT_OK;
 }
 
-extern "C" int rabit_linear_group(const rabit_layer* const* layers, const void* const* xs, void* const* ys,
-                                  int n_layers, int batch, void* stream) {
+extern "C" int rabit_linear(const rabit_layer* layer, const void* x, void* y, int batch, void* stream) {
+    return rabit_guarded("rabit_linear", [&] { return linear_call(layer, x, y, batch, stream); });
+}
+
+static int group_call(const rabit_layer* const* layers, const void* const* xs, void* const* ys, int n_layers, int batch, void* stream) {
     rabit_clear_error();
     if (!layers || !xs || !ys) return rabit_fail(RABIT_INVALID_ARG, "rabit_linear_group: null array");
     if (n_layers < 1) return rabit_fail(RABIT_INVALID_ARG, "rabit_linear_group: n_layers must be >= 1 (got %d)", n_layers);
@@ -325,6 +328,11 @@ extern "C" int rabit_linear_group(const rabit_layer* const* layers, const void* 
     }
     if (e != cudaSuccess) return rabit_fail(RABIT_CUDA_ERROR, "rabit_linear_group: launch failed: %s", cudaGetErrorString(e));
     return RABIT_OK;
+}
+
+extern "C" int rabit_linear_group(const rabit_layer* const* layers, const void* const* xs, void* const* ys,
+                                  int n_layers, int batch, void* stream) {
+    return rabit_guarded("rabit_linear_group", [&] { return group_call(layers, xs, ys, n_layers, batch, stream); });
 }
 
 extern "C" size_t rabit_stage_bytes(const rabit_layer* layer, int batch) {

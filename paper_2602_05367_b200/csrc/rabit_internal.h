@@ -37,6 +37,19 @@ void rabit_clear_error();
             return rabit_fail(RABIT_CUDA_ERROR, "%s failed: %s", #expr, cudaGetErrorString(e__)); \
     } while (0)
 
+// The body of an entry point that may allocate host memory (a remembered work split, say): none of them throws.
+#ifdef __cplusplus
+#include <new>
+template <typename F>
+inline int rabit_guarded(const char* name, F&& body) {
+    try {
+        return body();
+    } catch (const std::bad_alloc&) {
+        return rabit_fail(RABIT_INVALID_ARG, "%s: out of host memory", name);
+    }
+}
+#endif
+
 // geometry / layout (rabit_pack.cu)
 bool rabit_make_geom(int K, int M, int N, RabitGeom* out);          // hmax left at 0
 void rabit_fill_header(const RabitGeom& G, RabitHeader* hdr);

@@ -4,6 +4,8 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <exception>
+#include <functional>
 #include <thread>
 #include <vector>
 
@@ -195,10 +197,16 @@ bool rabit_build_meta(const uint16_t* g, const uint16_t* h, int K, int M, int N,
     return true;
 }
 
+static int pack_host(const uint32_t* planes, const uint16_t* g, const uint16_t* h, int K, int M, int N, void* out, size_t out_bytes);
+
 extern "C" int rabit_pack_host(const uint32_t* planes, const uint16_t* g, const uint16_t* h,
                                int K, int M, int N, void* out, size_t out_bytes) {
     rabit_clear_error();
     if (!planes || !g || !h || !out) return rabit_fail(RABIT_INVALID_ARG, "rabit_pack_host: null pointer");
+    return rabit_guarded("rabit_pack_host", [&] { return pack_host(planes, g, h, K, M, N, out, out_bytes); });
+}
+
+static int pack_host(const uint32_t* planes, const uint16_t* g, const uint16_t* h, int K, int M, int N, void* out, size_t out_bytes) {
     RabitGeom G;
     if (!rabit_make_geom(K, M, N, &G))
         return rabit_fail(RABIT_UNSUPPORTED_SHAPE, "rabit_pack_host: unsupported shape K=%d M=%d N=%d (need 1<=K<=3, M>=1, N%%32==0)", K, M, N);
@@ -233,17 +241,19 @@ extern "C" int rabit_pack_host(const uint32_t* planes, const uint16_t* g, const 
                 for (int cb = 0; cb < row_bytes; ++cb) lut[rabit_lut_byte_offset(G, k, row, cb)] = src[cb];
             }
     };
-    if (nthreads == 1) {
-        work(0);
-        work_lut(0);
-    } else {
+    auto share_out = [&](auto& part) {                              // what no thread is to be had for is done here
         std::vector<std::thread> pool;
-        for (int t = 0; t < nthreads; ++t) pool.emplace_back(work, t);
+        int started = 0;
+        try {
+            pool.reserve((size_t)nthreads);
+            for (; started < nthreads - 1; ++started) pool.emplace_back(std::ref(part), started);
+        } catch (const std::exception&) {
+        }
+        for (int t = started; t < nthreads; ++t) part(t);
         for (auto& th : pool) th.join();
-        pool.clear();
-        for (int t = 0; t < nthreads; ++t) pool.emplace_back(work_lut, t);
-        for (auto& th : pool) th.join();
-    }
+    };
+    share_out(work);
+    share_out(work_lut);
     uint16_t* gp = (uint16_t*)(base + hdr.off_g);
     uint16_t* hp = (uint16_t*)(base + hdr.off_h);
     for (int k = 0; k < K; ++k) {

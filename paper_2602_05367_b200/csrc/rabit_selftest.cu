@@ -51,9 +51,10 @@ __global__ void __launch_bounds__(512) stream_read_probe(const uint4* __restrict
 extern "C" int rabit_selftest_f16_plan(int K, int M, int N, int batch, int sms, int* bound_out, int max_out) {
     rabit_clear_error();
     if (!bound_out) return rabit_fail(RABIT_INVALID_ARG, "rabit_selftest_f16_plan: bound_out is NULL");
-    const int grid = rabit_gemv_f16_plan(K, M, N, batch, sms, bound_out, max_out);
-    if (grid < 0) return rabit_fail(RABIT_INVALID_ARG, "rabit_selftest_f16_plan: unsupported shape or too small an output array");
-    return grid;
+    return rabit_guarded("rabit_selftest_f16_plan", [&] {
+        const int grid = rabit_gemv_f16_plan(K, M, N, batch, sms, bound_out, max_out);
+        return grid < 0 ? rabit_fail(RABIT_INVALID_ARG, "rabit_selftest_f16_plan: unsupported shape or too small an output array") : grid;
+    });
 }
 
 extern "C" int rabit_selftest_gemm_plan(int n_layers, const int* M, const int* N, int K, int dequantised, int batch, int sms, int candidate,
