@@ -25,8 +25,8 @@
 //   4..19  expanders: four warpgroups (three if there are three paths) take the units in turn; warp q of a group owns
 //          tensor-memory lanes 32q..32q+31, i.e. the row blocks p = 2q, 2q + 1 of a sign tile.  tcgen05.st.16x256b takes a
 //          warp's registers in the same arrangement in which the tile keeps them (lane (gq, tq): rows gq, gq + 8, four
-//          consecutive columns at 4 tq), so a word of the tile becomes two operand registers with one byte permute, one
-//          shift and one logic instruction each.  Then (same warps) the epilogue: tcgen05.ld, g_k, sum of the paths, fp16,
+//          consecutive columns at 4 tq): a mask and a multiplication (in place of a shift) per word, then per two operand
+//          registers a byte permute, a logic instruction and a fused multiply-add.  Then (same warps) the epilogue: tcgen05.ld, g_k, sum of the paths, fp16,
 //          store.
 //
 // Work.  One CTA per SM.  An output tile is 128 weight rows x N batch columns, N a multiple of 16 chosen for the call.
@@ -37,10 +37,13 @@
 // one per SM, so that no last wave is left over.
 //
 // What bounds it (B200): a unit takes the larger of its four MMAs (32 clocks per 16 batch columns, and 52) and the expansion,
-// 130 clocks of issue, 181 measured at 16 columns and 188 at 48 (ALU pipe 63 % and 55 % busy).  A launch has 4 to 5 us beside
+// 172 clocks at 16 columns (28672 x 8192).  The expansion's 20 operations of the ALU pipe per tile and warp are 80 of them; without the
+// arithmetic a unit takes 143, without the MMAs 147, without stores 163, with none of the three 92: hand-overs between the roles (a wait
+// on a barrier takes some 100 clocks even if it need not wait) and all of them together, no single one.  Tried without gain: three units'
+// room per group (no faster), handing a unit over later so that the next one's loads come first (5 % slower).  A launch has 4 to 5 us beside
 // its units: of a 4096 x 4096 launch at 16 rows, in clocks of a median CTA, 3300 from the end of the dependency wait to the first MMA (tensor memory 800,
 // first weights seen 1300, x 820, first unit 370) and 3000 from the last MMA to the exit (sums and the atomics' answers 2260,
-// teardown 700).  14336 x 4096 at batch 48 51 -> 16.3 us, 28672 x 8192 at 16 55 -> 43.5, 5000 x 13824 with three paths at 200 209 -> 80
+// teardown 700).  14336 x 4096 at batch 48 16.3 -> 15.8 us, 28672 x 8192 at 16 43.5 -> 41.2 (28 operations a tile before), 5000 x 13824 with three paths at 200 209 -> 80
 // under sustained load, when the power cap sets the clock (68 to 70 alone).
 //
 // Every wait on a barrier of shared memory is bounded.  On a time-out the CTA skips its remaining waits and the producer starts no
@@ -167,6 +170,17 @@ struct Walk {
         slot += stride;
         if (slot >= size) { slot -= size; lap ^= 1u; }
     }
+};
+
+// a * m on the multiply-add pipe
+__device__ __forceinline__ uint32_t mul_lo(uint32_t a, uint32_t m) {
+    uint32_t r;
+    asm("mul.lo.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(m));
+    return r;
+}
+struct TileIn {                             // a lane's words of a sign tile and the input scales of its columns
+    uint4 w;
+    uint2 h[2];
 };
 
 // A task's passes: runs of groups inside one row tile, at most max16 groups each, cut evenly.
@@ -491,7 +505,11 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
         const int grp = (warp - 4) >> 2, q = warp & 3;        // tensor-memory lanes this warp may touch: 32q .. 32q + 31
         const int gq = lane >> 2, tq = lane & 3;
         const uint32_t lane_base = tmem_base + ((uint32_t)(32 * q) << 16);
-        const int shift = 6 - 2 * q;                          // bit p of a byte to its top: a shift by 7 - p, this for p = 2q + 1 and one more for p = 2q
+        // bits 2q and 2q + 1 of a byte to its top two: a multiplication by a power of two, 64 >> 2q, that the compiler does not know to be one (it
+        // goes to the multiply-add pipe instead of the one that the byte permutes and logic instructions fill)
+        const uint32_t keep = 0x03030303u << (2 * q);
+        uint32_t up = 64u >> (2 * q);
+        asm volatile("" : "+r"(up));
         // Integer instructions take two issue clocks each and bound this loop (80 of them a unit and warp are the expansion
         // itself), so everything around them is kept in few registers that only step: a group always has the same path, and
         // its units alternate between the same one or two places in tensor memory.
@@ -530,49 +548,76 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                 mbar_wait_stage(w_full0 + ww.slot * 8, ww.lap, abort_flag, &S.x_begun);
                 int sj = first;
                 for (; sj < n_here; sj += kStepsOn) {
-                    mbar_wait(bar, ((done >> lap_bit) & 1u) ^ 1u, abort_flag);             // (the first time round this is the barrier's previous phase: free)
-                    fence_after();
+                    const uint32_t parity = ((done >> lap_bit) & 1u) ^ 1u;                  // (the first time round this is the barrier's previous phase: free)
+                    const bool both = sj < whole;
                     if (!RABIT_IN_RANGE((dst & 0xFFFFu) - (tmem_base & 0xFFFFu) >= (uint32_t)P.a_col && (dst & 0xFFFFu) - (tmem_base & 0xFFFFu) + kUnitCols <= 512u && sj < kWSteps && ww.slot < w_stages &&
                                         bar >= smem_u32(&S.a_empty[0]) && bar <= smem_u32(&S.a_empty[units - 1]))) break;
-                    auto expand_tile = [&](int ct2) {
-                        uint32_t o[2][8];                                                  // [row block][16-column half, row half, column pair]
-                        // dequantised: sum_k +-g_k[row] h_k[col], accumulated from the last (smallest) path to the first with one
-                        // fused multiply-add per path
+                    auto load = [&](int kk, int ct2) {
+                        TileIn t;
+                        t.w = lds_v4(bits + (kk * kWTiles + ct2) * RABIT_TILE_BYTES);
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) o[0][i] = o[1][i] = 0u;
+                        for (int ah = 0; ah < 2; ++ah) t.h[ah] = lds_v2(hs + (kk * kWTiles * RABIT_TILE_COLS + 32 * ct2 + 16 * ah) * 2);
+                        return t;
+                    };
+                    // a tile of path kk into operand registers o[row block][16-column half, row half, column pair]
+                    auto expand = [&](const TileIn& t, int kk, uint32_t (&o)[2][8]) {
+                        const uint32_t word[4] = {mul_lo(t.w.x & keep, up), mul_lo(t.w.y & keep, up), mul_lo(t.w.z & keep, up), mul_lo(t.w.w & keep, up)};
 #pragma unroll
-                        for (int kk = DEQ ? K - 1 : 0; kk >= 0; --kk) {
-                            const uint4 wv = lds_v4(bits + (kk * kWTiles + ct2) * RABIT_TILE_BYTES);
-                            const uint32_t word[4] = {wv.x << shift, wv.y << shift, wv.z << shift, wv.w << shift};
+                        for (int ah = 0; ah < 2; ++ah)
 #pragma unroll
-                            for (int ah = 0; ah < 2; ++ah) {
-                                const uint2 hv = lds_v2(hs + (kk * kWTiles * RABIT_TILE_COLS + 32 * ct2 + 16 * ah) * 2);
+                            for (int rh = 0; rh < 2; ++rh)
 #pragma unroll
-                                for (int rh = 0; rh < 2; ++rh)
+                                for (int pair = 0; pair < 2; ++pair) {
+                                    // bytes [0, c0, 0, c1]: row block 2q + 1's bits at 15 and 31, row block 2q's one below, nothing else
+                                    const uint32_t v = __byte_perm(word[2 * ah + rh], 0u, pair ? 0x3424 : 0x1404);
+                                    const uint32_t hp = pair ? t.h[ah].y : t.h[ah].x, odd = (v & 0x80008000u) ^ hp;
+                                    // As an fp16 number v is 0 or 2 (the bit at 14) with the sign that odd has beside h, so h - v * odd is h or h - 2 h (exact)
+                                    const __half2 even2 = __hfma2(*reinterpret_cast<const __half2*>(&v), __hneg2(*reinterpret_cast<const __half2*>(&odd)), *reinterpret_cast<const __half2*>(&hp));
 #pragma unroll
-                                    for (int pair = 0; pair < 2; ++pair) {
-                                        // bytes [0, c0, 0, c1]: row block 2q + 1's bits at 15 and 31, row block 2q's one below
-                                        const uint32_t v = __byte_perm(word[2 * ah + rh], 0u, pair ? 0x3424 : 0x1404);
-                                        const uint32_t hp = pair ? hv.y : hv.x;
-                                        // bit 14 alone is the fp16 number 2: h - 2 h or h - 0 h, exact, and a floating operation costs half an integer one
-                                        const uint32_t two = v & 0x40004000u, odd = (v & 0x80008000u) ^ hp;
-                                        const __half2 h2 = *reinterpret_cast<const __half2*>(&hp);
-                                        const __half2 even2 = __hfma2(*reinterpret_cast<const __half2*>(&two), __hneg2(h2), h2);
-#pragma unroll
-                                        for (int pi = 0; pi < 2; ++pi) {
-                                            const __half2 m = pi ? *reinterpret_cast<const __half2*>(&odd) : even2;
-                                            uint32_t& a = o[pi][4 * ah + 2 * rh + pair];
-                                            const __half2 r = DEQ ? __hfma2(g_rows[DEQ ? kk : 0][pi][rh], m, *reinterpret_cast<const __half2*>(&a)) : m;
-                                            a = *reinterpret_cast<const uint32_t*>(&r);
-                                        }
+                                    for (int pi = 0; pi < 2; ++pi) {
+                                        const __half2 m = pi ? *reinterpret_cast<const __half2*>(&odd) : even2;
+                                        uint32_t& a = o[pi][4 * ah + 2 * rh + pair];
+                                        const __half2 r = DEQ ? __hfma2(g_rows[DEQ ? kk : 0][pi][rh], m, *reinterpret_cast<const __half2*>(&a)) : m;
+                                        a = *reinterpret_cast<const uint32_t*>(&r);
                                     }
-                            }
-                        }
+                                }
+                    };
+                    auto store = [&](int ct2, const uint32_t (&o)[2][8]) {
                         tmem_st_16x256b_x2(dst + ct2 * 16, o[0]);
                         tmem_st_16x256b_x2(dst + ct2 * 16 + (16u << 16), o[1]);
                     };
-                    expand_tile(0);
-                    if (sj < whole) expand_tile(1);
+                    uint32_t o[2][8];
+                    if constexpr (DEQ) {
+                        mbar_wait(bar, parity, abort_flag);
+                        fence_after();
+                        // dequantised: sum_k +-g_k[row] h_k[col], accumulated from the last (smallest) path to the first with one fused
+                        // multiply-add per path
+                        for (int ct2 = 0; ct2 < (both ? 2 : 1); ++ct2) {
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) o[0][i] = o[1][i] = 0u;
+#pragma unroll
+                            for (int kk = K - 1; kk >= 0; --kk) expand(load(kk, ct2), kk, o);
+                            store(ct2, o);
+                        }
+                    } else if constexpr (K == 3) {
+                        // Three groups have fewer warps to hide a unit's steps behind: its words are on their way and its place is asked for
+                        // first (5000 x 13824 at 16 / 48 rows 23.2 / 26.8 -> 22.0 / 25.2 us; with four groups no gain, with one path 2 % slower).
+                        const TileIn t0 = load(0, 0);
+                        const bool empty = mbar_test_wait(bar, parity);
+                        TileIn t1;
+                        if (both) t1 = load(0, 1);
+                        expand(t0, 0, o);
+                        if (!empty) mbar_wait(bar, parity, abort_flag);
+                        fence_after();
+                        store(0, o);
+                        if (both) { expand(t1, 0, o); store(1, o); }
+                    } else {
+                        mbar_wait(bar, parity, abort_flag);
+                        fence_after();
+                        expand(load(0, 0), 0, o);
+                        store(0, o);
+                        if (both) { expand(load(0, 1), 0, o); store(1, o); }
+                    }
                     bits += kStepsOn * 2 * RABIT_TILE_BYTES;
                     hs += kStepsOn * kStepCols * 2;
                     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
@@ -881,7 +926,7 @@ bool fill_resources(Plan& p, int K, int n_ops, int steps, bool one_box) {
 }
 
 // Clocks of a (step, path) unit, fitted on B200: four MMAs of the pass's batch columns, or the expansion of its two sign tiles
-// (about 130 clocks of integer issue and 50 around them; more if a group has only one unit's room in tensor memory and has
+// (its share of issue slots and the hand-overs around it; more if a group has only one unit's room in tensor memory and has
 // to wait for its MMAs).  Path-major: one warp issues everything and is the bound up to 16 groups (390 clocks at 7 groups, 510 at 13),
 // so that it pays only where the others expand a tile several times: 5000 x 13824 at batch 130 / 200 71 -> 56 / 75 -> 68 us.
 double unit_clocks(int n16, const Plan& p, int n_ops) {

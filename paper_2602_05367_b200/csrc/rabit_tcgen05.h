@@ -1,5 +1,5 @@
-// What the two tcgen05 kernels share (rabit_gemm_tc.cu, rabit_gemv_i8.cu): mbarriers with bounded waits, copies, shared-memory
-// operand descriptors, tensor memory.
+// What a tcgen05 kernel is made of (rabit_gemm_tc.cu): mbarriers with bounded waits, copies, shared-memory operand descriptors,
+// tensor memory.
 #ifndef RABIT_TCGEN05_H_
 #define RABIT_TCGEN05_H_
 
@@ -23,6 +23,12 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {      // (never asleep)
+    uint32_t ok;
+    asm volatile("{ .reg .pred p; mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
                  : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
