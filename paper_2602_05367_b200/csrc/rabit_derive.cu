@@ -10,6 +10,7 @@
 // sign(0) = +1 (bit 0).
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <cstring>
 
 #include "rabit_internal.h"
@@ -44,97 +45,155 @@ __device__ __forceinline__ int slice_byte(int K, int k, int rl, int group) {
     return ((rl >> 5) * K + k) * RABIT_LUT_PART_BYTES + (s >> 4) * 512 + l * 16 + (s & 15);
 }
 
-// One CTA per (row tile, slice of 256 columns), one warp per column tile; lane (gq, tq) owns rows 16p + gq + 8 alo and columns
-// 16 ah + 4 tq + c, which are the 16 bytes per path it owns in the sign tile.  The sign bit of a residual is shifted into two words
-// with one funnel shift each: in (c, p) order it is the tile's word (byte c, bit p), in (p, c) order a row's nibble, of which
-// two neighbouring lanes make a byte of the look-up blocks.  Bound: latency.  11008 x 4096 at K = 2 takes 47 to 48 us for a floor
-// of 32: 13.7 instructions per weight (loads, recurrence, both arrangements), issue slots 39 % and HBM 47 % busy, 15 warps per
-// SM mostly waiting for W, of which 128 registers a thread leave no more than a part ahead.
-// (Before: 43.9 us with a compare, a select and an OR per path and element, and 17 for a second kernel that gathered the
-// look-up blocks from the tiles.)
+// 16 bytes global -> shared, asynchronous, not through L1 (valid false: zeros)
+__device__ __forceinline__ void copy_async_16(uint32_t dst, const void* src, bool valid) {
+    const uint32_t size = valid ? 16u : 0u;
+    asm volatile("cp.async.cg.shared.global.L2::128B [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(size) : "memory");
+}
+template <int N>
+__device__ __forceinline__ void copy_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// A persistent CTA takes (row tile, slice of 256 columns) blocks in turn, one warp per column tile; lane (gq, tq) owns rows 16p + gq + 8 alo and
+// columns 16 ah + 4 tq + c, which are the 16 bytes per path it owns in the sign tile.  The sign bit of a residual is shifted into the
+// tile's word (byte c, bit p) with one funnel shift; transposed, two neighbouring lanes' words are four bytes of the look-up blocks each.
+// W comes in parts of 4 KB a warp (a quarter of its 128 x 32 weights) by asynchronous copies into a ring of three parts of its own in shared
+// memory, two ahead of the one at hand and across block borders; a lane reads back what it copied itself, so no barrier is involved.
+// The scales of the next block are fetched beside the work on this one.
+constexpr int kRingParts = 3;
+constexpr int kPartBytes = 32 * 8 * 16;
+template <int K>
+struct DeriveSmem {
+    static constexpr int kBytes = kWarps * kRingParts * kPartBytes;                          // behind the ring: the look-up bytes of a block
+    static constexpr int kScales = kBytes + 4 * K * RABIT_LUT_PART_BYTES;                    // then g and h of two blocks, fp32
+    static constexpr int kScaleFloats = (K - 1) * (RABIT_TILE_ROWS + RABIT_LUT_COLS);        // (the last path's are not needed)
+    static constexpr int kTotal = kScales + 2 * kScaleFloats * 4;
+};
 template <int K>
 __global__ void __launch_bounds__(kWarps * 32, 2)
 rabit_derive_kernel(RabitGeom G, const float* __restrict__ W, const __half* __restrict__ g, const __half* __restrict__ h,
-                    uint4* __restrict__ tiles, uint4* __restrict__ lut, const __grid_constant__ Fills F) {
-    __shared__ __align__(16) unsigned char bytes[4 * K * RABIT_LUT_PART_BYTES];
+                    uint4* __restrict__ tiles, uint4* __restrict__ lut, uint32_t n_blocks, const __grid_constant__ Fills F) {
+    using S = DeriveSmem<K>;
+    extern __shared__ __align__(16) unsigned char smem[];
+    unsigned char* bytes = smem + S::kBytes;
+    float* scales = reinterpret_cast<float*>(smem + S::kScales);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int rt = blockIdx.x / G.n_cs, cs = blockIdx.x - rt * G.n_cs, ct = cs * kWarps + warp;
     const int gq = lane >> 2, tq = lane & 3;
-    const bool inside = ct < G.n_ct;
+    const uint32_t ring = (uint32_t)__cvta_generic_to_shared(smem) + (uint32_t)(warp * kRingParts * kPartBytes + lane * 16);
 
-    // W in four parts of 8 x 16 bytes, the next one in flight while the current one is worked through
-    float4 w[2][8];
-    auto load = [&](int part, float4 (&dst)[8]) {
-        const int alo = part >> 1, ah = part & 1;
+    // part `part` of block b of W into ring slot `slot` (padded rows and columns, and blocks beyond the last: zeros, i.e. +1 signs)
+    auto fetch = [&](uint32_t b, int part, int slot) {
+        const int rt = (int)(b / (uint32_t)G.n_cs), ct = (int)(b - (uint32_t)rt * G.n_cs) * kWarps + warp, row0 = rt * RABIT_TILE_ROWS + gq + 8 * (part >> 1);
+        const bool inside = b < n_blocks && ct < G.n_ct;
+        const float* src = W + (size_t)row0 * G.N + ct * RABIT_TILE_COLS + 16 * (part & 1) + 4 * tq;
 #pragma unroll
         for (int p = 0; p < 8; ++p) {
-            const int row = rt * RABIT_TILE_ROWS + 16 * p + gq + 8 * alo;
-            dst[p] = make_float4(0.f, 0.f, 0.f, 0.f);     // padded rows and columns: +1 signs
-            if (inside && row < G.M) dst[p] = __ldcs(reinterpret_cast<const float4*>(W + (size_t)row * G.N + ct * RABIT_TILE_COLS + 16 * ah + 4 * tq));
+            const bool valid = inside && row0 + 16 * p < G.M;
+            copy_async_16(ring + (uint32_t)(slot * kPartBytes + p * 512), valid ? src + (size_t)(16 * p) * G.N : W, valid);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    // output and input scales of block b, a few per thread
+    constexpr int kPerThread = (S::kScaleFloats + kWarps * 32 - 1) / (kWarps * 32);
+    __half next[kPerThread > 0 ? kPerThread : 1];
+    auto fetch_scales = [&](uint32_t b) {
+        const int rt = (int)(b / (uint32_t)G.n_cs), cs = (int)(b - (uint32_t)rt * G.n_cs);
+#pragma unroll
+        for (int u = 0; u < kPerThread; ++u) {
+            const int i = threadIdx.x + u * kWarps * 32, k = i / (RABIT_TILE_ROWS + RABIT_LUT_COLS), j = i - k * (RABIT_TILE_ROWS + RABIT_LUT_COLS);
+            const int col = cs * RABIT_LUT_COLS + j - RABIT_TILE_ROWS;
+            next[u] = __half();
+            if (i < S::kScaleFloats && b < n_blocks) {
+                if (j < RABIT_TILE_ROWS) next[u] = g[(size_t)k * G.Mp + rt * RABIT_TILE_ROWS + j];       // (zero in padded rows)
+                else if (col < G.N) next[u] = h[(size_t)k * G.N + col];
+            }
         }
     };
-    load(0, w[0]);
-    do_fills(F);
-    uint32_t out[K][4];
+    auto keep_scales = [&](int buffer) {
 #pragma unroll
-    for (int part = 0; part < 4; ++part) {
-        if (part < 3) load(part + 1, w[(part + 1) & 1]);
-        const int alo = part >> 1, ah = part & 1;
-        float r[8][4];
-#pragma unroll
-        for (int p = 0; p < 8; ++p) {                     // (+ 0: a weight of -0 is +0, a NaN the positive one: bit 0)
-            const float4 v = w[part & 1][p];
-            r[p][0] = v.x + 0.f; r[p][1] = v.y + 0.f; r[p][2] = v.z + 0.f; r[p][3] = v.w + 0.f;
+        for (int u = 0; u < kPerThread; ++u) {
+            const int i = threadIdx.x + u * kWarps * 32;
+            if (i < S::kScaleFloats) scales[buffer * S::kScaleFloats + i] = __half2float(next[u]);
         }
+    };
+
+    fetch(blockIdx.x, 0, 0);
+    fetch(blockIdx.x, 1, 1);
+    fetch_scales(blockIdx.x);
+    do_fills(F);
+    keep_scales(0);
+    __syncthreads();
+    const uint32_t own_half = tq & 1 ? 0xF0F0F0F0u : 0x0F0F0F0Fu;
+    const int turn = tq & 1 ? 28 : 4;
+    int slot = 0, ahead = 2, buffer = 0;                  // ring slots of the part at hand and of the one to fetch
+    for (uint32_t b = blockIdx.x; b < n_blocks; b += gridDim.x, buffer ^= 1) {
+        const int rt = (int)(b / (uint32_t)G.n_cs), cs = (int)(b - (uint32_t)rt * G.n_cs), ct = cs * kWarps + warp;
+        const bool inside = ct < G.n_ct;
+        const float* gs = scales + buffer * S::kScaleFloats;
+        fetch_scales(b + gridDim.x);
+        uint32_t out[K][4];
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            uint32_t tile = 0u, nibbles = 0u;
+        for (int part = 0; part < 4; ++part) {
+            fetch(part < 2 ? b : b + gridDim.x, (part + 2) & 3, ahead);     // (into the slot of the part before this one)
+            ahead = ahead == kRingParts - 1 ? 0 : ahead + 1;
+            copy_async_wait<2>();
+            const int alo = part >> 1, ah = part & 1;
+            float r[8][4];
 #pragma unroll
-            for (int c = 3; c >= 0; --c)
+            for (int p = 0; p < 8; ++p) {                 // (+ 0: a weight of -0 is +0, a NaN the positive one: bit 0)
+                float4 v;
+                asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(ring + (uint32_t)(slot * kPartBytes + p * 512)) : "memory");
+                r[p][0] = v.x + 0.f; r[p][1] = v.y + 0.f; r[p][2] = v.z + 0.f; r[p][3] = v.w + 0.f;
+            }
+            slot = slot == kRingParts - 1 ? 0 : slot + 1;
 #pragma unroll
-                for (int p = 7; p >= 0; --p) tile = __funnelshift_l(__float_as_uint(r[p][c]), tile, 1);
+            for (int k = 0; k < K; ++k) {
+                uint32_t tile = 0u;
 #pragma unroll
-            for (int p = 7; p >= 0; --p)
+                for (int c = 3; c >= 0; --c)
 #pragma unroll
-                for (int c = 3; c >= 0; --c) nibbles = __funnelshift_l(__float_as_uint(r[p][c]), nibbles, 1);
-            out[k][alo | (ah << 1)] = tile;
-            if (k + 1 < K) {
-                float hv[4] = {0.f, 0.f, 0.f, 0.f};
-                if (inside) {
-                    const uint2 raw = *reinterpret_cast<const uint2*>(h + (size_t)k * G.N + ct * RABIT_TILE_COLS + 16 * ah + 4 * tq);
-                    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&raw.x)), b = __half22float2(*reinterpret_cast<const __half2*>(&raw.y));
-                    hv[0] = a.x; hv[1] = a.y; hv[2] = b.x; hv[3] = b.y;
-                }
+                    for (int p = 7; p >= 0; --p) tile = __funnelshift_l(__float_as_uint(r[p][c]), tile, 1);
+                out[k][alo | (ah << 1)] = tile;
+                if (k + 1 < K) {
+                    const float* gk = gs + k * (RABIT_TILE_ROWS + RABIT_LUT_COLS);
+                    const float4 hv = *reinterpret_cast<const float4*>(gk + RABIT_TILE_ROWS + warp * RABIT_TILE_COLS + 16 * ah + 4 * tq);
+                    const float hc[4] = {hv.x, hv.y, hv.z, hv.w};
 #pragma unroll
-                for (int p = 0; p < 8; ++p) {
-                    const float gv = __half2float(g[(size_t)k * G.Mp + rt * RABIT_TILE_ROWS + 16 * p + gq + 8 * alo]);   // (zero in padded rows)
+                    for (int p = 0; p < 8; ++p) {
+                        const float gv = gk[16 * p + gq + 8 * alo];
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const float gb = __uint_as_float(__float_as_uint(gv) ^ (__float_as_uint(r[p][c]) & 0x80000000u));   // g * B, exact
-                        r[p][c] = r[p][c] - gb * hv[c];   // the product is exact in fp32: one rounding
+                        for (int c = 0; c < 4; ++c) {
+                            const float gb = __uint_as_float(__float_as_uint(gv) ^ (__float_as_uint(r[p][c]) & 0x80000000u));   // g * B, exact
+                            r[p][c] = r[p][c] - gb * hc[c];   // the product is exact in fp32: one rounding
+                        }
                     }
                 }
+                // Bytes of the look-up blocks.  The word has bit p of byte c; with the two halves of its bytes transposed as 4 x 4 bit matrices byte i
+                // holds the columns of row block i in its low half, those of row block 4 + i in its high half.  The even lane of a pair has columns
+                // 0..3 of the byte group, the odd one columns 4..7; the even lane puts together the rows p = 0..3, the odd one p = 4..7.
+                uint32_t rows = tile, t = (rows ^ (rows >> 7)) & 0x00AA00AAu;
+                rows ^= t ^ (t << 7);
+                t = (rows ^ (rows >> 14)) & 0x0000CCCCu;
+                rows ^= t ^ (t << 14);
+                const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, rows, 1);
+                const uint32_t four = (rows & own_half) | (__funnelshift_l(other, other, turn) & ~own_half);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    bytes[slice_byte(K, k, 16 * (4 * (tq & 1) + i) + gq + 8 * alo, 4 * warp + 2 * ah + (tq >> 1))] = (unsigned char)(four >> (8 * i));
             }
-            // bytes of the look-up blocks: the even lane of a pair has columns 0..3 of the byte group, the odd one columns 4..7; the
-            // even lane puts together the rows p = 0..3, the odd one p = 4..7
-            const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, nibbles, 1);
-            const int odd = tq & 1;
-            uint32_t lo = ((odd ? other : nibbles) >> (16 * odd)) & 0xFFFFu, hi = ((odd ? nibbles : other) >> (16 * odd)) & 0xFFFFu;
-            lo = (lo | (lo << 8)) & 0x00FF00FFu; lo = (lo | (lo << 4)) & 0x0F0F0F0Fu;
-            hi = (hi | (hi << 8)) & 0x00FF00FFu; hi = (hi | (hi << 4)) & 0x0F0F0F0Fu;
-            const uint32_t four = lo | (hi << 4);
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                bytes[slice_byte(K, k, 16 * (4 * odd + i) + gq + 8 * alo, 4 * warp + 2 * ah + (tq >> 1))] = (unsigned char)(four >> (8 * i));
         }
-    }
-    if (inside) {
+        if (inside) {
 #pragma unroll
-        for (int k = 0; k < K; ++k) tiles[rabit_tile_pos(G, rt, k, ct) * 32 + lane] = make_uint4(out[k][0], out[k][1], out[k][2], out[k][3]);
+            for (int k = 0; k < K; ++k) tiles[rabit_tile_pos(G, rt, k, ct) * 32 + lane] = make_uint4(out[k][0], out[k][1], out[k][2], out[k][3]);
+        }
+        keep_scales(buffer ^ 1);
+        __syncthreads();
+        uint4* dst = lut + ((size_t)cs * G.n_rb + 4 * rt) * K * (RABIT_LUT_PART_BYTES / 16);
+        for (int i = threadIdx.x; i < 4 * K * (RABIT_LUT_PART_BYTES / 16); i += kWarps * 32) dst[i] = reinterpret_cast<const uint4*>(bytes)[i];
+        __syncthreads();
     }
-    __syncthreads();
-    uint4* dst = lut + ((size_t)cs * G.n_rb + 4 * rt) * K * (RABIT_LUT_PART_BYTES / 16);
-    for (int i = threadIdx.x; i < 4 * K * (RABIT_LUT_PART_BYTES / 16); i += kWarps * 32) dst[i] = reinterpret_cast<const uint4*>(bytes)[i];
+    copy_async_wait<0>();
 }
 
 // Canonical planes [K][M][N/32] -> look-up blocks: one warp per (slice, row block), lane = row.  A row's 32 bytes of the slice
@@ -200,6 +259,19 @@ void make_fills(const RabitHeader& hdr, char* base, Fills* F) {
     F->n_zero = (size_t)(hdr.off_lut - hdr.off_flags) / 16;
 }
 
+template <int K>
+cudaError_t launch_derive(const RabitGeom& G, const float* W, const __half* g, const __half* h, uint4* tiles, uint4* lut, uint32_t blocks, unsigned int grid, int device,
+                          const Fills& F, cudaStream_t stream) {
+    static bool done[64] = {};                            // function attributes are per device
+    if (device < 0 || device >= 64 || !done[device]) {
+        cudaError_t e = cudaFuncSetAttribute(rabit_derive_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, DeriveSmem<K>::kTotal);
+        if (e != cudaSuccess) return e;
+        if (device >= 0 && device < 64) done[device] = true;
+    }
+    rabit_derive_kernel<K><<<grid, kWarps * 32, DeriveSmem<K>::kTotal, stream>>>(G, W, g, h, tiles, lut, blocks, F);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 // Both write the signs in both arrangements, the header and the resting state of the exchange buffer and the flags; the scales
@@ -211,10 +283,14 @@ cudaError_t rabit_launch_derive(const RabitGeom& G, const RabitHeader& hdr, char
     make_fills(hdr, base, &F);
     const __half *g = reinterpret_cast<const __half*>(base + hdr.off_g), *h = reinterpret_cast<const __half*>(base + hdr.off_h);
     uint4 *tiles = reinterpret_cast<uint4*>(base + hdr.off_bits), *lut = reinterpret_cast<uint4*>(base + hdr.off_lut);
-    if (G.K == 1) rabit_derive_kernel<1><<<(unsigned int)blocks, kWarps * 32, 0, stream>>>(G, W, g, h, tiles, lut, F);
-    else if (G.K == 2) rabit_derive_kernel<2><<<(unsigned int)blocks, kWarps * 32, 0, stream>>>(G, W, g, h, tiles, lut, F);
-    else rabit_derive_kernel<3><<<(unsigned int)blocks, kWarps * 32, 0, stream>>>(G, W, g, h, tiles, lut, F);
-    return cudaGetLastError();
+    int device = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    if (e != cudaSuccess) return e;
+    const unsigned int grid = (unsigned int)std::min<long long>(blocks, 2LL * sms);
+    return G.K == 1 ? launch_derive<1>(G, W, g, h, tiles, lut, (uint32_t)blocks, grid, device, F, stream)
+         : G.K == 2 ? launch_derive<2>(G, W, g, h, tiles, lut, (uint32_t)blocks, grid, device, F, stream)
+                    : launch_derive<3>(G, W, g, h, tiles, lut, (uint32_t)blocks, grid, device, F, stream);
 }
 
 // `planes` may lie in the section of the sign tiles: the look-up blocks are made from the planes, the tiles from the look-up blocks.
