@@ -28,10 +28,11 @@
 //          consecutive columns at 4 tq): a mask and a multiplication (in place of a shift) per word, then per two operand
 //          registers a byte permute, a logic instruction and a fused multiply-add.  Then (same warps) the epilogue: tcgen05.ld, g_k, sum of the paths, fp16,
 //          store.
+//   20..23 stream kernels only: the epilogue of every pass but a task's last.
 //
 // Work.  One CTA per SM.  An output tile is 128 weight rows x N batch columns, N a multiple of 16 chosen for the call.
 // Up to 16 batch columns a CTA takes a contiguous range of (row tile, slice of 256 columns) pairs and the parts of a row tile meet in
-// its accumulate words (stream_plan), several layers in one launch if asked.  Otherwise make_plan() picks between: whole tiles;
+// its accumulate words (stream_plan; the stream kernels, NL > 1, up to four layers in a launch).  Otherwise make_plan() picks between: whole tiles;
 // tiles whose contraction is split over a cluster of 2 to 8 CTAs that add their partial results through distributed shared
 // memory (fixed order, no atomics); and, for long batches, contiguous ranges of 16-column groups in (row tile, group) order,
 // one per SM, so that no last wave is left over.
@@ -43,7 +44,7 @@
 // room per group (no faster), handing a unit over later so that the next one's loads come first (5 % slower).  A launch has 4 to 5 us beside
 // its units: of a 4096 x 4096 launch at 16 rows, in clocks of a median CTA, 3300 from the end of the dependency wait to the first MMA (tensor memory 800,
 // first weights seen 1300, x 820, first unit 370) and 3000 from the last MMA to the exit (sums and the atomics' answers 2260,
-// teardown 700).  14336 x 4096 at batch 48 16.3 -> 15.8 us, 28672 x 8192 at 16 43.5 -> 41.2 (28 operations a tile before), 5000 x 13824 with three paths at 200 209 -> 80
+// teardown 700).  14336 x 4096 at batch 48 16.3 -> 15.8 us, 28672 x 8192 at 16 43.5 -> 41.2 (28 operations a tile before) -> 40.2 (epilogues beside), 5000 x 13824 with three paths at 200 209 -> 80
 // under sustained load, when the power cap sets the clock (68 to 70 alone).
 //
 // Every wait on a barrier of shared memory is bounded.  On a time-out the CTA skips its remaining waits and the producer starts no
@@ -80,6 +81,7 @@ constexpr int kMaxWStages = 4;
 constexpr int kExpandGroups = 4;            // of four warps each
 constexpr int kExpandWarps = 4 * kExpandGroups;
 constexpr int kThreads = (4 + kExpandWarps) * 32;
+constexpr int kStreamThreads = kThreads + 128;             // stream kernels: four warps for the epilogues
 constexpr unsigned long long kSumMask = (1ULL << 55) - 1;
 
 constexpr int kMaxTasks = 512;
@@ -105,8 +107,7 @@ struct GemmParams {
     int n16;                                // groups of 16 batch columns
     int n_tasks;                            // tasks of the grid: one per CTA, or one per cluster if split > 1
     int chunks, chunk16;                    // > 0: a task is (row tile, chunk of chunk16 groups); 0: a contiguous range of groups
-    int n_groups, quot, rem;                // row tiles * n16 (stream: row tiles * n_cs, over all layers); that by n_tasks
-    int stream;                             // a task is a contiguous range of (row tile, slice) pairs, all of at most 16 batch columns
+    int n_groups, quot, rem;                // row tiles * n16 (stream kernels, NL > 1: row tiles * n_cs, over all layers); that by n_tasks
     int max16;                              // most groups one pass can accumulate
     int split;                              // CTAs (one cluster) that share the contraction of a task, up to 8
     int recv_off;                           // receive buffer of a split task, from the control block
@@ -133,8 +134,8 @@ struct Control {                            // ahead of the ring in shared memor
     unsigned long long w_empty[kMaxWStages];// every expander warp has read them
     unsigned long long a_ready[kMaxUnits];  // unit expanded
     unsigned long long a_empty[kMaxUnits];  // MMAs that read the unit retired
-    unsigned long long acc_ready;           // all MMAs of the pass retired
-    unsigned long long acc_empty;           // epilogue has read the accumulators
+    unsigned long long acc_ready[2];        // all MMAs of the pass retired (stream: by the parity of the pass, which has its own accumulators)
+    unsigned long long acc_empty[2];        // epilogue has read the accumulators
     unsigned long long drained[3];          // after a time-out: everything this accumulator's warp issued has retired
 #ifdef RABIT_CHECKED
     unsigned long long never;               // nothing arrives here (rabit_selftest_withhold)
@@ -214,20 +215,20 @@ struct PassWalker {
                 while (l + 1 < P.n_layers && g >= P.L[l + 1].pair0) ++l;
                 g -= P.L[l].pair0;
             }
-            const int per_rt = NL > 1 || P.stream ? P.L[l].n_cs : P.n16;
+            const int per_rt = NL > 1 ? P.L[l].n_cs : P.n16;
             rt = g / per_rt;
             c16 = g - rt * per_rt;
         }
     }
     __host__ __device__ bool next(const GemmParams<NL>& P, Pass& ps) {
         if (left <= 0) return false;
-        if (NL > 1 || P.stream) {
+        if (NL > 1) {
             const int n_cs = P.L[l].n_cs, run = min(left, n_cs - c16);
-            ps = Pass{l, rt, 0, 1, c16 * kSliceSteps, min((c16 + run) * kSliceSteps, NL > 1 ? (P.L[l].n_ct + 1) / 2 : s_hi), 0};
+            ps = Pass{l, rt, 0, 1, c16 * kSliceSteps, min((c16 + run) * kSliceSteps, (P.L[l].n_ct + 1) / 2), 0};
             left -= run;
             c16 = 0;
             ++rt;
-            if (NL > 1 && rt == P.L[l].n_rt) { rt = 0; ++l; }             // (a task that ends here never looks at the layer again)
+            if (rt == P.L[l].n_rt) { rt = 0; ++l; }                       // (a task that ends here never looks at the layer again)
             return true;
         }
         const int run = min(left, P.n16 - c16), pieces = run <= P.max16 ? 1 : (run + P.max16 - 1) / P.max16;
@@ -255,7 +256,7 @@ __host__ __device__ __forceinline__ int segment_arrivals(uint32_t first, uint32_
 // is a pass per path on one accumulator, the sum of the scaled passes stays in tensor memory beside it, and up to 13 groups fit
 // (5000 x 13824 at batch 200: each tile expanded once instead of three times).
 template <int K, bool DEQ, int NL, bool SEQ>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(NL > 1 ? kStreamThreads : kThreads, 1)
 rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_constant__ XMaps<NL> x_maps) {
     extern __shared__ unsigned char smem_raw[];
     // the swizzled x tiles need 1024-byte alignment; the launch reserves the slack
@@ -291,8 +292,10 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
         if (lane < kMaxWStages) { mbar_init(smem_u32(&S.w_full[lane]), 1); mbar_init(smem_u32(&S.w_empty[lane]), 4 * n_groups); }
         if (lane < kMaxUnits) { mbar_init(smem_u32(&S.a_ready[lane]), 4); mbar_init(smem_u32(&S.a_empty[lane]), 1); }
         if (lane == 0) {
-            mbar_init(smem_u32(&S.acc_ready), n_acc);
-            mbar_init(smem_u32(&S.acc_empty), kExpandWarps);
+            for (int i = 0; i < 2; ++i) {
+                mbar_init(smem_u32(&S.acc_ready[i]), n_acc);
+                mbar_init(smem_u32(&S.acc_empty[i]), NL > 1 ? 4 : kExpandWarps);
+            }
             S.abort_flag = 0;
             S.x_begun = -1;
 #ifdef RABIT_CHECKED
@@ -326,6 +329,83 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
         for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(d[i]);
+    };
+
+    // Stream: a pass's sums of this thread's row, batch columns [c0, c0 + n) (its scales are on their way).  A segment that is a whole row tile is stored;
+    // otherwise every output goes into its 64-bit accumulate word with one integer atomic (as in rabit_gemv_f16.cu: fixed-point grid
+    // of the packer, a segment of s slices shifted by s * 2^fix_bits, arrivals in bits 55..62, bit 63 = non-finite), and the thread
+    // whose add completes a word rounds it to fp16, stores y and clears it.
+    [[maybe_unused]] auto publish = [&](auto cols, const Pass& ps, int pass_i, int c0) {
+        constexpr int n = decltype(cols)::value;
+        const GemmLayer& L = layer(ps);
+        const int q = warp & 3, row = ps.rt * kTileM + q * 32 + lane, n_slices = (ps.s_hi - ps.s_lo + kSliceSteps - 1) / kSliceSteps, set = pass_i & 1;
+        // (in registers: read from the parameters between the atomics, each would be a wait)
+        const int M = L.M, Mp = L.Mp, n_cs = L.n_cs, fix_bits = L.fix_bits, n_here = P.batch - c0;
+        const float inv_unit = L.inv_unit, unit = L.unit, limit = L.limit * (float)n_slices;
+        __half* const y = L.y + (size_t)c0 * M + row;
+        unsigned long long* const word = L.acc + (size_t)c0 * Mp + row;
+        const int arrivals = segment_arrivals((uint32_t)(L.pair0 + ps.rt * n_cs), (uint32_t)n_cs, (uint32_t)P.n_tasks, (uint32_t)P.n_groups);
+        const uint32_t from = __shfl_sync(0xFFFFFFFFu, S.tmem_base, 0) + ((uint32_t)(32 * q) << 16) + (uint32_t)(set * n_acc * kGroupCols + c0);
+        mbar_wait(smem_u32(&S.acc_ready[set]), (uint32_t)(pass_i >> 1) & 1u, abort_flag);
+        __syncwarp();
+        fence_after();
+        float v[n];
+#pragma unroll
+        for (int i = 0; i < n; ++i) v[i] = 0.f;
+#pragma unroll
+        for (int m = 0; m < (n_ops == 1 ? 2 : n_ops); ++m) {
+            if (n_ops == 1 && m >= n_acc) break;
+            uint32_t d[n];
+            if constexpr (n == 16) tmem_ld16(from + (uint32_t)(m * kGroupCols), d);
+            else tmem_ld4(from + (uint32_t)(m * kGroupCols), d);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            const float gm = DEQ ? 1.f : scale(n_ops == 1 ? 0 : m);
+#pragma unroll
+            for (int i = 0; i < n; ++i) v[i] = fmaf(gm, __uint_as_float(d[i]), v[i]);
+        }
+        fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&S.acc_empty[set]));
+        if (n_slices == n_cs) {
+#pragma unroll
+            for (int i = 0; i < n; ++i)
+                if (i < n_here && row < M) y[(size_t)i * M] = __float2half_rn(v[i]);
+            return;
+        }
+        // inf or NaN: finite inputs cannot get beyond the limit
+        const unsigned long long bias = (unsigned long long)((long long)n_slices << fix_bits) + (1ULL << 55);
+        auto bad = [&](int i) { return !(fabsf(v[i] * inv_unit) < limit); };
+        auto contribution = [&](int i) { return (unsigned long long)(bad(i) ? 0LL : __float2ll_rn(v[i] * inv_unit)) + bias; };
+        auto poison = [&](int i) {                               // sticky: the add that follows never carries into bit 63
+            if (bad(i) && i < n_here && RABIT_IN_RANGE(row >= 0 && row < Mp && c0 + i < RABIT_LUT_MAX_BATCH)) atomicOr(word + (size_t)i * Mp, 1ULL << 63);
+        };
+        if constexpr (n == kGroupCols) {
+            // (many in a row: no branch between the adds.  20000 x 1024 at 16 rows 9.25 -> 8.95 us; with four a thread 4096 x 4096 7.35 -> 7.45)
+            uint32_t bads = 0u;
+#pragma unroll
+            for (int i = 0; i < n; ++i) bads |= bad(i) ? 1u : 0u;
+            if (bads != 0u) [[unlikely]] {
+#pragma unroll
+                for (int i = 0; i < n; ++i) poison(i);
+            }
+        }
+        unsigned long long old[n];
+        // all atomics of the thread back to back: nothing between them that could wait for an answer
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            old[i] = 0ULL;
+            if constexpr (n != kGroupCols) poison(i);
+            if (i < n_here && RABIT_IN_RANGE(row >= 0 && row < Mp && c0 + i < RABIT_LUT_MAX_BATCH)) old[i] = atomicAdd(word + (size_t)i * Mp, contribution(i));
+        }
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            if (i >= n_here || (int)((old[i] >> 55) & 0xFFu) != arrivals - 1) continue;       // other segments are still to come
+            const unsigned long long sum = (old[i] & kSumMask) + (contribution(i) & kSumMask);
+            const long long total = (long long)sum - ((long long)n_cs << fix_bits);
+            const bool poisoned = bad(i) || (old[i] >> 63) != 0;
+            if (row < M) y[(size_t)i * M] = poisoned ? __ushort_as_half((unsigned short)0x7FFF) : __float2half_rn(__ll2float_rn(total) * unit);
+            word[(size_t)i * Mp] = 0ULL;                         // resting state for the next call
+        }
     };
 
     auto weight_stages = [](const Pass& ps) { return (ps.s_hi - ps.s_lo + kWSteps - 1) / kWSteps; };
@@ -430,14 +510,17 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
             const int u_stride = n_ops == 1 ? n_acc : 1;         // steps from one of its units to the next
             const uint32_t full0 = smem_u32(&S.full[0]), empty0 = smem_u32(&S.empty[0]), a_ready0 = smem_u32(&S.a_ready[0]), a_empty0 = smem_u32(&S.a_empty[0]);
             const uint64_t bdesc0 = umma_desc(smem_u32(ring));
-            const uint32_t a0 = tmem_base + (uint32_t)P.a_col, d = tmem_base + (uint32_t)(m * P.max16 * kGroupCols);
+            const uint32_t a0 = tmem_base + (uint32_t)P.a_col, d0 = tmem_base + (uint32_t)(m * P.max16 * kGroupCols);
             const uint32_t step_bytes = (uint32_t)stage_bytes / (uint32_t)x_steps;
             int steps_before = 0;                                // of earlier passes
             PassWalker<NL, SEQ> w = first_pass;
             Pass ps;
             while (w.next(P, ps)) {
                 const uint32_t idesc = __shfl_sync(0xFFFFFFFFu, umma_idesc(ps.n * kGroupCols), 0);
-                if (pass_i > 0) mbar_wait(smem_u32(&S.acc_empty), (pass_i - 1) & 1, abort_flag);   // epilogue has drained the accumulators
+                // the epilogue of the pass that had these accumulators has read them
+                const int set = NL > 1 ? pass_i & 1 : 0;
+                const uint32_t d = NL > 1 ? __shfl_sync(0xFFFFFFFFu, d0 + (uint32_t)(set * n_acc * kGroupCols), 0) : d0;
+                if (NL > 1 ? pass_i > 1 : pass_i > 0) mbar_wait(smem_u32(&S.acc_empty[set]), (NL > 1 ? (pass_i >> 1) - 1 : pass_i - 1) & 1, abort_flag);
                 ++pass_i;
                 if (!RABIT_IN_RANGE(ps.n >= 1 && ps.n <= P.max16 && (m + 1) * P.max16 * kGroupCols <= P.a_col && P.a_col + units * kUnitCols <= 512)) break;
                 uint32_t accumulate = 0u;
@@ -493,14 +576,15 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                     xw.step(1, stages);
                 }
                 steps_before += s_hi - s_lo;
-                if (elected) umma_commit(smem_u32(&S.acc_ready));
+                const uint32_t passed = __shfl_sync(0xFFFFFFFFu, smem_u32(&S.acc_ready[set]), 0);
+                if (elected) umma_commit(passed);
                 __syncwarp();
             }
         };
         if (warp == 1) issue_units(std::integral_constant<int, 0>{});
         else if (warp == 2 && n_acc > 1) issue_units(std::integral_constant<int, 1>{});
         else if (warp == 3 && n_acc > 2) issue_units(std::integral_constant<int, 2>{});
-    } else if (warp >= 4) {
+    } else if (NL == 1 || warp < kThreads / 32) {
         // ============================ expanders, then epilogue ============================
         const int grp = (warp - 4) >> 2, q = warp & 3;        // tensor-memory lanes this warp may touch: 32q .. 32q + 31
         const int gq = lane >> 2, tq = lane & 3;
@@ -540,7 +624,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                         for (int rh = 0; rh < 2; ++rh)
                             g_rows[k][pi][rh] = __half2half2(L.g[(size_t)k * L.Mp + ps.rt * kTileM + 32 * q + 16 * pi + gq + 8 * rh]);
             }
-            load_scales(ps);
+            if (NL == 1 || w.left <= 0) load_scales(ps);
             int first = ((grp - u0 % n_groups + n_groups) % n_groups) / n_ops;   // the group's first step of the pass, and (unless its stride does not divide them) of each weight stage
             for (int j = 0; j < weight_stages(ps) && grp < n_groups; ++j) {
                 const int step0 = ps.s_lo + j * kWSteps, n_here = min(kWSteps, ps.s_hi - step0), whole = min(n_here, n_ct / 2 - step0);   // steps with two column tiles
@@ -635,68 +719,18 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
             }
             u0 += (ps.s_hi - ps.s_lo) * n_ops;
             if (split > 1 && (!SEQ || ps.path == P.paths - 1)) break;   // the cluster's epilogue follows the role branches
+            if constexpr (NL > 1) {
+                // A pass that another one follows is published by warps of their own, while this one is expanded (its accumulators are not
+                // those of the next); the last one by these, which are four times as many.
+                if (w.left <= 0) publish(std::integral_constant<int, 4>{}, ps, pass_i, 4 * grp);
+                ++pass_i;
+                continue;
+            }
             // ---- epilogue of this pass
-            mbar_wait(smem_u32(&S.acc_ready), pass_i & 1, abort_flag);
+            mbar_wait(smem_u32(&S.acc_ready[0]), pass_i & 1, abort_flag);
             ++pass_i;
             fence_after();
             const int row = ps.rt * kTileM + q * 32 + lane;
-            if (NL > 1 || P.stream) {
-                // Up to 16 batch columns, four per group.  A segment that is a whole row tile is stored; otherwise every output goes
-                // into its 64-bit accumulate word with one integer atomic (as in rabit_gemv_f16.cu: fixed-point grid of the packer,
-                // a segment of s slices shifted by s * 2^fix_bits, arrivals in bits 55..62, bit 63 = non-finite), and the thread
-                // whose add completes a word rounds it to fp16, stores y and clears it.
-                float v[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                for (int m = 0; m < (n_ops == 1 ? 2 : n_ops); ++m) {
-                    if (n_ops == 1 && m >= n_acc) break;
-                    uint32_t d[4];
-                    tmem_ld4(lane_base + (uint32_t)(m * P.max16 * kGroupCols + 4 * grp), d);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    const float gm = DEQ ? 1.f : scale(n_ops == 1 ? 0 : m);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) v[i] = fmaf(gm, __uint_as_float(d[i]), v[i]);
-                }
-                fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&S.acc_empty));
-                const int n_here = P.batch - 4 * grp;            // batch columns of this group, if positive
-                const int n_slices = (ps.s_hi - ps.s_lo + kSliceSteps - 1) / kSliceSteps;
-                if (n_slices == L.n_cs) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        if (i < n_here && row < L.M) L.y[(size_t)(4 * grp + i) * L.M + row] = __float2half_rn(v[i]);
-                    continue;
-                }
-                unsigned long long* word = L.acc + (size_t)(4 * grp) * L.Mp + row;
-                unsigned long long old[4], add[4];
-                uint32_t bad = 0u;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float scaled = v[i] * L.inv_unit;
-                    if (!(fabsf(scaled) < L.limit * (float)n_slices)) bad |= 1u << i;             // inf or NaN: finite inputs cannot get here
-                    const long long qv = (bad >> i) & 1u ? 0LL : __float2ll_rn(scaled);
-                    add[i] = (unsigned long long)(qv + ((long long)n_slices << L.fix_bits)) + (1ULL << 55);
-                }
-                // all atomics of the thread back to back: nothing between them that could wait for an answer
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    old[i] = 0ULL;
-                    if (i >= n_here || !RABIT_IN_RANGE(row >= 0 && row < L.Mp && 4 * grp + i < RABIT_LUT_MAX_BATCH)) continue;
-                    if ((bad >> i) & 1u) atomicOr(word + (size_t)i * L.Mp, 1ULL << 63);           // sticky: the add below never carries into bit 63
-                    old[i] = atomicAdd(word + (size_t)i * L.Mp, add[i]);
-                }
-                const int arrivals = segment_arrivals((uint32_t)((NL == 1 ? 0 : L.pair0) + ps.rt * L.n_cs), (uint32_t)L.n_cs, (uint32_t)P.n_tasks, (uint32_t)P.n_groups);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    if (i >= n_here || (int)((old[i] >> 55) & 0xFFu) != arrivals - 1) continue;   // other segments are still to come
-                    const unsigned long long sum = (old[i] & kSumMask) + (add[i] & kSumMask);
-                    const long long total = (long long)sum - ((long long)L.n_cs << L.fix_bits);
-                    const bool poisoned = ((bad >> i) & 1u) || (old[i] >> 63) != 0;
-                    if (row < L.M) L.y[(size_t)(4 * grp + i) * L.M + row] = poisoned ? __ushort_as_half((unsigned short)0x7FFF) : __float2half_rn(__ll2float_rn(total) * L.unit);
-                    word[(size_t)i * L.Mp] = 0ULL;               // resting state for the next call
-                }
-                continue;
-            }
             if constexpr (SEQ) {
                 if (ps.path < P.paths - 1) {
                     // a path that is not the last: its scaled result joins the sum beside the accumulator
@@ -715,7 +749,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                     fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&S.acc_empty));
+                    if (lane == 0) mbar_arrive(smem_u32(&S.acc_empty[0]));
                     continue;
                 }
             }
@@ -747,7 +781,17 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
             }
             fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&S.acc_empty));
+            if (lane == 0) mbar_arrive(smem_u32(&S.acc_empty[0]));
+        }
+    } else {
+        // ============================ epilogues of a stream task's passes, but for the last ============================
+        int pass_i = 0;
+        PassWalker<NL, SEQ> w = first_pass;
+        Pass ps;
+        while (w.next(P, ps) && w.left > 0) {
+            load_scales(ps);
+            publish(std::integral_constant<int, kGroupCols>{}, ps, pass_i, 0);
+            ++pass_i;
         }
     }
 
@@ -760,7 +804,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
         Pass ps;
         w.next(P, ps);
         if (warp >= 4) {
-            mbar_wait(smem_u32(&S.acc_ready), SEQ ? (P.paths - 1) & 1 : 0, abort_flag);
+            mbar_wait(smem_u32(&S.acc_ready[0]), SEQ ? (P.paths - 1) & 1 : 0, abort_flag);
             fence_after();
         }
         __syncwarp();
@@ -896,7 +940,7 @@ bool fill_resources(Plan& p, int K, int n_ops, int steps, bool one_box) {
     const int recv_bytes = p.split > 1 ? (p.chunk16 + p.split - 1) / p.split * p.split * kGroupCols * kTileM * 4 : 0;
     if (p.max16 * kGroupCols > 256) return false;
     const int turn = n_ops == 3 || p.seq ? 3 : 4;
-    auto free_units = [&](int n_acc) { return (512 - (n_acc + p.seq) * p.max16 * kGroupCols) / kUnitCols; };
+    auto free_units = [&](int n_acc) { return (512 - ((p.stream ? 2 : 1) * n_acc + p.seq) * p.max16 * kGroupCols) / kUnitCols; };   // (a stream: two sets of accumulators)
     // (one path: a second accumulator needs a step for each in every pass; a stream's shortest one is the last slice)
     p.n_acc = p.seq ? 1 : n_ops > 1 ? n_ops : (p.stream ? steps % kSliceSteps != 1 : steps >= 2) && free_units(2) >= turn ? 2 : 1;
     if (free_units(p.n_acc) < turn) return false;
@@ -934,21 +978,23 @@ double unit_clocks(int n16, const Plan& p, int n_ops) {
     return std::max(32.0 * n16 + 52.0, p.units >= 2 * (n_ops == 3 ? 3 : 4) ? 180.0 + 8.0 * n16 : n_ops == 3 ? 345.0 : 300.0);
 }
 
-// (group: the form for several layers)
-const void* kernel_for(int K, bool deq, bool group = false, bool seq = false) {
-    if (seq) return (const void*)rabit_gemm_tc_kernel<1, false, 1, true>;
-    if (group) return K == 1 ? (const void*)rabit_gemm_tc_kernel<1, false, kMaxGroup, false> : K == 2 ? (const void*)rabit_gemm_tc_kernel<2, false, kMaxGroup, false> : (const void*)rabit_gemm_tc_kernel<3, false, kMaxGroup, false>;
-    if (K == 1) return deq ? (const void*)rabit_gemm_tc_kernel<1, true, 1, false> : (const void*)rabit_gemm_tc_kernel<1, false, 1, false>;
-    if (K == 2) return deq ? (const void*)rabit_gemm_tc_kernel<2, true, 1, false> : (const void*)rabit_gemm_tc_kernel<2, false, 1, false>;
-    return deq ? (const void*)rabit_gemm_tc_kernel<3, true, 1, false> : (const void*)rabit_gemm_tc_kernel<3, false, 1, false>;
+// (stream: the form for contiguous ranges of up to kMaxGroup layers)
+template <int NL>
+const void* kernel_of(int K, bool deq) {
+    if (K == 1) return deq ? (const void*)rabit_gemm_tc_kernel<1, true, NL, false> : (const void*)rabit_gemm_tc_kernel<1, false, NL, false>;
+    if (K == 2) return deq ? (const void*)rabit_gemm_tc_kernel<2, true, NL, false> : (const void*)rabit_gemm_tc_kernel<2, false, NL, false>;
+    return deq ? (const void*)rabit_gemm_tc_kernel<3, true, NL, false> : (const void*)rabit_gemm_tc_kernel<3, false, NL, false>;
+}
+const void* kernel_for(int K, bool deq, bool stream = false, bool seq = false) {
+    return seq ? (const void*)rabit_gemm_tc_kernel<1, false, 1, true> : stream ? kernel_of<kMaxGroup>(K, deq) : kernel_of<1>(K, deq);
 }
 
 // Function attributes are per device.
-cudaError_t prepare_kernel(int K, bool deq, int device, bool group = false, bool seq = false) {
-    static bool done[64][10] = {};
-    const int slot = device >= 0 && device < 64 ? device : 0, inst = seq ? 9 : 3 * (K - 1) + (group ? 2 : deq ? 1 : 0);
+cudaError_t prepare_kernel(int K, bool deq, int device, bool stream = false, bool seq = false) {
+    static bool done[64][13] = {};
+    const int slot = device >= 0 && device < 64 ? device : 0, inst = seq ? 12 : 4 * (K - 1) + (stream ? 2 : 0) + (deq ? 1 : 0);
     if (done[slot][inst] && slot == device) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(kernel_for(K, deq, group, seq), cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(kernel_for(K, deq, stream, seq), cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
     if (e == cudaSuccess) done[slot][inst] = true;
     return e;
 }
@@ -974,7 +1020,11 @@ int resident_clusters(const void* kernel, int split, size_t smem, int sms) {
 constexpr double kPassClocks = 3000.0;               // pipeline fill and epilogue of a pass that nothing overlaps
 constexpr double kLaunchClocks = 8000.0;             // launch, first loads, last epilogue
 constexpr double kExchangeClocks = 2500.0;           // exchange of a split task
-constexpr double kPublishClocks = 1500.0;            // atomics of a part of a row tile, besides their throughput
+// Streams, fitted to 25 shapes x every task count (B200, 9 to 16 rows; 4 % rms, the split it picks 0.3 % slower than the best on average):
+// launch, unit of one, two or three paths, a further pass in a range, publishing parts of row tiles besides its throughput and that (sums per clock
+// over the GPU).  Before the epilogues had warps of their own a further pass cost 3000 and ranges that cross row tiles were avoided: 11008 x 4096
+// at 16 rows 14.7 -> 13.5 us, 14336 x 4096 with three paths 20.3 -> 18.9.
+constexpr double kStreamLaunch = 5600.0, kStreamUnit[3] = {208.0, 170.0, 166.0}, kStreamPass = 1300.0, kStreamPublish = 800.0, kStreamRate = 130.0;
 
 // Task counts worth an estimate: equal parts of every row tile (or nearly), and one task per SM.  Never more tasks than pairs: an
 // empty one would count among the arrivals of a row tile that it does not contribute to.  (Layers of unlike widths: parts for the
@@ -1006,7 +1056,7 @@ Plan stream_plan(int n_layers, const int* n_rt, const int* n_ct, int K, bool deq
     }
     if (most_cs > RABIT_LUT_MAX_SLICES || pairs >= kMaxPairs || sms > kMaxTasks || !fill_resources(p, K, n_ops, tail, wide_x)) return best;
     best.clocks = 1e300;
-    const double pair = kSliceSteps * n_ops * unit_clocks(1, p, n_ops);
+    const double pair = kSliceSteps * n_ops * kStreamUnit[n_ops - 1];
     int considered = 0;
     stream_task_counts(row_tiles, pairs, most_cs, sms, [&](long long tasks) {
         if (candidate >= 0 && considered++ != candidate) return;
@@ -1018,13 +1068,13 @@ Plan stream_plan(int n_layers, const int* n_rt, const int* n_ct, int K, bool deq
         for (long long at = 0; at < pairs;) {             // segment by segment
             const int n_cs = ((n_ct[l] + 1) / 2 + kSliceSteps - 1) / kSliceSteps;
             const long long t_end = pairs * (t + 1) / tasks, tile_end = at + n_cs - (at - base) % n_cs, end = std::min(t_end, tile_end);
-            c += (double)(end - at) * pair + (c > 0.0 ? kPassClocks : 0.0);
+            c += (double)(end - at) * pair + (c > 0.0 ? kStreamPass : 0.0);
             parts += end - at < n_cs;
             at = end;
             if (at == base + (long long)n_rt[l] * n_cs && l + 1 < n_layers) { base = at; ++l; }
             if (at == t_end) { worst = std::max(worst, c); c = 0.0; ++t; }
         }
-        p.clocks = kLaunchClocks + worst + (parts > 0 ? kPublishClocks + parts * 128.0 * batch / 80.0 : 0.0);
+        p.clocks = kStreamLaunch + worst + (parts > 0 ? kStreamPublish + parts * 128.0 * batch / kStreamRate : 0.0);
         if (p.clocks < best.clocks) best = p;
     });
     return best;
@@ -1144,14 +1194,13 @@ void fill_common(GemmParams<NL>& P, const Plan& p, int n_layers, int batch, long
     P.chunks = p.chunks; P.chunk16 = p.chunk16;
     P.n_groups = (int)std::min<long long>(0x7FFFFFFF, n_groups);          // (only read where it fits)
     P.quot = P.n_groups / P.n_tasks; P.rem = P.n_groups % P.n_tasks;
-    P.stream = p.stream;
     P.max16 = p.max16;
     P.split = p.split;
     P.recv_off = p.recv_off;
     P.stages = p.stages; P.stage_bytes = p.stage_bytes; P.x_steps = p.x_steps; P.w_stages = p.w_stages;
     P.box16 = p.box16;
     P.n_acc = p.n_acc;
-    P.units = p.units; P.a_col = (p.n_acc + p.seq) * p.max16 * kGroupCols;
+    P.units = p.units; P.a_col = ((p.stream ? 2 : 1) * p.n_acc + p.seq) * p.max16 * kGroupCols;
 #ifdef RABIT_CHECKED
     P.withhold = withhold;
 #endif
@@ -1209,7 +1258,7 @@ int rabit_gemm_tc_plan(int n_layers, const int (*shape)[2], int K, bool deq, int
     if (p.tasks < 1) return -1;
     const int h[8] = {p.tasks, p.split, p.stream, p.seq, p.max16, p.chunks, p.stages, p.n_acc};
     std::copy(h, h + 8, head);
-    if (n_layers > 1) {
+    if (p.stream) {
         GemmParams<kMaxGroup> P = {};
         return list_passes<kMaxGroup, false>(P, p, n_layers, shape, K, batch, out, max_passes);
     }
@@ -1233,12 +1282,9 @@ bool rabit_gemm_tc_group_supports(const rabit_layer* const* layers, int n_layers
     return pairs < kMaxPairs && sms_of(*layers[0]) <= kMaxTasks;
 }
 
-cudaError_t rabit_launch_gemm_tc_group(const rabit_layer* const* layers, int n_layers, const void* const* xs, void* const* ys, int batch, cudaStream_t stream) {
-    if (n_layers == 1) return rabit_launch_gemm_tc(*layers[0], xs[0], ys[0], batch, stream);
-    if (!rabit_gemm_tc_group_supports(layers, n_layers, batch)) return cudaErrorInvalidValue;
+// A stream launch: the plan's contiguous ranges over the layers.
+static cudaError_t launch_stream(const rabit_layer* const* layers, int n_layers, const void* const* xs, void* const* ys, int batch, bool dequantised, const Plan& p, cudaStream_t stream) {
     const int K = layers[0]->geom.K, device = layers[0]->device;
-    const Plan p = plan_for(layers, n_layers, false, batch);
-    if (p.tasks < 1) return cudaErrorInvalidValue;
     GemmParams<kMaxGroup> P;
     P.paths = K;
     XMaps<kMaxGroup> maps;
@@ -1252,11 +1298,11 @@ cudaError_t rabit_launch_gemm_tc_group(const rabit_layer* const* layers, int n_l
         pairs += G.n_rt * G.n_cs;
     }
     fill_common(P, p, n_layers, batch, pairs, layers[0]->withhold);
-    cudaError_t e = prepare_kernel(K, false, device, true);
+    cudaError_t e = prepare_kernel(K, dequantised, device, true);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned int)p.tasks);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(kStreamThreads);
     cfg.dynamicSmemBytes = p.smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -1265,7 +1311,15 @@ cudaError_t rabit_launch_gemm_tc_group(const rabit_layer* const* layers, int n_l
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     void* args[2] = {&P, &maps};
-    return cudaLaunchKernelExC(&cfg, kernel_for(K, false, true), args);
+    return cudaLaunchKernelExC(&cfg, kernel_for(K, dequantised, true), args);
+}
+
+cudaError_t rabit_launch_gemm_tc_group(const rabit_layer* const* layers, int n_layers, const void* const* xs, void* const* ys, int batch, cudaStream_t stream) {
+    if (n_layers == 1) return rabit_launch_gemm_tc(*layers[0], xs[0], ys[0], batch, stream);
+    if (!rabit_gemm_tc_group_supports(layers, n_layers, batch)) return cudaErrorInvalidValue;
+    const Plan p = plan_for(layers, n_layers, false, batch);
+    if (p.tasks < 1) return cudaErrorInvalidValue;
+    return launch_stream(layers, n_layers, xs, ys, batch, false, p, stream);
 }
 
 bool rabit_gemm_tc_supports(const rabit_layer& L, int batch) {
@@ -1279,6 +1333,10 @@ cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, i
     const RabitGeom& G = L.geom;
     const Plan p = plan_for(L, dequantised, batch);
     if (p.tasks < 1) return cudaErrorInvalidValue;
+    if (p.stream) {
+        const rabit_layer* one = &L;
+        return launch_stream(&one, 1, &x, &y, batch, dequantised, p, stream);
+    }
     XMaps<1> maps;
     cudaError_t e = x_tensor_map(x, G.N, batch, p.box16, p.x_steps, &maps.map[0]);
     if (e != cudaSuccess) return e;
@@ -1288,7 +1346,7 @@ cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, i
     GemmParams<1> P;
     P.paths = G.K;
     fill_layer(P.L[0], L, y, 0);
-    fill_common(P, p, 1, batch, (long long)G.n_rt * (p.stream ? G.n_cs : (batch + kGroupCols - 1) / kGroupCols), L.withhold);
+    fill_common(P, p, 1, batch, (long long)G.n_rt * ((batch + kGroupCols - 1) / kGroupCols), L.withhold);
 
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned int)(p.tasks * p.split));
