@@ -51,6 +51,18 @@ def test_derived_planes_bit_exact_and_layer_parity(K, M, N):
     layer.free()
 
 
+@pytest.mark.parametrize("K,M,N", [(1, 3000, 3488), (2, 5000, 2080), (3, 2600, 8224)])
+def test_derivation_with_several_blocks_per_cta(K, M, N):
+    """More blocks of 128 rows x 256 columns than CTAs at work, the last ones of a row tile and of a column of tiles ragged: the image is
+    the host packer's of the oracle's planes, byte for byte."""
+    import torch
+    import paper_2602_05367_b200 as rabit
+    W, g, h = _inputs(K, M, N, seed=K * 1000 + M + N)
+    layer = rabit.rabit_derive_pack(torch.from_numpy(W).cuda(), g, h)
+    assert np.array_equal(layer.dev_buf.cpu().numpy(), rabit.pack_host(orc.derive_planes(W, g, h, dtype=np.float32), g, h))
+    layer.free()
+
+
 def test_derive_then_run_on_one_stream_without_a_sync():
     """The decode kernel starts reading weights before its dependency wait; a layer derived on the same stream just
     before must still be seen complete (the library orders the two with a fill after the derivation kernels)."""

@@ -140,3 +140,15 @@ def test_gemm_split_contraction_across_a_cluster(K, M, N, batch, variant):
         check_against_oracle(L, x, y, tight=variant != DEQ, rows=rows)
     y2 = run_layer(L, x, variant)
     assert np.array_equal(y.view(np.uint16), y2.view(np.uint16))
+
+
+@pytest.mark.parametrize("K,M,N,batch", [
+    (1, 77000, 64, 9),       # four or five row tiles in every CTA's range, one step each
+    (2, 38000, 544, 13),     # six (row tile, slice) pairs a CTA: parts of row tiles at both ends, a whole one between, last step half
+    (3, 25700, 288, 16),
+])
+def test_several_row_tiles_in_a_range(K, M, N, batch):
+    """Up to 16 rows: passes alternate between two sets of accumulators, and all but a CTA's last are published beside the next."""
+    L = make_layer(M, N, K, key=(65, K, M, N))
+    x = make_x(batch, N, key=(65, M, N, batch))
+    check_against_oracle(L, x, run_layer(L, x, GEMM))
