@@ -10,10 +10,14 @@
 // fp32 add per EIGHT weights.  The input scale h_k is applied once per table (t = h * x), the signed
 // accumulation is the sum of table entries in fp32 registers, and every weight bit is read once.
 // Measured on B200, clocks per 2 KB block and SM on a layer of 114688 x 8192: the look-ups alone 67 (64 conflict-free wavefronts of
-// the shared-memory pipe; 8.9 TB/s over 148 SMs, above what HBM delivers), the whole loop 118 with one batch row (5.1 TB/s)
-// and 187 with two (look-ups alone 146).  One row: without the loads of the next blocks 99, without the atomics 115.5,
+// the shared-memory pipe; 8.9 TB/s over 148 SMs, above what HBM delivers), the whole loop 118 with one batch row (5.1 TB/s).
+// One row: without the loads of the next blocks 99, without the atomics 115.5,
 // without the look-ups 106: the loop waits for its weights, of which at most one block per warp (32 KB per SM) is under way.
-// Two rows: without the atomics 163, without the loads no faster: there the look-ups bound it.  (28672 x 8192: 15.0 and 22.9 us.)
+// Two rows: a look-up reads both rows' sums (8 bytes, 128 wavefronts a block whichever way) and one add takes both: 12 instructions instead
+// of 20 per word and path, and the next block's weights are loaded beside the look-ups instead of behind them.  28672 x 8192
+// 22.8 -> 20.9 us, 22016 x 4096 10.65 -> 9.95, 12288 x 4096 7.55 -> 7.0, one path 22016 x 4096 9.2 -> 7.5.  (The 8-byte look-ups without the
+// earlier loads: one path 8.2, two paths 28672 x 8192 24.1: warps then wait for weights.  The packed add for one row: two paths 3 % slower.)
+// One row: 28672 x 8192 15.0 us.
 //
 // Work split.  The layer is a grid of blocks (32 rows x 256 columns x K paths, K KB each) stored
 // slice-major; CTA c owns a contiguous range of block positions (cut on the host so that all CTAs cost
@@ -61,15 +65,15 @@ constexpr unsigned long long kSumMask = (1ULL << 55) - 1;
 // plus a constant that fits the load's immediate.  (Starting the tables on a 64 KB boundary instead costs 63 KB of slack and
 // sixteen registers for the table base.)
 constexpr int kSmemBase = 1024;
+// Two batch rows: entry e of (path k, byte group) is the pair of both rows' sums at  e * 256 + group * 8  of table k.
 template <int K, int NB>
 struct Tab {
-    static constexpr int kTables = (K + 1) / 2;                       // per batch row
-    static constexpr int kBytes = kTables * 65536;                    // per batch row
+    static constexpr int kBytes = (NB == 1 ? (K + 1) / 2 : K) * 65536;
     static constexpr int kTail = 256;                                 // behind the tables: the layer's descriptor and the CTA's range
     // Never so little that two CTAs share an SM: with 64 KB each the hardware put two CTAs of one launch on one SM wherever the
     // previous launch left room first, and a 4096 x 4096 layer went from 3.2 to 4.4 us.
-    static constexpr int kSmem = NB * kBytes + kTail > 116 * 1024 ? NB * kBytes + kTail : 116 * 1024;
-    __host__ __device__ static constexpr int offset(int k, int b) { return kSmemBase + b * kBytes + (k >> 1) * 65536 + (k & 1) * 128; }
+    static constexpr int kSmem = kBytes + kTail > 116 * 1024 ? kBytes + kTail : 116 * 1024;
+    __host__ __device__ static constexpr int offset(int k) { return kSmemBase + (NB == 1 ? (k >> 1) * 65536 + (k & 1) * 128 : k * 65536); }
 };
 
 template <int I, int N, typename F>
@@ -117,8 +121,24 @@ __device__ __forceinline__ float lds_f32(uint32_t addr) {
     asm volatile("ld.shared.f32 %0, [%1+%2];" : "=f"(v) : "r"(addr), "n"(OFF));
     return v;
 }
+// Pairs of fp32 numbers: one look-up and one add for both batch rows.
+template <int OFF>
+__device__ __forceinline__ unsigned long long lds_pair(uint32_t addr) {
+    unsigned long long v;
+    asm volatile("ld.shared.b64 %0, [%1+%2];" : "=l"(v) : "r"(addr), "n"(OFF));
+    return v;
+}
+__device__ __forceinline__ void add_pair(unsigned long long& sum, unsigned long long v) {
+    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(sum) : "l"(v));
+}
+__device__ __forceinline__ float2 pair_of(unsigned long long v) {
+    return make_float2(__uint_as_float((uint32_t)v), __uint_as_float((uint32_t)(v >> 32)));
+}
 __device__ __forceinline__ void sts_f32(uint32_t addr, float v) {
     asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ void sts_pair(uint32_t addr, float v0, float v1) {
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v0), "f"(v1) : "memory");
 }
 // Weights are read exactly once: no L1 allocation, 128-byte L2 sectors.
 __device__ __forceinline__ uint4 ldg_stream(const uint4* p) {
@@ -227,8 +247,8 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
     // The launch parameters live in constant memory, which is cold in every new launch: a first touch of one of its
     // lines costs a trip to L2.  Everything the CTA needs later is therefore copied to shared memory now, before the
     // dependency wait, so that none of those trips lands between the arrival of x and the end of the kernel.
-    LutLayer& layer_copy = *reinterpret_cast<LutLayer*>(smem + NB * T::kBytes);
-    CtaRange& range_copy = *reinterpret_cast<CtaRange*>(smem + NB * T::kBytes + 128);
+    LutLayer& layer_copy = *reinterpret_cast<LutLayer*>(smem + T::kBytes);
+    CtaRange& range_copy = *reinterpret_cast<CtaRange*>(smem + T::kBytes + 128);
     if (warp == 0) {
         const CtaRange r0 = P.range[blockIdx.x];
         const uint32_t* src = reinterpret_cast<const uint32_t*>(&P.layer[r0.layer]);
@@ -253,9 +273,12 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
     }
 
     const uint32_t tab0 = smem_u32(smem);                // == kSmemBase
-    // byte q of `bank0 + 0x10101010 * j`, modulo 128: bank offset (4 * group) of the group this lane visits in step 4j + q.  A
+    // One row: byte q of `bank0 + 0x10101010 * j`, modulo 128: bank offset (4 * group) of the group this lane visits in step 4j + q.  A
     // permute of (weight word, that) yields byte << 8 | bank offset (its upper bytes copy a sign bit that is always clear).
-    const uint32_t bank0 = (uint32_t)((lane * 4) & 127) | (uint32_t)((lane * 4 + 4) & 127) << 8 | (uint32_t)((lane * 4 + 8) & 127) << 16 | (uint32_t)((lane * 4 + 12) & 127) << 24;
+    // Two rows: offsets (8 * group) take all eight bits, so the ones of steps 4j, 4j + 1 and of 4j + 2, 4j + 3 sit a halfword each, modulo 256,
+    // and the permute's upper bytes are the clear byte between them.
+    const uint32_t lane4 = (uint32_t)lane * 4u;
+    const uint32_t bank0 = NB == 1 ? (lane4 & 127) | ((lane4 + 4) & 127) << 8 | ((lane4 + 8) & 127) << 16 | ((lane4 + 12) & 127) << 24 : ((2 * lane4) & 255) | ((2 * lane4 + 8) & 255) << 16;
     int cs = R.b0 / L.n_rb;
     int seg_rb0 = R.b0 - cs * L.n_rb;                    // row block of the first block of the current segment
     int seg_begin = 0, seg_end = min(n_blocks, L.n_rb - seg_rb0);       // blocks [seg_begin, seg_end) of the range use slice cs
@@ -281,14 +304,15 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
     // table of the slice whose h and x sit in hq / xq:  entry e of (path k, group) = sum_{bit<8} (e has bit ? -t : +t),  t = h * x
     auto build_table = [&]() {
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            const uint32_t xw[4] = {xq[b].x, xq[b].y, xq[b].z, xq[b].w};
+        for (int u = 0; u < kPairs; ++u) {
+            const int pi = warp + u * kWarps;
+            if (pi >= 8 * K) break;
+            const int k = pi >> 3, ehi = pi & 7;
+            const uint32_t hw[4] = {hq[u].x, hq[u].y, hq[u].z, hq[u].w};
+            float v[NB][32];
 #pragma unroll
-            for (int u = 0; u < kPairs; ++u) {
-                const int pi = warp + u * kWarps;
-                if (pi >= 8 * K) break;
-                const int k = pi >> 3, ehi = pi & 7;
-                const uint32_t hw[4] = {hq[u].x, hq[u].y, hq[u].z, hq[u].w};
+            for (int b = 0; b < NB; ++b) {
+                const uint32_t xw[4] = {xq[b].x, xq[b].y, xq[b].z, xq[b].w};
                 float t[8];
 #pragma unroll
                 for (int w = 0; w < 4; ++w) {
@@ -297,21 +321,24 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
                     t[2 * w] = hf.x * xf.x;                              // exact: two 11-bit significands
                     t[2 * w + 1] = hf.y * xf.y;
                 }
-                float v[32];
-                v[0] = (ehi & 1 ? -t[5] : t[5]) + (ehi & 2 ? -t[6] : t[6]) + (ehi & 4 ? -t[7] : t[7])
-                     + (((t[0] + t[1]) + (t[2] + t[3])) + t[4]);
+                v[b][0] = (ehi & 1 ? -t[5] : t[5]) + (ehi & 2 ? -t[6] : t[6]) + (ehi & 4 ? -t[7] : t[7])
+                        + (((t[0] + t[1]) + (t[2] + t[3])) + t[4]);
 #pragma unroll
                 for (int bit = 0; bit < 5; ++bit) {
                     const float m2 = -2.f * t[bit];
 #pragma unroll
-                    for (int e = 0; e < (1 << bit); ++e) v[e | (1 << bit)] = v[e] + m2;
+                    for (int e = 0; e < (1 << bit); ++e) v[b][e | (1 << bit)] = v[b][e] + m2;
                 }
-                const uint32_t dst = tab0 + b * T::kBytes + (k >> 1) * 65536 + (ehi * 32) * 256 + (k & 1) * 128 + lane * 4;
-#pragma unroll
-                for (int e = 0; e < 32; ++e)
-                    if (RABIT_IN_RANGE(dst + e * 256 >= tab0 && dst + e * 256 + 4 <= tab0 + (uint32_t)(NB * T::kBytes)))
-                        sts_f32(dst + e * 256, v[e]);
             }
+            // (the start of the tables as a register or as a constant: either way round the other form loses, by allocation of registers, 28672 x 8192
+            // 14.9 -> 15.3 us with one row, 20.9 -> 23.6 with two)
+            const uint32_t dst = (NB == 1 ? tab0 + (k >> 1) * 65536 + (k & 1) * 128 : (uint32_t)T::offset(k)) + (ehi * 32) * 256 + lane * (4 * NB);
+#pragma unroll
+            for (int e = 0; e < 32; ++e)
+                if (RABIT_IN_RANGE(dst + e * 256 >= tab0 && dst + e * 256 + 4 * NB <= tab0 + (uint32_t)T::kBytes)) {
+                    if constexpr (NB == 1) sts_f32(dst + e * 256, v[0][e]);
+                    else sts_pair(dst + e * 256, v[0][e], v[1][e]);
+                }
         }
     };
     // makes the table of block bb's slice the current one; every warp crosses every slice border of the range here
@@ -390,43 +417,55 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
         }
 #endif
 
-        float acc[NB][K][2];
+        // sums of the even and the odd byte groups, two rows' as pairs
+        std::conditional_t<NB == 1, float, unsigned long long> acc[K][2];
 #pragma unroll
-        for (int b = 0; b < NB; ++b)
-#pragma unroll
-            for (int k = 0; k < K; ++k) acc[b][k][0] = acc[b][k][1] = 0.f;
-        // (the next block's weights are loaded into the registers that the look-ups have used up, all together behind the last of
-        // them: the other warps' look-ups cover the wait.  Half by half, each as soon as its registers are free, is no faster with one batch
-        // row and slower with two: 28672 x 8192 23.9 against 22.9 us)
+        for (int k = 0; k < K; ++k) acc[k][0] = acc[k][1] = 0;
+        // The next block's weights.  One row: into the registers that the look-ups have used up, all together behind the last of them: the
+        // other warps' look-ups cover the wait (into registers of their own behind the first step 28672 x 8192 15.0 -> 16.8 us).  Two rows, whose
+        // look-ups take longer than the wait: into registers of their own behind the first of the eight steps (28672 x 8192 20.9 us; behind the
+        // second 21.9, the fourth 24.5, the last 24.1; above this block's scales and atomics 21.4).
+        [[maybe_unused]] Blk<NB == 1 ? 1 : K> ahead;
+        if constexpr (NB > 1) ahead = cur;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            const uint32_t bank = (bank0 + 0x10101010u * (uint32_t)j) & 0x7F7F7F7Fu;
+            const uint32_t bank = NB == 1 ? (bank0 + 0x10101010u * (uint32_t)j) & 0x7F7F7F7Fu : (bank0 + 0x00200020u * (uint32_t)j) & 0x00F800F8u;
+            const uint32_t bank2 = (bank0 + 0x00200020u * (uint32_t)j + 0x00100010u) & 0x00F800F8u;
             static_for<0, K>([&](auto kc) {
                 constexpr int k = decltype(kc)::value;
                 const uint4 part = cur.v[2 * k + (j >> 2)];
                 const uint32_t w = (j & 3) == 0 ? part.x : (j & 3) == 1 ? part.y : (j & 3) == 2 ? part.z : part.w;
                 // sign byte << 8 | bank offset, from one permute
-                const uint32_t a0 = prmt(w, bank, 0xCC04), a1 = prmt(w, bank, 0xCC15);
-                const uint32_t a2 = prmt(w, bank, 0xCC26), a3 = prmt(w, bank, 0xCC37);
+                const uint32_t a0 = prmt(w, bank, NB == 1 ? 0xCC04 : 0x5504), a1 = prmt(w, bank, NB == 1 ? 0xCC15 : 0x5516);
+                const uint32_t a2 = prmt(w, NB == 1 ? bank : bank2, NB == 1 ? 0xCC26 : 0x5524), a3 = prmt(w, NB == 1 ? bank : bank2, NB == 1 ? 0xCC37 : 0x5536);
 #ifdef RABIT_CHECKED
                 {
-                    const uint32_t hi = 65536u - 128u;                   // with the path offset added: inside table k >> 1
+                    const uint32_t hi = NB == 1 ? 65536u - 128u : 65536u;   // with the path offset added: inside its table
                     if (!RABIT_IN_RANGE(a0 < hi && a1 < hi && a2 < hi && a3 < hi)) return;
                 }
 #endif
-                static_for<0, NB>([&](auto bc) {
-                    constexpr int b = decltype(bc)::value;
-                    acc[b][k][0] += lds_f32<T::offset(k, b)>(a0);
-                    acc[b][k][1] += lds_f32<T::offset(k, b)>(a1);
-                    acc[b][k][0] += lds_f32<T::offset(k, b)>(a2);
-                    acc[b][k][1] += lds_f32<T::offset(k, b)>(a3);
-                });
+                if constexpr (NB == 1) {
+                    acc[k][0] += lds_f32<T::offset(k)>(a0);
+                    acc[k][1] += lds_f32<T::offset(k)>(a1);
+                    acc[k][0] += lds_f32<T::offset(k)>(a2);
+                    acc[k][1] += lds_f32<T::offset(k)>(a3);
+                } else {
+                    const unsigned long long v0 = lds_pair<T::offset(k)>(a0), v1 = lds_pair<T::offset(k)>(a1), v2 = lds_pair<T::offset(k)>(a2), v3 = lds_pair<T::offset(k)>(a3);
+                    add_pair(acc[k][0], v0);
+                    add_pair(acc[k][1], v1);
+                    add_pair(acc[k][0], v2);
+                    add_pair(acc[k][1], v3);
+                }
             });
-            if (j == 7 && next_ok) { load_half<K>(cur, 0, range_base, bb_next, lane); load_half<K>(cur, 1, range_base, bb_next, lane); }
+            if (j == (NB == 1 ? 7 : 0) && next_ok) {
+                if constexpr (NB == 1) { load_half<K>(cur, 0, range_base, bb_next, lane); load_half<K>(cur, 1, range_base, bb_next, lane); }
+                else { load_half<K>(ahead, 0, range_base, bb_next, lane); load_half<K>(ahead, 1, range_base, bb_next, lane); }
+            }
         }
+        if constexpr (NB > 1) cur = ahead;
 #ifdef RABIT_TRACE
         if (i == 0) RABIT_STAMP(7);                                     // first block's look-ups issued
-        if (i < 11 && use_here_u64(__float_as_uint(acc[0][0][0] + acc[0][0][1] + acc[0][K - 1][0] + acc[0][K - 1][1])) != 0x13572468u) RABIT_STAMP(10 + 5 * i);   // look-ups answered
+        if (i < 11 && use_here_u64((unsigned long long)(acc[0][0] + acc[0][1] + acc[K - 1][0] + acc[K - 1][1])) != 0x13572468u) RABIT_STAMP(10 + 5 * i);   // look-ups answered
 #endif
 #pragma unroll
         for (int b = 0; b < NB; ++b) pd[b].old = use_here_u64(pd[b].old);
@@ -443,7 +482,16 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
         for (int b = 0; b < NB; ++b) {
             float p = 0.f;
 #pragma unroll
-            for (int k = 0; k < K; ++k) p += __half2float(__ushort_as_half(graw[k])) * (acc[b][k][0] + acc[b][k][1]);
+            for (int k = 0; k < K; ++k) {
+                float sum;
+                if constexpr (NB == 1) {
+                    sum = acc[k][0] + acc[k][1];
+                } else {
+                    const float2 even = pair_of(acc[k][0]), odd = pair_of(acc[k][1]);
+                    sum = b == 0 ? even.x + odd.x : even.y + odd.y;
+                }
+                p += __half2float(__ushort_as_half(graw[k])) * sum;
+            }
             const float scaled = p * inv_unit;
             const bool bad = !(fabsf(scaled) < limit);                    // inf or NaN: finite inputs cannot get here
             const long long qv = bad ? 0LL : __float2ll_rn(scaled);
@@ -477,7 +525,7 @@ struct Cost {
 // for the cut.  (The block's figure is in clocks of an earlier loop: it takes 118 now.)
 // (the table figure is a fit: the split that minimises the measured step time charges a table about 26 blocks, far
 // more than its 430 cycles of stores, because a rebuild in mid-range also stops every warp at two barriers)
-// (two batch rows: a quarter less measured best, 22016 x 4096 11.5 -> 10.9 us, with one path 9.8 -> 9.3)
+// (two batch rows: a quarter less measures best; 22016 x 4096 10.2, 9.9, 9.85 us and 28672 x 8192 20.9, 20.9, 21.3 with 1900, 1700, 1500)
 Cost cost_of(int K, int nb) { return Cost{(long long)nb * (70 * K + 30), (long long)nb * ((nb == 1 ? 2200 : 1700) * K) + 100}; }
 
 // CTAs a layer of n_cs x n_rb blocks needs when no CTA may cost more than `limit`; writes the cuts if asked.

@@ -272,3 +272,15 @@ def test_tiny_and_huge_magnitudes_keep_their_precision():
         err, tol = check_against_oracle(L, xn, y.cpu().numpy())
         assert (err <= 0.3 * tol).all()          # far inside: only the fp16 output rounding is left
     layer.free()
+
+
+@pytest.mark.parametrize("K,M,N", [(1, 33, 32), (2, 33, 32), (1, 5000, 1184), (2, 200, 65280), (2, 12000, 544), (2, 4096, 4096)])
+def test_two_rows_are_one_row_twice(K, M, N):
+    """The two-row kernel looks both rows up at once, in the one-row kernel's order of additions: the outputs are the same bits.  (One block
+    and less than a slice; several blocks a warp; a block at most; the most slices.)"""
+    L = make_layer(M, N, K, key=(72, K, M, N))
+    x = make_x(2, N, key=(72, M, N))
+    both = run_layer(L, x, 5)
+    check_against_oracle(L, x, both)
+    for b in (0, 1):
+        assert np.array_equal(both[b].view(np.uint16), run_layer(L, x[b:b + 1], 5)[0].view(np.uint16))
