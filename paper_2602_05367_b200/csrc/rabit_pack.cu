@@ -54,6 +54,7 @@ bool rabit_make_geom(int K, int M, int N, RabitGeom* out) {
 //     65504 * max_i sum_k |g_k[i]| * max_{k, slice} sum_{j in slice} |h_k[j]|,
 // so a grid of 2^unit_exp whose 2^fix_bits steps cover twice that bound can never overflow, and with
 // fix_bits = 54 - ceil(log2(slices)) the sum of all slices (each shifted to be non-negative) stays below 2^55.
+
 // |value| of every fp16 magnitude (sign bit cleared), converted once: the scans below are table look-ups
 static const float* half_magnitude_table() {
     static const std::vector<float> table = [] {
@@ -63,33 +64,64 @@ static const float* half_magnitude_table() {
     }();
     return table.data();
 }
+static uint32_t top_magnitude(const uint16_t* v, size_t n) {
+    int16_t top = 0;
+    for (size_t i = 0; i < n; ++i) top = std::max<int16_t>(top, (int16_t)(v[i] & 0x7FFF));
+    return (uint32_t)top;
+}
 
 void rabit_scale_meta(const uint16_t* g, const uint16_t* h, int K, int M, int N, RabitGeom* G) {
+    // per path the largest |h| (fp16 magnitudes order like their bit patterns; the first NaN wins and sticks, so a NaN scale makes
+    // the bound NaN); the largest sum of |h| over a slice of 256 columns; the largest sum of |g| over the paths of a row
     const float* mag = half_magnitude_table();
-    // one pass over h: per path the largest |h| (fp16 magnitudes order like their bit patterns; the first NaN wins and
-    // sticks, so a NaN scale makes the bound NaN) and per slice of 256 columns the sum of |h|, added in column order
-    double hsum_max = 0.0;
+    double hsum_max = 0.0, gsum_max = 0.0;
+    uint32_t top[RABIT_MAX_K], most = top_magnitude(g, (size_t)K * M);
     for (int k = 0; k < K; ++k) {
-        const uint16_t* hk = h + (size_t)k * N;
-        uint32_t top = 0, first_nan = 0;
-        for (int j0 = 0; j0 < N; j0 += RABIT_LUT_COLS) {
-            const int j1 = j0 + RABIT_LUT_COLS < N ? j0 + RABIT_LUT_COLS : N;
-            double s = 0.0;
-            for (int j = j0; j < j1; ++j) {
-                const uint32_t m = hk[j] & 0x7FFFu;
-                if (m > 0x7C00u && first_nan == 0) first_nan = m;
-                top = m > top ? m : top;
-                s += (double)mag[m];
-            }
-            if (s > hsum_max || s != s) hsum_max = s;
-        }
-        G->hmax[k] = mag[first_nan ? first_nan : top];
+        top[k] = top_magnitude(h + (size_t)k * N, (size_t)N);
+        most = std::max(most, top[k]);
     }
-    double gsum_max = 0.0;
-    for (int i = 0; i < M; ++i) {
-        double s = 0.0;
-        for (int k = 0; k < K; ++k) s += (double)mag[g[(size_t)k * M + i] & 0x7FFFu];
-        if (s > gsum_max || s != s) gsum_max = s;
+    if (most < 0x7C00u) {
+        // All finite, the usual case.  Sums of 256 multiples of 2^-24 below 2^16 are exact in double in any order, so four run side by side.
+        for (int k = 0; k < K; ++k) {
+            const uint16_t* hk = h + (size_t)k * N;
+            G->hmax[k] = mag[top[k]];
+            for (int j0 = 0; j0 < N; j0 += RABIT_LUT_COLS) {
+                const int j1 = j0 + RABIT_LUT_COLS < N ? j0 + RABIT_LUT_COLS : N;
+                double s[4] = {};
+                for (int j = j0; j < j1; j += 4)              // (N is a multiple of 32)
+                    for (int u = 0; u < 4; ++u) s[u] += (double)mag[hk[j + u] & 0x7FFFu];
+                hsum_max = std::max(hsum_max, (s[0] + s[1]) + (s[2] + s[3]));
+            }
+        }
+        double m[4] = {};
+        for (int i = 0; i < M; i += 4)
+            for (int u = 0; u < 4 && i + u < M; ++u) {
+                double s = 0.0;
+                for (int k = 0; k < K; ++k) s += (double)mag[g[(size_t)k * M + i + u] & 0x7FFFu];
+                m[u] = std::max(m[u], s);
+            }
+        gsum_max = std::max(std::max(m[0], m[1]), std::max(m[2], m[3]));
+    } else {
+        for (int k = 0; k < K; ++k) {
+            const uint16_t* hk = h + (size_t)k * N;
+            uint32_t first_nan = 0;
+            for (int j0 = 0; j0 < N; j0 += RABIT_LUT_COLS) {
+                const int j1 = j0 + RABIT_LUT_COLS < N ? j0 + RABIT_LUT_COLS : N;
+                double s = 0.0;
+                for (int j = j0; j < j1; ++j) {
+                    const uint32_t v = hk[j] & 0x7FFFu;
+                    if (v > 0x7C00u && first_nan == 0) first_nan = v;
+                    s += (double)mag[v];
+                }
+                if (s > hsum_max || s != s) hsum_max = s;
+            }
+            G->hmax[k] = mag[first_nan ? first_nan : top[k]];
+        }
+        for (int i = 0; i < M; ++i) {
+            double s = 0.0;
+            for (int k = 0; k < K; ++k) s += (double)mag[g[(size_t)k * M + i] & 0x7FFFu];
+            if (s > gsum_max || s != s) gsum_max = s;
+        }
     }
     int clog = 0;
     while ((1 << clog) < G->n_cs) ++clog;
