@@ -165,10 +165,10 @@ static int linear_call(const rabit_layer* layer, const void* x, void* y, int bat
 
     int variant = layer->variant;
     if (variant == 0) {
-        if (rabit_gemv_lut_supports(*layer, batch)) {
+        if (rabit_gemv_lut_supports(*layer, batch) && rabit_gemv_lut_preferred(&layer, 1, batch)) {
             variant = 5;
         } else if (batch <= RABIT_MAX_GEMV_BATCH && rabit_gemv_f16_supports(*layer, kF16Rows)) {
-            variant = 6;                    // the f16 GEMV, beyond kF16Rows the GEMM (also two rows of three paths, whose tables do not fit)
+            variant = 6;                    // the f16 GEMV, beyond kF16Rows the GEMM (also two rows of small layers of three paths)
         } else if (batch <= RABIT_MAX_GEMV_BATCH) {
             variant = rabit_gemv_mma_supports(*layer, batch) ? 2 : 1;
             // Layers of more than 255 slices, or beyond the f16 GEMV's 32-bit offsets.  From 5 batch rows on the integer-MMA GEMV
@@ -262,9 +262,12 @@ static int group_call(const rabit_layer* const* layers, const void* const* xs, v
             return rabit_fail(RABIT_INVALID_ARG, "rabit_linear_group: the layers live on device %d but device %d is current", layers[0]->device, dev);
     }
     {
-        bool lut = rabit_gemv_lut_group_supports(layers, n_layers, batch);
-        for (int l = 0; l < n_layers && lut; ++l) lut = layers[l]->variant == 0 || layers[l]->variant == 5;
-        if (lut) {
+        bool lut = rabit_gemv_lut_group_supports(layers, n_layers, batch), forced = false;
+        for (int l = 0; l < n_layers && lut; ++l) {
+            lut = layers[l]->variant == 0 || layers[l]->variant == 5;
+            forced = forced || layers[l]->variant == 5;
+        }
+        if (lut && (forced || rabit_gemv_lut_preferred(layers, n_layers, batch))) {
             cudaError_t e = rabit_launch_gemv_lut_group(layers, n_layers, xs, ys, batch, st, nullptr, nullptr);
             if (e != cudaSuccess) return rabit_fail(RABIT_CUDA_ERROR, "rabit_linear_group: launch failed: %s", cudaGetErrorString(e));
             return RABIT_OK;
@@ -284,7 +287,7 @@ static int group_call(const rabit_layer* const* layers, const void* const* xs, v
             if (e != cudaSuccess) return rabit_fail(RABIT_CUDA_ERROR, "rabit_linear_group: launch failed: %s", cudaGetErrorString(e));
             return RABIT_OK;
         }
-        if (f16 && batch <= kF16Rows && !rabit_gemv_lut_supports(*layers[0], batch) && rabit_gemv_f16_group_supports(layers, n_layers, batch)) {
+        if (f16 && batch <= kF16Rows && !(rabit_gemv_lut_supports(*layers[0], batch) && rabit_gemv_lut_preferred(layers, n_layers, batch)) && rabit_gemv_f16_group_supports(layers, n_layers, batch)) {
             cudaError_t e = rabit_launch_gemv_f16_group(layers, n_layers, xs, ys, batch, st);
             if (e != cudaSuccess) return rabit_fail(RABIT_CUDA_ERROR, "rabit_linear_group: launch failed: %s", cudaGetErrorString(e));
             return RABIT_OK;

@@ -421,12 +421,13 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
         std::conditional_t<NB == 1, float, unsigned long long> acc[K][2];
 #pragma unroll
         for (int k = 0; k < K; ++k) acc[k][0] = acc[k][1] = 0;
+        constexpr bool kAhead = NB > 1 && K < 3;                        // (three paths: 24 registers that there are not, 22016 x 4096 16.1 instead of 15.2 us)
         // The next block's weights.  One row: into the registers that the look-ups have used up, all together behind the last of them: the
         // other warps' look-ups cover the wait (into registers of their own behind the first step 28672 x 8192 15.0 -> 16.8 us).  Two rows, whose
         // look-ups take longer than the wait: into registers of their own behind the first of the eight steps (28672 x 8192 20.9 us; behind the
         // second 21.9, the fourth 24.5, the last 24.1; above this block's scales and atomics 21.4).
-        [[maybe_unused]] Blk<NB == 1 ? 1 : K> ahead;
-        if constexpr (NB > 1) ahead = cur;
+        [[maybe_unused]] Blk<!kAhead ? 1 : K> ahead;
+        if constexpr (kAhead) ahead = cur;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const uint32_t bank = NB == 1 ? (bank0 + 0x10101010u * (uint32_t)j) & 0x7F7F7F7Fu : (bank0 + 0x00200020u * (uint32_t)j) & 0x00F800F8u;
@@ -457,12 +458,12 @@ rabit_gemv_lut_kernel(const __grid_constant__ LutParams P) {
                     add_pair(acc[k][1], v3);
                 }
             });
-            if (j == (NB == 1 ? 7 : 0) && next_ok) {
-                if constexpr (NB == 1) { load_half<K>(cur, 0, range_base, bb_next, lane); load_half<K>(cur, 1, range_base, bb_next, lane); }
+            if (j == (!kAhead ? 7 : 0) && next_ok) {
+                if constexpr (!kAhead) { load_half<K>(cur, 0, range_base, bb_next, lane); load_half<K>(cur, 1, range_base, bb_next, lane); }
                 else { load_half<K>(ahead, 0, range_base, bb_next, lane); load_half<K>(ahead, 1, range_base, bb_next, lane); }
             }
         }
-        if constexpr (NB > 1) cur = ahead;
+        if constexpr (kAhead) cur = ahead;
 #ifdef RABIT_TRACE
         if (i == 0) RABIT_STAMP(7);                                     // first block's look-ups issued
         if (i < 11 && use_here_u64((unsigned long long)(acc[0][0] + acc[0][1] + acc[K - 1][0] + acc[K - 1][1])) != 0x13572468u) RABIT_STAMP(10 + 5 * i);   // look-ups answered
@@ -590,7 +591,7 @@ cudaError_t launch_inst(const LutParams& P, int grid, int device, cudaStream_t s
 cudaError_t launch_k(int K, int batch, const LutParams& P, int grid, int device, cudaStream_t stream) {
     if (K == 1) return batch == 1 ? launch_inst<1, 1>(P, grid, device, stream) : launch_inst<1, 2>(P, grid, device, stream);
     if (K == 2) return batch == 1 ? launch_inst<2, 1>(P, grid, device, stream) : launch_inst<2, 2>(P, grid, device, stream);
-    return launch_inst<3, 1>(P, grid, device, stream);
+    return batch == 1 ? launch_inst<3, 1>(P, grid, device, stream) : launch_inst<3, 2>(P, grid, device, stream);
 }
 
 }  // namespace
@@ -610,9 +611,19 @@ static bool smem_base_ok(int device) {
 
 bool rabit_gemv_lut_supports(const rabit_layer& L, int batch) {
     if (batch < 1 || batch > 2 || !smem_base_ok(L.device)) return false;
-    if (L.geom.K == 3 && batch > 1) return false;                        // four 64 KB tables do not fit into shared memory
     if (L.geom.n_cs > RABIT_LUT_MAX_SLICES) return false;
     return (long long)L.geom.n_cs * L.geom.n_rb < (1LL << 30) && L.d_lut != nullptr && L.d_acc != nullptr;
+}
+
+// Whether it is the faster one for layers that it can run.  Against the f16 GEMV only two rows of three paths are ever not: its tables take
+// a table's build (three of 64 KB) per CTA and pay from about four blocks of 32 rows x 256 columns per SM on (B200, us, f16 GEMV against this:
+// 2000 x 1024 (256 blocks) 3.67 / 4.1, 2048 x 2048 (512) 4.1 / 4.2, 1024 x 4096 (512) 4.1 / 4.0, 11008 x 512 (688) 5.0 / 4.6, 2048 x 3072 (768)
+// 5.0 / 4.3, 4096 x 4096 7.4 / 5.7, 22016 x 4096 24.2 / 15.2, 28672 x 8192 54.0 / 31.8).
+bool rabit_gemv_lut_preferred(const rabit_layer* const* layers, int n_layers, int batch) {
+    if (layers[0]->geom.K < 3 || batch == 1) return true;
+    long long blocks = 0;
+    for (int l = 0; l < n_layers; ++l) blocks += (long long)layers[l]->geom.n_cs * layers[l]->geom.n_rb;
+    return blocks > 4LL * (layers[0]->sm_count > 0 ? layers[0]->sm_count : 148);
 }
 
 bool rabit_gemv_lut_group_supports(const rabit_layer* const* layers, int n_layers, int batch) {

@@ -96,6 +96,7 @@ int rabit_gemv_f16_plan(int K, int M, int N, int batch, int sms, int* bound_out,
 // table-driven GEMV (rabit_gemv_lut.cu); acc_override / status_override redirect the scratch (nullptr: the image's own)
 cudaError_t rabit_launch_gemv_lut(const rabit_layer& L, const void* x, void* y, int batch, cudaStream_t stream);
 bool rabit_gemv_lut_supports(const rabit_layer& L, int batch);
+bool rabit_gemv_lut_preferred(const rabit_layer* const* layers, int n_layers, int batch);
 int rabit_gemv_lut_max_rows();
 bool rabit_gemv_lut_group_supports(const rabit_layer* const* layers, int n_layers, int batch);
 cudaError_t rabit_launch_gemv_lut_group(const rabit_layer* const* layers, int n_layers, const void* const* xs, void* const* ys,

@@ -274,7 +274,8 @@ def test_tiny_and_huge_magnitudes_keep_their_precision():
     layer.free()
 
 
-@pytest.mark.parametrize("K,M,N", [(1, 33, 32), (2, 33, 32), (1, 5000, 1184), (2, 200, 65280), (2, 12000, 544), (2, 4096, 4096)])
+@pytest.mark.parametrize("K,M,N", [(1, 33, 32), (2, 33, 32), (1, 5000, 1184), (2, 200, 65280), (2, 12000, 544), (2, 4096, 4096),
+                                   (3, 33, 32), (3, 5000, 1184), (3, 200, 65280)])
 def test_two_rows_are_one_row_twice(K, M, N):
     """The two-row kernel looks both rows up at once, in the one-row kernel's order of additions: the outputs are the same bits.  (One block
     and less than a slice; several blocks a warp; a block at most; the most slices.)"""
@@ -284,3 +285,25 @@ def test_two_rows_are_one_row_twice(K, M, N):
     check_against_oracle(L, x, both)
     for b in (0, 1):
         assert np.array_equal(both[b].view(np.uint16), run_layer(L, x[b:b + 1], 5)[0].view(np.uint16))
+
+
+@pytest.mark.parametrize("M,variant", [(2304, 6), (2432, 5)])
+def test_two_rows_of_three_paths_either_side_of_the_line(M, variant):
+    """Two rows of three paths: tables from four blocks of 32 rows x 256 columns per SM on, the f16 GEMV below (148 SMs: 576 and 608 blocks),
+    alone and as a group whose blocks count together."""
+    import torch
+    import paper_2602_05367_b200 as rabit
+    L = make_layer(M, 2048, 3, key=(73, M))
+    x = make_x(2, 2048, key=(73, M))
+    y = run_layer(L, x, 0)
+    check_against_oracle(L, x, y)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert np.array_equal(y.view(np.uint16), run_layer(L, x, variant).view(np.uint16))
+    layers = [rabit.rabit_pack(L.planes, L.g, L.h) for _ in range(2)]
+    xd = torch.from_numpy(x).cuda()
+    ys = [torch.zeros((2, M), dtype=torch.float16, device="cuda") for _ in layers]
+    rabit.rabit_linear_group(layers, [xd, xd], ys)
+    for yg in ys:
+        assert np.array_equal(yg.cpu().numpy().view(np.uint16), run_layer(L, x, 5).view(np.uint16))
+    for layer in layers:
+        layer.free()
