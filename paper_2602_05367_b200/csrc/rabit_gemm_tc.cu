@@ -20,7 +20,7 @@
 //          dependency wait.  (Few, large copies: with one per step and path, and x in boxes of 16 rows, this warp was
 //          what the CTA waited for: 28672 x 8192 at batch 512 390 us with boxes of 16 rows, 350 with two boxes a step.)
 //   1..3   warp 1 allocates tensor memory; each issues the MMAs of the units of one accumulator and commits units and stages
-//          back (a unit is a step of one path; one path uses two accumulators for alternate steps, added in the epilogue).
+//          back (a unit is a step of one path; one path uses up to four accumulators in turn, added in the epilogue).
 //          One issuing warp took about 430 clocks per unit, mostly its own waits, where the four MMAs need 2 N.
 //   4..19  expanders: four warpgroups (three if there are three paths) take the units in turn; warp q of a group owns
 //          tensor-memory lanes 32q..32q+31, i.e. the row blocks p = 2q, 2q + 1 of a sign tile.  tcgen05.st.16x256b takes a
@@ -28,7 +28,7 @@
 //          consecutive columns at 4 tq): a mask and a multiplication (in place of a shift) per word, then per two operand
 //          registers a byte permute, a logic instruction and a fused multiply-add.  Then (same warps) the epilogue: tcgen05.ld, g_k, sum of the paths, fp16,
 //          store.
-//   20..23 stream kernels only: the epilogue of every pass but a task's last.
+//   then   the fourth issuing warp, where there is one; in stream kernels four warps for the epilogue of every pass but a task's last.
 //
 // Work.  One CTA per SM.  An output tile is 128 weight rows x N batch columns, N a multiple of 16 chosen for the call.
 // Up to 16 batch columns a CTA takes a contiguous range of (row tile, slice of 256 columns) pairs and the parts of a row tile meet in
@@ -80,8 +80,11 @@ constexpr int kWTiles = 2 * kWSteps, kWBytes = kWTiles * (RABIT_TILE_BYTES + RAB
 constexpr int kMaxWStages = 4;
 constexpr int kExpandGroups = 4;            // of four warps each
 constexpr int kExpandWarps = 4 * kExpandGroups;
-constexpr int kThreads = (4 + kExpandWarps) * 32;
-constexpr int kStreamThreads = kThreads + 128;             // stream kernels: four warps for the epilogues
+constexpr int kFourthIssuer = 4 + kExpandWarps;
+constexpr int kMaxAcc = 4;                  // accumulators
+// Threads of an instance: one operand per step (one path, or the dequantised form) has a fourth issuing warp, stream kernels four warps
+// for the epilogues.
+__host__ __device__ constexpr int threads_of(bool one_op, bool stream) { return (kFourthIssuer + (one_op ? 1 : 0) + (stream ? 4 : 0)) * 32; }
 constexpr unsigned long long kSumMask = (1ULL << 55) - 1;
 
 constexpr int kMaxTasks = 512;
@@ -136,7 +139,7 @@ struct Control {                            // ahead of the ring in shared memor
     unsigned long long a_empty[kMaxUnits];  // MMAs that read the unit retired
     unsigned long long acc_ready[2];        // all MMAs of the pass retired (stream: by the parity of the pass, which has its own accumulators)
     unsigned long long acc_empty[2];        // epilogue has read the accumulators
-    unsigned long long drained[3];          // after a time-out: everything this accumulator's warp issued has retired
+    unsigned long long drained[kMaxAcc];          // after a time-out: everything this accumulator's warp issued has retired
 #ifdef RABIT_CHECKED
     unsigned long long never;               // nothing arrives here (rabit_selftest_withhold)
 #endif
@@ -256,7 +259,7 @@ __host__ __device__ __forceinline__ int segment_arrivals(uint32_t first, uint32_
 // is a pass per path on one accumulator, the sum of the scaled passes stays in tensor memory beside it, and up to 13 groups fit
 // (5000 x 13824 at batch 200: each tile expanded once instead of three times).
 template <int K, bool DEQ, int NL, bool SEQ>
-__global__ void __launch_bounds__(NL > 1 ? kStreamThreads : kThreads, 1)
+__global__ void __launch_bounds__(threads_of((DEQ || K == 1) && !SEQ, NL > 1), 1)
 rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_constant__ XMaps<NL> x_maps) {
     extern __shared__ unsigned char smem_raw[];
     // the swizzled x tiles need 1024-byte alignment; the launch reserves the slack
@@ -271,12 +274,13 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
         const uint32_t word = reinterpret_cast<const uint32_t*>(&P)[warp * 16];
         asm volatile("" ::"r"(word));
     }
-    if (warp == kThreads / 32 - 1 && lane < (NL == 1 ? 1 : P.n_layers)) asm volatile("prefetch.tensormap [%0];" ::"l"(&x_maps.map[NL == 1 ? 0 : lane]) : "memory");
+    if (warp == kFourthIssuer - 1 && lane < (NL == 1 ? 1 : P.n_layers)) asm volatile("prefetch.tensormap [%0];" ::"l"(&x_maps.map[NL == 1 ? 0 : lane]) : "memory");
     auto layer = [&](const Pass& ps) -> const GemmLayer& { return P.L[NL == 1 ? 0 : ps.l]; };
     unsigned char* ring = smem + kControlBytes;
     unsigned char* w_ring = ring + P.stages * P.stage_bytes;
     constexpr int n_ops = DEQ ? 1 : K;                            // operand units (and accumulators) per step
     constexpr int n_groups = n_ops == 3 || SEQ ? 3 : 4;                  // expander groups at work
+    constexpr int n_fourth = n_ops == 1 && !SEQ ? 1 : 0;                 // whether there is a fourth issuing warp
     const int stages = P.stages, w_stages = P.w_stages, units = P.units, x_steps = P.x_steps, n_acc = P.n_acc;
     const int stage_bytes = P.stage_bytes;
     volatile int* abort_flag = &S.abort_flag;
@@ -353,7 +357,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
 #pragma unroll
         for (int i = 0; i < n; ++i) v[i] = 0.f;
 #pragma unroll
-        for (int m = 0; m < (n_ops == 1 ? 2 : n_ops); ++m) {
+        for (int m = 0; m < (n_ops == 1 ? kMaxAcc : n_ops); ++m) {
             if (n_ops == 1 && m >= n_acc) break;
             uint32_t d[n];
             if constexpr (n == 16) tmem_ld16(from + (uint32_t)(m * kGroupCols), d);
@@ -498,7 +502,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
             *(volatile int*)&S.x_begun = it;
         }
         __syncwarp();
-    } else if (warp < 4) {
+    } else if (warp < 4 || (n_fourth && warp == kFourthIssuer)) {
         // ===================================== MMA issuers =====================================
         // Warp 1 + m issues the units u = m, m + n_acc, ... into accumulator m.  (The whole warp walks the loop, one elected lane
         // issues: see the header.)
@@ -530,7 +534,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                     const int n_here = min(x_steps, s_hi - s);
                     mbar_wait_stage(full0 + xw.slot * 8, xw.lap, abort_flag, &S.x_begun);
                     const uint64_t bdesc = bdesc0 + (uint64_t)((xw.slot * stage_bytes) >> 4);
-                    int si = n_ops == 1 && n_acc > 1 ? (m ^ (steps_before + s - s_lo)) & 1 : 0;
+                    int si = n_ops == 1 ? (m - (steps_before + s - s_lo)) & (n_acc - 1) : 0;   // (1, 2 or 4 accumulators)
                     auto issue = [&](uint32_t a, int step, bool first) {
                         const uint64_t bd = bdesc + (uint64_t)((step * step_bytes) >> 4);
                         umma_f16_ts(d, a, bd, idesc, first ? accumulate : 1u);
@@ -584,7 +588,8 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
         if (warp == 1) issue_units(std::integral_constant<int, 0>{});
         else if (warp == 2 && n_acc > 1) issue_units(std::integral_constant<int, 1>{});
         else if (warp == 3 && n_acc > 2) issue_units(std::integral_constant<int, 2>{});
-    } else if (NL == 1 || warp < kThreads / 32) {
+        else if (n_fourth && warp == kFourthIssuer && n_acc > 3) issue_units(std::integral_constant<int, 3>{});
+    } else if (warp < kFourthIssuer) {
         // ============================ expanders, then epilogue ============================
         const int grp = (warp - 4) >> 2, q = warp & 3;        // tensor-memory lanes this warp may touch: 32q .. 32q + 31
         const int gq = lane >> 2, tq = lane & 3;
@@ -761,7 +766,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                     for (int i = 0; i < 16; ++i) v[i] = 0.f;
                     if constexpr (SEQ) path_sum(c, v);
 #pragma unroll
-                    for (int m = 0; m < (n_ops == 1 ? 2 : n_ops); ++m) {
+                    for (int m = 0; m < (n_ops == 1 ? kMaxAcc : n_ops); ++m) {
                         if (n_ops == 1 && m >= n_acc) break;
                         uint32_t d[16];
                         tmem_ld16(lane_base + (uint32_t)((m * P.max16 + c) * kGroupCols), d);
@@ -803,7 +808,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
         PassWalker<NL, SEQ> w = first_pass;
         Pass ps;
         w.next(P, ps);
-        if (warp >= 4) {
+        if (warp >= 4 && warp < kFourthIssuer) {
             mbar_wait(smem_u32(&S.acc_ready[0]), SEQ ? (P.paths - 1) & 1 : 0, abort_flag);
             fence_after();
         }
@@ -811,7 +816,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
         if (SEQ) cluster_sync_all();                           // the receive buffer lies in the rings: every CTA's are done with
         float* recv = reinterpret_cast<float*>(smem + P.recv_off);
-        if (warp >= 4) {
+        if (warp >= 4 && warp < kFourthIssuer) {
             const int grp = (warp - 4) >> 2, q = warp & 3, r_in = q * 32 + lane;
 #pragma unroll 1
             for (int c = grp; c < ps.n; c += kExpandGroups) {
@@ -820,7 +825,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                 for (int i = 0; i < 16; ++i) v[i] = 0.f;
                 if constexpr (SEQ) path_sum(c, v);
 #pragma unroll
-                for (int m = 0; m < (n_ops == 1 ? 2 : n_ops); ++m) {
+                for (int m = 0; m < (n_ops == 1 ? kMaxAcc : n_ops); ++m) {
                     if (n_ops == 1 && m >= n_acc) break;
                     uint32_t d[16];
                     tmem_ld16(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)((m * P.max16 + c) * kGroupCols), d);
@@ -838,7 +843,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
         }
         __syncwarp();
         cluster_sync_all();
-        if (warp >= 4) {
+        if (warp >= 4 && warp < kFourthIssuer) {
             const int et = (warp - 4) * 32 + lane, r_in = et & (kTileM - 1), hh = et >> 7;  // four threads per row, every fourth column each
             const int row = ps.rt * kTileM + r_in;
             for (int c = (int)crank; c < ps.n; c += split)
@@ -863,12 +868,12 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
     if (gave_up) [[unlikely]] {
         // Copies and MMAs under way must not outlive the shared and tensor memory they work on.  (All of it in one branch of its
         // own: with the ordinary path running through it a launch took 0.1 us longer.)
-        if (tid < 3) mbar_init(smem_u32(&S.drained[tid]), 1);
+        if (tid < kMaxAcc) mbar_init(smem_u32(&S.drained[tid]), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         __syncthreads();
         const long long t0 = clock64();
-        if (warp >= 1 && warp <= 3) {                            // (an arrival once all that this lane issued has retired)
-            const uint32_t bar = smem_u32(&S.drained[warp - 1]);
+        if ((warp >= 1 && warp <= 3) || (n_fourth && warp == kFourthIssuer)) {   // (an arrival once all that this lane issued has retired)
+            const uint32_t bar = smem_u32(&S.drained[warp <= 3 ? warp - 1 : 3]);
             if (elect_one()) umma_commit(bar);
             __syncwarp();
             while (!mbar_try_wait(bar, 0u) && clock64() - t0 <= kWaitLimitCycles) { }
@@ -941,8 +946,15 @@ bool fill_resources(Plan& p, int K, int n_ops, int steps, bool one_box) {
     if (p.max16 * kGroupCols > 256) return false;
     const int turn = n_ops == 3 || p.seq ? 3 : 4;
     auto free_units = [&](int n_acc) { return (512 - ((p.stream ? 2 : 1) * n_acc + p.seq) * p.max16 * kGroupCols) / kUnitCols; };   // (a stream: two sets of accumulators)
-    // (one path: a second accumulator needs a step for each in every pass; a stream's shortest one is the last slice)
-    p.n_acc = p.seq ? 1 : n_ops > 1 ? n_ops : (p.stream ? steps % kSliceSteps != 1 : steps >= 2) && free_units(2) >= turn ? 2 : 1;
+    // One operand per step: up to four accumulators, if every pass has a step for each (a stream's shortest one is the last slice) and x comes in
+    // several steps a stage (every issuing warp sees every stage: with one step in each 3894 x 14304 at 42 18.6 -> 19.5 us) and
+    // the contraction is long enough to pay for adding them up (8 steps, 2000 x 4096 at 64 7.1 -> 7.3; 16, 4096 x 4096 at 32 7.17 -> 7.26; 32,
+    // 600 x 16384 at 20 8.35 -> 7.8).  One or two
+    // issuing warps were what such layers waited for up to 64 batch columns (one path, 28672 x 8192 at 16 26.5 -> 25.5 us, 14336 x 4096 at 48 10.85 -> 10.45;
+    // with two paths, whose two warps issue pairs of units, four of them are 2 to 4 % slower).
+    p.n_acc = n_ops;
+    if (n_ops == 1 && !p.seq)
+        for (int more = 2; more <= (one_box && (p.stream || steps >= 24) ? kMaxAcc : 2) && steps >= more && free_units(more) >= (more == 2 ? turn : 2 * turn); more *= 2) p.n_acc = more;
     if (free_units(p.n_acc) < turn) return false;
     p.units = free_units(p.n_acc) >= 2 * turn ? 2 * turn : turn;
     const int step_bytes = (p.max16 + p.box16 - 1) / p.box16 * p.box16 * kGroupCols * kStepCols * 2;
@@ -1000,10 +1012,10 @@ cudaError_t prepare_kernel(int K, bool deq, int device, bool stream = false, boo
 }
 
 // How many clusters of `split` CTAs of this kernel the device places at once (a cluster sits inside one GPC).
-int resident_clusters(const void* kernel, int split, size_t smem, int sms) {
+int resident_clusters(const void* kernel, int threads, int split, size_t smem, int sms) {
     cudaLaunchConfig_t q = {};
     q.gridDim = dim3((unsigned int)((sms / split) * split));
-    q.blockDim = dim3(kThreads);
+    q.blockDim = dim3((unsigned int)threads);
     q.dynamicSmemBytes = smem;
     cudaLaunchAttribute qa[1];
     qa[0].id = cudaLaunchAttributeClusterDimension;
@@ -1024,7 +1036,7 @@ constexpr double kExchangeClocks = 2500.0;           // exchange of a split task
 // launch, unit of one, two or three paths, a further pass in a range, publishing parts of row tiles besides its throughput and that (sums per clock
 // over the GPU).  Before the epilogues had warps of their own a further pass cost 3000 and ranges that cross row tiles were avoided: 11008 x 4096
 // at 16 rows 14.7 -> 13.5 us, 14336 x 4096 with three paths 20.3 -> 18.9.
-constexpr double kStreamLaunch = 5600.0, kStreamUnit[3] = {208.0, 170.0, 166.0}, kStreamPass = 1300.0, kStreamPublish = 800.0, kStreamRate = 130.0;
+constexpr double kStreamLaunch = 5600.0, kStreamUnit[3] = {199.0, 170.0, 166.0}, kStreamPass = 1300.0, kStreamPublish = 800.0, kStreamRate = 130.0;
 
 // Task counts worth an estimate: equal parts of every row tile (or nearly), and one task per SM.  Never more tasks than pairs: an
 // empty one would count among the arrivals of a row tile that it does not contribute to.  (Layers of unlike widths: parts for the
@@ -1044,14 +1056,14 @@ Plan stream_plan(int n_layers, const int* n_rt, const int* n_ct, int K, bool deq
     p.stream = p.split = p.max16 = p.box16 = 1;
     const int n_ops = deq ? 1 : K;
     long long pairs = 0, row_tiles = 0;
-    int most_cs = 0, tail = 2;                            // tail: steps of a last slice, 1 if any layer's has just one
+    int most_cs = 0, tail = kSliceSteps;                  // tail: steps of the shortest last slice
     bool wide_x = true;
     for (int l = 0; l < n_layers; ++l) {
         const int steps = (n_ct[l] + 1) / 2, n_cs = (steps + kSliceSteps - 1) / kSliceSteps;
         pairs += (long long)n_rt[l] * n_cs;
         row_tiles += n_rt[l];
         most_cs = std::max(most_cs, n_cs);
-        if (steps % kSliceSteps == 1) tail = 1;
+        if (steps % kSliceSteps != 0) tail = std::min(tail, steps % kSliceSteps);
         wide_x = wide_x && n_ct[l] % 2 == 0;
     }
     if (most_cs > RABIT_LUT_MAX_SLICES || pairs >= kMaxPairs || sms > kMaxTasks || !fill_resources(p, K, n_ops, tail, wide_x)) return best;
@@ -1105,7 +1117,7 @@ Plan make_plan(int n_rt, int n_steps, int K, bool deq, int batch, int sms, int d
                 const long long ctas = (long long)p.tasks * split;
                 if (split > 1 && (n_steps / split < 4 || ctas > sms)) continue;
                 if (!fill_resources(p, seq ? 1 : K, seq ? 1 : n_ops, n_steps / split, wide_x)) continue;
-                if (split > 1 && device >= 0 && (prepare_kernel(K, deq, device, false, seq != 0) != cudaSuccess || resident_clusters(kernel_for(K, deq, false, seq != 0), split, p.smem, sms) < p.tasks)) continue;
+                if (split > 1 && device >= 0 && (prepare_kernel(K, deq, device, false, seq != 0) != cudaSuccess || resident_clusters(kernel_for(K, deq, false, seq != 0), threads_of(n_ops == 1 && !seq, false), split, p.smem, sms) < p.tasks)) continue;
                 const double rounds = (double)((ctas + sms - 1) / sms);
                 p.clocks = kLaunchClocks + (split > 1 ? kExchangeClocks * (1 + seq) : 0.0) + rounds * ((n_steps + split - 1) / split) * n_ops * unit_clocks(p.chunk16, p, seq ? 1 : n_ops) +
                            (rounds * (seq ? K : 1) - 1.0) * kPassClocks;
@@ -1302,7 +1314,7 @@ static cudaError_t launch_stream(const rabit_layer* const* layers, int n_layers,
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned int)p.tasks);
-    cfg.blockDim = dim3(kStreamThreads);
+    cfg.blockDim = dim3((unsigned int)threads_of(K == 1 || dequantised, true));
     cfg.dynamicSmemBytes = p.smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -1350,7 +1362,7 @@ cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, i
 
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned int)(p.tasks * p.split));
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3((unsigned int)threads_of((G.K == 1 || dequantised) && !p.seq, false));
     cfg.dynamicSmemBytes = p.smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];

@@ -39,7 +39,7 @@ def test_clearing_the_status_restores_the_whole_scratch(batch):
 
 @pytest.mark.parametrize("shapes,batch,variant,stages", [
     ([(2, 2560, 8192)], 12, 3, (0, 2)),                     # ranges of (row tile, slice) pairs
-    ([(1, 2560, 8192)], 12, 3, (1,)),                       # two accumulators for one path
+    ([(1, 2560, 8192)], 12, 3, (1,)),                       # four accumulators for one path
     ([(2, 3000, 8192)], 48, 3, (0, 3)),                     # the contraction over clusters
     ([(3, 2500, 8192)], 200, 3, (2, 20)),                   # path after path, over clusters
     ([(2, 20000, 1024)], 300, 3, (3,)),                     # several passes of 16-column groups a CTA

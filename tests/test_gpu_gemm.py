@@ -152,3 +152,13 @@ def test_several_row_tiles_in_a_range(K, M, N, batch):
     L = make_layer(M, N, K, key=(65, K, M, N))
     x = make_x(batch, N, key=(65, M, N, batch))
     check_against_oracle(L, x, run_layer(L, x, GEMM))
+
+
+@pytest.mark.parametrize("batch", [16, 40, 64, 65])
+@pytest.mark.parametrize("N", [64, 160, 320, 384, 448, 1024])
+def test_one_path_accumulators(N, batch):
+    """One operand per step: one, two or four accumulators, by the steps of the shortest pass (a last slice of one to four steps, fewer steps
+    than accumulators) and by the room that 64 and 65 columns leave."""
+    L = make_layer(700, N, 1, key=(66, N))
+    x = make_x(batch, N, key=(66, N, batch))
+    check_against_oracle(L, x, run_layer(L, x, GEMM))
