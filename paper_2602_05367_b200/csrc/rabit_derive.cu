@@ -60,15 +60,18 @@ __device__ __forceinline__ void copy_async_wait() {
 // tile's word (byte c, bit p) with one funnel shift; transposed, two neighbouring lanes' words are four bytes of the look-up blocks each.
 // W comes in parts of 4 KB a warp (a quarter of its 128 x 32 weights) by asynchronous copies into a ring of three parts of its own in shared
 // memory, two ahead of the one at hand and across block borders; a lane reads back what it copied itself, so no barrier is involved.
-// The scales of the next block are fetched beside the work on this one.
+// The scales of the next block are fetched beside the work on this one.  Two CTAs per SM, which for three paths takes scales of one block only in
+// shared memory (of two 48.6 us, one CTA per SM, instead of 42.6).  Bound: HBM with one path (11008 x 4096, 200 MB in and out: 32 us), beyond that the
+// recurrence's instructions beside it; two paths 36.5 (47.9 with W in registers, at most a part ahead), 28672 x 8192 161 (256).
 constexpr int kRingParts = 3;
 constexpr int kPartBytes = 32 * 8 * 16;
 template <int K>
 struct DeriveSmem {
     static constexpr int kBytes = kWarps * kRingParts * kPartBytes;                          // behind the ring: the look-up bytes of a block
-    static constexpr int kScales = kBytes + 4 * K * RABIT_LUT_PART_BYTES;                    // then g and h of two blocks, fp32
+    static constexpr int kScales = kBytes + 4 * K * RABIT_LUT_PART_BYTES;                    // then g and h of the block, fp32
     static constexpr int kScaleFloats = (K - 1) * (RABIT_TILE_ROWS + RABIT_LUT_COLS);        // (the last path's are not needed)
-    static constexpr int kTotal = kScales + 2 * kScaleFloats * 4;
+    static constexpr int kTotal = kScales + kScaleFloats * 4;
+    static_assert(2 * (kTotal + 1024) <= 228 * 1024, "two CTAs per SM");
 };
 template <int K>
 __global__ void __launch_bounds__(kWarps * 32, 2)
@@ -110,11 +113,11 @@ rabit_derive_kernel(RabitGeom G, const float* __restrict__ W, const __half* __re
             }
         }
     };
-    auto keep_scales = [&](int buffer) {
+    auto keep_scales = [&]() {
 #pragma unroll
         for (int u = 0; u < kPerThread; ++u) {
             const int i = threadIdx.x + u * kWarps * 32;
-            if (i < S::kScaleFloats) scales[buffer * S::kScaleFloats + i] = __half2float(next[u]);
+            if (i < S::kScaleFloats) scales[i] = __half2float(next[u]);
         }
     };
 
@@ -122,15 +125,14 @@ rabit_derive_kernel(RabitGeom G, const float* __restrict__ W, const __half* __re
     fetch(blockIdx.x, 1, 1);
     fetch_scales(blockIdx.x);
     do_fills(F);
-    keep_scales(0);
+    keep_scales();
     __syncthreads();
     const uint32_t own_half = tq & 1 ? 0xF0F0F0F0u : 0x0F0F0F0Fu;
     const int turn = tq & 1 ? 28 : 4;
-    int slot = 0, ahead = 2, buffer = 0;                  // ring slots of the part at hand and of the one to fetch
-    for (uint32_t b = blockIdx.x; b < n_blocks; b += gridDim.x, buffer ^= 1) {
+    int slot = 0, ahead = 2;                              // ring slots of the part at hand and of the one to fetch
+    for (uint32_t b = blockIdx.x; b < n_blocks; b += gridDim.x) {
         const int rt = (int)(b / (uint32_t)G.n_cs), cs = (int)(b - (uint32_t)rt * G.n_cs), ct = cs * kWarps + warp;
         const bool inside = ct < G.n_ct;
-        const float* gs = scales + buffer * S::kScaleFloats;
         fetch_scales(b + gridDim.x);
         uint32_t out[K][4];
 #pragma unroll
@@ -156,7 +158,7 @@ rabit_derive_kernel(RabitGeom G, const float* __restrict__ W, const __half* __re
                     for (int p = 7; p >= 0; --p) tile = __funnelshift_l(__float_as_uint(r[p][c]), tile, 1);
                 out[k][alo | (ah << 1)] = tile;
                 if (k + 1 < K) {
-                    const float* gk = gs + k * (RABIT_TILE_ROWS + RABIT_LUT_COLS);
+                    const float* gk = scales + k * (RABIT_TILE_ROWS + RABIT_LUT_COLS);
                     const float4 hv = *reinterpret_cast<const float4*>(gk + RABIT_TILE_ROWS + warp * RABIT_TILE_COLS + 16 * ah + 4 * tq);
                     const float hc[4] = {hv.x, hv.y, hv.z, hv.w};
 #pragma unroll
@@ -187,8 +189,8 @@ rabit_derive_kernel(RabitGeom G, const float* __restrict__ W, const __half* __re
 #pragma unroll
             for (int k = 0; k < K; ++k) tiles[rabit_tile_pos(G, rt, k, ct) * 32 + lane] = make_uint4(out[k][0], out[k][1], out[k][2], out[k][3]);
         }
-        keep_scales(buffer ^ 1);
         __syncthreads();
+        keep_scales();                                    // (nobody reads this block's any more)
         uint4* dst = lut + ((size_t)cs * G.n_rb + 4 * rt) * K * (RABIT_LUT_PART_BYTES / 16);
         for (int i = threadIdx.x; i < 4 * K * (RABIT_LUT_PART_BYTES / 16); i += kWarps * 32) dst[i] = reinterpret_cast<const uint4*>(bytes)[i];
         __syncthreads();
