@@ -142,7 +142,7 @@ static bool ranges_overlap(const void* a, size_t an, const void* b, size_t bn) {
 
 // Rows up to which the f16 GEMV is the faster of the two tensor-core kernels: its MMAs carry eight rows, a second set for 9 to
 // 16 makes it slower than the GEMM, which costs the same from 1 to 16 (B200, us at 8 / 9 / 16 rows against the GEMM:
-// 4096 x 4096 6.8 / 8.4 / 8.9 against 7.8, 14336 x 4096 13 / 18.3 / 20.6 against 16.0, 28672 x 8192 38 / 54 / 55 against 44).
+// 4096 x 4096 6.8 / 8.4 / 8.9 against 7.5, 14336 x 4096 13 / 18.3 / 20.6 against 14.6, 28672 x 8192 38 / 54 / 55 against 40).
 static const int kF16Rows = 8;
 
 static int linear_call(const rabit_layer* layer, const void* x, void* y, int batch, void* stream) {
