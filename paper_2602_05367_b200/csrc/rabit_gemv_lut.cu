@@ -526,8 +526,9 @@ struct Cost {
 // for the cut.  (The block's figure is in clocks of an earlier loop: it takes 118 now.)
 // (the table figure is a fit: the split that minimises the measured step time charges a table about 26 blocks, far
 // more than its 430 cycles of stores, because a rebuild in mid-range also stops every warp at two barriers)
-// (two batch rows: a quarter less measures best; 22016 x 4096 10.2, 9.9, 9.85 us and 28672 x 8192 20.9, 20.9, 21.3 with 1900, 1700, 1500)
-Cost cost_of(int K, int nb) { return Cost{(long long)nb * (70 * K + 30), (long long)nb * ((nb == 1 ? 2200 : 1700) * K) + 100}; }
+// (two batch rows: a quarter less measures best; 22016 x 4096 10.2, 9.9, 9.85 us and 28672 x 8192 20.9, 20.9, 21.3 with 1900, 1700, 1500;
+// of three paths 5000 x 13824 14.35, 14.15, 12.95, 22016 x 4096 15.2, 15.2, 14.8, 28672 x 8192 32.05, 32.0, 32.2 with 2400, 1700, 1200)
+Cost cost_of(int K, int nb) { return Cost{(long long)nb * (70 * K + 30), (long long)nb * ((nb == 1 ? 2200 : K == 3 ? 1200 : 1700) * K) + 100}; }
 
 // CTAs a layer of n_cs x n_rb blocks needs when no CTA may cost more than `limit`; writes the cuts if asked.
 int ctas_needed(int n_cs, int n_rb, const Cost& C, long long limit, std::vector<int>* cuts) {
@@ -618,7 +619,7 @@ bool rabit_gemv_lut_supports(const rabit_layer& L, int batch) {
 // Whether it is the faster one for layers that it can run.  Against the f16 GEMV only two rows of three paths are ever not: its tables take
 // a table's build (three of 64 KB) per CTA and pay from about four blocks of 32 rows x 256 columns per SM on (B200, us, f16 GEMV against this:
 // 2000 x 1024 (256 blocks) 3.67 / 4.1, 2048 x 2048 (512) 4.1 / 4.2, 1024 x 4096 (512) 4.1 / 4.0, 11008 x 512 (688) 5.0 / 4.6, 2048 x 3072 (768)
-// 5.0 / 4.3, 4096 x 4096 7.4 / 5.7, 22016 x 4096 24.2 / 15.2, 28672 x 8192 54.0 / 31.8).
+// 5.0 / 4.3, 4096 x 4096 7.4 / 5.7, 22016 x 4096 24.2 / 14.8, 28672 x 8192 54.0 / 32.0).
 bool rabit_gemv_lut_preferred(const rabit_layer* const* layers, int n_layers, int batch) {
     if (layers[0]->geom.K < 3 || batch == 1) return true;
     long long blocks = 0;
