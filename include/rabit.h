@@ -251,6 +251,14 @@ RABIT_API int rabit_selftest_gemm_plan(int n_layers, const int* M, const int* N,
                              int* head_out, int* passes_out, int max_passes);
 
 /*
+ * Test aid (no counterpart in the paper; host only, no GPU needed): by which of the tcgen05 GEMM's barriers the warps that publish pass `pass`
+ * (from 0) of a task of `passes` passes learn that its MMAs are done.  Returns the barrier; parity_out (HOST, one int) receives the parity
+ * of the phase that they wait for.  stream: 1 for tasks that are ranges of (row tile, slice) pairs, where four warps publish every
+ * pass but the last and the expanding warps the last; 0 for all others, where the expanding warps publish every pass.
+ */
+RABIT_API int rabit_selftest_gemm_ready(int stream, int pass, int passes, int* parity_out);
+
+/*
  * Measurement aid (no counterpart in the paper): one kernel that reads `bytes` bytes of device memory once with
  * 128-bit streaming loads and keeps nothing.  Timed by the caller with CUDA events over a buffer much larger than L2
  * it gives the read-only HBM bandwidth this GPU delivers to plain loads, the natural ceiling of the decode GEMV.

@@ -137,7 +137,7 @@ struct Control {                            // ahead of the ring in shared memor
     unsigned long long w_empty[kMaxWStages];// every expander warp has read them
     unsigned long long a_ready[kMaxUnits];  // unit expanded
     unsigned long long a_empty[kMaxUnits];  // MMAs that read the unit retired
-    unsigned long long acc_ready[2];        // all MMAs of the pass retired (stream: by the parity of the pass, which has its own accumulators)
+    unsigned long long acc_ready[3];        // all MMAs of the pass retired (which one: ready_of)
     unsigned long long acc_empty[2];        // epilogue has read the accumulators
     unsigned long long drained[kMaxAcc];          // after a time-out: everything this accumulator's warp issued has retired
 #ifdef RABIT_CHECKED
@@ -247,6 +247,18 @@ struct PassWalker {
     }
 };
 
+// Which of the acc_ready barriers says that all MMAs of a task's pass have retired, and the parity of that phase.  A wait by parity tells a phase
+// from the one before it and from no other, so whoever waits for a barrier waits for every phase of it in turn.  In a stream task the warps
+// for the epilogues do that with the two of the alternating passes; the expanders, which publish the last pass only and may be several
+// passes ahead of the MMAs when they come to it (as many as the unit ring holds, and a group without units all of them), have a barrier of its own.
+struct Ready {
+    int bar;
+    uint32_t parity;
+};
+__host__ __device__ __forceinline__ Ready ready_of(bool stream, int pass_i, bool last) {
+    return !stream ? Ready{0, (uint32_t)pass_i & 1u} : last ? Ready{2, 0u} : Ready{pass_i & 1, (uint32_t)(pass_i >> 1) & 1u};
+}
+
 // Segments of a row tile of stream tasks: the tasks that touch its n_cs pairs, the first of which is pair `first` of n_pairs.  No task
 // is empty.  (pairs < kMaxPairs and tasks <= kMaxTasks: 32 bits hold the products)
 __host__ __device__ __forceinline__ int segment_arrivals(uint32_t first, uint32_t n_cs, uint32_t tasks, uint32_t n_pairs) {
@@ -296,10 +308,8 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
         if (lane < kMaxWStages) { mbar_init(smem_u32(&S.w_full[lane]), 1); mbar_init(smem_u32(&S.w_empty[lane]), 4 * n_groups); }
         if (lane < kMaxUnits) { mbar_init(smem_u32(&S.a_ready[lane]), 4); mbar_init(smem_u32(&S.a_empty[lane]), 1); }
         if (lane == 0) {
-            for (int i = 0; i < 2; ++i) {
-                mbar_init(smem_u32(&S.acc_ready[i]), n_acc);
-                mbar_init(smem_u32(&S.acc_empty[i]), NL > 1 ? 4 : kExpandWarps);
-            }
+            for (int i = 0; i < 3; ++i) mbar_init(smem_u32(&S.acc_ready[i]), n_acc);
+            for (int i = 0; i < 2; ++i) mbar_init(smem_u32(&S.acc_empty[i]), NL > 1 ? 4 : kExpandWarps);
             S.abort_flag = 0;
             S.x_begun = -1;
 #ifdef RABIT_CHECKED
@@ -339,8 +349,9 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
     // otherwise every output goes into its 64-bit accumulate word with one integer atomic (as in rabit_gemv_f16.cu: fixed-point grid
     // of the packer, a segment of s slices shifted by s * 2^fix_bits, arrivals in bits 55..62, bit 63 = non-finite), and the thread
     // whose add completes a word rounds it to fp16, stores y and clears it.
-    [[maybe_unused]] auto publish = [&](auto cols, const Pass& ps, int pass_i, int c0) {
+    [[maybe_unused]] auto publish = [&](auto cols, auto is_last, const Pass& ps, int pass_i, int c0) {
         constexpr int n = decltype(cols)::value;
+        constexpr bool last = decltype(is_last)::value;
         const GemmLayer& L = layer(ps);
         const int q = warp & 3, row = ps.rt * kTileM + q * 32 + lane, n_slices = (ps.s_hi - ps.s_lo + kSliceSteps - 1) / kSliceSteps, set = pass_i & 1;
         // (in registers: read from the parameters between the atomics, each would be a wait)
@@ -350,7 +361,8 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
         unsigned long long* const word = L.acc + (size_t)c0 * Mp + row;
         const int arrivals = segment_arrivals((uint32_t)(L.pair0 + ps.rt * n_cs), (uint32_t)n_cs, (uint32_t)P.n_tasks, (uint32_t)P.n_groups);
         const uint32_t from = __shfl_sync(0xFFFFFFFFu, S.tmem_base, 0) + ((uint32_t)(32 * q) << 16) + (uint32_t)(set * n_acc * kGroupCols + c0);
-        mbar_wait(smem_u32(&S.acc_ready[set]), (uint32_t)(pass_i >> 1) & 1u, abort_flag);
+        const Ready ready = ready_of(true, pass_i, last);
+        mbar_wait(smem_u32(&S.acc_ready[ready.bar]), ready.parity, abort_flag);
         __syncwarp();
         fence_after();
         float v[n];
@@ -369,7 +381,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
         }
         fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&S.acc_empty[set]));
+        if (!last && lane == 0) mbar_arrive(smem_u32(&S.acc_empty[set]));     // (nothing follows the last pass)
         if (n_slices == n_cs) {
 #pragma unroll
             for (int i = 0; i < n; ++i)
@@ -580,7 +592,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                     xw.step(1, stages);
                 }
                 steps_before += s_hi - s_lo;
-                const uint32_t passed = __shfl_sync(0xFFFFFFFFu, smem_u32(&S.acc_ready[set]), 0);
+                const uint32_t passed = __shfl_sync(0xFFFFFFFFu, smem_u32(&S.acc_ready[ready_of(NL > 1, pass_i - 1, w.left <= 0).bar]), 0);
                 if (elected) umma_commit(passed);
                 __syncwarp();
             }
@@ -727,12 +739,13 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
             if constexpr (NL > 1) {
                 // A pass that another one follows is published by warps of their own, while this one is expanded (its accumulators are not
                 // those of the next); the last one by these, which are four times as many.
-                if (w.left <= 0) publish(std::integral_constant<int, 4>{}, ps, pass_i, 4 * grp);
+                if (w.left <= 0) publish(std::integral_constant<int, 4>{}, std::true_type{}, ps, pass_i, 4 * grp);
                 ++pass_i;
                 continue;
             }
             // ---- epilogue of this pass
-            mbar_wait(smem_u32(&S.acc_ready[0]), pass_i & 1, abort_flag);
+            const Ready ready = ready_of(false, pass_i, false);
+            mbar_wait(smem_u32(&S.acc_ready[ready.bar]), ready.parity, abort_flag);
             ++pass_i;
             fence_after();
             const int row = ps.rt * kTileM + q * 32 + lane;
@@ -795,7 +808,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
         Pass ps;
         while (w.next(P, ps) && w.left > 0) {
             load_scales(ps);
-            publish(std::integral_constant<int, kGroupCols>{}, ps, pass_i, 0);
+            publish(std::integral_constant<int, kGroupCols>{}, std::false_type{}, ps, pass_i, 0);
             ++pass_i;
         }
     }
@@ -1276,6 +1289,13 @@ int rabit_gemm_tc_plan(int n_layers, const int (*shape)[2], int K, bool deq, int
     }
     GemmParams<1> P = {};
     return p.seq ? list_passes<1, true>(P, p, 1, shape, K, batch, out, max_passes) : list_passes<1, false>(P, p, 1, shape, K, batch, out, max_passes);
+}
+
+// The same function that the kernel uses (see rabit_selftest_gemm_ready).
+int rabit_gemm_tc_ready(bool stream, int pass_i, bool last, int* parity) {
+    const Ready r = ready_of(stream, pass_i, last);
+    *parity = (int)r.parity;
+    return r.bar;
 }
 
 int rabit_gemm_tc_max_group() { return kMaxGroup; }

@@ -107,6 +107,7 @@ int rabit_gemm_tc_max_group();
 bool rabit_gemm_tc_group_supports(const rabit_layer* const* layers, int n_layers, int batch);
 cudaError_t rabit_launch_gemm_tc_group(const rabit_layer* const* layers, int n_layers, const void* const* xs, void* const* ys, int batch, cudaStream_t stream);
 int rabit_gemm_tc_plan(int n_layers, const int (*shape)[2], int K, bool deq, int batch, int sms, int candidate, int head[8], int* out, int max_passes);   // host only: the work split
+int rabit_gemm_tc_ready(bool stream, int pass_i, bool last, int* parity);   // host only: who waits for what
 double rabit_gemm_tc_estimate_us(const rabit_layer& L, int batch);
 
 #endif  // RABIT_INTERNAL_H_

@@ -68,6 +68,13 @@ extern "C" int rabit_selftest_gemm_plan(int n_layers, const int* M, const int* N
     return n;
 }
 
+extern "C" int rabit_selftest_gemm_ready(int stream, int pass, int passes, int* parity_out) {
+    rabit_clear_error();
+    if (!parity_out) return rabit_fail(RABIT_INVALID_ARG, "rabit_selftest_gemm_ready: parity_out is NULL");
+    if (pass < 0 || pass >= passes) return rabit_fail(RABIT_INVALID_ARG, "rabit_selftest_gemm_ready: pass %d of %d", pass, passes);
+    return rabit_gemm_tc_ready(stream != 0, pass, pass == passes - 1, parity_out);
+}
+
 extern "C" int rabit_selftest_stream_read(const void* src_dev, size_t bytes, unsigned int* sink_dev, void* stream) {
     rabit_clear_error();
     if (!src_dev || ((uintptr_t)src_dev & 15u)) return rabit_fail(RABIT_INVALID_ARG, "rabit_selftest_stream_read: src_dev must be a 16-byte aligned device pointer");

@@ -2,6 +2,7 @@
 yields must cover the layer exactly once, and the number of contributions at which an accumulate word counts as complete must
 be the number that arrive.  The view and the kernel share the walk and the count."""
 import collections
+import ctypes
 import random
 
 import numpy as np
@@ -112,6 +113,32 @@ def test_random_groups_and_every_split_that_is_weighed():
                 assert candidate >= 1
                 break
             check_ranges(p, shapes, sms)
+
+
+@pytest.mark.parametrize("stream", [0, 1])
+def test_nobody_waits_for_a_phase_further_off_than_the_next(stream):
+    """A wait by parity cannot tell a phase from the one two before it, so a warp that waits for a barrier must wait for every phase
+    of it in turn.  One phase completes per pass that the barrier belongs to; with ranges of pairs one group of warps publishes all passes but
+    the last, another (which may come to it passes ahead of the MMAs) the last."""
+    lib = binding.raw_lib()
+    parity = ctypes.c_int()
+    for passes in range(1, 12):
+        ready = []
+        for i in range(passes):
+            ready.append((lib.rabit_selftest_gemm_ready(stream, i, passes, ctypes.byref(parity)), parity.value))
+            assert ready[i][0] >= 0
+        phase, of_bar = [], collections.Counter()
+        for bar, _ in ready:
+            phase.append(of_bar[bar])
+            of_bar[bar] += 1
+        for role in ([range(passes - 1), range(passes - 1, passes)] if stream else [range(passes)]):
+            waited = collections.Counter()
+            for i in role:
+                bar, par = ready[i]
+                assert phase[i] == waited[bar], f"pass {i} of {passes}: the wait is {phase[i] - waited[bar]} phases on from the last"
+                assert par == phase[i] & 1
+                waited[bar] += 1
+    assert lib.rabit_selftest_gemm_ready(stream, 3, 3, ctypes.byref(parity)) == -1 and lib.rabit_selftest_gemm_ready(stream, 0, 1, None) == -1
 
 
 def test_what_the_view_refuses():

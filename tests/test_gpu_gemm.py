@@ -162,3 +162,54 @@ def test_one_path_accumulators(N, batch):
     L = make_layer(700, N, 1, key=(66, N))
     x = make_x(batch, N, key=(66, N, batch))
     check_against_oracle(L, x, run_layer(L, x, GEMM))
+
+
+@pytest.mark.parametrize("K,shapes,variant,passes", [
+    (1, [(56832, 64)], 0, 3),           # three passes of one unit in every CTA: of the four expanding groups one has no unit at all
+    (1, [(128256, 64)], 0, 7),
+    (2, [(128256, 64)], 0, 7),
+    (2, [(128256, 128)], GEMM, 7),
+    (2, [(128256, 64)], 4, 7),          # (dequantised: one unit a step)
+    (3, [(57000, 64)], 0, 4),           # three paths: a fourth group that never has a unit
+    (3, [(77000, 64)], 0, 5),
+    (3, [(40000, 288)], GEMM, 3),
+    (1, [(14336, 64)] * 4, 0, 4),
+    (2, [(11008, 64)] * 4, 0, 3),
+    (3, [(14336, 512)] * 3, 0, 3),
+])
+def test_short_passes_are_published_complete(K, shapes, variant, passes):
+    """Ranges of several short passes, whose expanding warps are far ahead of the MMAs when they come to publish the last one: it must not be read
+    before its MMAs are done.  Other activations in every call, and another layer in between, so that what an earlier launch left in
+    tensor memory is never the right answer."""
+    import torch
+    import paper_2602_05367_b200 as rabit
+    from tests.test_gemm_plan import plan
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    if sms == 148:
+        listed = plan(shapes, K, 16, deq=int(variant == 4)).passes[:, 0].tolist()
+        assert max(listed.count(t) for t in set(listed)) == passes
+    Ls = [make_layer(M, N, K, key=(67, i, K, M, N)) for i, (M, N) in enumerate(shapes)]
+    between = make_layer(2560, 8192, K, key=(68, K))
+    layers = [rabit.rabit_pack(L.planes, L.g, L.h) for L in Ls]
+    other = rabit.rabit_pack(between.planes, between.g, between.h)
+    xo = torch.from_numpy(make_x(16, 8192, key=(68,))).cuda()
+    for layer in layers:
+        layer.set_variant(variant)
+    N = shapes[0][1]
+    xs = [make_x(16, N, key=(67, N, i)) for i in range(4)]
+    xd = [torch.from_numpy(x).cuda() for x in xs]
+    ys = [[torch.zeros((16, M), dtype=torch.float16, device="cuda") for M, _ in shapes] for _ in xs]
+    for i, x in enumerate(xd):
+        if i & 1:
+            rabit.rabit_linear(other, xo)
+        if len(layers) == 1:
+            rabit.rabit_linear(layers[0], x, ys[i][0])
+        else:
+            rabit.rabit_linear_group(layers, [x] * len(layers), ys[i])
+    torch.cuda.synchronize()
+    for x, y in zip(xs, ys):
+        for L, layer, yl in zip(Ls, layers, y):
+            assert layer.status() == 0, rabit.last_error()
+            check_against_oracle(L, x, yl.cpu().numpy(), tight=variant != 4)
+    for layer in layers + [other]:
+        layer.free()
