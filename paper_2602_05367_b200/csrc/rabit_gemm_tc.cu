@@ -1059,11 +1059,12 @@ int resident_clusters(const void* kernel, int threads, int split, size_t smem, i
 constexpr double kPassClocks = 3000.0;               // pipeline fill and epilogue of a pass that nothing overlaps
 constexpr double kLaunchClocks = 8000.0;             // launch, first loads, last epilogue
 constexpr double kExchangeClocks = 2500.0;           // exchange of a split task
-// Streams, fitted to 25 shapes x every task count (B200, 9 to 16 rows; 4 % rms, the split it picks 0.3 % slower than the best on average):
-// launch, unit of one, two or three paths, a further pass in a range, publishing parts of row tiles besides its throughput and that (sums per clock
-// over the GPU).  Before the epilogues had warps of their own a further pass cost 3000 and ranges that cross row tiles were avoided: 11008 x 4096
-// at 16 rows 14.7 -> 13.5 us, 14336 x 4096 with three paths 20.3 -> 18.9.
-constexpr double kStreamLaunch = 5600.0, kStreamUnit[3] = {199.0, 170.0, 166.0}, kStreamPass = 1300.0, kStreamPublish = 800.0, kStreamRate = 130.0;
+// Streams, fitted to 470 shapes (128 to 28672 rows, 64 to 13824 columns, one to three paths, 9 and 16 batch rows) x their task counts (B200): launch, unit of
+// one, two or three paths, a further pass in a range; and where a range ends in a part of a row tile, publishing that part (the atomics and their
+// answers; those of earlier parts run beside the next pass) and the throughput of all such ends, in sums per clock over the GPU.  The split that
+// they pick is 0.2 % slower than the best on average, 4.5 % at most.  (Every part counted, publishing at 800 clocks, a pass at 1300: 1.0 % and 17 %;
+// 256 x 512 with two paths, whose two slices are better not split, 3.75 against 4.35 us, 14336 x 4096 with three paths 20.0 on 112 tasks against 18.55 on 148.)
+constexpr double kStreamLaunch = 5600.0, kStreamUnit[3] = {195.0, 185.0, 175.0}, kStreamPass = 1150.0, kStreamPublish = 2050.0, kStreamRate = 140.0;
 
 // Task counts worth an estimate: equal parts of every row tile (or nearly), and one task per SM.  Never more tasks than pairs: an
 // empty one would count among the arrivals of a row tile that it does not contribute to.  (Layers of unlike widths: parts for the
@@ -1101,19 +1102,19 @@ Plan stream_plan(int n_layers, const int* n_rt, const int* n_ct, int K, bool deq
         if (candidate >= 0 && considered++ != candidate) return;
         p.tasks = (int)tasks;
         double worst = 0.0;
-        long long parts = 0, base = 0, t = 0;             // segments that are not whole row tiles
+        long long parts = 0, base = 0, t = 0;             // tasks that end in a segment that is not a whole row tile
         int l = 0;
         double c = 0.0;
         for (long long at = 0; at < pairs;) {             // segment by segment
             const int n_cs = ((n_ct[l] + 1) / 2 + kSliceSteps - 1) / kSliceSteps;
             const long long t_end = pairs * (t + 1) / tasks, tile_end = at + n_cs - (at - base) % n_cs, end = std::min(t_end, tile_end);
             c += (double)(end - at) * pair + (c > 0.0 ? kStreamPass : 0.0);
-            parts += end - at < n_cs;
+            const bool part = end - at < n_cs;
             at = end;
             if (at == base + (long long)n_rt[l] * n_cs && l + 1 < n_layers) { base = at; ++l; }
-            if (at == t_end) { worst = std::max(worst, c); c = 0.0; ++t; }
+            if (at == t_end) { worst = std::max(worst, c + (part ? kStreamPublish : 0.0)); parts += part; c = 0.0; ++t; }
         }
-        p.clocks = kStreamLaunch + worst + (parts > 0 ? kStreamPublish + parts * 128.0 * batch / kStreamRate : 0.0);
+        p.clocks = kStreamLaunch + worst + parts * 128.0 * batch / kStreamRate;
         if (p.clocks < best.clocks) best = p;
     });
     return best;
