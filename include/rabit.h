@@ -122,8 +122,6 @@ RABIT_API int rabit_derive_pack(const float* W_dev, const uint16_t* g, const uin
  * GEMM launch, whichever the library's cost estimate for the shape favours.  A GEMM with few output tiles splits a tile's
  * contraction over CTAs.  fp32 (or exact integer) accumulation, one rounding to fp16 at the end;
  * an inf or NaN in a batch row of x makes that row of y non-finite and leaves the other rows untouched.
- * A layer may have been packed with an infinite or NaN scale: the outputs that it takes part in are then infinite or NaN (above
- * 16 rows infinite, with the sign that +-1 gives it, where the sum is).
  */
 RABIT_API int rabit_linear(const rabit_layer* layer, const void* x, void* y, int batch, void* stream);
 

@@ -58,7 +58,6 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
-#include <cmath>
 #include <cstddef>
 #include <type_traits>
 #include <vector>
@@ -270,10 +269,8 @@ __host__ __device__ __forceinline__ int segment_arrivals(uint32_t first, uint32_
 // its own x, of which the layers may share one).  SEQ (an instance with K = 1): path-major, for three paths.  Three accumulators
 // leave room for 8 groups of columns at most, so wider batches expanded every tile two or three times; here a task
 // is a pass per path on one accumulator, the sum of the scaled passes stays in tensor memory beside it, and up to 13 groups fit
-// (5000 x 13824 at batch 200: each tile expanded once instead of three times).  FINITE: no input scale is infinite.  (The instances for layers with
-// an infinite one, whose outputs are then infinite or NaN too, take another way of flipping half the signs.  That way for all layers
-// costs 5 %, 28672 x 8192 at 16 rows 40.1 -> 42.3 us, and a branch between the two inside the loop 2 %, with three paths 10.)
-template <int K, bool DEQ, int NL, bool SEQ, bool FINITE>
+// (5000 x 13824 at batch 200: each tile expanded once instead of three times).
+template <int K, bool DEQ, int NL, bool SEQ>
 __global__ void __launch_bounds__(threads_of((DEQ || K == 1) && !SEQ, NL > 1), 1)
 rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_constant__ XMaps<NL> x_maps) {
     extern __shared__ unsigned char smem_raw[];
@@ -675,10 +672,8 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                                     // bytes [0, c0, 0, c1]: row block 2q + 1's bits at 15 and 31, row block 2q's one below, nothing else
                                     const uint32_t v = __byte_perm(word[2 * ah + rh], 0u, pair ? 0x3424 : 0x1404);
                                     const uint32_t hp = pair ? t.h[ah].y : t.h[ah].x, odd = (v & 0x80008000u) ^ hp;
-                                    // As an fp16 number v is 0 or 2 (the bit at 14) with the sign that odd has beside h, so h - v * odd is h or h - 2 h, exact for every
-                                    // finite h; an infinite one has to be multiplied with the sign, 1 - |v|
-                                    const __half2 h2 = *reinterpret_cast<const __half2*>(&hp), v2 = *reinterpret_cast<const __half2*>(&v);
-                                    const __half2 even2 = FINITE ? __hfma2(v2, __hneg2(*reinterpret_cast<const __half2*>(&odd)), h2) : __hmul2(h2, __hsub2(__float2half2_rn(1.f), __habs2(v2)));
+                                    // As an fp16 number v is 0 or 2 (the bit at 14) with the sign that odd has beside h, so h - v * odd is h or h - 2 h (exact)
+                                    const __half2 even2 = __hfma2(*reinterpret_cast<const __half2*>(&v), __hneg2(*reinterpret_cast<const __half2*>(&odd)), *reinterpret_cast<const __half2*>(&hp));
 #pragma unroll
                                     for (int pi = 0; pi < 2; ++pi) {
                                         const __half2 m = pi ? *reinterpret_cast<const __half2*>(&odd) : even2;
@@ -1008,32 +1003,23 @@ double unit_clocks(int n16, const Plan& p, int n_ops) {
     return std::max(32.0 * n16 + 52.0, p.units >= 2 * (n_ops == 3 ? 3 : 4) ? 180.0 + 8.0 * n16 : n_ops == 3 ? 345.0 : 300.0);
 }
 
-// (stream: the form for contiguous ranges of up to kMaxGroup layers; finite: no layer has an infinite input scale)
-template <int NL, bool FINITE>
+// (stream: the form for contiguous ranges of up to kMaxGroup layers)
+template <int NL>
 const void* kernel_of(int K, bool deq) {
-    if (K == 1) return deq ? (const void*)rabit_gemm_tc_kernel<1, true, NL, false, FINITE> : (const void*)rabit_gemm_tc_kernel<1, false, NL, false, FINITE>;
-    if (K == 2) return deq ? (const void*)rabit_gemm_tc_kernel<2, true, NL, false, FINITE> : (const void*)rabit_gemm_tc_kernel<2, false, NL, false, FINITE>;
-    return deq ? (const void*)rabit_gemm_tc_kernel<3, true, NL, false, FINITE> : (const void*)rabit_gemm_tc_kernel<3, false, NL, false, FINITE>;
+    if (K == 1) return deq ? (const void*)rabit_gemm_tc_kernel<1, true, NL, false> : (const void*)rabit_gemm_tc_kernel<1, false, NL, false>;
+    if (K == 2) return deq ? (const void*)rabit_gemm_tc_kernel<2, true, NL, false> : (const void*)rabit_gemm_tc_kernel<2, false, NL, false>;
+    return deq ? (const void*)rabit_gemm_tc_kernel<3, true, NL, false> : (const void*)rabit_gemm_tc_kernel<3, false, NL, false>;
 }
-template <bool FINITE>
-const void* kernel_of(int K, bool deq, bool stream, bool seq) {
-    return seq ? (const void*)rabit_gemm_tc_kernel<1, false, 1, true, FINITE> : stream ? kernel_of<kMaxGroup, FINITE>(K, deq) : kernel_of<1, FINITE>(K, deq);
-}
-const void* kernel_for(int K, bool deq, bool stream, bool seq, bool finite) {
-    return finite ? kernel_of<true>(K, deq, stream, seq) : kernel_of<false>(K, deq, stream, seq);
-}
-bool finite_scales(const rabit_layer& L) {
-    for (int k = 0; k < L.geom.K; ++k)
-        if (!(L.geom.hmax[k] < HUGE_VALF)) return false;
-    return true;
+const void* kernel_for(int K, bool deq, bool stream = false, bool seq = false) {
+    return seq ? (const void*)rabit_gemm_tc_kernel<1, false, 1, true> : stream ? kernel_of<kMaxGroup>(K, deq) : kernel_of<1>(K, deq);
 }
 
 // Function attributes are per device.
-cudaError_t prepare_kernel(int K, bool deq, int device, bool stream, bool seq, bool finite) {
-    static bool done[64][26] = {};
-    const int slot = device >= 0 && device < 64 ? device : 0, inst = (seq ? 12 : 4 * (K - 1) + (stream ? 2 : 0) + (deq ? 1 : 0)) + (finite ? 0 : 13);
+cudaError_t prepare_kernel(int K, bool deq, int device, bool stream = false, bool seq = false) {
+    static bool done[64][13] = {};
+    const int slot = device >= 0 && device < 64 ? device : 0, inst = seq ? 12 : 4 * (K - 1) + (stream ? 2 : 0) + (deq ? 1 : 0);
     if (done[slot][inst] && slot == device) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(kernel_for(K, deq, stream, seq, finite), cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(kernel_for(K, deq, stream, seq), cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
     if (e == cudaSuccess) done[slot][inst] = true;
     return e;
 }
@@ -1145,7 +1131,7 @@ Plan make_plan(int n_rt, int n_steps, int K, bool deq, int batch, int sms, int d
                 const long long ctas = (long long)p.tasks * split;
                 if (split > 1 && (n_steps / split < 4 || ctas > sms)) continue;
                 if (!fill_resources(p, seq ? 1 : K, seq ? 1 : n_ops, n_steps / split, wide_x)) continue;
-                if (split > 1 && device >= 0 && (prepare_kernel(K, deq, device, false, seq != 0, true) != cudaSuccess || resident_clusters(kernel_for(K, deq, false, seq != 0, true), threads_of(n_ops == 1 && !seq, false), split, p.smem, sms) < p.tasks)) continue;
+                if (split > 1 && device >= 0 && (prepare_kernel(K, deq, device, false, seq != 0) != cudaSuccess || resident_clusters(kernel_for(K, deq, false, seq != 0), threads_of(n_ops == 1 && !seq, false), split, p.smem, sms) < p.tasks)) continue;
                 const double rounds = (double)((ctas + sms - 1) / sms);
                 p.clocks = kLaunchClocks + (split > 1 ? kExchangeClocks * (1 + seq) : 0.0) + rounds * ((n_steps + split - 1) / split) * n_ops * unit_clocks(p.chunk16, p, seq ? 1 : n_ops) +
                            (rounds * (seq ? K : 1) - 1.0) * kPassClocks;
@@ -1345,9 +1331,7 @@ static cudaError_t launch_stream(const rabit_layer* const* layers, int n_layers,
         pairs += G.n_rt * G.n_cs;
     }
     fill_common(P, p, n_layers, batch, pairs, layers[0]->withhold);
-    bool finite = true;
-    for (int l = 0; l < n_layers; ++l) finite = finite && finite_scales(*layers[l]);
-    cudaError_t e = prepare_kernel(K, dequantised, device, true, false, finite);
+    cudaError_t e = prepare_kernel(K, dequantised, device, true);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned int)p.tasks);
@@ -1360,7 +1344,7 @@ static cudaError_t launch_stream(const rabit_layer* const* layers, int n_layers,
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     void* args[2] = {&P, &maps};
-    return cudaLaunchKernelExC(&cfg, kernel_for(K, dequantised, true, false, finite), args);
+    return cudaLaunchKernelExC(&cfg, kernel_for(K, dequantised, true), args);
 }
 
 cudaError_t rabit_launch_gemm_tc_group(const rabit_layer* const* layers, int n_layers, const void* const* xs, void* const* ys, int batch, cudaStream_t stream) {
@@ -1389,8 +1373,7 @@ cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, i
     XMaps<1> maps;
     cudaError_t e = x_tensor_map(x, G.N, batch, p.box16, p.x_steps, &maps.map[0]);
     if (e != cudaSuccess) return e;
-    const bool finite = finite_scales(L);
-    e = prepare_kernel(G.K, dequantised, L.device, false, p.seq != 0, finite);
+    e = prepare_kernel(G.K, dequantised, L.device, false, p.seq != 0);
     if (e != cudaSuccess) return e;
 
     GemmParams<1> P;
@@ -1413,5 +1396,5 @@ cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, i
     cfg.attrs = attr;
     cfg.numAttrs = p.split > 1 ? 2 : 1;
     void* args[2] = {&P, &maps};
-    return cudaLaunchKernelExC(&cfg, kernel_for(G.K, dequantised, false, p.seq != 0, finite), args);
+    return cudaLaunchKernelExC(&cfg, kernel_for(G.K, dequantised, false, p.seq != 0), args);
 }
