@@ -82,9 +82,11 @@ constexpr int kExpandGroups = 4;            // of four warps each
 constexpr int kExpandWarps = 4 * kExpandGroups;
 constexpr int kFourthIssuer = 4 + kExpandWarps;
 constexpr int kMaxAcc = 4;                  // accumulators
-// Threads of an instance: one operand per step (one path, or the dequantised form) has a fourth issuing warp, stream kernels four warps
-// for the epilogues.
-__host__ __device__ constexpr int threads_of(bool one_op, bool stream) { return (kFourthIssuer + (one_op ? 1 : 0) + (stream ? 4 : 0)) * 32; }
+// Most accumulators of an instance.  The dequantised form of several paths, one operand per step too, has two: its expanders have more to do for
+// a step than an issuing warp (with four, two paths 14336 x 4096 at 40 rows 16.5 -> 17.0 us).
+__host__ __device__ constexpr int most_acc(int K, bool deq, bool seq) { return seq ? 1 : !deq ? (K == 1 ? kMaxAcc : K) : K == 1 ? kMaxAcc : 2; }
+// Threads of an instance: a fourth issuing warp if there may be four accumulators, in stream kernels four warps for the epilogues.
+__host__ __device__ constexpr int threads_of(int K, bool deq, bool seq, bool stream) { return (kFourthIssuer + (most_acc(K, deq, seq) > 3 ? 1 : 0) + (stream ? 4 : 0)) * 32; }
 constexpr unsigned long long kSumMask = (1ULL << 55) - 1;
 
 constexpr int kMaxTasks = 512;
@@ -271,7 +273,7 @@ __host__ __device__ __forceinline__ int segment_arrivals(uint32_t first, uint32_
 // is a pass per path on one accumulator, the sum of the scaled passes stays in tensor memory beside it, and up to 13 groups fit
 // (5000 x 13824 at batch 200: each tile expanded once instead of three times).
 template <int K, bool DEQ, int NL, bool SEQ>
-__global__ void __launch_bounds__(threads_of((DEQ || K == 1) && !SEQ, NL > 1), 1)
+__global__ void __launch_bounds__(threads_of(K, DEQ, SEQ, NL > 1), 1)
 rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_constant__ XMaps<NL> x_maps) {
     extern __shared__ unsigned char smem_raw[];
     // the swizzled x tiles need 1024-byte alignment; the launch reserves the slack
@@ -292,7 +294,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
     unsigned char* w_ring = ring + P.stages * P.stage_bytes;
     constexpr int n_ops = DEQ ? 1 : K;                            // operand units (and accumulators) per step
     constexpr int n_groups = n_ops == 3 || SEQ ? 3 : 4;                  // expander groups at work
-    constexpr int n_fourth = n_ops == 1 && !SEQ ? 1 : 0;                 // whether there is a fourth issuing warp
+    constexpr int max_acc = most_acc(K, DEQ, SEQ), n_fourth = max_acc > 3 ? 1 : 0;   // (n_fourth: whether there is a fourth issuing warp)
     const int stages = P.stages, w_stages = P.w_stages, units = P.units, x_steps = P.x_steps, n_acc = P.n_acc;
     const int stage_bytes = P.stage_bytes;
     volatile int* abort_flag = &S.abort_flag;
@@ -369,7 +371,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
 #pragma unroll
         for (int i = 0; i < n; ++i) v[i] = 0.f;
 #pragma unroll
-        for (int m = 0; m < (n_ops == 1 ? kMaxAcc : n_ops); ++m) {
+        for (int m = 0; m < max_acc; ++m) {
             if (n_ops == 1 && m >= n_acc) break;
             uint32_t d[n];
             if constexpr (n == 16) tmem_ld16(from + (uint32_t)(m * kGroupCols), d);
@@ -662,7 +664,9 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                     };
                     // a tile of path kk into operand registers o[row block][16-column half, row half, column pair]
                     auto expand = [&](const TileIn& t, int kk, uint32_t (&o)[2][8]) {
-                        const uint32_t word[4] = {mul_lo(t.w.x & keep, up), mul_lo(t.w.y & keep, up), mul_lo(t.w.z & keep, up), mul_lo(t.w.w & keep, up)};
+                        // (dequantised, three paths: the multiply-add pipe has enough to do already, 14336 x 4096 at 16 rows 21.2 -> 20.9 us; wider passes 6 % slower)
+                        auto top = [&](uint32_t w) { return DEQ && K == 3 && NL > 1 ? (w & keep) << (6 - 2 * q) : mul_lo(w & keep, up); };
+                        const uint32_t word[4] = {top(t.w.x), top(t.w.y), top(t.w.z), top(t.w.w)};
 #pragma unroll
                         for (int ah = 0; ah < 2; ++ah)
 #pragma unroll
@@ -779,7 +783,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                     for (int i = 0; i < 16; ++i) v[i] = 0.f;
                     if constexpr (SEQ) path_sum(c, v);
 #pragma unroll
-                    for (int m = 0; m < (n_ops == 1 ? kMaxAcc : n_ops); ++m) {
+                    for (int m = 0; m < max_acc; ++m) {
                         if (n_ops == 1 && m >= n_acc) break;
                         uint32_t d[16];
                         tmem_ld16(lane_base + (uint32_t)((m * P.max16 + c) * kGroupCols), d);
@@ -838,7 +842,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                 for (int i = 0; i < 16; ++i) v[i] = 0.f;
                 if constexpr (SEQ) path_sum(c, v);
 #pragma unroll
-                for (int m = 0; m < (n_ops == 1 ? kMaxAcc : n_ops); ++m) {
+                for (int m = 0; m < max_acc; ++m) {
                     if (n_ops == 1 && m >= n_acc) break;
                     uint32_t d[16];
                     tmem_ld16(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)((m * P.max16 + c) * kGroupCols), d);
@@ -954,7 +958,8 @@ struct Plan {
 
 // Ring, tensor-memory and shared-memory figures of passes of up to max16 groups; false if they do not fit.  The units are a
 // multiple of the expander groups and of the accumulators (see Walk).
-bool fill_resources(Plan& p, int K, int n_ops, int steps, bool one_box) {
+bool fill_resources(Plan& p, int K, bool deq, int steps, bool one_box) {
+    const int n_ops = deq || p.seq ? 1 : K;
     const int recv_bytes = p.split > 1 ? (p.chunk16 + p.split - 1) / p.split * p.split * kGroupCols * kTileM * 4 : 0;
     if (p.max16 * kGroupCols > 256) return false;
     const int turn = n_ops == 3 || p.seq ? 3 : 4;
@@ -967,7 +972,7 @@ bool fill_resources(Plan& p, int K, int n_ops, int steps, bool one_box) {
     // with two paths, whose two warps issue pairs of units, four of them are 2 to 4 % slower).
     p.n_acc = n_ops;
     if (n_ops == 1 && !p.seq)
-        for (int more = 2; more <= (one_box && (p.stream || steps >= 24) ? kMaxAcc : 2) && steps >= more && free_units(more) >= (more == 2 ? turn : 2 * turn); more *= 2) p.n_acc = more;
+        for (int more = 2; more <= std::min(most_acc(K, deq, false), one_box && (p.stream || steps >= 24) ? kMaxAcc : 2) && steps >= more && free_units(more) >= (more == 2 ? turn : 2 * turn); more *= 2) p.n_acc = more;
     if (free_units(p.n_acc) < turn) return false;
     p.units = free_units(p.n_acc) >= 2 * turn ? 2 * turn : turn;
     const int step_bytes = (p.max16 + p.box16 - 1) / p.box16 * p.box16 * kGroupCols * kStepCols * 2;
@@ -1080,7 +1085,7 @@ Plan stream_plan(int n_layers, const int* n_rt, const int* n_ct, int K, bool deq
         if (steps % kSliceSteps != 0) tail = std::min(tail, steps % kSliceSteps);
         wide_x = wide_x && n_ct[l] % 2 == 0;
     }
-    if (most_cs > RABIT_LUT_MAX_SLICES || pairs >= kMaxPairs || sms > kMaxTasks || !fill_resources(p, K, n_ops, tail, wide_x)) return best;
+    if (most_cs > RABIT_LUT_MAX_SLICES || pairs >= kMaxPairs || sms > kMaxTasks || !fill_resources(p, K, deq, tail, wide_x)) return best;
     best.clocks = 1e300;
     const double pair = kSliceSteps * n_ops * kStreamUnit[n_ops - 1];
     int considered = 0;
@@ -1130,8 +1135,8 @@ Plan make_plan(int n_rt, int n_steps, int K, bool deq, int batch, int sms, int d
                 p.tasks = n_rt * chunks;
                 const long long ctas = (long long)p.tasks * split;
                 if (split > 1 && (n_steps / split < 4 || ctas > sms)) continue;
-                if (!fill_resources(p, seq ? 1 : K, seq ? 1 : n_ops, n_steps / split, wide_x)) continue;
-                if (split > 1 && device >= 0 && (prepare_kernel(K, deq, device, false, seq != 0) != cudaSuccess || resident_clusters(kernel_for(K, deq, false, seq != 0), threads_of(n_ops == 1 && !seq, false), split, p.smem, sms) < p.tasks)) continue;
+                if (!fill_resources(p, seq ? 1 : K, deq, n_steps / split, wide_x)) continue;
+                if (split > 1 && device >= 0 && (prepare_kernel(K, deq, device, false, seq != 0) != cudaSuccess || resident_clusters(kernel_for(K, deq, false, seq != 0), threads_of(K, deq, seq != 0, false), split, p.smem, sms) < p.tasks)) continue;
                 const double rounds = (double)((ctas + sms - 1) / sms);
                 p.clocks = kLaunchClocks + (split > 1 ? kExchangeClocks * (1 + seq) : 0.0) + rounds * ((n_steps + split - 1) / split) * n_ops * unit_clocks(p.chunk16, p, seq ? 1 : n_ops) +
                            (rounds * (seq ? K : 1) - 1.0) * kPassClocks;
@@ -1150,9 +1155,9 @@ Plan make_plan(int n_rt, int n_steps, int K, bool deq, int batch, int sms, int d
             // most passes of a range are cut to this size: two boxes of it make one step
             const int run = std::min(per_sm, n16), pieces = (run + p.max16 - 1) / p.max16;
             p.box16 = ((run + pieces - 1) / pieces + 1) / 2;
-            if (fill_resources(p, K, n_ops, n_steps, false)) break;
+            if (fill_resources(p, K, deq, n_steps, false)) break;
         }
-        if (fill_resources(p, K, n_ops, n_steps, false)) {
+        if (fill_resources(p, K, deq, n_steps, false)) {
             double worst = 0.0;
             for (int t = 0; t < sms; ++t) {
                 long long g = groups * t / sms;
@@ -1335,7 +1340,7 @@ static cudaError_t launch_stream(const rabit_layer* const* layers, int n_layers,
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned int)p.tasks);
-    cfg.blockDim = dim3((unsigned int)threads_of(K == 1 || dequantised, true));
+    cfg.blockDim = dim3((unsigned int)threads_of(K, dequantised, false, true));
     cfg.dynamicSmemBytes = p.smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -1383,7 +1388,7 @@ cudaError_t rabit_launch_gemm_tc(const rabit_layer& L, const void* x, void* y, i
 
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned int)(p.tasks * p.split));
-    cfg.blockDim = dim3((unsigned int)threads_of((G.K == 1 || dequantised) && !p.seq, false));
+    cfg.blockDim = dim3((unsigned int)threads_of(G.K, dequantised, p.seq != 0, false));
     cfg.dynamicSmemBytes = p.smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];

@@ -145,7 +145,7 @@ def test_gemm_split_contraction_across_a_cluster(K, M, N, batch, variant):
 @pytest.mark.parametrize("K,M,N,batch", [
     (1, 77000, 64, 9),       # four or five row tiles in every CTA's range, one step each
     (2, 38000, 544, 13),     # six (row tile, slice) pairs a CTA: parts of row tiles at both ends, a whole one between, last step half
-    (3, 25700, 288, 16),
+    (3, 25700, 288, 16),     # one or two passes (more of them: test_short_passes_are_published_complete)
 ])
 def test_several_row_tiles_in_a_range(K, M, N, batch):
     """Up to 16 rows: passes alternate between two sets of accumulators, and all but a CTA's last are published beside the next."""
@@ -157,11 +157,29 @@ def test_several_row_tiles_in_a_range(K, M, N, batch):
 @pytest.mark.parametrize("batch", [16, 40, 64, 65])
 @pytest.mark.parametrize("N", [64, 160, 320, 384, 448, 1024])
 def test_one_path_accumulators(N, batch):
-    """One operand per step: one, two or four accumulators, by the steps of the shortest pass (a last slice of one to four steps, fewer steps
-    than accumulators) and by the room that 64 and 65 columns leave."""
+    """One operand per step: one, two or four accumulators up to 16 rows, by the steps of the shortest pass (a last slice of one to four steps, fewer
+    steps than accumulators); one or two beyond (four: test_four_accumulators)."""
     L = make_layer(700, N, 1, key=(66, N))
     x = make_x(batch, N, key=(66, N, batch))
     check_against_oracle(L, x, run_layer(L, x, GEMM))
+
+
+@pytest.mark.parametrize("K,M,N,batch,variant,split", [
+    (1, 14336, 1536, 33, GEMM, 1), (1, 14336, 1536, 64, GEMM, 1),    # 24 steps, the fewest
+    (1, 9000, 1600, 48, GEMM, 1),                                    # 25 steps: a unit more in the first accumulator
+    (1, 300, 16384, 33, GEMM, 8), (1, 600, 15488, 20, GEMM, 8),      # over clusters: 32 steps a CTA, 30 or 31
+    (1, 14336, 1536, 48, DEQ, 1), (1, 600, 16384, 20, DEQ, 8),
+])
+def test_four_accumulators(K, M, N, batch, variant, split):
+    """One path, more than 16 rows, a long contraction: a fourth issuing warp, the sums of four accumulators added."""
+    import torch
+    from tests.test_gemm_plan import plan
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        p = plan([(M, N)], K, batch, deq=int(variant == DEQ))
+        assert (p.n_acc, p.split, p.stream) == (4, split, 0)
+    L = make_layer(M, N, K, key=(70, K, M, N))
+    x = make_x(batch, N, key=(70, N, batch))
+    check_against_oracle(L, x, run_layer(L, x, variant), tight=variant != DEQ)
 
 
 @pytest.mark.parametrize("K,shapes,variant,passes", [
