@@ -122,6 +122,8 @@ RABIT_API int rabit_derive_pack(const float* W_dev, const uint16_t* g, const uin
  * GEMM launch, whichever the library's cost estimate for the shape favours.  A GEMM with few output tiles splits a tile's
  * contraction over CTAs.  fp32 (or exact integer) accumulation, one rounding to fp16 at the end;
  * an inf or NaN in a batch row of x makes that row of y non-finite and leaves the other rows untouched.
+ * Scales are meant to be finite: the outputs that an infinite or NaN scale takes part in are infinite or NaN, which of the two
+ * depends on the kernel.
  */
 RABIT_API int rabit_linear(const rabit_layer* layer, const void* x, void* y, int batch, void* stream);
 

@@ -676,7 +676,7 @@ rabit_gemm_tc_kernel(const __grid_constant__ GemmParams<NL> P, const __grid_cons
                                     // bytes [0, c0, 0, c1]: row block 2q + 1's bits at 15 and 31, row block 2q's one below, nothing else
                                     const uint32_t v = __byte_perm(word[2 * ah + rh], 0u, pair ? 0x3424 : 0x1404);
                                     const uint32_t hp = pair ? t.h[ah].y : t.h[ah].x, odd = (v & 0x80008000u) ^ hp;
-                                    // As an fp16 number v is 0 or 2 (the bit at 14) with the sign that odd has beside h, so h - v * odd is h or h - 2 h (exact)
+                                    // As an fp16 number v is 0 or 2 (the bit at 14) with the sign that odd has beside h, so h - v * odd is h or h - 2 h (exact; NaN if h is infinite)
                                     const __half2 even2 = __hfma2(*reinterpret_cast<const __half2*>(&v), __hneg2(*reinterpret_cast<const __half2*>(&odd)), *reinterpret_cast<const __half2*>(&hp));
 #pragma unroll
                                     for (int pi = 0; pi < 2; ++pi) {

@@ -231,3 +231,12 @@ def test_short_passes_are_published_complete(K, shapes, variant, passes):
             check_against_oracle(L, x, yl.cpu().numpy(), tight=variant != 4)
     for layer in layers + [other]:
         layer.free()
+
+
+@pytest.mark.parametrize("K,batch,variant", [(1, 1, 0), (2, 2, 0), (3, 5, 0), (1, 9, 0), (2, 16, 0), (3, 16, 0), (1, 17, 0), (2, 40, 0), (3, 200, 0), (2, 16, DEQ), (2, 40, DEQ)])
+def test_infinite_input_scale(K, batch, variant):
+    """One infinite input scale: every output that it takes part in (all of them) is infinite or NaN, in every kernel."""
+    M, N = 400, 1088
+    L = make_layer(M, N, K, key=(69, K))
+    L.h[K - 1, 77] = np.float16(np.inf)
+    assert not np.isfinite(run_layer(L, make_x(batch, N, key=(69, batch)), variant)).any()
