@@ -26,7 +26,7 @@ def test_small_shapes_pass_under_the_checked_build():
     cmd = [sys.executable, "-m", "pytest", "-x", "-q", "-m", "gpu", os.path.join(ROOT, "tests", "test_gpu_parity.py"),
            os.path.join(ROOT, "tests", "test_gpu_group.py"), os.path.join(ROOT, "tests", "test_gpu_failure.py"),
            os.path.join(ROOT, "tests", "test_gpu_gemm.py"), os.path.join(ROOT, "tests", "test_gpu_edges.py"),
-           "-k", "small_shapes or structured or outlier or repeated or group or withheld or gemm_shapes or small_batches or splits or dequantised"]
+           "-k", "small_shapes or structured or outlier or repeated or group or withheld or gemm_shapes or small_batches or splits or dequantised or several or accumulators or short_passes or two_rows"]
     proc = subprocess.run(cmd, cwd=ROOT, env=env, capture_output=True, text=True, timeout=1200)
     assert proc.returncode == 0, proc.stdout[-3000:] + proc.stderr[-2000:]
     assert " passed" in proc.stdout
