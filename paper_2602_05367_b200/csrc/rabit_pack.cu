@@ -46,15 +46,6 @@ bool rabit_make_geom(int K, int M, int N, RabitGeom* out) {
     return true;
 }
 
-// Everything the header records about the scales: max_j |h_k[j]| per path (the integer-MMA GEMV derives its
-// fixed-point scale from it) and the fixed-point grid of the table-driven GEMV's accumulate words.
-//
-// That GEMV adds, per output row, one partial sum per 256-column slice into a 64-bit word with an integer
-// atomic.  A partial sum is bounded, for ANY finite fp16 activations, by
-//     65504 * max_i sum_k |g_k[i]| * max_{k, slice} sum_{j in slice} |h_k[j]|,
-// so a grid of 2^unit_exp whose 2^fix_bits steps cover twice that bound can never overflow, and with
-// fix_bits = 54 - ceil(log2(slices)) the sum of all slices (each shifted to be non-negative) stays below 2^55.
-
 // |value| of every fp16 magnitude (sign bit cleared), converted once: the scans below are table look-ups
 static const float* half_magnitude_table() {
     static const std::vector<float> table = [] {
@@ -70,6 +61,14 @@ static uint32_t top_magnitude(const uint16_t* v, size_t n) {
     return (uint32_t)top;
 }
 
+// Everything the header records about the scales: max_j |h_k[j]| per path (the integer-MMA GEMV derives its
+// fixed-point scale from it) and the fixed-point grid of the table-driven GEMV's accumulate words.
+//
+// That GEMV adds, per output row, one partial sum per 256-column slice into a 64-bit word with an integer
+// atomic.  A partial sum is bounded, for ANY finite fp16 activations, by
+//     65504 * max_i sum_k |g_k[i]| * max_{k, slice} sum_{j in slice} |h_k[j]|,
+// so a grid of 2^unit_exp whose 2^fix_bits steps cover twice that bound can never overflow, and with
+// fix_bits = 54 - ceil(log2(slices)) the sum of all slices (each shifted to be non-negative) stays below 2^55.
 void rabit_scale_meta(const uint16_t* g, const uint16_t* h, int K, int M, int N, RabitGeom* G) {
     // per path the largest |h| (fp16 magnitudes order like their bit patterns; the first NaN wins and sticks, so a NaN scale makes
     // the bound NaN); the largest sum of |h| over a slice of 256 columns; the largest sum of |g| over the paths of a row
