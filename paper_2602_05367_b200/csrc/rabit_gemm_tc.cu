@@ -1055,7 +1055,8 @@ constexpr double kExchangeClocks = 2500.0;           // exchange of a split task
 // answers; those of earlier parts run beside the next pass) and the throughput of all such ends, in sums per clock over the GPU.  The split that
 // they pick is 0.2 % slower than the best on average, 4.5 % at most.  (Every part counted, publishing at 800 clocks, a pass at 1300: 1.0 % and 17 %;
 // 256 x 512 with two paths, whose two slices are better not split, 3.75 against 4.35 us, 14336 x 4096 with three paths 20.0 on 112 tasks against 18.55 on 148.)
-constexpr double kStreamLaunch = 5600.0, kStreamUnit[3] = {195.0, 185.0, 175.0}, kStreamPass = 1150.0, kStreamPublish = 2050.0, kStreamRate = 140.0;
+// The dequantised form's one unit a step takes kStreamDeq more for every path after the first (4096 x 4096 and 14336 x 4096 at 16 rows with one, two and three paths).
+constexpr double kStreamLaunch = 5600.0, kStreamUnit[3] = {195.0, 185.0, 175.0}, kStreamDeq = 210.0, kStreamPass = 1150.0, kStreamPublish = 2050.0, kStreamRate = 140.0;
 
 // Task counts worth an estimate: equal parts of every row tile (or nearly), and one task per SM.  Never more tasks than pairs: an
 // empty one would count among the arrivals of a row tile that it does not contribute to.  (Layers of unlike widths: parts for the
@@ -1087,7 +1088,7 @@ Plan stream_plan(int n_layers, const int* n_rt, const int* n_ct, int K, bool deq
     }
     if (most_cs > RABIT_LUT_MAX_SLICES || pairs >= kMaxPairs || sms > kMaxTasks || !fill_resources(p, K, deq, tail, wide_x)) return best;
     best.clocks = 1e300;
-    const double pair = kSliceSteps * n_ops * kStreamUnit[n_ops - 1];
+    const double pair = kSliceSteps * (n_ops * kStreamUnit[n_ops - 1] + (deq ? (K - 1) * kStreamDeq : 0.0));
     int considered = 0;
     stream_task_counts(row_tiles, pairs, most_cs, sms, [&](long long tasks) {
         if (candidate >= 0 && considered++ != candidate) return;

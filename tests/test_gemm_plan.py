@@ -125,6 +125,12 @@ def test_what_the_estimates_choose_up_to_16_rows(K, M, N, tasks):
     assert plan([(M, N)], K, 16).tasks == tasks
 
 
+@pytest.mark.parametrize("K,M,N,tasks", [(2, 700, 1024, 24), (2, 3000, 1024, 96)])
+def test_what_they_choose_for_the_dequantised_form(K, M, N, tasks):
+    """Its units take longer with every path: with those of one path such layers were not split, 700 x 1024 4.6 -> 5.7 us and 3000 x 1024 5.0 -> 5.75."""
+    assert plan([(M, N)], K, 16, deq=1).tasks == tasks
+
+
 @pytest.mark.parametrize("stream", [0, 1])
 def test_nobody_waits_for_a_phase_further_off_than_the_next(stream):
     """A wait by parity cannot tell a phase from the one two before it, so a warp that waits for a barrier must wait for every phase
